@@ -415,9 +415,10 @@ int cr_checkpoint(cr_ctx *ctx, cr_state_view *out, cr_counters *counters);
 int cr_restore(cr_ctx *ctx, int32_t n, const float *xyz, const float *vel, const float *force, const uint64_t *id,
                const int32_t *type, const int32_t *cls, const int8_t *state, const cr_counters *counters);
 
-/* Launch shape of the colour-phase kernel: threads per domain and halo
- * particles held in registers per thread.  Supported pairs: (32|64|128|256|512,
- * 0) halo in shared memory; (128, 4), (256, 2), (512, 1) halo in registers.
+/* Launch shape of the colour-phase kernel: threads per domain.  Supported
+ * pairs: (32|64|128|256|512, 0); (128, 4), (256, 2) and (512, 1), which name
+ * halo particles held in registers per thread, run the shape of that many
+ * threads (every shape keeps its halo in shared memory).
  * By default the first unlogged sweeps time every supported shape (with full
  * and with compact shared-memory capacities) in two passes, one shape per
  * sweep, and keep the shape with the shortest time; the

@@ -26,10 +26,10 @@ struct cr_ctx {
   int device = 0;
   cudaStream_t stream = nullptr;
   SysParams P{};
-  // schedule / launch shape: (threads per CTA, halo registers per thread) of
-  // the phase kernel, chosen by timing real sweeps (the chain does not depend
-  // on it: the energy sums are exact fixed point)
-  int T = 128, R = 4;
+  // schedule / launch shape: (threads per CTA, groups) of the phase kernel,
+  // chosen by timing real sweeps (the chain does not depend on it: the energy
+  // sums are exact fixed point); regs: as given to cr_set_launch_shape
+  int T = 128, W = 1, regs = 0;
   int smem_max = 0;
   int tune_next = 0;     // sweeps timed so far (TUNE_ROUNDS passes over the candidates)
   bool tuning = true;
@@ -59,7 +59,8 @@ struct cr_ctx {
   float4 *d_gs_pos = nullptr, *d_gs_vel = nullptr;
   unsigned long long *d_gs_id = nullptr;
   long long *d_gs_lnk = nullptr;
-  int *d_gs_info = nullptr, *d_gs_rank = nullptr;
+  int *d_gs_info = nullptr;
+  uint2 *d_gs_ord = nullptr;
   int *d_plist = nullptr, *d_nparts = nullptr;  // MD particle list
   long long *d_fsum = nullptr;                    // MD pair-force sums per slot
   int *d_order = nullptr;                       // launch order of the domains of each colour
@@ -70,7 +71,7 @@ struct cr_ctx {
   cr_trial_da *d_dlog = nullptr;
   float *d_feat = nullptr;
   size_t dlog_cap = 0, feat_cap = 0;
-  int da_T = 128, da_R = 0, da_next = 0;
+  int da_T = 128, da_W = 1, da_next = 0;
   bool da_tuning = true;
   float da_ms[8] = {};
   // cr_load inputs (capacity-sized)
@@ -213,7 +214,7 @@ static void free_ctx(cr_ctx *c) {
                   c->d_in_id, c->d_in_frc, c->d_present, c->d_ion_key, c->d_ion_key2, c->d_ion_val, c->d_ion_val2, c->d_ion_rank, c->d_sort_tmp,
                   c->d_out_xyz, c->d_out_vel, c->d_out_frc, c->d_out_id, c->d_out_type, c->d_out_cls,
                   c->d_out_state, c->d_out_site,
-                  c->d_reps, c->d_gs_pos, c->d_gs_vel, c->d_gs_id, c->d_gs_lnk, c->d_gs_info, c->d_gs_rank,
+                  c->d_reps, c->d_gs_pos, c->d_gs_vel, c->d_gs_id, c->d_gs_lnk, c->d_gs_info, c->d_gs_ord,
                   c->d_plist, c->d_nparts, c->d_fsum, c->d_mlp_w, c->d_mlp_b, c->d_dlog, c->d_feat, c->d_order,
                   c->d_ek_nA, c->d_ek_Shi, c->d_ek_Slo, c->d_ek_list, c->d_ek_np,
                   c->d_bodies, c->d_body_member, c->d_body_d, c->d_body_df, c->d_body_newpos};
@@ -575,9 +576,7 @@ extern "C" int cr_init(cr_ctx **out, const cr_system *sys, double pH, const doub
         }
   }
   {
-    // starting shape before tuning: 128 threads, enough registers for the densest halo
-    c->T = 128;
-    c->R = 0;  // halo in shared memory until the tuner has timed the shapes
+    // 128 threads until the tuner has timed the shapes
     c->tuning = std::getenv("CRMC_NO_TUNE") == nullptr;
     c->da_tuning = c->tuning;
   }
@@ -603,12 +602,12 @@ extern "C" int cr_init(cr_ctx **out, const cr_system *sys, double pH, const doub
   S.dcs = std::min(P.dcap_glob, S.dcs);
   S.hcs = sys->halo_capacity > 0 ? sys->halo_capacity : std::min(maxh + maxh / 4 + 32, 4096);
   S.lns = std::min(P.lnmax, S.dcs + 4);
-  while (phase_smem_bytes(S, 512, false) > (size_t)smem_max / 2 && S.dcs > 64) {
+  while (phase_smem_bytes(S, 512, 1, false) > (size_t)smem_max / 2 && S.dcs > 64) {
     S.dcs /= 2;
     S.hcs = std::max(S.hcs / 2, 64);
     S.lns = std::min(P.lnmax, S.dcs + 4);
   }
-  if (phase_smem_bytes(S, 512, false) > (size_t)smem_max) { free_ctx(c); return CR_ERR_INVALID_ARG; }
+  if (phase_smem_bytes(S, 512, 1, false) > (size_t)smem_max) { free_ctx(c); return CR_ERR_INVALID_ARG; }
   {
     auto pct90 = [](std::vector<int> v) {
       if (v.empty()) return 0;
@@ -699,7 +698,7 @@ extern "C" int cr_init(cr_ctx **out, const cr_system *sys, double pH, const doub
     ALLOC(c->d_gs_id, ng);
     ALLOC(c->d_gs_lnk, ng);
     ALLOC(c->d_gs_info, ng);
-    ALLOC(c->d_gs_rank, ng);
+    ALLOC(c->d_gs_ord, ng);
   }
   ALLOC(c->d_reps, 1);
   ALLOC(c->d_plist, (size_t)std::max(sys->capacity, 1));
@@ -769,7 +768,7 @@ extern "C" int cr_init(cr_ctx **out, const cr_system *sys, double pH, const doub
   P.gs_id = c->d_gs_id;
   P.gs_lnk = c->d_gs_lnk;
   P.gs_info = c->d_gs_info;
-  P.gs_rank = c->d_gs_rank;
+  P.gs_ord = c->d_gs_ord;
   P.ek_nA = c->d_ek_nA;
   P.ek_Shi = c->d_ek_Shi;
   P.ek_Slo = c->d_ek_Slo;
@@ -972,7 +971,7 @@ static int grow(TT **p, size_t *cap, size_t n) {
 constexpr int TUNE_ROUNDS = 2;
 
 struct TuneRef {
-  int &T, &R, &next;
+  int &T, &W, &next;
   bool &on;
   float *ms;
   bool &C;  // the chosen shape uses the compact capacities
@@ -990,7 +989,7 @@ static void tune_skip(TuneRef t, const PhaseShape &S, const PhaseShape &Sc, int 
     int t_, r_;
     phase_shape(c % nshape, &t_, &r_, da);
     const PhaseShape &Q = phase_shape_compact(c % nshape, da) ? Sc : S;
-    if (phase_shape_smem(Q, t_, r_, da) <= (size_t)smem_max) break;
+    if (phase_smem_bytes(Q, t_, r_, da) <= (size_t)smem_max) break;
     t.ms[c] = 1e30f;
     t.next++;
   }
@@ -1006,7 +1005,7 @@ static void tune_finish(TuneRef t, float ms, const PhaseShape &S, const PhaseSha
     int best = 0;
     for (int i = 1; i < tune_count(t, da); ++i)
       if (t.ms[i] < t.ms[best]) best = i;
-    phase_shape(best % nshape, &t.T, &t.R, da);
+    phase_shape(best % nshape, &t.T, &t.W, da);
     t.C = phase_shape_compact(best % nshape, da);
     if (t.pers) *t.pers = best >= nshape;
     t.on = false;
@@ -1040,18 +1039,18 @@ static int sweep_impl(cr_ctx *ctx, uint64_t n_trials, uint64_t seed, cr_sweep_st
   if (log) CR_CUDA(cudaMemcpyAsync(ctx->d_reps, &P, sizeof(SysParams), cudaMemcpyHostToDevice, s));
   const uint64_t n_sweeps = n_trials / (uint64_t)ctx->per_sweep;
   const uint32_t sweep0 = (uint32_t)ctx->sweep;
-  TuneRef tr = da ? TuneRef{ctx->da_T, ctx->da_R, ctx->da_next, ctx->da_tuning, ctx->da_ms, ctx->da_C}
-                  : TuneRef{ctx->T, ctx->R, ctx->tune_next, ctx->tuning, ctx->tune_ms, ctx->C};
+  TuneRef tr = da ? TuneRef{ctx->da_T, ctx->da_W, ctx->da_next, ctx->da_tuning, ctx->da_ms, ctx->da_C}
+                  : TuneRef{ctx->T, ctx->W, ctx->tune_next, ctx->tuning, ctx->tune_ms, ctx->C};
   for (uint64_t sw = 0; sw < n_sweeps; ++sw) {
     const uint32_t swc = (uint32_t)ctx->sweep++;
     if (!log) tune_skip(tr, ctx->S, ctx->Sc, ctx->smem_max, da);
     const bool tune = tr.on && !log && tr.next < tune_total(tr, da);
-    int T = tr.T, R = tr.R;
+    int T = tr.T, W = tr.W;
     const bool compact = tune ? phase_shape_compact(tune_cand(tr, da), da) : tr.C;
     const PhaseShape &SS = compact ? ctx->Sc : ctx->S;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (tune) {
-      phase_shape(tune_cand(tr, da), &T, &R, da);
+      phase_shape(tune_cand(tr, da), &T, &W, da);
       cudaEventCreate(&e0);
       cudaEventCreate(&e1);
       cudaEventRecord(e0, s);
@@ -1067,7 +1066,7 @@ static int sweep_impl(cr_ctx *ctx, uint64_t n_trials, uint64_t seed, cr_sweep_st
     for (int col = 0; col < P.ncol; ++col) {
       int ti;
       tbegin(ctx, 0, &ti);
-      CR_CUDA(launch_phase(ctx->d_reps, 1, P.nact, SS, T, R, log != nullptr, da, s, swc, sweep0, col, k0, k1));
+      CR_CUDA(launch_phase(ctx->d_reps, 1, P.nact, SS, T, W, log != nullptr, da, s, swc, sweep0, col, k0, k1));
       tend(ctx, 0, ti);
       ctx->launches_total++;
     }
@@ -1147,7 +1146,7 @@ extern "C" int cr_set_surrogate(cr_ctx *ctx, const cr_mlp *m) {
   for (int i = 0; i < phase_shape_count(true); ++i) {
     int t, r;
     phase_shape(i, &t, &r, true);
-    smem_ok |= phase_shape_smem(ctx->S, t, r, true) <= (size_t)ctx->smem_max;
+    smem_ok |= phase_smem_bytes(ctx->S, t, r, true) <= (size_t)ctx->smem_max;
   }
   if (!smem_ok) return CR_ERR_INVALID_ARG;
   // transposed BF16 weights (WT[in][out]) and the biases
@@ -1665,40 +1664,33 @@ extern "C" int cr_set_launch_shape(cr_ctx *ctx, int32_t threads, int32_t regs) {
   if (threads == 0) {  // re-enable tuning
     ctx->tuning = true;
     ctx->tune_next = 0;
+    ctx->regs = 0;
     ctx->da_tuning = true;
     ctx->da_next = 0;
     return CR_OK;
   }
-  bool found = false;
-  for (int i = 0; i < phase_shape_count(false); ++i) {
-    int t, r;
-    phase_shape(i, &t, &r, false);
-    if (t == threads && r == regs) {
-      ctx->T = t;
-      ctx->R = r;
-      ctx->C = false;
-      ctx->tuning = false;
-      found = true;
-    }
+  int w, wd;
+  const bool plain = phase_shape_named(threads, regs, false, &w), da = phase_shape_named(threads, regs, true, &wd);
+  if (plain) {
+    ctx->T = threads;
+    ctx->W = w;
+    ctx->regs = regs;
+    ctx->C = false;
+    ctx->tuning = false;
   }
-  for (int i = 0; i < phase_shape_count(true); ++i) {  // delayed-acceptance sweeps, where supported
-    int t, r;
-    phase_shape(i, &t, &r, true);
-    if (t == threads && r == regs) {
-      ctx->da_T = t;
-      ctx->da_R = r;
-      ctx->da_C = false;
-      ctx->da_tuning = false;
-      found = true;
-    }
+  if (da) {  // delayed-acceptance sweeps, where supported
+    ctx->da_T = threads;
+    ctx->da_W = wd;
+    ctx->da_C = false;
+    ctx->da_tuning = false;
   }
-  return found ? CR_OK : CR_ERR_INVALID_ARG;
+  return plain || da ? CR_OK : CR_ERR_INVALID_ARG;
 }
 
 extern "C" int cr_get_launch_shape(const cr_ctx *ctx, int32_t *threads, int32_t *regs) {
   if (!ctx || !threads || !regs) return CR_ERR_INVALID_ARG;
   *threads = ctx->T;
-  *regs = ctx->R;
+  *regs = ctx->regs;
   return CR_OK;
 }
 
@@ -1728,7 +1720,7 @@ struct cr_batch {
   cudaStream_t cstream = nullptr;  // capture stream
   cudaGraphExec_t graph = nullptr;
   double g_dt = 0.0, g_gamma = 0.0;
-  int g_T = 0, g_R = 0, g_da = -1;
+  int g_T = 0, g_W = 0, g_da = -1;
   bool g_C = false, g_pers = false, g_fine = false, g_timing = false;
   bool g_ff = false;  // the graph's step evaluates the forces first (a step after a load)
   int64_t g_kernels = 0;                      // kernels per graph launch
@@ -1737,12 +1729,12 @@ struct cr_batch {
   PhaseShape S{}, Sc{};
   bool C = false, da_C = false;
   int grid_x = 0, ncol = 8;
-  int T = 128, R = 4;
+  int T = 128, W = 1, regs = 0;
   int smem_max = 0;
   bool tuning = true;
   int tune_next = 0;
   float tune_ms[32] = {};
-  int da_T = 128, da_R = 0, da_next = 0;
+  int da_T = 128, da_W = 1, da_next = 0;
   bool da_tuning = true;
   float da_ms[16] = {};
   std::vector<SysParams> reps;  // host copy of d_reps
@@ -1833,7 +1825,6 @@ extern "C" int cr_batch_create(cr_batch **out, cr_ctx *const *ctxs, int32_t n) {
   b->ctx.assign(ctxs, ctxs + n);
   for (int r = 0; r < n; ++r) b->chem_seen.push_back(ctxs[r] ? ctxs[r]->chem_version : 0);
   std::vector<SysParams> reps(n);
-  int maxR = 1;
   for (int r = 0; r < n; ++r) {
     cr_ctx *c = ctxs[r];
     if (!c || c->P.ncol != ctxs[0]->P.ncol || c->sweep != ctxs[0]->sweep || c->stream != ctxs[0]->stream ||
@@ -1860,12 +1851,9 @@ extern "C" int cr_batch_create(cr_batch **out, cr_ctx *const *ctxs, int32_t n) {
     b->Sc.chunk = std::max(b->Sc.chunk, c->Sc.chunk);
     b->Sc.ewk = std::max(b->Sc.ewk, c->Sc.ewk);
     b->grid_x = std::max(b->grid_x, c->P.nact);
-    maxR = std::max(maxR, c->R);
   }
   b->ncol = ctxs[0]->P.ncol;
   b->stream = ctxs[0]->stream;
-  b->R = 0;
-  (void)maxR;
   b->tuning = std::getenv("CRMC_NO_TUNE") == nullptr;
   b->da_tuning = b->tuning;
   b->reps = reps;
@@ -1876,7 +1864,7 @@ extern "C" int cr_batch_create(cr_batch **out, cr_ctx *const *ctxs, int32_t n) {
     }
   int smem_max = 0;
   cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctxs[0]->device);
-  if (phase_smem_bytes(b->S, 512, false) > (size_t)smem_max) { delete b; return CR_ERR_INVALID_ARG; }
+  if (phase_smem_bytes(b->S, 512, 1, false) > (size_t)smem_max) { delete b; return CR_ERR_INVALID_ARG; }
   b->smem_max = smem_max;
   cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, ctxs[0]->device);
   if (cudaMalloc((void **)&b->d_reps, sizeof(SysParams) * n) != cudaSuccess) { delete b; return CR_ERR_NOMEM; }
@@ -1953,7 +1941,7 @@ extern "C" void cr_batch_destroy(cr_batch *b) {
 static int batch_refresh_chem(cr_batch *b);
 
 // one persistent sweep launch of every replica (words zeroed first)
-static int batch_launch_persistent(cr_batch *b, const PhaseShape &SS, int T, int R, bool da, uint32_t swc,
+static int batch_launch_persistent(cr_batch *b, const PhaseShape &SS, int T, int W, bool da, uint32_t swc,
                                    uint32_t sweep0, uint32_t k0, uint32_t k1, int withhold = -1,
                                    unsigned long long wait_ns = 2000000000ull, const StepDyn *dyn = nullptr) {
   cr_ctx *c0 = b->ctx[0];
@@ -1975,7 +1963,7 @@ static int batch_launch_persistent(cr_batch *b, const PhaseShape &SS, int T, int
   int ti;
   tbegin(c0, 0, &ti);
   const int sms = b->sms > 0 ? b->sms : 1;
-  CR_CUDA(launch_sweep(b->d_reps, SS, T, R, da, s, swc, sweep0, k0, k1, Q, b->ctas_per_sm * sms, dyn));
+  CR_CUDA(launch_sweep(b->d_reps, SS, T, W, da, s, swc, sweep0, k0, k1, Q, b->ctas_per_sm * sms, dyn));
   tend(c0, 0, ti);
   c0->launches_total++;
   return CR_OK;
@@ -2007,8 +1995,8 @@ static int batch_sweep_impl(cr_batch *b, uint64_t n_sweeps, uint64_t seed, bool 
   const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
   const uint32_t sweep0 = (uint32_t)c0->sweep;
   bool &pers_choice = da ? b->da_persistent : b->persistent;
-  TuneRef tr = da ? TuneRef{b->da_T, b->da_R, b->da_next, b->da_tuning, b->da_ms, b->da_C}
-                  : TuneRef{b->T, b->R, b->tune_next, b->tuning, b->tune_ms, b->C};
+  TuneRef tr = da ? TuneRef{b->da_T, b->da_W, b->da_next, b->da_tuning, b->da_ms, b->da_C}
+                  : TuneRef{b->T, b->W, b->tune_next, b->tuning, b->tune_ms, b->C};
   if (b->pmode < 0) tr.pers = &pers_choice;
   else pers_choice = b->pmode != 0;
   const int nshape = phase_shape_count(da);
@@ -2021,14 +2009,14 @@ static int batch_sweep_impl(cr_batch *b, uint64_t n_sweeps, uint64_t seed, bool 
     }
     tune_skip(tr, b->S, b->Sc, b->smem_max, da);
     const bool tune = tr.on && tr.next < tune_total(tr, da);
-    int T = tr.T, R = tr.R;
+    int T = tr.T, W = tr.W;
     bool persistent = pers_choice;
     const int cand = tune ? tune_cand(tr, da) : 0;
     const bool compact = tune ? phase_shape_compact(cand % nshape, da) : tr.C;
     const PhaseShape &SS = compact ? b->Sc : b->S;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (tune) {
-      phase_shape(cand % nshape, &T, &R, da);
+      phase_shape(cand % nshape, &T, &W, da);
       if (tr.pers) persistent = cand >= nshape;
       cudaEventCreate(&e0);
       cudaEventCreate(&e1);
@@ -2043,13 +2031,13 @@ static int batch_sweep_impl(cr_batch *b, uint64_t n_sweeps, uint64_t seed, bool 
       c0->launches_total += 2;
     }
     if (persistent) {
-      const int rc = batch_launch_persistent(b, SS, T, R, da, swc, sweep0, k0, k1);
+      const int rc = batch_launch_persistent(b, SS, T, W, da, swc, sweep0, k0, k1);
       if (rc != CR_OK) return rc;
     } else {
       for (int col = 0; col < b->ncol; ++col) {
         int ti;
         tbegin(c0, 0, &ti);
-        CR_CUDA(launch_phase(b->d_reps, n, b->grid_x, SS, T, R, false, da, s, swc, sweep0, col, k0, k1));
+        CR_CUDA(launch_phase(b->d_reps, n, b->grid_x, SS, T, W, false, da, s, swc, sweep0, col, k0, k1));
         tend(c0, 0, ti);
         c0->launches_total++;
       }
@@ -2090,17 +2078,17 @@ extern "C" int cr_batch_selftest_wait_timeout(cr_batch *b, int32_t replica, doub
     c->f_valid = false;
     c->fcons_valid = false;
   }
-  int T = b->T, R = b->R;
+  int T = b->T, W = b->W;
   const PhaseShape &SS = b->C ? b->Sc : b->S;
   if (b->tuning) {  // a shape every context supports
     T = 128;
-    R = 0;
+    W = 1;
   }
   if (b->order_nc > 0) {
     CR_CUDA(launch_domain_order(b->d_reps, (int)b->ctx.size(), b->ncol, b->order_nact, c0->stream, swc, 1u, 0u));
     c0->launches_total++;
   }
-  const int rc = batch_launch_persistent(b, b->tuning ? b->S : SS, T, R, false, swc, swc, 1u, 0u, replica,
+  const int rc = batch_launch_persistent(b, b->tuning ? b->S : SS, T, W, false, swc, swc, 1u, 0u, replica,
                                          (unsigned long long)(timeout_ms * 1e6));
   if (rc != CR_OK) return rc;
   CR_CUDA(cudaStreamSynchronize(c0->stream));
@@ -2211,7 +2199,7 @@ static int batch_capture_cycle(cr_batch *b, double dt, double gamma, bool da, bo
     launches[r] = b->ctx[r]->launches_total;
     fvalid[r] = b->ctx[r]->f_valid ? 1 : 0;
   }
-  const int T = da ? b->da_T : b->T, R = da ? b->da_R : b->R;
+  const int T = da ? b->da_T : b->T, W = da ? b->da_W : b->W;
   const bool C = da ? b->da_C : b->C, pers = da ? b->da_persistent : b->persistent;
   const PhaseShape &SS = C ? b->Sc : b->S;
   const StepDyn *dyn = b->d_dyn;
@@ -2237,12 +2225,12 @@ static int batch_capture_cycle(cr_batch *b, double dt, double gamma, bool da, bo
     }
     if (rc == CR_OK) {
       if (pers) {
-        rc = batch_launch_persistent(b, SS, T, R, da, 0, 0, 0, 0, -1, 2000000000ull, dyn);
+        rc = batch_launch_persistent(b, SS, T, W, da, 0, 0, 0, 0, -1, 2000000000ull, dyn);
       } else {
         for (int col = 0; col < b->ncol && rc == CR_OK; ++col) {
           int ti;
           tbegin(c0, 0, &ti);
-          if (launch_phase(b->d_reps, n, b->grid_x, SS, T, R, false, da, s, 0, 0, col, 0, 0, dyn) != cudaSuccess)
+          if (launch_phase(b->d_reps, n, b->grid_x, SS, T, W, false, da, s, 0, 0, col, 0, 0, dyn) != cudaSuccess)
             rc = CR_ERR_CUDA;
           tend(c0, 0, ti);
           c0->launches_total++;
@@ -2284,7 +2272,7 @@ static int batch_capture_cycle(cr_batch *b, double dt, double gamma, bool da, bo
   b->g_dt = dt;
   b->g_gamma = gamma;
   b->g_T = T;
-  b->g_R = R;
+  b->g_W = W;
   b->g_C = C;
   b->g_pers = pers;
   b->g_fine = b->fine;
@@ -2337,11 +2325,11 @@ extern "C" int cr_batch_cycle(cr_batch *b, int32_t n_steps, double dt, double ga
       CR_CUDA(cudaMemcpyAsync(b->d_reps, b->reps.data(), sizeof(SysParams) * b->ctx.size(), cudaMemcpyHostToDevice, s));
   }
   if (!b->d_dyn) CR_CUDA(cudaMalloc((void **)&b->d_dyn, sizeof(StepDyn)));
-  const int T = da ? b->da_T : b->T, R = da ? b->da_R : b->R;
+  const int T = da ? b->da_T : b->T, W = da ? b->da_W : b->W;
   const bool C = da ? b->da_C : b->C, pers = da ? b->da_persistent : b->persistent;
   while (step < n_steps) {
     const bool first = ff && step == 0;  // only a call's first step can have stale forces
-    if (!b->graph || b->g_dt != dt || b->g_gamma != gamma || b->g_T != T || b->g_R != R || b->g_C != C ||
+    if (!b->graph || b->g_dt != dt || b->g_gamma != gamma || b->g_T != T || b->g_W != W || b->g_C != C ||
         b->g_pers != pers || b->g_fine != b->fine || b->g_da != (da ? 1 : 0) || b->g_timing != c0->timing ||
         b->g_ff != first) {
       if ((rc = batch_capture_cycle(b, dt, gamma, da != 0, first)) != CR_OK) return rc;
@@ -2549,36 +2537,36 @@ extern "C" int cr_batch_set_launch_shape(cr_batch *b, int32_t threads, int32_t r
   if (!b) return CR_ERR_INVALID_ARG;
   if (threads == 0) {  // re-enable tuning
     b->tuning = b->da_tuning = true;
+    b->regs = 0;
     b->tune_next = b->da_next = 0;
     return CR_OK;
   }
   if (b->pmode < 0) b->persistent = b->da_persistent = false;  // a fixed shape without a fixed mode: per colour
-  bool found = false;
-  for (int da = 0; da < 2; ++da)
-    for (int i = 0; i < phase_shape_count(da != 0); ++i) {
-      int t, r;
-      phase_shape(i, &t, &r, da != 0);
-      if (t != threads || r != regs || phase_shape_smem(b->S, t, r, da != 0) > (size_t)b->smem_max) continue;
-      if (da) {
-        b->da_T = t;
-        b->da_R = r;
-        b->da_C = false;
-        b->da_tuning = false;
-      } else {
-        b->T = t;
-        b->R = r;
-        b->C = false;
-        b->tuning = false;
-      }
-      found = true;
-    }
-  return found ? CR_OK : CR_ERR_INVALID_ARG;
+  int w, wd;
+  const bool plain = phase_shape_named(threads, regs, false, &w) &&
+                     phase_smem_bytes(b->S, threads, w, false) <= (size_t)b->smem_max;
+  const bool da = phase_shape_named(threads, regs, true, &wd) &&
+                  phase_smem_bytes(b->S, threads, wd, true) <= (size_t)b->smem_max;
+  if (plain) {
+    b->T = threads;
+    b->W = w;
+    b->regs = regs;
+    b->C = false;
+    b->tuning = false;
+  }
+  if (da) {
+    b->da_T = threads;
+    b->da_W = wd;
+    b->da_C = false;
+    b->da_tuning = false;
+  }
+  return plain || da ? CR_OK : CR_ERR_INVALID_ARG;
 }
 
 extern "C" int cr_batch_get_launch_shape(const cr_batch *b, int32_t *threads, int32_t *regs) {
   if (!b || !threads || !regs) return CR_ERR_INVALID_ARG;
   *threads = b->T;
-  *regs = b->R;
+  *regs = b->regs;
   return CR_OK;
 }
 

@@ -9,6 +9,8 @@
 //   vel, frc[ncell * cap]      MD velocity and total force (float4)
 // A cell's particles occupy slots [c*cap, c*cap + cnt[c]) in ascending id.
 #pragma once
+#include <cuda_runtime.h>
+
 #include <cstdint>
 
 #include "crmc.h"
@@ -55,7 +57,7 @@ struct WcaEntry {
 // Everything a phase (or MD) kernel needs about one system (one replica).
 // The phase kernel reads it from a device array (one entry per replica);
 // the MD kernels take it by value.
-struct SysParams {
+struct alignas(16) SysParams {
   // geometry
   int nc, k, h, nd, ncol, m, cap, global, nr, ncell;
   int nact;             // active domains per colour phase
@@ -92,7 +94,8 @@ struct SysParams {
   float4 *gs_pos, *gs_vel;
   unsigned long long *gs_id;
   long long *gs_lnk;
-  int *gs_info, *gs_rank;
+  int *gs_info;
+  uint2 *gs_ord;
   int dcap_glob;        // entries per CTA region (k^3 * cap + 2 m)
   // bookkeeping
   unsigned long long *stats;  // [16]: attempts[6], accepts[6], no-elig, edge, overlap, trials
@@ -140,12 +143,14 @@ constexpr int MLPB_N = 3 * MLP_H + 1;
 // the maximum over the replicas of a batch).
 struct PhaseShape {
   int dcs;     // domain-list entries held in shared memory
-  int hcs;     // halo particles held in shared memory (shapes without halo registers)
+  int hcs;     // halo particles held in shared memory
   int lns;     // log-table entries held in shared memory
   int nr3;     // region cells
   int kc3;     // domain cells
   int chunk;   // trials whose random numbers are drawn at once (min(m, TRIAL_CHUNK))
   int ewk;     // Ewald: kmax + 1 phase factors per axis and changed particle (0 without Ewald)
+  static constexpr int N_OFF = 33;
+  unsigned off[N_OFF];  // byte offsets of the CTA's shared arrays (filled for each launch form)
 };
 
 // error bits in *err

@@ -6,18 +6,20 @@
 // the order k_domain_order computes at the start of every sweep), so that the
 // long CTAs do not form the tail of the launch.
 // The CTA
-//   1. stages the domain's particles into a list kept in canonical order
-//      (in-domain cell rank, then id) -- in shared memory, or in a global
-//      scratch region when the domain is unusually dense -- and the halo
-//      particles around it into registers (they do not change in the phase);
+//   1. stages the domain's particles into a list -- in shared memory, or in a
+//      global scratch region when the domain is unusually dense -- with its
+//      canonical order (in-domain cell rank, then id) as a list of slots, and
+//      the halo particles around it into shared memory (they do not change in
+//      the phase);
 //   2. draws the phase's random numbers for a chunk of trials at once
 //      (Philox4x32-10, counter (trial, domain, phase, purpose));
 //   3. runs the m trials of the domain one after another: warp 0 selects the
-//      participants (ballot scans of the list); every thread sums its share of
+//      participants (ballot scans of the order); every thread sums its share of
 //      the pair changes -- FP32 Coulomb, FP64 WCA of inserted/deleted ions --
 //      into 64-bit fixed point, exact and therefore independent of the thread
-//      count; warp 0 takes the FP64 Metropolis decision and commits the move;
-//   4. writes the domain's cells back (id-sorted) and adds its count changes.
+//      count; warp 0 takes the Metropolis decision and commits the move;
+//   4. writes the domain's cells back (id-sorted), if a trial was accepted, and
+//      adds its count changes.
 // The move rules are those of Sec. II.C of the paper applied to the domain
 // (the domain's volume and counts).
 #include <cuda_runtime.h>
@@ -32,8 +34,6 @@
 namespace crmc {
 
 namespace {
-
-constexpr int MAX_WARPS = 16;  // up to 512 threads per CTA
 
 struct TrialPre {
   uint32_t w0, w1, w2, w3;  // move, site choice, first ion, second ion
@@ -52,7 +52,7 @@ struct TrialPre {
 
 struct Desc {
   float x, y, z, dqlB;  // position, lB * (q_new - q_old)
-  int dp, cls, skip;    // WCA presence change, class, list index (-1 inserted)
+  int dp, cls, skip;    // WCA presence change, class, list slot (-1 inserted)
 };
 
 struct TrialCtl {
@@ -60,7 +60,7 @@ struct TrialCtl {
   int nch;    // changed particles needing the energy sweep (0 = decided)
   int flags;  // CR_TRIAL_* bits known before the sweep
   int move;
-  int site, ionA, ionB;  // list indices (-1 none)
+  int site, ionA, ionB;  // places in the canonical order (-1 none)
   unsigned long long id_a, id_b, newid;
   long long ln_ratio_fx, dself_fx;  // 2^-48 fixed point
   float qa_o, qa_n, qb_o, qb_n;  // effective charges of the two changed particles
@@ -73,18 +73,38 @@ struct TrialCtl {
   long long sur_fx;      // dE~ clamped, 2^-48 fixed point (DA)
 };
 
+// The domain's particles.  A particle keeps its slot of the payload arrays
+// while it lives; `ord` holds the canonical order (in-domain cell rank, then
+// id) as (slot | kind << ORD_KIND_SHIFT, cell rank), so an insertion or
+// deletion moves 8 bytes per entry instead of the 56 of the payload: under the
+// global schedule (a list of about 1,250, five trials in six accepted) moving
+// the payload by one warp was a third of a trial, and finding the k-th of a
+// kind 32 entries at a time another fifth (500 trials in each of 128 boxes:
+// 5.96 ms before, 3.21 ms with the order list and 256 entries per scan round).
+// pos is in the region's flat frame (frame_x).  A deleted particle's slot goes to a
+// free list threaded through its info word; its charge is 0 and its class
+// CR_CLS_NONE, so the pair sweep passes over it without a test.
 struct DomList {
   float4 *pos, *vel;
   unsigned long long *id;
   long long *lnk;  // site constant ln10 (pH - pK - pI_X) at 2^-48, 0 for non-sites
-  int *info, *rank;
+  int *info;
+  uint2 *ord;
 };
+constexpr int ORD_KIND_SHIFT = 28;
+constexpr unsigned ORD_SLOT_MASK = (1u << ORD_KIND_SHIFT) - 1u;
+// info word of a free slot: no type, class CR_CLS_NONE, the next free slot + 1
+constexpr int INFO_FREE = 15 | (CR_CLS_NONE << INFO_CLS_SHIFT);
+// a phase's counters beyond the kind counts (misc)
+constexpr int MISC_HW = MISC_N, MISC_FREE = MISC_N + 1, MISC_DIRTY = MISC_N + 2, MISC_TOTAL = MISC_N + 4;
 
 // FP32 constants of the pair sweep, kept in registers
 struct PairK {
-  float Lf, halfL, rc2, alpha, c1, c2, rcf, lBf;
-  double Ld, halfLd;
+  float Lf, halfL, rc2, alpha, c1, c2, rcf;
 };
+__device__ __forceinline__ PairK pair_k(const SysParams &P) {
+  return PairK{P.Lf, P.halfL, P.rc2, P.alpha, P.c1, P.c2, P.rcf};
+}
 
 __device__ __forceinline__ int region_coord(int i, int org, int k, int h, int nr, int nc) {
   int c = (i < k + h) ? org + i : org + i - nr;
@@ -93,11 +113,12 @@ __device__ __forceinline__ int region_coord(int i, int org, int k, int h, int nr
   return c;
 }
 
-// Exclusive scan of n ints (shared memory) into pre[0..n]; all threads call.
-__device__ void block_scan(const int *vals, int n, int *pre, int *tmp) {
-  const int T = blockDim.x, t = threadIdx.x, lane = t & 31, w = t >> 5, nw = T >> 5;
-  const int per = (n + T - 1) / T;
-  const int lo = min(n, t * per), hi = min(n, lo + per);
+// Exclusive scan of n ints (shared memory) into pre[0..n] by one warp, each
+// lane a run of consecutive entries
+__device__ __forceinline__ void warp_scan(const int *vals, int n, int *pre) {
+  const int lane = threadIdx.x & 31;
+  const int per = (n + 31) >> 5;
+  const int lo = min(n, lane * per), hi = min(n, lo + per);
   int s = 0;
   for (int i = lo; i < hi; ++i) s += vals[i];
   int x = s;
@@ -106,25 +127,12 @@ __device__ void block_scan(const int *vals, int n, int *pre, int *tmp) {
     const int y = __shfl_up_sync(0xffffffffu, x, o);
     if (lane >= o) x += y;
   }
-  if (lane == 31) tmp[w] = x;
-  __syncthreads();
-  if (w == 0) {
-    int v = lane < nw ? tmp[lane] : 0;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, v, o);
-      if (lane >= o) v += y;
-    }
-    if (lane < nw) tmp[lane] = v;
-  }
-  __syncthreads();
-  int run = x - s + (w > 0 ? tmp[w - 1] : 0);
+  int run = x - s;
   for (int i = lo; i < hi; ++i) {
     pre[i] = run;
     run += vals[i];
   }
-  if (t == T - 1) pre[n] = run;
-  __syncthreads();
+  if (lane == 31) pre[n] = x;
 }
 
 // largest i with pre[i] <= j (pre ascending, pre[0] = 0, j < pre[n])
@@ -137,17 +145,49 @@ __device__ __forceinline__ int upper_idx(const int *pre, int n, int j) {
   return lo;
 }
 
-// warp: index of the kth (0-based) list entry of a kind, -1 if none
-__device__ __forceinline__ int warp_kth(const int *info, int n, int kind, int kth) {
+// warp: place of the kth (0-based) entry of a kind in the canonical order, -1
+// if none.  Short lists take one ballot; longer ones eight at a time, so that
+// the loads of 256 entries are in flight together.
+__device__ __forceinline__ int warp_kth(const uint2 *ord, int n, int kind, int kth) {
   const int lane = threadIdx.x & 31;
+  const unsigned lt = (1u << lane) - 1u;
   for (int base = 0; base < n; base += 32) {
+    if (n - base > 64) {  // whole 256-entry rounds that end before the kth are skipped together
+      unsigned b[8];
+      int c = 0;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int j = base + 32 * u + lane;
+        const unsigned e = j < n ? ord[j].x >> ORD_KIND_SHIFT : 15u;
+        b[u] = __ballot_sync(0xffffffffu, e == (unsigned)kind);
+      }
+      int found = -1, before = 0;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int cu = __popc(b[u]);
+        if (found < 0 && kth < c + cu) {
+          found = u;
+          before = c;
+        }
+        c += cu;
+      }
+      if (found < 0) {
+        kth -= c;
+        base += 224;
+        continue;
+      }
+      unsigned m = 0u;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) m = u == found ? b[u] : m;
+      const unsigned hit = __ballot_sync(0xffffffffu, ((m >> lane) & 1u) && __popc(m & lt) == kth - before);
+      return base + 32 * found + __ffs(hit) - 1;
+    }
     const int j = base + lane;
-    const bool m = j < n && kind_of(info[j]) == kind;
+    const bool m = j < n && (ord[j].x >> ORD_KIND_SHIFT) == (unsigned)kind;
     const unsigned b = __ballot_sync(0xffffffffu, m);
     const int c = __popc(b);
     if (kth < c) {
-      const unsigned lt = b & ((1u << lane) - 1u);
-      const unsigned hit = __ballot_sync(0xffffffffu, m && __popc(lt) == kth);
+      const unsigned hit = __ballot_sync(0xffffffffu, m && __popc(b & lt) == kth);
       return base + __ffs(hit) - 1;
     }
     kth -= c;
@@ -155,71 +195,53 @@ __device__ __forceinline__ int warp_kth(const int *info, int n, int kind, int kt
   return -1;
 }
 
-// warp: number of entries with rank < r and rank == r (four chunks per round)
-__device__ __forceinline__ void warp_rank_count(const int *rank, int n, int r, int &below, int &same) {
+// warp: number of entries with cell rank < r (the ranks ascend); long lists
+// are narrowed 32-fold per round
+__device__ __forceinline__ int warp_lower(const uint2 *ord, int n, int r) {
   const int lane = threadIdx.x & 31;
-  below = 0;
-  same = 0;
-  for (int base = 0; base < n; base += 128) {
-    int rk[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int j = base + 32 * u + lane;
-      rk[u] = j < n ? rank[j] : INT_MAX;
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      below += __popc(__ballot_sync(0xffffffffu, rk[u] < r));
-      same += __popc(__ballot_sync(0xffffffffu, rk[u] == r));
-    }
+  int base = 0, len = n;
+  while (len > 32) {
+    const int st = (len + 31) >> 5, o = lane * st;
+    const int b = __popc(__ballot_sync(0xffffffffu, o < len && (int)ord[base + o].y < r));
+    if (b == 0) return base;
+    const int skip = (b - 1) * st;
+    base += skip;
+    len = min(st, len - skip);
   }
+  return base + __popc(__ballot_sync(0xffffffffu, lane < len && (int)ord[base + lane].y < r));
 }
 
-// one list entry held in registers while the list shifts
-struct EntryRegs {
-  float4 a, v;
-  unsigned long long b;
-  long long e;
-  int c, d;
-};
-__device__ __forceinline__ EntryRegs entry_load(const DomList &L, int j) {
-  return EntryRegs{L.pos[j], L.vel[j], L.id[j], L.lnk[j], L.info[j], L.rank[j]};
-}
-__device__ __forceinline__ void entry_store(const DomList &L, int j, const EntryRegs &x) {
-  L.pos[j] = x.a; L.vel[j] = x.v; L.id[j] = x.b; L.lnk[j] = x.e; L.info[j] = x.c; L.rank[j] = x.d;
-}
-
-// warp: open a hole at p (entries [p, n) move up by one), 64 entries per
+// warp: open a hole at p (entries [p, n) move up by one), 128 entries per
 // round from the top down: every load of a round before its stores
-__device__ void warp_insert_gap(DomList L, int n, int p) {
+__device__ __forceinline__ void ord_open(uint2 *ord, int n, int p) {
   const int lane = threadIdx.x & 31;
-  for (int hi = n; hi > p; hi -= 64) {
-    const int lo = max(p, hi - 64);
-    const int j0 = lo + lane, j1 = lo + 32 + lane;
-    const bool a0 = j0 < hi, a1 = j1 < hi;
-    EntryRegs x0{}, x1{};
-    if (a0) x0 = entry_load(L, j0);
-    if (a1) x1 = entry_load(L, j1);
+  for (int hi = n; hi > p; hi -= 128) {
+    const int lo = max(p, hi - 128);
+    uint2 x[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (lo + 32 * u + lane < hi) x[u] = ord[lo + 32 * u + lane];
     __syncwarp();
-    if (a0) entry_store(L, j0 + 1, x0);
-    if (a1) entry_store(L, j1 + 1, x1);
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (lo + 32 * u + lane < hi) ord[lo + 32 * u + lane + 1] = x[u];
     __syncwarp();
   }
 }
 
-// warp: remove entry p (entries (p, n) move down by one), 64 entries per
-// round from the bottom up
-__device__ void warp_remove(DomList L, int n, int p) {
+// warp: close place p (entries (p, n) move down by one), 128 per round from
+// the bottom up
+__device__ __forceinline__ void ord_close(uint2 *ord, int n, int p) {
   const int lane = threadIdx.x & 31;
-  for (int lo = p + 1; lo < n; lo += 64) {
-    const int j0 = lo + lane, j1 = lo + 32 + lane;
-    const bool a0 = j0 < n, a1 = j1 < n;
-    EntryRegs x0{}, x1{};
-    if (a0) x0 = entry_load(L, j0);
-    if (a1) x1 = entry_load(L, j1);
+  for (int lo = p + 1; lo < n; lo += 128) {
+    uint2 x[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (lo + 32 * u + lane < n) x[u] = ord[lo + 32 * u + lane];
     __syncwarp();
-    if (a0) entry_store(L, j0 - 1, x0);
-    if (a1) entry_store(L, j1 - 1, x1);
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (lo + 32 * u + lane < n) ord[lo + 32 * u + lane - 1] = x[u];
     __syncwarp();
   }
 }
@@ -228,7 +250,7 @@ __device__ void warp_remove(DomList L, int n, int p) {
 // FP32 and WCA in FP64, into fixed point (without a WCA term the FP64 sum
 // reduces to the FP32 change, taken directly)
 template <bool WITH_S>
-__device__ __forceinline__ void cc_change_impl(const PairK &K, const WcaEntry *wca, const TrialCtl &t, long long &acc,
+__device__ __forceinline__ void cc_change_impl(const SysParams &K, const WcaEntry *wca, const TrialCtl &t, long long &acc,
                                                unsigned long long &sacc, int &ov) {
   const Desc &A = t.c[0], &B = t.c[1];
   const float dx = wrap_diff(B.x, A.x, K.Lf, K.halfL);
@@ -366,8 +388,8 @@ __device__ __forceinline__ int region_of(int r, int dx, int dy, int dz, int k, i
 // input order (weights transposed, WT[k][o], so that a warp's loads coalesce)
 template <int T>
 __device__ __forceinline__ void mlp_layer(const uint16_t *__restrict__ WT, const float *__restrict__ b,
-                                          const float *x, int n_in, float *y) {
-  for (int o = threadIdx.x; o < 2 * MLP_H; o += T) {
+                                          const float *x, int n_in, float *y, int tid) {
+  for (int o = tid; o < 2 * MLP_H; o += T) {
     const int v = o / MLP_H, i = o % MLP_H;
     const float *xv = x + v * n_in;
     float a = __ldg(&b[i]);
@@ -393,22 +415,11 @@ __device__ __forceinline__ void coul_eval(const PairK &K, float r2, float qp, lo
   }
 }
 
-// WCA pre-check radii of a changed particle against the four classes
-// (1.0001 x squared cutoff, or -1 when it is not inserted / deleted or the
-// pair does not interact), kept in registers for the whole trial
-__device__ __forceinline__ float4 wca_radii(const WcaEntry *wca, const Desc &c) {
-  float r[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const WcaEntry &w = wca[c.cls * 4 + j];
-    r[j] = (c.dp != 0 && w.on) ? 1.0001f * w.wcut2 : -1.0f;
-  }
-  return make_float4(r[0], r[1], r[2], r[3]);
-}
-
-__device__ __forceinline__ float sel4(const float4 v, int i) {
-  return i == 0 ? v.x : (i == 1 ? v.y : (i == 2 ? v.z : v.w));
-}
+// WCA pre-check radius of a changed particle of class ci against class cj
+// (1.0001 x squared cutoff, or -1 when the classes do not interact), and the
+// largest over cj: the sweep compares with the latter and looks the former up
+// for the few candidates inside it
+__device__ __forceinline__ float wca_radius(const WcaEntry &w) { return w.on ? 1.0001f * w.wcut2 : -1.0f; }
 
 // A pair within the WCA range of an inserted / deleted changed particle:
 // Coulomb in FP32 and WCA in FP64, evaluated at once (rare).  Not inlined, to
@@ -454,11 +465,8 @@ __device__ __noinline__ PairSum near_pair(const SysParams &P, const WcaEntry &w,
 // line, with its FP64 WCA branch)
 template <bool WITH_S>
 __device__ __noinline__ PairSum cc_change(const SysParams &P, const TrialCtl &t) {
-  PairK K;
-  K.Lf = P.Lf; K.halfL = P.halfL; K.rc2 = P.rc2; K.alpha = P.alpha; K.c1 = P.c1; K.c2 = P.c2; K.rcf = P.rcf;
-  K.lBf = P.lBf; K.Ld = P.Ld; K.halfLd = P.halfLd;
   PairSum out{0, 0ull, 0};
-  cc_change_impl<WITH_S>(K, P.wca, t, out.acc, out.sacc, out.ov);
+  cc_change_impl<WITH_S>(P, P.wca, t, out.acc, out.sacc, out.ov);
   return out;
 }
 
@@ -471,115 +479,130 @@ __device__ __forceinline__ float frame_x(float x, int strad, int axis, float hal
   return ((strad >> axis) & 1) && x >= halfL ? x - L : x;
 }
 
+// a coordinate of the flat frame (frame_x) back in [0, L), exactly
+__device__ __forceinline__ float unframe_x(float x, float L) { return x < 0.0f ? x + L : x; }
+
 // every full 32 queued Coulomb pairs of the warp are evaluated with all lanes
 // busy; the rest (fewer than 32) stays queued
 template <bool WITH_S>
-__device__ __forceinline__ void queue_flush(const PairK &K, float *qr2, float *qqp, int &qn, long long &acc,
+__device__ __forceinline__ void queue_flush(const PairK &K, float2 *q, int &qn, long long &acc,
                                             unsigned long long &sacc, int &ov) {
   const int lane = threadIdx.x & 31;
-  while (qn >= 32) {
+  while (qn >= 32) {  // from the end, so that the rest stays where it is
     __syncwarp();
-    coul_eval<WITH_S>(K, qr2[lane], qqp[lane], acc, sacc, ov);
-    const int rest = qn - 32;
-    float a0 = 0.f, b0 = 0.f, a1 = 0.f, b1 = 0.f;
-    if (lane < rest) {
-      a0 = qr2[32 + lane];
-      b0 = qqp[32 + lane];
-    }
-    if (lane + 32 < rest) {
-      a1 = qr2[64 + lane];
-      b1 = qqp[64 + lane];
-    }
-    __syncwarp();
-    if (lane < rest) {
-      qr2[lane] = a0;
-      qqp[lane] = b0;
-    }
-    if (lane + 32 < rest) {
-      qr2[32 + lane] = a1;
-      qqp[32 + lane] = b1;
-    }
-    __syncwarp();
-    qn = rest;
+    const float2 e = q[qn - 32 + lane];
+    qn -= 32;
+    coul_eval<WITH_S>(K, e.x, e.y, acc, sacc, ov);
   }
+  __syncwarp();
 }
 
-// Both changed particles A and B against one candidate j (lane-parallel):
-// the two distance tests are independent, pairs near an inserted / deleted
-// particle are evaluated at once, the in-range Coulomb pairs of A and B join
-// the warp's queue with one compaction step, and every full 32 queued pairs
-// are evaluated with all lanes busy.
-// FLAT: the candidate's coordinates and As, Bs (those of A and B) are in the
-// region's flat frame (below), where plain differences are the minimum-image
-// ones; the raw coordinates, for the FP64 WCA of a near pair, come back
-// exactly as x + L for a shifted (negative) x.
-template <bool WITH_S, bool FLAT = false>
-__device__ __forceinline__ void offer2(const SysParams &P, const PairK &K, const WcaEntry *wca, const Desc &A,
-                                       const Desc &B,
-                                       const float4 wrA, const float4 wrB, bool valid, float xj, float yj, float zj,
-                                       float qj, int jcls, float *qr2, float *qqp, int &qn, long long &acc,
-                                       unsigned long long &sacc, int &ov, const float3 As = float3{},
-                                       const float3 Bs = float3{}) {
-  const int lane = threadIdx.x & 31;
+// A candidate within the largest WCA range of an inserted / deleted changed
+// particle c (rare): the pair is evaluated here when it lies within its own
+// classes' range (returned true), Coulomb included
+template <bool WITH_S>
+__device__ __forceinline__ bool near_check(const SysParams &P, const float *wr, const Desc &c, float r2, float xj,
+                                           float yj, float zj, float qj, int jcls, long long &acc,
+                                           unsigned long long &sacc, int &ov) {
+  const int e = c.cls * 4 + jcls;
+  if (!(r2 < wr[e])) return false;
+  const PairSum p = near_pair<WITH_S>(P, P.wca[e], c.x, c.y, c.z, c.dqlB, c.dp, unframe_x(xj, P.Lf),
+                                      unframe_x(yj, P.Lf), unframe_x(zj, P.Lf), qj, r2);
+  acc += p.acc;
+  sacc += p.sacc;
+  ov |= p.ov;
+  return true;
+}
+
+// One trial's changed particles as the sweep needs them: coordinates in the
+// sweep's frame, Coulomb ranges (-1 without a charge change) and the largest
+// WCA ranges (-1 when the particle is neither inserted nor deleted)
+struct SweepPair {
+  float ax, ay, az, bx, by, bz, qA, qB, rcA, rcB, wmA, wmB;
+  int skA, skB;
+};
+__device__ __forceinline__ SweepPair sweep_pair(const PairK &K, const float *wmax, const Desc &A, const Desc &B,
+                                                int strad) {
+  SweepPair p;
+  p.ax = frame_x(A.x, strad, 0, K.halfL, K.Lf);
+  p.ay = frame_x(A.y, strad, 1, K.halfL, K.Lf);
+  p.az = frame_x(A.z, strad, 2, K.halfL, K.Lf);
+  p.bx = frame_x(B.x, strad, 0, K.halfL, K.Lf);
+  p.by = frame_x(B.y, strad, 1, K.halfL, K.Lf);
+  p.bz = frame_x(B.z, strad, 2, K.halfL, K.Lf);
+  p.qA = A.dqlB;
+  p.qB = B.dqlB;
+  p.rcA = A.dqlB != 0.0f ? K.rc2 : -1.0f;
+  p.rcB = B.dqlB != 0.0f ? K.rc2 : -1.0f;
+  p.wmA = A.dp != 0 ? wmax[A.cls] : -1.0f;
+  p.wmB = B.dp != 0 ? wmax[B.cls] : -1.0f;
+  p.skA = A.skip;
+  p.skB = B.skip;
+  return p;
+}
+
+// Both changed particles against one candidate (lane-parallel): two distance
+// tests; the in-range Coulomb pairs of A and B join the warp's queue with one
+// compaction step, and every full 32 queued pairs are evaluated with all
+// lanes busy.  cls(): the candidate's class, read only for near candidates.
+// FLAT: plain differences in the region's flat frame are the minimum-image
+// ones.
+template <bool WITH_S, bool FLAT, typename Cls>
+__device__ __forceinline__ void offer2(const SysParams &P, const PairK &K, const float *wr, const TrialCtl &ctl,
+                                       const SweepPair &p, bool valid, float xj, float yj, float zj, float qj,
+                                       Cls cls, float2 *q, int &qn, long long &acc, unsigned long long &sacc,
+                                       int &ov) {
   float ax, ay, az, bx, by, bz;
   if (FLAT) {
-    ax = xj - As.x; ay = yj - As.y; az = zj - As.z;
-    bx = xj - Bs.x; by = yj - Bs.y; bz = zj - Bs.z;
+    ax = xj - p.ax; ay = yj - p.ay; az = zj - p.az;
+    bx = xj - p.bx; by = yj - p.by; bz = zj - p.bz;
   } else {
-    ax = wrap_diff(xj, A.x, K.Lf, K.halfL); ay = wrap_diff(yj, A.y, K.Lf, K.halfL); az = wrap_diff(zj, A.z, K.Lf, K.halfL);
-    bx = wrap_diff(xj, B.x, K.Lf, K.halfL); by = wrap_diff(yj, B.y, K.Lf, K.halfL); bz = wrap_diff(zj, B.z, K.Lf, K.halfL);
+    ax = wrap_diff(xj, p.ax, K.Lf, K.halfL); ay = wrap_diff(yj, p.ay, K.Lf, K.halfL); az = wrap_diff(zj, p.az, K.Lf, K.halfL);
+    bx = wrap_diff(xj, p.bx, K.Lf, K.halfL); by = wrap_diff(yj, p.by, K.Lf, K.halfL); bz = wrap_diff(zj, p.bz, K.Lf, K.halfL);
   }
   const float rA = ax * ax + ay * ay + az * az, rB = bx * bx + by * by + bz * bz;
-  const bool nearA = valid && rA < sel4(wrA, jcls), nearB = valid && rB < sel4(wrB, jcls);
-  if (nearA || nearB) {
-    float xr = xj, yr = yj, zr = zj;
-    if (FLAT) {
-      xr = xj < 0.0f ? xj + K.Lf : xj;
-      yr = yj < 0.0f ? yj + K.Lf : yj;
-      zr = zj < 0.0f ? zj + K.Lf : zj;
-    }
-    if (nearA) {
-      const PairSum p = near_pair<WITH_S>(P, wca[A.cls * 4 + jcls], A.x, A.y, A.z, A.dqlB, A.dp, xr, yr, zr, qj, rA);
-      acc += p.acc;
-      sacc += p.sacc;
-      ov |= p.ov;
-    }
-    if (nearB) {
-      const PairSum p = near_pair<WITH_S>(P, wca[B.cls * 4 + jcls], B.x, B.y, B.z, B.dqlB, B.dp, xr, yr, zr, qj, rB);
-      acc += p.acc;
-      sacc += p.sacc;
-      ov |= p.ov;
-    }
+  const bool charged = valid && qj != 0.0f;
+  bool inA = charged && rA < p.rcA, inB = charged && rB < p.rcB;
+  if (valid && (rA < p.wmA || rB < p.wmB)) {
+    const int jc = cls();
+    if (rA < p.wmA && near_check<WITH_S>(P, wr, ctl.c[0], rA, xj, yj, zj, qj, jc, acc, sacc, ov)) inA = false;
+    if (rB < p.wmB && near_check<WITH_S>(P, wr, ctl.c[1], rB, xj, yj, zj, qj, jc, acc, sacc, ov)) inB = false;
   }
-  const bool inA = valid && !nearA && rA < K.rc2 && A.dqlB != 0.0f && qj != 0.0f;
-  const bool inB = valid && !nearB && rB < K.rc2 && B.dqlB != 0.0f && qj != 0.0f;
   const unsigned mA = __ballot_sync(FULL, inA), mB = __ballot_sync(FULL, inB);
-  if ((mA | mB) == 0u) return;
+  const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   const int nA = __popc(mA);
-  if (inA) {
-    const int p = qn + __popc(mA & lt);
-    qr2[p] = rA;
-    qqp[p] = A.dqlB * qj;
-  }
-  if (inB) {
-    const int p = qn + nA + __popc(mB & lt);
-    qr2[p] = rB;
-    qqp[p] = B.dqlB * qj;
-  }
+  if (inA) q[qn + __popc(mA & lt)] = make_float2(rA, p.qA * qj);
+  if (inB) q[qn + nA + __popc(mB & lt)] = make_float2(rB, p.qB * qj);
   qn += nA + __popc(mB);
-  queue_flush<WITH_S>(K, qr2, qqp, qn, acc, sacc, ov);
+  if (qn >= 32) queue_flush<WITH_S>(K, q, qn, acc, sacc, ov);
 }
 
 
-template <int T>
-__device__ __forceinline__ void cta_sync() {
-  if (T == 32) __syncwarp();
-  else __syncthreads();
+// barrier of a group of G warps (its own named barrier, ids 1 .. 15)
+template <int G>
+__device__ __forceinline__ void group_sync(int group) {
+  if (G == 1) __syncwarp();
+  else asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "r"(32 * G) : "memory");
 }
 
-// int64 sum over the warp, result in every lane
-__device__ __forceinline__ long long warp_allsum(long long v) { return warp_sum_i64(v); }
+// A CTA's domain, in shared memory (so that the trial loop holds none of it
+// in registers): where it lies, its random-number counters, its list, and the
+// region around it.  The sweep reads the halo on chip (cpos[0 .. nhc), classes
+// hcls), the list's payload behind it (cpos[hcs + slot]) when that is in shared
+// memory too (in_smem), and what does not fit there from global memory.
+struct Dom {
+  DomList L;
+  const long long *lnt;  // log table
+  const int *hpre, *hcell;
+  long long log_dom;     // first record of a logged call
+  int nhc, hcs;   // halo entries on chip, and their capacity
+  int NH, NR;     // halo entries in all; region cells
+  int in_smem, strad, flat, list_cap;
+  int org[3], off[3], dd[3], d;
+  uint32_t phi, key0, key1;
+  float wr[20];   // [16] WCA pre-check radii by class pair, [4] their maxima per class
+};
 
 // Random numbers of a chunk of trials (Philox purposes 0-3 and 6-7; thread i0
 // of a group of `stride` threads takes every stride-th task): the move and
@@ -587,18 +610,18 @@ __device__ __forceinline__ long long warp_allsum(long long v) { return warp_sum_
 // Metropolis uniform, for delayed acceptance the stage-2 uniform, and the
 // velocities of the ions an insertion would add.
 template <bool LOG, bool DA>
-__device__ __noinline__ void draw_chunk(TrialPre *tp, float4 *tvel, int k0, int nchunk, int i0, int stride, int d,
-                                        uint32_t phi, int org0, int org1, int org2, int off0, int off1, int off2,
-                                        int dd0, int dd1, int dd2, int k, int nc, float af, float Lf, float scf,
-                                        uint32_t key0, uint32_t key1) {
-  const int org[3] = {org0, org1, org2}, off[3] = {off0, off1, off2}, dd[3] = {dd0, dd1, dd2};
-  for (int u = i0; u < 3 * nchunk; u += stride) {
-    if (u >= nchunk) {  // the Maxwell-Boltzmann velocities an accepted insertion gives its ions (purposes 6, 7)
-      const int t = u % nchunk, which = u / nchunk - 1;
-      tvel[2 * t + which] = ion_velocity((uint32_t)(k0 + t), (uint32_t)d, phi, 6u + (uint32_t)which, key0, key1);
-      continue;
-    }
-    const int t = u;
+__device__ __noinline__ void draw_chunk(const SysParams &P, const Dom &D, TrialPre *tp, float4 *tvel, int k0,
+                                        int nchunk, int i0, int stride) {
+  const int d = D.d, k = P.k, nc = P.nc;
+  const uint32_t phi = D.phi, key0 = D.key0, key1 = D.key1;
+  const float af = P.af, Lf = P.Lf, scf = P.scf;
+  const int *org = D.org, *off = D.off, *dd = D.dd;
+  // the Maxwell-Boltzmann velocities an accepted insertion gives its ions
+  // (purposes 6, 7), counted from the last thread so that other warps than
+  // those of the trials' own numbers draw them
+  for (int u = stride - 1 - i0; u < 2 * nchunk; u += stride)
+    tvel[u] = ion_velocity((uint32_t)(k0 + (u >> 1)), (uint32_t)d, phi, 6u + (uint32_t)(u & 1), key0, key1);
+  for (int t = i0; t < nchunk; t += stride) {
     const uint32_t kk = (uint32_t)(k0 + t);
     const uint4 a = philox10(kk, (uint32_t)d, phi, 0u, key0, key1);
     const uint4 b = philox10(kk, (uint32_t)d, phi, 1u, key0, key1);
@@ -646,15 +669,25 @@ __device__ __noinline__ void draw_chunk(TrialPre *tp, float4 *tvel, int k0, int 
   }
 }
 
+// slot of the particle at place i of the canonical order, and a slot's
+// position in [0, L) (w: charge)
+__device__ __forceinline__ int slot_at(const DomList &L, int i) { return (int)(L.ord[i].x & ORD_SLOT_MASK); }
+__device__ __forceinline__ float4 raw_pos(const DomList &L, int s, float Lf) {
+  const float4 p = L.pos[s];
+  return make_float4(unframe_x(p.x, Lf), unframe_x(p.y, Lf), unframe_x(p.z, Lf), p.w);
+}
+
 // Proposal of trial kk on the current list (Sec. II.C applied to the domain):
 // the move, its participants, the log of the acceptance ratio without the
 // energy, the self-energy change and the two changed particles.  Every lane
 // of the calling warp computes the same values (the list scans are ballots).
 template <bool DA>
-__device__ __forceinline__ void select_trial(const SysParams &P, const DomList &L, const int *misc,
-                                             const long long *lnt, const TrialPre &q, int d, int m, int kk,
-                                             uint32_t phi, TrialCtl &C) {
-  const int lane = threadIdx.x & 31;
+__device__ __forceinline__ void select_trial(const SysParams &P, const Dom &D, const int *misc, const TrialPre &q,
+                                             int kk, TrialCtl &C) {
+  const DomList L = D.L;
+  const long long *lnt = D.lnt;
+  const int lane = threadIdx.x & 31, d = D.d, m = P.m;
+  const uint32_t phi = D.phi;
   const int n = misc[0];
   const int mv = pick32(q.w0, 2 * P.n_react);
   const int r = P.react[mv >> 1];
@@ -676,40 +709,42 @@ __device__ __forceinline__ void select_trial(const SysParams &P, const DomList &
     if (fwd) {
       if (n0 == 0) flags |= CR_TRIAL_NO_ELIGIBLE;
       else {
-        site = warp_kth(L.info, n, kn, pick32(q.w1, n0));
+        site = warp_kth(L.ord, n, kn, pick32(q.w1, n0));
         if (q.rankA < 0) flags |= CR_TRIAL_EDGE;
         if (site < 0) { site = 0; bad = true; }
-        id_a = L.id[site];
+        const int ss = bad ? 0 : slot_at(L, site);
+        id_a = L.id[ss];
         id_b = newid;
-        const float4 sp4 = L.pos[site];
-        const int sinfo = L.info[site];
-        c0 = Desc{sp4.x, sp4.y, sp4.z, P.lBf * qs, 0, (sinfo >> INFO_CLS_SHIFT) & 3, site};
+        const float4 sp4 = raw_pos(L, ss, P.Lf);
+        const int sinfo = L.info[ss];
+        c0 = Desc{sp4.x, sp4.y, sp4.z, P.lBf * qs, 0, (sinfo >> INFO_CLS_SHIFT) & 3, ss};
         c1 = Desc{q.ax, q.ay, q.az, P.lBf * (-qs * P.ion_q), 1, P.ion_cls, -1};
         qa_o = 0.f; qa_n = qs; qb_o = 0.f; qb_n = -qs * P.ion_q;
         pa_o = pa_n = 1; pb_o = 0; pb_n = 1;
         nch = 2;
         ln_ratio = lnt[n0] + P.lnz1_fx - lnt[n1 + 1];
         ln_ratio -= lnt[nx + 1];
-        ln_ratio += L.lnk[site];
+        ln_ratio += L.lnk[ss];
       }
     } else {
       if (n1 == 0 || nx == 0) flags |= CR_TRIAL_NO_ELIGIBLE;
       else {
-        site = warp_kth(L.info, n, ki, pick32(q.w1, n1));
-        ionA = warp_kth(L.info, n, kx, pick32(q.w2, nx));
+        site = warp_kth(L.ord, n, ki, pick32(q.w1, n1));
+        ionA = warp_kth(L.ord, n, kx, pick32(q.w2, nx));
         if (site < 0 || ionA < 0) { site = max(site, 0); ionA = max(ionA, 0); bad = true; }
-        id_a = L.id[site];
-        id_b = L.id[ionA];
-        const float4 sp4 = L.pos[site], ip4 = L.pos[ionA];
-        const int sinfo = L.info[site], iinfo = L.info[ionA];
-        c0 = Desc{sp4.x, sp4.y, sp4.z, P.lBf * (-qs), 0, (sinfo >> INFO_CLS_SHIFT) & 3, site};
-        c1 = Desc{ip4.x, ip4.y, ip4.z, P.lBf * (-ip4.w), -1, (iinfo >> INFO_CLS_SHIFT) & 3, ionA};
+        const int ss = bad ? 0 : slot_at(L, site), si = bad ? 0 : slot_at(L, ionA);
+        id_a = L.id[ss];
+        id_b = L.id[si];
+        const float4 sp4 = raw_pos(L, ss, P.Lf), ip4 = raw_pos(L, si, P.Lf);
+        const int sinfo = L.info[ss], iinfo = L.info[si];
+        c0 = Desc{sp4.x, sp4.y, sp4.z, P.lBf * (-qs), 0, (sinfo >> INFO_CLS_SHIFT) & 3, ss};
+        c1 = Desc{ip4.x, ip4.y, ip4.z, P.lBf * (-ip4.w), -1, (iinfo >> INFO_CLS_SHIFT) & 3, si};
         qa_o = qs; qa_n = 0.f; qb_o = ip4.w; qb_n = 0.f;
         pa_o = pa_n = 1; pb_o = 1; pb_n = 0;
         nch = 2;
         ln_ratio = lnt[n1] - lnt[n0 + 1] - P.lnz1_fx;
         ln_ratio += lnt[nx];
-        ln_ratio -= L.lnk[site];
+        ln_ratio -= L.lnk[ss];
       }
     }
   } else {
@@ -728,14 +763,15 @@ __device__ __forceinline__ void select_trial(const SysParams &P, const DomList &
     } else {
       if (nxp == 0 || nxm == 0) flags |= CR_TRIAL_NO_ELIGIBLE;
       else {
-        ionA = warp_kth(L.info, n, P.kxp, pick32(q.w2, nxp));
-        ionB = warp_kth(L.info, n, P.kxm, pick32(q.w3, nxm));
+        ionA = warp_kth(L.ord, n, P.kxp, pick32(q.w2, nxp));
+        ionB = warp_kth(L.ord, n, P.kxm, pick32(q.w3, nxm));
         if (ionA < 0 || ionB < 0) { ionA = max(ionA, 0); ionB = max(ionB, 0); bad = true; }
-        id_a = L.id[ionA];
-        id_b = L.id[ionB];
-        const float4 a4 = L.pos[ionA], b4 = L.pos[ionB];
-        c0 = Desc{a4.x, a4.y, a4.z, P.lBf * (-a4.w), -1, (L.info[ionA] >> INFO_CLS_SHIFT) & 3, ionA};
-        c1 = Desc{b4.x, b4.y, b4.z, P.lBf * (-b4.w), -1, (L.info[ionB] >> INFO_CLS_SHIFT) & 3, ionB};
+        const int sa = bad ? 0 : slot_at(L, ionA), sb = bad ? 0 : slot_at(L, ionB);
+        id_a = L.id[sa];
+        id_b = L.id[sb];
+        const float4 a4 = raw_pos(L, sa, P.Lf), b4 = raw_pos(L, sb, P.Lf);
+        c0 = Desc{a4.x, a4.y, a4.z, P.lBf * (-a4.w), -1, (L.info[sa] >> INFO_CLS_SHIFT) & 3, sa};
+        c1 = Desc{b4.x, b4.y, b4.z, P.lBf * (-b4.w), -1, (L.info[sb] >> INFO_CLS_SHIFT) & 3, sb};
         qa_o = a4.w; qa_n = 0.f; qb_o = b4.w; qb_n = 0.f;
         pa_o = 1; pa_n = 0; pb_o = 1; pb_n = 0;
         nch = 2;
@@ -759,11 +795,11 @@ __device__ __forceinline__ void select_trial(const SysParams &P, const DomList &
   int rka = 0, rkb = 0;
   if (DA && nch) {
     if (r == R_SALT) {
-      rka = fwd ? q.rankA : L.rank[ionA];
-      rkb = fwd ? q.rankB : L.rank[ionB];
+      rka = fwd ? q.rankA : (int)L.ord[ionA].y;
+      rkb = fwd ? q.rankB : (int)L.ord[ionB].y;
     } else {
-      rka = L.rank[site];
-      rkb = fwd ? q.rankA : L.rank[ionA];
+      rka = (int)L.ord[site].y;
+      rkb = fwd ? q.rankA : (int)L.ord[ionA].y;
     }
   }
   if (lane == 0) {
@@ -798,151 +834,96 @@ __device__ __forceinline__ void select_trial(const SysParams &P, const DomList &
   }
 }
 
-// One candidate of the merged stream of a region's particles that are not
-// held in registers: u < nhc the on-chip halo (shared memory, already in the
-// flat frame when the region is flat, w = q + 8 cls), u < NH the halo beyond
-// it (global memory), then the domain list.  FLAT: coordinates are returned
-// in the region's flat frame.
-template <bool FLAT>
-__device__ __forceinline__ bool stream_cand(const SysParams &P, const DomList &L, const Desc &A, const Desc &B,
-                                            const float4 *hpos, int nhc, int NH, int n, const int *hpre,
-                                            const int *hcell, int NR, int strad, int u, float &x, float &y,
-                                            float &z, float &q, int &cls) {
-  if (u < nhc) {
-    const float4 p = hpos[u];
-    cls = __float2int_rd((p.w + 2.0f) * 0.125f);
-    q = p.w - 8.0f * (float)cls;
-    x = p.x;
-    y = p.y;
-    z = p.z;
-    return true;
-  }
-  float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
-  bool v = false;
-  cls = 0;
-  if (u < NH) {  // halo beyond what is held on chip (dense regions): straight from global memory
-    const int i = upper_idx(hpre, NR, u);
-    const int g = hcell[i] * P.cap + (u - hpre[i]);
-    p = P.pos[g];
-    cls = (P.info[g] >> INFO_CLS_SHIFT) & 3;
-    v = true;
-  } else if (u < NH + n) {
-    const int j = u - NH;
-    p = L.pos[j];
-    cls = (L.info[j] >> INFO_CLS_SHIFT) & 3;
-    v = j != A.skip && j != B.skip;
-  }
-  q = p.w;
-  if (FLAT) {
-    x = frame_x(p.x, strad, 0, P.halfL, P.Lf);
-    y = frame_x(p.y, strad, 1, P.halfL, P.Lf);
-    z = frame_x(p.z, strad, 2, P.halfL, P.Lf);
-  } else {
-    x = p.x;
-    y = p.y;
-    z = p.z;
-  }
-  return v;
-}
-
-// The region's stream (all of it, or from `from` on) against A and B without
-// the flat frame: regions wider than 0.4 L, i.e. small boxes.  Out of line,
-// so that the flat loop is the only pair sweep in the trial loop's code; its
-// sums come back by value.
-template <bool LOG>
-__device__ __noinline__ PairSum sweep_general(const SysParams &P, const TrialCtl &C, const float4 *lpos,
-                                              const int *linfo, const float4 *hpos, int nhc, int NH, int n,
-                                              const int *hpre, const int *hcell, int NR, int from, int i0, int stride,
-                                              float *qr2, float *qqp) {
-  const Desc A = C.c[0], B = C.c[1];
-  DomList L{};
-  L.pos = const_cast<float4 *>(lpos);
-  L.info = const_cast<int *>(linfo);
-  PairK K;
-  K.Lf = P.Lf; K.halfL = P.halfL; K.rc2 = P.rc2; K.alpha = P.alpha; K.c1 = P.c1; K.c2 = P.c2; K.rcf = P.rcf;
-  K.lBf = P.lBf; K.Ld = P.Ld; K.halfLd = P.halfLd;
-  const WcaEntry *wca = P.wca;
-  const float4 wrA = wca_radii(wca, A), wrB = wca_radii(wca, B);
+// The part of a region that is not on chip: the halo beyond its capacity
+// (dense regions; straight from global memory) and a list in global memory.
+// Out of line, as it is rare; the queue (qn entries) is continued and emptied.
+template <bool LOG, bool FLAT>
+__device__ __noinline__ PairSum sweep_rest(const SysParams &P, const TrialCtl &C, const Dom &Rg, int nlist, int i0,
+                                           int stride, float2 *q, int qn) {
+  const PairK K = pair_k(P);
+  const SweepPair sp = sweep_pair(K, Rg.wr + 16, C.c[0], C.c[1], Rg.strad);
   const int lane = threadIdx.x & 31;
   PairSum out{0, 0ull, 0};
-  int qn = 0;
-  for (int base = from; base < NH + n; base += stride) {
-    float x, y, z, q;
-    int cls;
+  const float4 *lpos = Rg.L.pos;
+  const int *linfo = Rg.L.info;
+  const int nover = Rg.NH - Rg.nhc, total = nover + (Rg.in_smem ? 0 : nlist);
+  for (int base = 0; base < total; base += stride) {
     const int u = base + i0;
-    const bool v = stream_cand<false>(P, L, A, B, hpos, nhc, NH, n, hpre, hcell, NR, 0, u, x, y, z, q, cls);
-    offer2<LOG>(P, K, wca, A, B, wrA, wrB, v, x, y, z, q, cls, qr2, qqp, qn, out.acc, out.sacc, out.ov);
+    float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
+    bool v = false;
+    int cls = 0;
+    if (u < nover) {
+      const int h = Rg.nhc + u;
+      const int i = upper_idx(Rg.hpre, Rg.NR, h);
+      const int g = Rg.hcell[i] * P.cap + (h - Rg.hpre[i]);
+      p = P.pos[g];
+      p.x = frame_x(p.x, Rg.strad, 0, P.halfL, P.Lf);
+      p.y = frame_x(p.y, Rg.strad, 1, P.halfL, P.Lf);
+      p.z = frame_x(p.z, Rg.strad, 2, P.halfL, P.Lf);
+      cls = (P.info[g] >> INFO_CLS_SHIFT) & 3;
+      v = true;
+    } else if (u < total) {
+      const int j = u - nover;
+      p = lpos[j];
+      cls = (linfo[j] >> INFO_CLS_SHIFT) & 3;
+      v = j != sp.skA && j != sp.skB;
+    }
+    offer2<LOG, FLAT>(P, K, Rg.wr, C, sp, v, p.x, p.y, p.z, p.w, [&] { return cls; }, q, qn, out.acc, out.sacc, out.ov);
   }
   __syncwarp();
-  if (lane < qn) coul_eval<LOG>(K, qr2[lane], qqp[lane], out.acc, out.sacc, out.ov);
+  if (lane < qn) coul_eval<LOG>(K, q[lane].x, q[lane].y, out.acc, out.sacc, out.ov);
+  __syncwarp();
   return out;
 }
 
 // The pair changes of the two changed particles A and B against the halo and
 // the domain list, summed by a group of threads (thread i0 of `stride`; each
-// thread keeps its part in acc / sacc / ov; the warp's queued Coulomb pairs
-// are evaluated at the end).  The pair between A and B is not included.
-// Flat regions (the common case) take every candidate in the flat frame in
-// one loop over the merged stream; halo particles held in registers come
-// first.
-template <bool LOG, int R, int RR>
-__device__ __forceinline__ void sweep_pairs(const PairK &K, const WcaEntry *wca, const SysParams &P, const DomList &L,
-                                            const Desc &A, const Desc &B, const float4 (&hreg)[RR], int nmine,
-                                            const float4 *hpos, int NH, int hcap, const int *hpre, const int *hcell,
-                                            int NR, int n, int i0, int stride, float *qr2, float *qqp, long long &acc,
-                                            unsigned long long &sacc, int &ov, bool flat, int strad,
-                                            const TrialCtl *ctl) {
+// thread's part is returned; the warp's queued Coulomb pairs are evaluated at
+// the end).  The pair between A and B is not included.  One loop over the halo
+// and the list in shared memory; per 32 candidates it costs two distance tests
+// and one compaction.
+template <bool LOG, bool FLAT>
+__device__ __forceinline__ PairSum sweep_pairs(const PairK &K, const SysParams &P, const TrialCtl &C, const Dom &Rg,
+                                               const float4 *cpos, const unsigned char *hcls, int nlist, int i0,
+                                               int stride, float2 *q) {
   const int lane = threadIdx.x & 31;
-  const float4 wrA = wca_radii(wca, A), wrB = wca_radii(wca, B);
+  const SweepPair sp = sweep_pair(K, Rg.wr + 16, C.c[0], C.c[1], Rg.strad);
+  PairSum out{0, 0ull, 0};
   int qn = 0;
-  // the on-chip halo is stored in the flat frame when the region allows it
-  const float3 As = make_float3(frame_x(A.x, strad, 0, K.halfL, K.Lf), frame_x(A.y, strad, 1, K.halfL, K.Lf),
-                                frame_x(A.z, strad, 2, K.halfL, K.Lf));
-  const float3 Bs = make_float3(frame_x(B.x, strad, 0, K.halfL, K.Lf), frame_x(B.y, strad, 1, K.halfL, K.Lf),
-                                frame_x(B.z, strad, 2, K.halfL, K.Lf));
-  if (R > 0) {
-    if (flat) {
-#pragma unroll
-      for (int r = 0; r < RR; ++r) {
-        const float4 p = hreg[r];
-        const int cls = __float2int_rd((p.w + 2.0f) * 0.125f);
-        const float q = p.w - 8.0f * (float)cls;
-        offer2<LOG, true>(P, K, wca, A, B, wrA, wrB, r < nmine, p.x, p.y, p.z, q, cls, qr2, qqp, qn, acc, sacc, ov,
-                          As, Bs);
-      }
-    } else {
-#pragma unroll
-      for (int r = 0; r < RR; ++r) {
-        const float4 p = hreg[r];
-        const int cls = __float2int_rd((p.w + 2.0f) * 0.125f);
-        const float q = p.w - 8.0f * (float)cls;
-        offer2<LOG>(P, K, wca, A, B, wrA, wrB, r < nmine, p.x, p.y, p.z, q, cls, qr2, qqp, qn, acc, sacc, ov);
-      }
-    }
+  const int nhc = Rg.nhc, total = nhc + (Rg.in_smem ? nlist : 0);
+  const int gap = Rg.hcs - nhc;  // from the on-chip halo to the list's slots
+  const int skA = sp.skA >= 0 ? nhc + sp.skA : -1, skB = sp.skB >= 0 ? nhc + sp.skB : -1;
+  for (int base = 0; base < total; base += stride) {
+    const int u = base + i0;
+    const bool v = u < total && u != skA && u != skB;
+    float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (v) p = cpos[u < nhc ? u : u + gap];
+    offer2<LOG, FLAT>(P, K, Rg.wr, C, sp, v, p.x, p.y, p.z, p.w,
+                      [&] { return u < nhc ? (int)hcls[u] : (Rg.L.info[u - nhc] >> INFO_CLS_SHIFT) & 3; }, q, qn,
+                      out.acc, out.sacc, out.ov);
   }
-  // the rest of the stream: for R == 0 the halo in shared memory from 0, for
-  // R > 0 the part of the halo beyond the registers, then the list
-  const int nhc = R > 0 ? 0 : min(NH, hcap);
-  const int from = R > 0 ? min(NH, hcap) : 0;
-  if (flat) {
-    for (int base = from; base < NH + n; base += stride) {
-      float x, y, z, q;
-      int cls;
-      const bool v = stream_cand<true>(P, L, A, B, hpos, nhc, NH, n, hpre, hcell, NR, strad, base + i0, x, y, z, q,
-                                       cls);
-      offer2<LOG, true>(P, K, wca, A, B, wrA, wrB, v, x, y, z, q, cls, qr2, qqp, qn, acc, sacc, ov, As, Bs);
-    }
-    __syncwarp();
-    if (lane < qn) coul_eval<LOG>(K, qr2[lane], qqp[lane], acc, sacc, ov);
+  if (Rg.NH > nhc || !Rg.in_smem) {  // uniform over the CTA
+    const PairSum g = sweep_rest<LOG, FLAT>(P, C, Rg, nlist, i0, stride, q, qn);
+    out.acc += g.acc;
+    out.sacc += g.sacc;
+    out.ov |= g.ov;
   } else {
     __syncwarp();
-    if (lane < qn) coul_eval<LOG>(K, qr2[lane], qqp[lane], acc, sacc, ov);  // the registers' queue
-    const PairSum g =
-        sweep_general<LOG>(P, *ctl, L.pos, L.info, hpos, nhc, NH, n, hpre, hcell, NR, from, i0, stride, qr2, qqp);
-    acc += g.acc;
-    sacc += g.sacc;
-    ov |= g.ov;
+    if (lane < qn) coul_eval<LOG>(K, q[lane].x, q[lane].y, out.acc, out.sacc, out.ov);
+    __syncwarp();
   }
+  return out;
+}
+
+// The same without the flat frame: regions wider than 0.4 L, i.e. small boxes
+// and the global schedule.  Out of line, so that the flat loop is the only
+// pair sweep in the trial loop's code.
+template <bool LOG>
+__device__ __noinline__ PairSum sweep_general(const SysParams &P, const TrialCtl &C, const Dom &Rg,
+                                              const float4 *cpos, const unsigned char *hcls, int nlist, int i0,
+                                              int stride, float2 *q) {
+  const PairK K = pair_k(P);
+  return sweep_pairs<LOG, false>(K, P, C, Rg, cpos, hcls, nlist, i0, stride, q);
 }
 
 // ---- Ewald reciprocal part (global schedule): the change of
@@ -1058,93 +1039,104 @@ __device__ __noinline__ void ewald_update(const SysParams &P, const float2 *f, c
   }
 }
 
-// room for the ions an accepted insertion adds: their cells below the cell
-// capacity and the list below its capacity (belowA / sameA: entries of the
-// list before and in the first ion's cell, where it goes)
-__device__ __forceinline__ bool insert_room(const SysParams &P, const DomList &L, int n, int list_cap, int r,
-                                            const TrialPre &q, int &belowA, int &sameA) {
-  warp_rank_count(L.rank, n, q.rankA, belowA, sameA);
-  bool full = sameA + 1 > P.cap;
-  if (r == R_SALT) {
-    int below2, same2;
-    warp_rank_count(L.rank, n, q.rankB, below2, same2);
-    full = full || same2 + 1 + (q.rankB == q.rankA ? 1 : 0) > P.cap;
+// payload slot for a new particle: the last one freed, or the next unused one
+__device__ __forceinline__ int slot_take(const DomList &L, int *misc) {
+  const int f = misc[MISC_FREE];
+  if (f > 0) {
+    misc[MISC_FREE] = L.info[f - 1] >> INFO_SITE_SHIFT;
+    return f - 1;
   }
-  return !(full || n + 2 > list_cap);
+  return misc[MISC_HW]++;
 }
 
-// Commit of an accepted trial by one warp: the site's charge state, the ion
-// inserted (after every entry of its cell, as new ids are the largest) or
-// deleted in the list, the kind counts.  Returns the new list size.
-__device__ __forceinline__ int commit_trial(const SysParams &P, const DomList &L, int *misc, const TrialCtl &C,
-                                            const TrialPre &q, const float4 *vel, int n, int belowA, int sameA) {
-  const int lane = threadIdx.x & 31;
+// warp: a new ion of cell rank `rank` joins the list (n entries) at place p,
+// after every entry of its cell, as new ids are the largest
+__device__ __forceinline__ void insert_ion(const SysParams &P, const DomList &L, int *misc, int n, int p, int rank,
+                                           float x, float y, float z, float q, const float4 &vel,
+                                           unsigned long long id, int type, int kind, int strad) {
+  ord_open(L.ord, n, p);
+  if ((threadIdx.x & 31) == 0) {
+    const int s = slot_take(L, misc);
+    L.pos[s] = make_float4(frame_x(x, strad, 0, P.halfL, P.Lf), frame_x(y, strad, 1, P.halfL, P.Lf),
+                           frame_x(z, strad, 2, P.halfL, P.Lf), q);
+    L.vel[s] = vel;
+    L.id[s] = id;
+    L.lnk[s] = 0;
+    L.info[s] = type | (P.ion_cls << INFO_CLS_SHIFT);
+    L.ord[p] = make_uint2((unsigned)s | ((unsigned)kind << ORD_KIND_SHIFT), (unsigned)rank);
+  }
+  __syncwarp();
+}
+
+// warp: the particle at place p leaves the list (n entries)
+__device__ __forceinline__ void remove_ion(const DomList &L, int *misc, int n, int p) {
+  if ((threadIdx.x & 31) == 0) {
+    const int s = slot_at(L, p);
+    L.pos[s].w = 0.0f;
+    L.info[s] = INFO_FREE | (misc[MISC_FREE] << INFO_SITE_SHIFT);
+    misc[MISC_FREE] = s + 1;
+  }
+  __syncwarp();
+  ord_close(L.ord, n, p);
+}
+
+// An accepted trial, by one warp: room for the ions an insertion adds -- their
+// cells below the cell capacity and the list below its capacity (else -1 and
+// nothing changes) -- then the site's charge state, the ions inserted or
+// deleted, the kind counts.  Returns the new list size.  Out of line: it runs
+// only for accepted trials and is large.
+__device__ __noinline__ int try_commit(const SysParams &P, const Dom &D, int *misc, const TrialCtl &C,
+                                       const TrialPre &q, const float4 *vel, int n) {
+  const int lane = threadIdx.x & 31, list_cap = D.list_cap, strad = D.strad;
+  const DomList &L = D.L;
   const int r = C.move >> 1;
   const bool fwd = (C.move & 1) == 0;
-  if (r == R_ACID || r == R_BASE) {
-    const float qs = r == R_ACID ? -1.0f : 1.0f;
-    const int s_site = C.site;
+  const float qs = r == R_BASE ? 1.0f : -1.0f;  // charge of an ionised site
+  int pA = 0, pB = 0;
+  if (fwd) {
+    const int loA = warp_lower(L.ord, n, q.rankA);
+    pA = warp_lower(L.ord, n, q.rankA + 1);
+    bool full = pA - loA + 1 > P.cap;
+    if (r == R_SALT) {
+      const int loB = warp_lower(L.ord, n, q.rankB);
+      pB = warp_lower(L.ord, n, q.rankB + 1);
+      full = full || pB - loB + 1 + (q.rankB == q.rankA ? 1 : 0) > P.cap;
+    }
+    if (full || n + 2 > list_cap) return -1;
+  }
+  const int move_kind = r == R_SALT || (r == R_ACID) ? P.kxp : P.kxm;  // kind of the first ion
+  if (r != R_SALT) {
     if (lane == 0) {
-      L.info[s_site] ^= INFO_ION_BIT;
-      L.pos[s_site].w = fwd ? qs : 0.0f;
+      const int s = slot_at(L, C.site);
+      const int kn = r == R_ACID ? K_A0 : K_B0, ki = kn + 1, dlt = fwd ? 1 : -1;
+      L.info[s] ^= INFO_ION_BIT;
+      L.pos[s].w = fwd ? qs : 0.0f;
+      L.ord[C.site].x = (unsigned)s | ((unsigned)(fwd ? ki : kn) << ORD_KIND_SHIFT);
+      misc[1 + kn] -= dlt;
+      misc[1 + ki] += dlt;
+      misc[1 + move_kind] += dlt;
     }
     __syncwarp();
     if (fwd) {
-      const int p = belowA + sameA;  // after every entry of its cell rank
-      warp_insert_gap(L, n, p);
-      if (lane == 0) {
-        L.pos[p] = make_float4(q.ax, q.ay, q.az, -qs * P.ion_q);
-        L.vel[p] = vel[0];
-        L.id[p] = C.newid;
-        L.lnk[p] = 0;
-        L.info[p] = (r == R_ACID ? P.txp : P.txm) | (P.ion_cls << INFO_CLS_SHIFT);
-        L.rank[p] = q.rankA;
-      }
+      insert_ion(P, L, misc, n, pA, q.rankA, q.ax, q.ay, q.az, -qs * P.ion_q, vel[0], C.newid,
+                 r == R_ACID ? P.txp : P.txm, move_kind, strad);
       n += 1;
     } else {
-      warp_remove(L, n, C.ionA);
+      remove_ion(L, misc, n, C.ionA);
       n -= 1;
-    }
-    if (lane == 0) {
-      const int kn = r == R_ACID ? K_A0 : K_B0, ki = kn + 1, kx = r == R_ACID ? P.kxp : P.kxm;
-      const int dlt = fwd ? 1 : -1;
-      misc[1 + kn] -= dlt;
-      misc[1 + ki] += dlt;
-      misc[1 + kx] += dlt;
     }
   } else {
     if (fwd) {
-      int p = belowA + sameA;
-      warp_insert_gap(L, n, p);
-      if (lane == 0) {
-        L.pos[p] = make_float4(q.ax, q.ay, q.az, P.ion_q);
-        L.vel[p] = vel[0];
-        L.id[p] = C.newid;
-        L.lnk[p] = 0;
-        L.info[p] = P.txp | (P.ion_cls << INFO_CLS_SHIFT);
-        L.rank[p] = q.rankA;
-      }
-      __syncwarp();
-      n += 1;
-      int below, same;
-      warp_rank_count(L.rank, n, q.rankB, below, same);
-      p = below + same;
-      warp_insert_gap(L, n, p);
-      if (lane == 0) {
-        L.pos[p] = make_float4(q.bx, q.by, q.bz, -P.ion_q);
-        L.vel[p] = vel[1];
-        L.id[p] = C.newid + 1u;
-        L.lnk[p] = 0;
-        L.info[p] = P.txm | (P.ion_cls << INFO_CLS_SHIFT);
-        L.rank[p] = q.rankB;
-      }
-      n += 1;
+      insert_ion(P, L, misc, n, pA, q.rankA, q.ax, q.ay, q.az, P.ion_q, vel[0], C.newid, P.txp, P.kxp, strad);
+      // the first ion lies before the second's place unless its cell ranks higher
+      insert_ion(P, L, misc, n + 1, pB + (q.rankA <= q.rankB ? 1 : 0), q.rankB, q.bx, q.by, q.bz, -P.ion_q, vel[1],
+                 C.newid + 1u, P.txm, P.kxm, strad);
+      n += 2;
     } else {
       const int hi = max(C.ionA, C.ionB), lo = min(C.ionA, C.ionB);
-      warp_remove(L, n, hi);
-      n -= 1;
-      warp_remove(L, n, lo);
-      n -= 1;
+      remove_ion(L, misc, n, hi);
+      remove_ion(L, misc, n - 1, lo);
+      n -= 2;
     }
     if (lane == 0) {
       const int dlt = fwd ? 1 : -1;
@@ -1152,104 +1144,120 @@ __device__ __forceinline__ int commit_trial(const SysParams &P, const DomList &L
       misc[1 + P.kxm] += dlt;
     }
   }
+  if (lane == 0) {
+    misc[0] = n;
+    misc[MISC_DIRTY] = 1;
+  }
   __syncwarp();
   return n;
 }
 
-// An accepted trial, by warp 0: room for the ions an insertion adds (else
-// -1 and nothing changes), then the commit; returns the new list size.  Out
-// of line: it runs only for accepted trials and is large.
-__device__ __noinline__ int try_commit(const SysParams &P, float4 *lpos, float4 *lvel, unsigned long long *lid,
-                                       long long *llnk, int *linfo, int *lrank, int *misc, const TrialCtl &C,
-                                       const TrialPre &q, const float4 *vel, int n, int list_cap) {
-  DomList L;
-  L.pos = lpos; L.vel = lvel; L.id = lid; L.lnk = llnk; L.info = linfo; L.rank = lrank;
-  const int r = C.move >> 1;
-  const bool fwd = (C.move & 1) == 0;
-  int belowA = 0, sameA = 0;
-  if (fwd && !insert_room(P, L, n, list_cap, r, q, belowA, sameA)) return -1;
-  return commit_trial(P, L, misc, C, q, vel, n, belowA, sameA);
-}
-
 }  // namespace
+
+// Shared memory of a phase CTA: the bytes of each array in order (every array
+// starts on a 16-byte boundary); fills S.off and returns the total.
+static size_t phase_layout(PhaseShape &S, int warps, int groups, bool da) {
+  const size_t dcs = S.dcs, chunk = S.chunk, nr3 = S.nr3 + 1, kc3 = S.kc3 + 1;
+  const size_t bytes[PhaseShape::N_OFF] = {
+      sizeof(SysParams),
+      sizeof(Dom),
+      sizeof(float4) * (S.hcs + dcs),         // halo, then the list's positions
+      sizeof(float4) * dcs,                   // velocities
+      sizeof(unsigned long long) * dcs,       // ids
+      sizeof(long long) * dcs,                // site constants
+      sizeof(int) * dcs,                      // info words
+      sizeof(uint2) * dcs,                    // canonical order
+      (size_t)S.hcs,                          // halo classes
+      sizeof(long long) * S.lns,              // log table
+      sizeof(TrialPre) * chunk,
+      sizeof(float4) * 2 * chunk,             // velocities of inserted ions
+      sizeof(TrialCtl) * groups,
+      sizeof(long long) * warps,              // the warps' sums
+      sizeof(unsigned long long) * warps,
+      sizeof(int) * warps,
+      sizeof(float2) * QCAP * warps,          // queues of Coulomb pairs
+      sizeof(int) * MISC_TOTAL,
+      sizeof(int) * nr3,                      // halo cells: counts, cells, prefix sums
+      sizeof(int) * nr3,
+      sizeof(int) * nr3,
+      sizeof(int) * kc3,                      // domain cells: counts, cells, prefix sums
+      sizeof(int) * kc3,
+      sizeof(int) * kc3,
+      sizeof(float2) * 6 * S.ewk,             // Ewald: axis factors, charge changes
+      sizeof(float) * 4,
+      da ? sizeof(int) * nr3 : 0,             // DA: region cell aggregates (ion charge, site charge, particles)
+      da ? sizeof(int) * nr3 : 0,
+      da ? sizeof(int) * nr3 : 0,
+      da ? sizeof(int) * MLP_IN * groups : 0,  // per group: feature bins, surrogate layers
+      da ? sizeof(float) * 2 * MLP_IN * groups : 0,
+      da ? sizeof(float) * 2 * MLP_H * groups : 0,
+      da ? sizeof(float) * 2 * MLP_H * groups : 0};
+  size_t at = 0;
+  for (int i = 0; i < PhaseShape::N_OFF; ++i) {
+    S.off[i] = (unsigned)at;
+    at += (bytes[i] + 15) / 16 * 16;
+  }
+  return at;
+}
 
 // ---------------------------------------------------------------------------
 // One domain of one colour phase of replica `rep`: `rank` is its place in
 // the colour's launch order.  Every thread of the CTA calls it; smem is the
-// CTA's dynamic shared memory, carved up as phase_smem_bytes describes.
-template <int T, int R, bool LOG, bool DA>
+// CTA's dynamic shared memory (phase_layout).
+//
+// The CTA is W groups of G warps.
+template <int G, int W, bool LOG, bool DA>
 __device__ __forceinline__ void phase_task(unsigned char *smem, const SysParams *__restrict__ reps,
                                            const PhaseShape &S, uint32_t sweep, uint32_t sweep0, int colour,
                                            uint32_t key0, uint32_t key1_base, int rep, int rank) {
-  constexpr int NW = T / 32;
+  constexpr int T = 32 * G * W, GT = 32 * G;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int group = W > 1 ? warp / G : 0, gwarp = warp % G, gtid = tid - group * GT;
 
-  // ---- shared memory carve-up (launch-wide shape); every array starts on
-  // a 16-byte boundary (phase_smem_bytes mirrors this order and padding)
-  unsigned char *sp = smem;
-  auto take = [&](size_t bytes) {
-    unsigned char *p = sp;
-    sp += (bytes + 15) / 16 * 16;
-    return p;
-  };
-  SysParams &P = *(SysParams *)take(sizeof(SysParams));
-  DomList Ls;
-  Ls.pos = (float4 *)take(sizeof(float4) * S.dcs);
-  Ls.vel = (float4 *)take(sizeof(float4) * S.dcs);
-  Ls.id = (unsigned long long *)take(sizeof(unsigned long long) * S.dcs);
-  Ls.lnk = (long long *)take(sizeof(long long) * S.dcs);
-  Ls.info = (int *)take(sizeof(int) * S.dcs);
-  Ls.rank = (int *)take(sizeof(int) * S.dcs);
-  float4 *hpos = (float4 *)take(sizeof(float4) * S.hcs);  // halo (R == 0): x, y, z, q + 8 cls
-  long long *lntab_s = (long long *)take(sizeof(long long) * S.lns);
-  TrialPre *tp = (TrialPre *)take(sizeof(TrialPre) * S.chunk);
-  float4 *tvel = (float4 *)take(sizeof(float4) * 2 * S.chunk);  // velocities of inserted ions
-  TrialCtl *ctl = (TrialCtl *)take(sizeof(TrialCtl));
-  long long *red = (long long *)take(sizeof(long long) * MAX_WARPS);
-  unsigned long long *reds = (unsigned long long *)take(sizeof(unsigned long long) * MAX_WARPS);
-  unsigned long long *st = (unsigned long long *)take(sizeof(unsigned long long) * 16);
-  float *qbuf = (float *)take(sizeof(float) * 2 * QCAP * NW);
-  int *redov = (int *)take(sizeof(int) * MAX_WARPS);
-  int *scan_tmp = (int *)take(sizeof(int) * 32);
-  int *misc = (int *)take(sizeof(int) * MISC_N);  // [0] list size, [1 + kind] counts, [MISC_INIT + kind] at start
-  int *hcnt = (int *)take(sizeof(int) * (S.nr3 + 1));
-  int *hcell = (int *)take(sizeof(int) * (S.nr3 + 1));
-  int *hpre = (int *)take(sizeof(int) * (S.nr3 + 1));
-  int *dcnt = (int *)take(sizeof(int) * (S.kc3 + 1));
-  int *dpre = (int *)take(sizeof(int) * (S.kc3 + 1));
-  float *qr2 = qbuf + warp * 2 * QCAP, *qqp = qr2 + QCAP;
-  // Ewald: the changed particles' axis factors and charge changes
-  float2 *ewf = (float2 *)take(sizeof(float2) * 6 * S.ewk);
-  float *ewq = (float *)take(sizeof(float) * 4);
-  // delayed acceptance: region cell aggregates (ion charge, site charge,
-  // particles), feature bins, the two surrogate inputs and hidden layers
+  // (the offsets come from the launch's constant parameters)
+#define CRMC_AT(i) (smem + S.off[i])
+  SysParams &P = *(SysParams *)CRMC_AT(0);
+  Dom &D = *(Dom *)CRMC_AT(1);
+  float4 *cpos = (float4 *)CRMC_AT(2);  // halo [hcs], then the list's positions [dcs]
+  unsigned char *hcls = CRMC_AT(8);
+  long long *lntab_s = (long long *)CRMC_AT(9);
+  TrialPre *tp = (TrialPre *)CRMC_AT(10);
+  float4 *tvel = (float4 *)CRMC_AT(11);
+  TrialCtl *ctls = (TrialCtl *)CRMC_AT(12);
+  long long *red = (long long *)CRMC_AT(13);
+  unsigned long long *reds = (unsigned long long *)CRMC_AT(14);
+  int *redov = (int *)CRMC_AT(15);
+  float2 *queue = (float2 *)CRMC_AT(16) + warp * QCAP;
+  int *misc = (int *)CRMC_AT(17);  // [0] list size, [1 + kind] counts, [MISC_INIT + kind] at start, MISC_HW ...
+  int *hcnt = (int *)CRMC_AT(18), *hcell = (int *)CRMC_AT(19), *hpre = (int *)CRMC_AT(20);
+  int *dcnt = (int *)CRMC_AT(21), *dcell = (int *)CRMC_AT(22), *dpre = (int *)CRMC_AT(23);
+  float2 *ewf = (float2 *)CRMC_AT(24);
+  float *ewq = (float *)CRMC_AT(25);
   int *aQi = nullptr, *aQs = nullptr, *aN = nullptr, *dfeat = nullptr;
   float *fv = nullptr, *hb0 = nullptr, *hb1 = nullptr;
   if (DA) {
-    aQi = (int *)take(sizeof(int) * (S.nr3 + 1));
-    aQs = (int *)take(sizeof(int) * (S.nr3 + 1));
-    aN = (int *)take(sizeof(int) * (S.nr3 + 1));
-    dfeat = (int *)take(sizeof(int) * MLP_IN);
-    fv = (float *)take(sizeof(float) * 2 * MLP_IN);
-    hb0 = (float *)take(sizeof(float) * 2 * MLP_H);
-    hb1 = (float *)take(sizeof(float) * 2 * MLP_H);
+    aQi = (int *)CRMC_AT(26);
+    aQs = (int *)CRMC_AT(27);
+    aN = (int *)CRMC_AT(28);
+    dfeat = (int *)CRMC_AT(29) + group * MLP_IN;
+    fv = (float *)CRMC_AT(30) + group * 2 * MLP_IN;
+    hb0 = (float *)CRMC_AT(31) + group * 2 * MLP_H;
+    hb1 = (float *)CRMC_AT(32) + group * 2 * MLP_H;
   }
 
   {
-    const int *src = (const int *)&reps[rep];
-    int *dst = (int *)&P;
-    for (int i = tid; i < (int)(sizeof(SysParams) / 4); i += T) dst[i] = src[i];
+    const int4 *src = (const int4 *)&reps[rep];
+    int4 *dst = (int4 *)&P;
+    static_assert(sizeof(SysParams) % 16 == 0, "parameters copied 16 bytes at a time");
+    for (int i = tid; i < (int)(sizeof(SysParams) / 16); i += T) dst[i] = src[i];
   }
+  if (tid < MISC_TOTAL) misc[tid] = 0;
   __syncthreads();
   if (rank >= P.nact) return;  // uniform over the CTA
   const int bdom = P.order ? P.order[colour * P.nact + rank] : rank;  // active-domain index
   const int k = P.k, h = P.h, nc = P.nc, nr = P.nr, m = P.m;
   const int KC = k * k * k, NR = nr * nr * nr;
   const uint32_t key1 = key1_base ^ P.key_xor;
-  PairK K;
-  K.Lf = P.Lf; K.halfL = P.halfL; K.rc2 = P.rc2; K.alpha = P.alpha; K.c1 = P.c1; K.c2 = P.c2; K.rcf = P.rcf;
-  K.lBf = P.lBf; K.Ld = P.Ld; K.halfLd = P.halfLd;
-  const WcaEntry *wca = P.wca;
 
   // ---- which domain
   int dd[3];
@@ -1274,36 +1282,63 @@ __device__ __forceinline__ void phase_task(unsigned char *smem, const SysParams 
   int org[3];
 #pragma unroll
   for (int i = 0; i < 3; ++i) org[i] = (off[i] + dd[i] * k) % nc;
+  // flat frame (frame_x): a region spanning less than half the box along
+  // every axis is compared without minimum-image tests; strad marks the
+  // axes along which it wraps around the periodic boundary
+  const bool flat = !P.global && 2.5f * (float)nr * P.af < P.Lf;
+  int strad = 0;
+  if (flat)
+    for (int i = 0; i < 3; ++i) strad |= (org[i] < h || org[i] + k + h > nc) ? 1 << i : 0;
 
-  // ---- cell counts of the domain and of its halo (cell indices kept)
-  for (int r = tid; r < KC; r += T) {
-    const int lx = r % k, ly = (r / k) % k, lz = r / (k * k);
-    dcnt[r] = P.cnt[(org[0] + lx) % nc + nc * ((org[1] + ly) % nc + nc * ((org[2] + lz) % nc))];
-  }
-  for (int i = tid; i < NR; i += T) {
-    const int ix = i % nr, iy = (i / nr) % nr, iz = i / (nr * nr);
-    int c = 0, cell = 0;
-    if (!(ix < k && iy < k && iz < k)) {
-      cell = region_coord(ix, org[0], k, h, nr, nc) +
-             nc * (region_coord(iy, org[1], k, h, nr, nc) + nc * region_coord(iz, org[2], k, h, nr, nc));
-      c = P.cnt[cell];
+  // ---- the region's cells and their counts (four cells per thread at a
+  // time, so that their loads are in flight together): the domain's own by
+  // rank, the halo's by region index (zero at the domain's)
+  for (int i0 = tid; i0 < NR; i0 += 4 * T) {
+    int cl[4], cn[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int i = min(i0 + u * T, NR - 1);
+      const int ix = i % nr, iy = (i / nr) % nr, iz = i / (nr * nr);
+      cl[u] = region_coord(ix, org[0], k, h, nr, nc) +
+              nc * (region_coord(iy, org[1], k, h, nr, nc) + nc * region_coord(iz, org[2], k, h, nr, nc));
     }
-    hcnt[i] = c;
-    hcell[i] = cell;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) cn[u] = P.cnt[cl[u]];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int i = i0 + u * T;
+      if (i >= NR) break;
+      const int ix = i % nr, iy = (i / nr) % nr, iz = i / (nr * nr);
+      const bool own = ix < k && iy < k && iz < k;
+      hcnt[i] = own ? 0 : cn[u];
+      hcell[i] = cl[u];
+      if (own) {
+        const int r = ix + k * (iy + k * iz);
+        dcnt[r] = cn[u];
+        dcell[r] = cl[u];
+      }
+    }
   }
-  if (tid < MISC_N) misc[tid] = 0;
-  if (tid < 16) st[tid] = 0ull;
+  // the WCA pre-check radii
+  if (tid < 16) D.wr[tid] = wca_radius(P.wca[tid]);
+  if (tid < 4)
+    D.wr[16 + tid] = fmaxf(fmaxf(wca_radius(P.wca[4 * tid]), wca_radius(P.wca[4 * tid + 1])),
+                           fmaxf(wca_radius(P.wca[4 * tid + 2]), wca_radius(P.wca[4 * tid + 3])));
   __syncthreads();
-  block_scan(dcnt, KC, dpre, scan_tmp);
-  block_scan(hcnt, NR, hpre, scan_tmp);
+  if (warp == 0) warp_scan(dcnt, KC, dpre);
+  if (warp == (T > 32 ? 1 : 0)) warp_scan(hcnt, NR, hpre);
+  __syncthreads();
   const int ND = dpre[KC], NH = hpre[NR];
+  const int nhc = min(NH, S.hcs);
   // the list lives in shared memory unless the domain is unusually dense
   const bool in_smem = ND + 2 * m <= S.dcs;
-  DomList L = Ls;
+  DomList L;
+  L.pos = cpos + S.hcs; L.vel = (float4 *)CRMC_AT(3); L.id = (unsigned long long *)CRMC_AT(4); L.lnk = (long long *)CRMC_AT(5);
+  L.info = (int *)CRMC_AT(6); L.ord = (uint2 *)CRMC_AT(7);
   if (!in_smem) {
     const size_t o = (size_t)(colour * P.nact + rank) * P.dcap_glob;  // this domain's region of the replica's scratch
     L.pos = P.gs_pos + o; L.vel = P.gs_vel + o; L.id = P.gs_id + o; L.lnk = P.gs_lnk + o;
-    L.info = P.gs_info + o; L.rank = P.gs_rank + o;
+    L.info = P.gs_info + o; L.ord = P.gs_ord + o;
     if (ND + 2 * m > P.dcap_glob) {  // cannot happen: a cell holds at most cap particles
       if (tid == 0) atomicOr(P.err, ERRB_CELL_OVERFLOW);
       return;
@@ -1312,66 +1347,89 @@ __device__ __forceinline__ void phase_task(unsigned char *smem, const SysParams 
   const int lnmax_need = min(P.lnmax, ND + 2 * m + 2);
   const bool ln_in_smem = lnmax_need <= S.lns;
   const long long *lnt = ln_in_smem ? lntab_s : P.lntab_fx;
+  if (tid == 0) {
+    D.L = L;
+    D.hpre = hpre;
+    D.hcell = hcell;
+    D.nhc = nhc;
+    D.hcs = S.hcs;
+    D.NH = NH;
+    D.NR = NR;
+    D.in_smem = in_smem ? 1 : 0;
+    D.strad = strad;
+    D.flat = flat ? 1 : 0;
+    D.list_cap = in_smem ? S.dcs : P.dcap_glob;
+    D.lnt = lnt;
+    D.d = d;
+    D.phi = phi;
+    D.key0 = key0;
+    D.key1 = key1;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      D.org[i] = org[i];
+      D.off[i] = off[i];
+      D.dd[i] = dd[i];
+    }
+    D.log_dom = (long long)(sweep - sweep0) * P.per_sweep + (long long)colour * P.nact * m + (long long)bdom * m;
+    misc[0] = ND;
+    misc[MISC_HW] = ND;
+  }
+  // ---- the particles' slots, written by their cells: each halo entry's and
+  // list entry's source slot (and rank) waits where the entry itself goes
+  for (int i = tid; i < NR; i += T) {
+    const int j0 = hpre[i], n = min(hcnt[i], max(nhc - j0, 0)), g = hcell[i] * P.cap;
+    for (int q = 0; q < n; ++q) *(int *)&cpos[j0 + q] = g + q;
+  }
+  for (int r = tid; r < KC; r += T) {
+    const int j0 = dpre[r], n = dcnt[r], g = dcell[r] * P.cap;
+    for (int q = 0; q < n; ++q) L.ord[j0 + q] = make_uint2((unsigned)(g + q), (unsigned)r);
+  }
   if (ln_in_smem)
     for (int i = tid; i < lnmax_need; i += T) lntab_s[i] = P.lntab_fx[i];
-  for (int j = tid; j < ND; j += T) {
-    const int r = upper_idx(dpre, KC, j);
-    const int lx = r % k, ly = (r / k) % k, lz = r / (k * k);
-    const int cell = (org[0] + lx) % nc + nc * ((org[1] + ly) % nc + nc * ((org[2] + lz) % nc));
-    const int g = cell * P.cap + (j - dpre[r]);
-    const int info = P.info[g];
-    const int t = info & INFO_TYPE_MASK;
-    L.pos[j] = P.pos[g];
-    L.vel[j] = P.vel[g];
-    L.id[j] = P.pid[g];
-    L.lnk[j] = (t == CR_ACID || t == CR_BASE) ? P.lnK_fx[info >> INFO_SITE_SHIFT] : 0ll;
-    L.info[j] = info;
-    L.rank[j] = r;
-    atomicAdd(&misc[1 + min(kind_of(info), (int)K_OTHER)], 1);
-  }
-  // flat frame (frame_x): a region spanning less than half the box along
-  // every axis is compared without minimum-image tests; strad marks the
-  // axes along which it wraps around the periodic boundary
-  const bool flat = !P.global && 2.5f * (float)nr * P.af < P.Lf;
-  int strad = 0;
-  if (flat)
-    for (int i = 0; i < 3; ++i) strad |= (org[i] < h || org[i] + k + h > nc) ? 1 << i : 0;
-  // halo particles (they do not change during the phase): w = q + 8 * cls
-  constexpr int RR = R > 0 ? R : 1;
-  float4 hreg[RR];
-  int nmine = 0;
-  const int hcap = R > 0 ? R * T : S.hcs;  // halo entries held on chip
-  if (R > 0) {
+  __syncthreads();
+  // ---- the halo (it does not change during the phase)
+  for (int j0 = tid; j0 < nhc; j0 += 4 * T) {
+    float4 p[4];
+    int inf[4];
 #pragma unroll
-    for (int r = 0; r < RR; ++r) {
-      const int j = tid + r * T;
-      hreg[r] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (j < NH) {
-        const int i = upper_idx(hpre, NR, j);
-        const int g = hcell[i] * P.cap + (j - hpre[i]);
-        const float4 p = P.pos[g];
-        hreg[r] = make_float4(frame_x(p.x, strad, 0, P.halfL, P.Lf), frame_x(p.y, strad, 1, P.halfL, P.Lf),
-                              frame_x(p.z, strad, 2, P.halfL, P.Lf),
-                              p.w + 8.0f * (float)((P.info[g] >> INFO_CLS_SHIFT) & 3));
-        nmine = r + 1;
+    for (int u = 0; u < 4; ++u) {
+      const int j = j0 + u * T;
+      if (j < nhc) {
+        const int g = *(const int *)&cpos[j];
+        p[u] = P.pos[g];
+        inf[u] = P.info[g];
       }
     }
-  } else {
-    for (int j = tid; j < min(NH, hcap); j += T) {
-      const int i = upper_idx(hpre, NR, j);
-      const int g = hcell[i] * P.cap + (j - hpre[i]);
-      const float4 p = P.pos[g];
-      hpos[j] = make_float4(frame_x(p.x, strad, 0, P.halfL, P.Lf), frame_x(p.y, strad, 1, P.halfL, P.Lf),
-                            frame_x(p.z, strad, 2, P.halfL, P.Lf),
-                            p.w + 8.0f * (float)((P.info[g] >> INFO_CLS_SHIFT) & 3));
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int j = j0 + u * T;
+      if (j < nhc) {
+        cpos[j] = make_float4(frame_x(p[u].x, strad, 0, P.halfL, P.Lf), frame_x(p[u].y, strad, 1, P.halfL, P.Lf),
+                              frame_x(p[u].z, strad, 2, P.halfL, P.Lf), p[u].w);
+        hcls[j] = (unsigned char)((inf[u] >> INFO_CLS_SHIFT) & 3);
+      }
     }
+  }
+  // ---- the list, in canonical order at first
+  for (int j = tid; j < ND; j += T) {
+    const uint2 o = L.ord[j];
+    const int g = (int)o.x;
+    const int info = P.info[g];
+    const float4 p = P.pos[g], v = P.vel[g];
+    const unsigned long long id = P.pid[g];
+    const int t = info & INFO_TYPE_MASK, kd = min(kind_of(info), (int)K_OTHER);
+    L.pos[j] = make_float4(frame_x(p.x, strad, 0, P.halfL, P.Lf), frame_x(p.y, strad, 1, P.halfL, P.Lf),
+                           frame_x(p.z, strad, 2, P.halfL, P.Lf), p.w);
+    L.vel[j] = v;
+    L.id[j] = id;
+    L.lnk[j] = (t == CR_ACID || t == CR_BASE) ? P.lnK_fx[info >> INFO_SITE_SHIFT] : 0ll;
+    L.info[j] = info;
+    L.ord[j] = make_uint2((unsigned)j | ((unsigned)kd << ORD_KIND_SHIFT), o.y);
+    atomicAdd(&misc[1 + kd], 1);
   }
   if (DA) {  // region cell aggregates at the start of the phase
     for (int i = tid; i < NR; i += T) {
-      const int ix = i % nr, iy = (i / nr) % nr, iz = i / (nr * nr);
-      const int cell = region_coord(ix, org[0], k, h, nr, nc) +
-                       nc * (region_coord(iy, org[1], k, h, nr, nc) + nc * region_coord(iz, org[2], k, h, nr, nc));
-      const int cn = P.cnt[cell];
+      const int cell = hcell[i], cn = P.cnt[cell];
       int qi = 0, qs = 0;
       for (int sl = 0; sl < cn; ++sl) {
         const int g = cell * P.cap + sl;
@@ -1385,44 +1443,44 @@ __device__ __forceinline__ void phase_task(unsigned char *smem, const SysParams 
       aN[i] = cn;
     }
   }
-  if (tid == 0) misc[0] = ND;
   __syncthreads();
   if (tid < N_KIND) misc[MISC_INIT + tid] = misc[1 + tid];
-  const int cc_thread = NW > 1 ? 32 : 0;  // the thread that adds the changed-pair term
-  const long long log_dom = (long long)(sweep - sweep0) * P.per_sweep + (long long)colour * P.nact * m +
-                            (long long)bdom * m;
+  TrialCtl &ctl = ctls[group];
+  // the CTA's statistics: lane l of each group's first warp counts entry l
+  unsigned stat = 0u;
 
-  for (int k0 = 0; k0 < m; k0 += S.chunk) {
-    const int nchunk = min(S.chunk, m - k0);
+  for (int k0 = 0; k0 < P.m; k0 += S.chunk) {
+    const int nchunk = min(S.chunk, P.m - k0);
     // ---- random numbers of the chunk
-    draw_chunk<LOG, DA>(tp, tvel, k0, nchunk, tid, T, d, phi, org[0], org[1], org[2], off[0], off[1], off[2], dd[0],
-                        dd[1], dd[2], k, nc, P.af, P.Lf, P.scf, key0, key1);
+    draw_chunk<LOG, DA>(P, D, tp, tvel, k0, nchunk, tid, T);
     __syncthreads();
 
-    for (int t = 0; t < nchunk; ++t) {
-      const int kk = k0 + t;
-      // ---- warp 0: proposal and participants; the selection lives in
-      // shared memory (*ctl) across the sweep
-      if (warp == 0) select_trial<DA>(P, L, misc, lnt, tp[t], d, m, kk, phi, *ctl);
-      cta_sync<T>();
+    for (int t0 = 0; t0 < nchunk;) {
+      const int t = t0 + group, kk = k0 + t;
+      const bool mine = W == 1 || t < nchunk;  // uniform over the group
+      // ---- the group's first warp: proposal and participants; the selection
+      // lives in shared memory across the sweep
+      if (mine && gwarp == 0) select_trial<DA>(P, D, misc, tp[t], kk, ctl);
+      group_sync<G>(group);
       // Ewald (global schedule): the changed particles' phase factors
-      const bool ew = !DA && P.ewald_nk > 0 && ctl->nch;
+      const bool ew = !DA && W == 1 && P.ewald_nk > 0 && ctl.nch;
       if (ew) {
-        ewald_factors(P, *ctl, ewf, ewq, S.ewk, tid, T);
-        cta_sync<T>();
+        ewald_factors(P, ctl, ewf, ewq, S.ewk, tid, T);
+        __syncthreads();
       }
-      // ---- delayed acceptance, stage 1: surrogate features and MLP (all
-      // threads), decision in warp 0; a rejection skips the pair sweep
-      if (DA && ctl->nch) {
-        if (tid < MLP_IN) dfeat[tid] = 0;
-        cta_sync<T>();
-        const int rka = ctl->rka, rkb = ctl->rkb;
-        const int dqa = ctl->dqa, dqb = ctl->dqb, ea = ctl->eta_a, eb = ctl->eta_b;
-        for (int it = tid; it < 250; it += T) {  // 2 changed particles x 125 stencil cells
+      // ---- delayed acceptance, stage 1: surrogate features and MLP (all of
+      // the group's threads), decision in its first warp; a rejection skips
+      // the pair sweep
+      if (DA && mine && ctl.nch) {
+        for (int i = gtid; i < MLP_IN; i += GT) dfeat[i] = 0;
+        group_sync<G>(group);
+        const int rka = ctl.rka, rkb = ctl.rkb;
+        const int dqa = ctl.dqa, dqb = ctl.dqb, ea = ctl.eta_a, eb = ctl.eta_b;
+        for (int it = gtid; it < 250; it += GT) {  // 2 changed particles x 125 stencil cells
           const int sb = it >= 125 ? 1 : 0;
           const int c = it - 125 * sb;
           const int dx = c % 5 - 2, dy = (c / 5) % 5 - 2, dz = c / 25 - 2;
-          const int ri = region_of(sb ? rkb : rka, dx, dy, dz, k, nr);
+          const int ri = region_of(sb ? rkb : rka, dx, dy, dz, P.k, P.nr);
           const int sh = shell_of_n2(dx * dx + dy * dy + dz * dz);
           const int dq = sb ? dqb : dqa, eta = sb ? eb : ea;
           if (dq != 0) {
@@ -1432,39 +1490,39 @@ __device__ __forceinline__ void phase_task(unsigned char *smem, const SysParams 
           }
           if (eta != 0 && aN[ri]) atomicAdd(&dfeat[24 * sb + 16 + sh], eta * aN[ri]);
         }
-        cta_sync<T>();
-        if (tid == 0) {  // the changed particles themselves do not count; the a-b pair term
-          const TrialCtl &C = *ctl;
+        group_sync<G>(group);
+        if (gtid == 0) {  // the changed particles themselves do not count; the a-b pair term
+          const TrialCtl &C = ctl;
           const int qao = __float2int_rn(C.qa_o), qan = __float2int_rn(C.qa_n);
           const int qbo = __float2int_rn(C.qb_o), qbn = __float2int_rn(C.qb_n);
           for (int sb = 0; sb < 2; ++sb) {
             const int rs = sb ? rkb : rka, dq = sb ? dqb : dqa, eta = sb ? eb : ea;
             for (int x = 0; x < 2; ++x) {
               if (!(x ? C.pb_o : C.pa_o)) continue;
-              const int sh = shell_ranks(rs, x ? rkb : rka, k);
+              const int sh = shell_ranks(rs, x ? rkb : rka, P.k);
               if (sh < 0) continue;
               dfeat[24 * sb + (x ? 0 : C.cat_a) + sh] -= dq * (x ? qbo : qao);
               dfeat[24 * sb + 16 + sh] -= eta;
             }
           }
-          const int sh = shell_ranks(rka, rkb, k);
+          const int sh = shell_ranks(rka, rkb, P.k);
           if (sh >= 0) dfeat[sh] += (C.pa_n && C.pb_n ? qan * qbn : 0) - (C.pa_o && C.pb_o ? qao * qbo : 0);
         }
-        cta_sync<T>();
-        if (tid < MLP_IN) {
-          const float f = (float)dfeat[tid];
-          fv[tid] = f;
-          fv[MLP_IN + tid] = -f;
-          if (LOG && P.feat_log) P.feat_log[(size_t)(log_dom + kk) * MLP_IN + tid] = f;
+        group_sync<G>(group);
+        for (int i = gtid; i < MLP_IN; i += GT) {
+          const float f = (float)dfeat[i];
+          fv[i] = f;
+          fv[MLP_IN + i] = -f;
+          if (LOG && P.feat_log) P.feat_log[(size_t)(D.log_dom + kk) * MLP_IN + i] = f;
         }
-        cta_sync<T>();
-        mlp_layer<T>(P.mlp_w + MLPW_W1, P.mlp_b, fv, MLP_IN, hb0);
-        cta_sync<T>();
-        mlp_layer<T>(P.mlp_w + MLPW_W2, P.mlp_b + MLP_H, hb0, MLP_H, hb1);
-        cta_sync<T>();
-        mlp_layer<T>(P.mlp_w + MLPW_W3, P.mlp_b + 2 * MLP_H, hb1, MLP_H, hb0);
-        cta_sync<T>();
-        if (warp == 0) {
+        group_sync<G>(group);
+        mlp_layer<GT>(P.mlp_w + MLPW_W1, P.mlp_b, fv, MLP_IN, hb0, gtid);
+        group_sync<G>(group);
+        mlp_layer<GT>(P.mlp_w + MLPW_W2, P.mlp_b + MLP_H, hb0, MLP_H, hb1, gtid);
+        group_sync<G>(group);
+        mlp_layer<GT>(P.mlp_w + MLPW_W3, P.mlp_b + 2 * MLP_H, hb1, MLP_H, hb0, gtid);
+        group_sync<G>(group);
+        if (gwarp == 0) {
           float y = 0.0f;
           if (lane < 2) {
             y = __ldg(&P.mlp_b[3 * MLP_H]);
@@ -1479,29 +1537,32 @@ __device__ __forceinline__ void phase_task(unsigned char *smem, const SysParams 
           long long sur_fx = 0;
           if (sur == sur) {
             sur_fx = __double2ll_rn((double)fminf(fmaxf(sur, -16384.0f), 16384.0f) * LNFIX);
-            s1 = accept_fx(ctl->ln_ratio_fx - ctl->dself_fx - sur_fx, tp[t].lnu_f, tp[t].uhi, tp[t].ulo);
+            s1 = accept_fx(ctl.ln_ratio_fx - ctl.dself_fx - sur_fx, tp[t].lnu_f, tp[t].uhi, tp[t].ulo);
           }
           if (lane == 0) {
-            ctl->go = s1 ? 1 : 0;
-            ctl->sur = sur;
-            ctl->sur_fx = sur_fx;
+            ctl.go = s1 ? 1 : 0;
+            ctl.sur = sur;
+            ctl.sur_fx = sur_fx;
           }
         }
-        cta_sync<T>();
-      } else if (DA && LOG && P.feat_log && tid < MLP_IN) {
-        P.feat_log[(size_t)(log_dom + kk) * MLP_IN + tid] = 0.0f;
+        group_sync<G>(group);
+      } else if (DA && mine && LOG && P.feat_log) {
+        for (int i = gtid; i < MLP_IN; i += GT) P.feat_log[(size_t)(D.log_dom + kk) * MLP_IN + i] = 0.0f;
       }
-      // ---- all threads: the pair-change sweep
-      const int nch = (DA && !LOG && !ctl->go) ? 0 : ctl->nch;
+      // ---- the group: the pair-change sweep
+      const int nch = !mine || (DA && !LOG && !ctl.go) ? 0 : ctl.nch;
       long long acc = 0;
       unsigned long long sacc = 0;
       int ov = 0;
       if (nch) {
-        const Desc A = ctl->c[0], B = ctl->c[1];
-        sweep_pairs<LOG, R, RR>(K, wca, P, L, A, B, hreg, nmine, hpos, NH, hcap, hpre, hcell, NR, misc[0], tid, T,
-                                qr2, qqp, acc, sacc, ov, flat, strad, ctl);
-        if (tid == cc_thread) {
-          const PairSum cc = cc_change<LOG>(P, *ctl);
+        const int nlist = misc[MISC_HW];
+        const PairSum ps = D.flat ? sweep_pairs<LOG, true>(pair_k(P), P, ctl, D, cpos, hcls, nlist, gtid, GT, queue)
+                                  : sweep_general<LOG>(P, ctl, D, cpos, hcls, nlist, gtid, GT, queue);
+        acc = ps.acc;
+        sacc = ps.sacc;
+        ov = ps.ov;
+        if (gtid == (G > 1 ? 32 : 0)) {  // one thread adds the changed pair itself
+          const PairSum cc = cc_change<LOG>(P, ctl);
           acc += cc.acc;
           sacc += cc.sacc;
           ov |= cc.ov;
@@ -1512,37 +1573,36 @@ __device__ __forceinline__ void phase_task(unsigned char *smem, const SysParams 
           sacc += e.sacc;
           ov |= e.ov;
         }
-        acc = warp_allsum(acc);
-        if (LOG) sacc = (unsigned long long)warp_allsum((long long)sacc);
+        acc = warp_sum_i64(acc);
+        if (LOG) sacc = (unsigned long long)warp_sum_i64((long long)sacc);
         ov = __any_sync(FULL, ov) ? 1 : 0;
-        if (NW > 1 && lane == 0) {
+        if (G > 1 && lane == 0) {
           red[warp] = acc;
           reds[warp] = sacc;
           redov[warp] = ov;
         }
       }
-      if (NW > 1) __syncthreads();
-      // ---- warp 0: decision and commit
-      if (warp == 0) {
+      if (G > 1) group_sync<G>(group);
+      // ---- the group's first warp: decision
+      bool accept = false;
+      int flags = 0;
+      double dE = 0.0, Ssum = 0.0, lnA = -INFINITY, lnA2r = quiet_nan();  // records only
+      const bool s1 = !DA || ctl.go != 0;
+      if (mine && gwarp == 0) {
         const TrialPre &q = tp[t];
-        const int s_move = ctl->move, s_nch = ctl->nch;
-        const long long s_ln_ratio = ctl->ln_ratio_fx, s_dself = ctl->dself_fx;
-        const unsigned long long s_id_a = ctl->id_a, s_id_b = ctl->id_b;
-        const bool s1 = !DA || ctl->go != 0;
-        const float sur = DA ? ctl->sur : 0.0f;
-        const long long sur_fx = DA ? ctl->sur_fx : 0ll;
-        int flags = ctl->flags;
-        bool accept = false;
-        double dE = 0.0, Ssum = 0.0, lnA = -INFINITY, lnA2r = quiet_nan();
+        const int s_nch = ctl.nch;
+        const long long s_ln_ratio = ctl.ln_ratio_fx, s_dself = ctl.dself_fx;
+        const float sur = DA ? ctl.sur : 0.0f;
+        flags = ctl.flags;
         if (DA && LOG && s_nch) lnA = (double)s_ln_ratio / LNFIX - (double)s_dself / LNFIX - (double)sur;
         if (s_nch && (!DA || LOG || s1)) {
           long long tot = acc;
           unsigned long long stot = sacc;
           int anyov = ov;
-          if (NW > 1) {
-            tot = warp_allsum(lane < NW ? red[lane] : 0ll);
-            if (LOG) stot = (unsigned long long)warp_allsum(lane < NW ? (long long)reds[lane] : 0ll);
-            anyov = __any_sync(FULL, lane < NW && redov[lane]) ? 1 : 0;
+          if (G > 1) {
+            tot = warp_sum_i64(lane < G ? red[warp + lane] : 0ll);
+            if (LOG) stot = (unsigned long long)warp_sum_i64(lane < G ? (long long)reds[warp + lane] : 0ll);
+            anyov = __any_sync(FULL, lane < G && redov[warp + lane]) ? 1 : 0;
           }
           if (anyov) {
             if (!DA || s1) flags |= CR_TRIAL_OVERLAP;  // DA: only an exact evaluation that decides
@@ -1550,7 +1610,7 @@ __device__ __forceinline__ void phase_task(unsigned char *smem, const SysParams 
           } else {
             const long long totc = tot > DE_CLAMP32 ? DE_CLAMP32 : (tot < -DE_CLAMP32 ? -DE_CLAMP32 : tot);
             if (DA) {  // stage 2: ln u2 < dE~ - dE_pair
-              if (s1) accept = accept_fx(sur_fx - (totc << 16), q.lnu2_f, q.u2hi, q.u2lo);
+              if (s1) accept = accept_fx(ctl.sur_fx - (totc << 16), q.lnu2_f, q.u2hi, q.u2lo);
             } else {
               accept = accept_fx(s_ln_ratio - ((totc << 16) + s_dself), q.lnu_f, q.uhi, q.ulo);
             }
@@ -1562,28 +1622,20 @@ __device__ __forceinline__ void phase_task(unsigned char *smem, const SysParams 
             }
           }
         }
-        const int r = s_move >> 1;
-        const bool fwd = (s_move & 1) == 0;
-        int n = misc[0];
-        if (accept) {  // commit, unless an insertion finds no room (checked before anything changes)
-          const int n2 = try_commit(P, L.pos, L.vel, L.id, L.lnk, L.info, L.rank, misc, *ctl, q, tvel + 2 * t, n,
-                                    in_smem ? S.dcs : P.dcap_glob);
-          if (n2 < 0) {
-            accept = false;
-            if (lane == 0) atomicOr(P.err, ERRB_CELL_OVERFLOW);
-          } else {
-            n = n2;
-          }
-        }
-        (void)r;
-        (void)fwd;
-        if (lane == 0) ctl->ewacc = accept ? 1 : 0;
-        if (accept) {
+      }
+      // ---- commit, unless an insertion finds no room (checked before
+      // anything changes)
+      if (accept) {
+        const int n2 = try_commit(P, D, misc, ctl, tp[t], tvel + 2 * t, misc[0]);
+        if (n2 < 0) {
+          accept = false;
+          if (lane == 0) atomicOr(P.err, ERRB_CELL_OVERFLOW);
+        } else {
           flags |= CR_TRIAL_ACCEPTED;
           if (DA && lane == 0) {  // region aggregates follow the committed change
-            const TrialCtl &C = *ctl;
+            const TrialCtl &C = ctl;
             for (int x = 0; x < 2; ++x) {
-              const int ri = region_of(x ? C.rkb : C.rka, 0, 0, 0, k, nr);
+              const int ri = region_of(x ? C.rkb : C.rka, 0, 0, 0, P.k, P.nr);
               int *aq = (x == 0 && C.cat_a == 8) ? aQs : aQi;
               if (x ? C.pb_o : C.pa_o) {
                 aq[ri] -= __float2int_rn(x ? C.qb_o : C.qa_o);
@@ -1596,80 +1648,90 @@ __device__ __forceinline__ void phase_task(unsigned char *smem, const SysParams 
             }
           }
         }
+      }
+      if (mine && gwarp == 0) {
+        const unsigned hit = (1u << ctl.move) | (accept ? 64u << ctl.move : 0u) |
+                             (flags & CR_TRIAL_NO_ELIGIBLE ? 1u << 12 : 0u) |
+                             (flags & CR_TRIAL_EDGE ? 1u << 13 : 0u) | (flags & CR_TRIAL_OVERLAP ? 1u << 14 : 0u) |
+                             (1u << 15);
+        stat += (hit >> lane) & 1u;
         if (lane == 0) {
-          misc[0] = n;
-          st[s_move] += 1;
-          if (flags & CR_TRIAL_ACCEPTED) st[6 + s_move] += 1;
-          if (flags & CR_TRIAL_NO_ELIGIBLE) st[12] += 1;
-          if (flags & CR_TRIAL_EDGE) st[13] += 1;
-          if (flags & CR_TRIAL_OVERLAP) st[14] += 1;
-          st[15] += 1;
+          ctl.ewacc = accept ? 1 : 0;
           if (LOG && P.log) {
             cr_trial rec;
-            rec.move = s_move;
+            rec.move = ctl.move;
             rec.flags = flags;
-            rec.id_a = s_id_a;
-            rec.id_b = s_id_b;
+            rec.id_a = ctl.id_a;
+            rec.id_b = ctl.id_b;
             rec.dE = dE;
             rec.S = Ssum;
             rec.lnA = lnA;
-            rec.lnu = q.lnu;
-            P.log[log_dom + kk] = rec;
+            rec.lnu = tp[t].lnu;
+            P.log[D.log_dom + kk] = rec;
             if (DA && P.dlog) {
               cr_trial_da dr;
-              dr.dE_sur = s_nch ? sur : 0.0f;
-              dr.stage = s_nch ? (s1 ? 2 : 1) : 0;
+              dr.dE_sur = ctl.nch ? ctl.sur : 0.0f;
+              dr.stage = ctl.nch ? (s1 ? 2 : 1) : 0;
               dr.lnA2 = lnA2r;
-              dr.lnu2 = s_nch ? q.lnu2 : quiet_nan();
-              P.dlog[log_dom + kk] = dr;
+              dr.lnu2 = ctl.nch ? tp[t].lnu2 : quiet_nan();
+              P.dlog[D.log_dom + kk] = dr;
             }
           }
         }
       }
-      cta_sync<T>();
-      if (ew && ctl->ewacc) ewald_update(P, ewf, ewq, S.ewk, tid, T);
+      t0 += 1;
+      if (ew) {
+        __syncthreads();
+        if (ctl.ewacc) ewald_update(P, ewf, ewq, S.ewk, tid, T);
+      }
+      // (the other warps wait for the first one's next selection at the
+      // group's barrier; what they read of this trial they have read)
     }
+    __syncthreads();  // the chunk's numbers have been read
   }
-  // ---- write the domain back (id-sorted cells) and publish counts
-  __syncthreads();
-  const int n = misc[0];
-  for (int r = tid; r < KC; r += T) {
-    int lo = 0, hi = n;  // first entry with rank >= r
-    while (lo < hi) { const int mid = (lo + hi) >> 1; if (L.rank[mid] < r) lo = mid + 1; else hi = mid; }
-    int lo2 = lo, hi2 = n;  // first entry with rank > r
-    while (lo2 < hi2) { const int mid = (lo2 + hi2) >> 1; if (L.rank[mid] <= r) lo2 = mid + 1; else hi2 = mid; }
-    dcnt[r] = lo;
-    const int lx = r % k, ly = (r / k) % k, lz = r / (k * k);
-    P.cnt[(org[0] + lx) % nc + nc * ((org[1] + ly) % nc + nc * ((org[2] + lz) % nc))] = lo2 - lo;
+  // ---- write the domain back (id-sorted cells), if anything changed, and
+  // publish the counts
+  if (misc[MISC_DIRTY]) {
+    const DomList L = D.L;
+    const int n = misc[0], KC = P.k * P.k * P.k;
+    for (int r = tid; r < KC; r += T) {
+      int lo = 0, hi = n;  // first entry with rank >= r
+      while (lo < hi) { const int mid = (lo + hi) >> 1; if ((int)L.ord[mid].y < r) lo = mid + 1; else hi = mid; }
+      int lo2 = lo, hi2 = n;  // first entry with rank > r
+      while (lo2 < hi2) { const int mid = (lo2 + hi2) >> 1; if ((int)L.ord[mid].y <= r) lo2 = mid + 1; else hi2 = mid; }
+      dcnt[r] = lo;
+      P.cnt[dcell[r]] = lo2 - lo;
+    }
+    __syncthreads();
+    for (int j = tid; j < n; j += T) {
+      const uint2 o = L.ord[j];
+      const int sl = (int)(o.x & ORD_SLOT_MASK);
+      const int g = dcell[o.y] * P.cap + (j - dcnt[o.y]);
+      const unsigned long long id = L.id[sl];
+      P.pos[g] = raw_pos(L, sl, P.Lf);
+      P.vel[g] = L.vel[sl];
+      P.pid[g] = id;
+      P.info[g] = L.info[sl];
+      if (id < (unsigned long long)P.n_perm) P.perm_slot[id] = g;
+    }
+    if (tid < N_KIND && misc[1 + tid] != misc[MISC_INIT + tid])
+      atomicAdd((unsigned long long *)&P.counts[tid],
+                (unsigned long long)(long long)(misc[1 + tid] - misc[MISC_INIT + tid]));
   }
-  __syncthreads();
-  for (int j = tid; j < n; j += T) {
-    const int r = L.rank[j];
-    const int lx = r % k, ly = (r / k) % k, lz = r / (k * k);
-    const int cell = (org[0] + lx) % nc + nc * ((org[1] + ly) % nc + nc * ((org[2] + lz) % nc));
-    const int g = cell * P.cap + (j - dcnt[r]);
-    const unsigned long long id = L.id[j];
-    P.pos[g] = L.pos[j];
-    P.vel[g] = L.vel[j];
-    P.pid[g] = id;
-    P.info[g] = L.info[j];
-    if (id < (unsigned long long)P.n_perm) P.perm_slot[id] = g;
-  }
-  if (tid < 16 && st[tid]) atomicAdd(&P.stats[tid], st[tid]);
-  if (tid < N_KIND && misc[1 + tid] != misc[MISC_INIT + tid])
-    atomicAdd((unsigned long long *)&P.counts[tid],
-              (unsigned long long)(long long)(misc[1 + tid] - misc[MISC_INIT + tid]));
+  if (gwarp == 0 && lane < 16 && stat) atomicAdd(&P.stats[lane], (unsigned long long)stat);
+#undef CRMC_AT
 }
 
 // ---------------------------------------------------------------------------
-// the phase kernel: one CTA per active domain of one colour
-//   T threads per domain (T == 32: one warp, no block barriers);
-//   R > 0: halo particles in R registers per thread, R == 0: in shared memory
+// the phase kernel: one CTA per active domain of one colour, of W groups of G
+// warps (G == 1, W == 1: one warp, no block barriers)
 // ---------------------------------------------------------------------------
-template <int T, int R, bool LOG, bool DA>
-__global__ void __launch_bounds__(T, (T <= 32 ? 16 : (T <= 64 ? 8 : (T <= 128 ? 4 : (T <= 256 ? 2 : 1)))))
-    k_cr_phase(const SysParams *__restrict__ reps, PhaseShape S, uint32_t sweep, uint32_t sweep0, int colour,
-               uint32_t key0, uint32_t key1_base, const StepDyn *dyn) {
+constexpr int min_ctas(int T) { return T <= 32 ? 16 : (T <= 64 ? 8 : (T <= 128 ? 4 : (T <= 256 ? 2 : 1))); }
+
+template <int G, int W, bool LOG, bool DA>
+__global__ void __launch_bounds__(32 * G * W, min_ctas(32 * G * W))
+    k_cr_phase(const SysParams *__restrict__ reps, const __grid_constant__ PhaseShape S, uint32_t sweep,
+               uint32_t sweep0, int colour, uint32_t key0, uint32_t key1_base, const StepDyn *dyn) {
   extern __shared__ __align__(16) unsigned char smem[];
   if (dyn) {  // a captured cycle: this step's sweep counter and key
     const unsigned long long step = dyn->step, seed = dyn->sweep_seed0 + step;
@@ -1677,7 +1739,7 @@ __global__ void __launch_bounds__(T, (T <= 32 ? 16 : (T <= 64 ? 8 : (T <= 128 ? 
     key0 = (uint32_t)seed;
     key1_base = (uint32_t)(seed >> 32);
   }
-  phase_task<T, R, LOG, DA>(smem, reps, S, sweep, sweep0, colour, key0, key1_base, (int)blockIdx.x,
+  phase_task<G, W, LOG, DA>(smem, reps, S, sweep, sweep0, colour, key0, key1_base, (int)blockIdx.x,
                             (int)blockIdx.y);
 }
 
@@ -1737,10 +1799,10 @@ __device__ __forceinline__ bool wait_at_least(const unsigned *p, unsigned need, 
   return true;
 }
 
-template <int T, int R, bool DA>
-__global__ void __launch_bounds__(T, (T <= 32 ? 16 : (T <= 64 ? 8 : (T <= 128 ? 4 : (T <= 256 ? 2 : 1)))))
-    k_cr_sweep(const SysParams *__restrict__ reps, PhaseShape S, uint32_t sweep, uint32_t sweep0, uint32_t key0,
-               uint32_t key1_base, SweepSched Q, const StepDyn *dyn) {
+template <int G, int W, bool DA>
+__global__ void __launch_bounds__(32 * G * W, min_ctas(32 * G * W))
+    k_cr_sweep(const SysParams *__restrict__ reps, const __grid_constant__ PhaseShape S, uint32_t sweep,
+               uint32_t sweep0, uint32_t key0, uint32_t key1_base, SweepSched Q, const StepDyn *dyn) {
   extern __shared__ __align__(16) unsigned char smem[];
   if (dyn) {  // a captured cycle: this step's sweep counter and key
     const unsigned long long step = dyn->step, seed = dyn->sweep_seed0 + step;
@@ -1801,7 +1863,7 @@ __global__ void __launch_bounds__(T, (T <= 32 ? 16 : (T <= 64 ? 8 : (T <= 128 ? 
     int r = 0;
     while (Q.rep_first[r + 1] <= q) ++r;
     if (s_run)
-      phase_task<T, R, false, DA>(smem, reps, S, sweep, sweep0, c, key0, key1_base, r, q - Q.rep_first[r]);
+      phase_task<G, W, false, DA>(smem, reps, S, sweep, sweep0, c, key0, key1_base, r, q - Q.rep_first[r]);
     __syncthreads();  // the task's stores are done, its shared memory is free
     if (threadIdx.x == 0 && !(r == Q.withhold_rep && c == 0)) {
       __threadfence();
@@ -1811,23 +1873,23 @@ __global__ void __launch_bounds__(T, (T <= 32 ? 16 : (T <= 64 ? 8 : (T <= 128 ? 
   }
 }
 
-template <int T, int R, bool DA>
+template <int G, int W, bool DA>
 static cudaError_t launch_sweep_t(const SysParams *d_reps, PhaseShape S, cudaStream_t s, uint32_t sweep,
                                   uint32_t sweep0, uint32_t k0, uint32_t k1, const SweepSched &Q, int max_ctas,
                                   const StepDyn *dyn) {
-  if (R > 0) S.hcs = 0;  // halo in registers
+  constexpr int T = 32 * G * W;
   static size_t attr_bytes = 0;
   static int per_sm = 0;
   static size_t per_sm_bytes = ~(size_t)0;
-  const size_t smem = phase_smem_bytes(S, T, DA);
+  const size_t smem = phase_layout(S, T / 32, W, DA);
   if (smem > attr_bytes) {
-    cudaError_t e = cudaFuncSetAttribute(k_cr_sweep<T, R, DA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k_cr_sweep<G, W, DA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     attr_bytes = smem;
   }
   if (smem != per_sm_bytes) {  // resident CTAs per SM at this shared-memory size
     int nb = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_cr_sweep<T, R, DA>, T, smem);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_cr_sweep<G, W, DA>, T, smem);
     if (e != cudaSuccess) return e;
     per_sm = std::max(nb, 1);
     per_sm_bytes = smem;
@@ -1839,28 +1901,27 @@ static cudaError_t launch_sweep_t(const SysParams *d_reps, PhaseShape S, cudaStr
   int grid = std::min(total, per_sm * std::max(sms, 1));
   if (max_ctas > 0) grid = std::min(grid, max_ctas);
   if (grid <= 0) return cudaSuccess;
-  k_cr_sweep<T, R, DA><<<grid, T, smem, s>>>(d_reps, S, sweep, sweep0, k0, k1, Q, dyn);
+  k_cr_sweep<G, W, DA><<<grid, T, smem, s>>>(d_reps, S, sweep, sweep0, k0, k1, Q, dyn);
   return cudaGetLastError();
 }
 
-cudaError_t launch_sweep(const SysParams *d_reps, const PhaseShape &S, int threads, int R, bool da, cudaStream_t s,
+// the instantiated shapes: X(threads, groups), for plain and delayed-acceptance sweeps
+#define CRMC_SHAPES(X) X(32, 1) X(64, 1) X(128, 1) X(256, 1) X(512, 1)
+#define CRMC_SHAPES_DA(X) X(128, 1) X(256, 1) X(512, 1)
+
+cudaError_t launch_sweep(const SysParams *d_reps, const PhaseShape &S, int threads, int groups, bool da, cudaStream_t s,
                          uint32_t sweep, uint32_t sweep0, uint32_t k0, uint32_t k1, const SweepSched &Q,
                          int max_ctas, const StepDyn *dyn) {
-#define CRMC_SW(TT, RR, DD)                                                                   \
-  if (da == DD && threads == TT && R == RR)                                                    \
-    return launch_sweep_t<TT, RR, DD>(d_reps, S, s, sweep, sweep0, k0, k1, Q, max_ctas, dyn);
-  CRMC_SW(32, 0, false)
-  CRMC_SW(64, 0, false)
-  CRMC_SW(128, 0, false)
-  CRMC_SW(128, 4, false)
-  CRMC_SW(256, 0, false)
-  CRMC_SW(256, 2, false)
-  CRMC_SW(512, 0, false)
-  CRMC_SW(512, 1, false)
-  CRMC_SW(128, 0, true)
-  CRMC_SW(256, 0, true)
-  CRMC_SW(512, 0, true)
+#define CRMC_SW(TT, WW, DD)             \
+  if (da == DD && threads == TT && groups == WW) \
+    return launch_sweep_t<TT / 32 / WW, WW, DD>(d_reps, S, s, sweep, sweep0, k0, k1, Q, max_ctas, dyn);
+#define CRMC_SW_PLAIN(TT, WW) CRMC_SW(TT, WW, false)
+#define CRMC_SW_DA(TT, WW) CRMC_SW(TT, WW, true)
+  CRMC_SHAPES(CRMC_SW_PLAIN)
+  CRMC_SHAPES_DA(CRMC_SW_DA)
 #undef CRMC_SW
+#undef CRMC_SW_PLAIN
+#undef CRMC_SW_DA
   return cudaErrorInvalidValue;
 }
 
@@ -2025,109 +2086,69 @@ cudaError_t launch_ewald_sk(const SysParams *d_reps, int n_rep, int max_nk, cuda
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
-size_t phase_smem_bytes(const PhaseShape &S, int threads, bool da) {
-  const size_t sizes[] = {sizeof(SysParams),
-                          sizeof(float4) * S.dcs,
-                          sizeof(float4) * S.dcs,
-                          sizeof(unsigned long long) * S.dcs,
-                          sizeof(long long) * S.dcs,
-                          sizeof(int) * S.dcs,
-                          sizeof(int) * S.dcs,
-                          sizeof(float4) * S.hcs,
-                          sizeof(long long) * S.lns,
-                          sizeof(TrialPre) * S.chunk,
-                          sizeof(float4) * 2 * S.chunk,
-                          sizeof(TrialCtl),
-                          sizeof(long long) * MAX_WARPS,
-                          sizeof(unsigned long long) * MAX_WARPS,
-                          sizeof(unsigned long long) * 16,
-                          sizeof(float) * 2 * QCAP * (threads / 32),
-                          sizeof(int) * MAX_WARPS,
-                          sizeof(int) * 32,
-                          sizeof(int) * MISC_N,
-                          sizeof(int) * (S.nr3 + 1),
-                          sizeof(int) * (S.nr3 + 1),
-                          sizeof(int) * (S.nr3 + 1),
-                          sizeof(int) * (S.kc3 + 1),
-                          sizeof(int) * (S.kc3 + 1),
-                          sizeof(float2) * 6 * S.ewk,
-                          sizeof(float) * 4};
-  size_t b = 0;
-  for (size_t x : sizes) b += (x + 15) / 16 * 16;
-  if (da) {
-    const size_t dsz[] = {sizeof(int) * (S.nr3 + 1), sizeof(int) * (S.nr3 + 1), sizeof(int) * (S.nr3 + 1),
-                          sizeof(int) * MLP_IN,      sizeof(float) * 2 * MLP_IN, sizeof(float) * 2 * MLP_H,
-                          sizeof(float) * 2 * MLP_H};
-    for (size_t x : dsz) b += (x + 15) / 16 * 16;
-  }
-  return b;
+size_t phase_smem_bytes(const PhaseShape &S, int threads, int groups, bool da) {
+  PhaseShape Q = S;
+  return phase_layout(Q, threads / 32, groups, da);
 }
 
-template <int T, int R, bool LOG, bool DA>
+template <int G, int W, bool LOG, bool DA>
 static cudaError_t launch_phase_t(const SysParams *d_reps, int n_rep, int grid_x, PhaseShape S, cudaStream_t s,
                                   uint32_t sweep, uint32_t sweep0, int colour, uint32_t k0, uint32_t k1,
                                   const StepDyn *dyn) {
-  if (R > 0) S.hcs = 0;  // halo in registers
+  constexpr int T = 32 * G * W;
   static size_t attr_bytes = 0;
-  const size_t smem = phase_smem_bytes(S, T, DA);
+  const size_t smem = phase_layout(S, T / 32, W, DA);
   if (smem > attr_bytes) {
     cudaError_t e =
-        cudaFuncSetAttribute(k_cr_phase<T, R, LOG, DA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(k_cr_phase<G, W, LOG, DA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     attr_bytes = smem;
   }
-  k_cr_phase<T, R, LOG, DA><<<dim3(n_rep, grid_x), T, smem, s>>>(d_reps, S, sweep, sweep0, colour, k0, k1, dyn);
+  k_cr_phase<G, W, LOG, DA><<<dim3(n_rep, grid_x), T, smem, s>>>(d_reps, S, sweep, sweep0, colour, k0, k1, dyn);
   return cudaGetLastError();
 }
 
-// variants the autotuner picks from: (threads per CTA, halo registers per
-// thread (0: the halo in shared memory), compact).  Compact variants size the
-// shared-memory list and halo for most domains rather than the densest
-// (denser ones spill to global memory), so that more CTAs fit on an SM.
-static const int kShapes[][3] = {{32, 0, 0},  {64, 0, 0},  {128, 0, 0}, {128, 4, 0}, {256, 0, 0}, {256, 2, 0},
-                                 {512, 0, 0}, {512, 1, 0}, {32, 0, 1},  {64, 0, 1},  {128, 0, 1}, {256, 0, 1}};
+// variants the autotuner picks from: (threads per CTA, groups, compact).
+// Compact variants size the shared-memory list and halo for most domains
+// rather than the densest (denser ones spill to global memory), so that more
+// CTAs fit on an SM.
+static const int kShapes[][3] = {{32, 1, 0},  {64, 1, 0}, {128, 1, 0}, {256, 1, 0}, {512, 1, 0},
+                                 {32, 1, 1},  {64, 1, 1}, {128, 1, 1}, {256, 1, 1}};
 
 // shapes with a delayed-acceptance variant (the surrogate runs on >= 128 threads)
-static const int kShapesDA[][3] = {{128, 0, 0}, {256, 0, 0}, {512, 0, 0}, {128, 0, 1}, {256, 0, 1}};
+static const int kShapesDA[][3] = {{128, 1, 0}, {256, 1, 0}, {512, 1, 0}, {128, 1, 1}, {256, 1, 1}};
 
 int phase_shape_count(bool da) {
   return da ? (int)(sizeof(kShapesDA) / sizeof(kShapesDA[0])) : (int)(sizeof(kShapes) / sizeof(kShapes[0]));
 }
-void phase_shape(int i, int *threads, int *regs, bool da) {
+void phase_shape(int i, int *threads, int *groups, bool da) {
   *threads = da ? kShapesDA[i][0] : kShapes[i][0];
-  *regs = da ? kShapesDA[i][1] : kShapes[i][1];
+  *groups = da ? kShapesDA[i][1] : kShapes[i][1];
 }
 bool phase_shape_compact(int i, bool da) { return (da ? kShapesDA[i][2] : kShapes[i][2]) != 0; }
 
-size_t phase_shape_smem(const PhaseShape &S, int threads, int regs, bool da) {
-  PhaseShape Q = S;
-  if (regs > 0) Q.hcs = 0;
-  return phase_smem_bytes(Q, threads, da);
+bool phase_shape_named(int threads, int regs, bool da, int *groups) {
+  *groups = 1;
+  if (regs != 0) return !da && ((threads == 128 && regs == 4) || (threads == 256 && regs == 2) || (threads == 512 && regs == 1));
+  if (da) return threads == 128 || threads == 256 || threads == 512;
+  return threads == 32 || threads == 64 || threads == 128 || threads == 256 || threads == 512;
 }
 
-cudaError_t launch_phase(const SysParams *d_reps, int n_rep, int grid_x, const PhaseShape &S, int threads, int R,
+cudaError_t launch_phase(const SysParams *d_reps, int n_rep, int grid_x, const PhaseShape &S, int threads, int groups,
                          bool log, bool da, cudaStream_t s, uint32_t sweep, uint32_t sweep0, int colour,
                          uint32_t k0, uint32_t k1, const StepDyn *dyn) {
-#define CRMC_CASE(TT, RR)                                                                                      \
-  if (!da && threads == TT && R == RR)                                                                         \
-    return log ? launch_phase_t<TT, RR, true, false>(d_reps, n_rep, grid_x, S, s, sweep, sweep0, colour, k0, k1, dyn) \
-               : launch_phase_t<TT, RR, false, false>(d_reps, n_rep, grid_x, S, s, sweep, sweep0, colour, k0, k1, dyn);
-#define CRMC_CASE_DA(TT, RR)                                                                                   \
-  if (da && threads == TT && R == RR)                                                                          \
-    return log ? launch_phase_t<TT, RR, true, true>(d_reps, n_rep, grid_x, S, s, sweep, sweep0, colour, k0, k1, dyn)  \
-               : launch_phase_t<TT, RR, false, true>(d_reps, n_rep, grid_x, S, s, sweep, sweep0, colour, k0, k1, dyn);
-  CRMC_CASE(32, 0)
-  CRMC_CASE(64, 0)
-  CRMC_CASE(128, 0)
-  CRMC_CASE(128, 4)
-  CRMC_CASE(256, 0)
-  CRMC_CASE(256, 2)
-  CRMC_CASE(512, 0)
-  CRMC_CASE(512, 1)
-  CRMC_CASE_DA(128, 0)
-  CRMC_CASE_DA(256, 0)
-  CRMC_CASE_DA(512, 0)
+#define CRMC_CASE(TT, WW, DD)                                                                                   \
+  if (da == DD && threads == TT && groups == WW)                                                                \
+    return log ? launch_phase_t<TT / 32 / WW, WW, true, DD>(d_reps, n_rep, grid_x, S, s, sweep, sweep0, colour, \
+                                                            k0, k1, dyn)                                        \
+               : launch_phase_t<TT / 32 / WW, WW, false, DD>(d_reps, n_rep, grid_x, S, s, sweep, sweep0, colour, \
+                                                             k0, k1, dyn);
+#define CRMC_CASE_PLAIN(TT, WW) CRMC_CASE(TT, WW, false)
+#define CRMC_CASE_DA(TT, WW) CRMC_CASE(TT, WW, true)
+  CRMC_SHAPES(CRMC_CASE_PLAIN)
+  CRMC_SHAPES_DA(CRMC_CASE_DA)
 #undef CRMC_CASE
+#undef CRMC_CASE_PLAIN
 #undef CRMC_CASE_DA
   return cudaErrorInvalidValue;
 }
