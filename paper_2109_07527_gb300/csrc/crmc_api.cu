@@ -26,17 +26,16 @@ struct cr_ctx {
   int device = 0;
   cudaStream_t stream = nullptr;
   SysParams P{};
-  // schedule / launch shape: (threads per CTA, groups) of the phase kernel,
-  // chosen by timing real sweeps (the chain does not depend on it: the energy
-  // sums are exact fixed point); regs: as given to cr_set_launch_shape
-  int T = 128, W = 1, regs = 0;
+  // launch form of the phase kernel, chosen by timing real sweeps (the chain
+  // does not depend on it: the energy sums are exact fixed point); regs: as
+  // given to cr_set_launch_shape
+  PhaseForm F{128, 1, 1, 16, 0};
+  int regs = 0;
   int smem_max = 0;
-  int tune_next = 0;     // sweeps timed so far (TUNE_ROUNDS passes over the candidates)
+  int tune_next = 0;     // sweeps timed so far
   bool tuning = true;
   float tune_ms[16] = {};
-  PhaseShape S{};   // shared-memory capacities for the densest domain
-  PhaseShape Sc{};  // compact capacities (most domains; denser ones spill to global memory)
-  bool C = false, da_C = false;  // the tuned shapes use Sc
+  PhaseShape S{};  // shared-memory capacities
   SysParams *d_reps = nullptr;  // device copy of P (the phase kernel reads it)
   int64_t per_sweep = 0;
   // sizes
@@ -71,7 +70,8 @@ struct cr_ctx {
   cr_trial_da *d_dlog = nullptr;
   float *d_feat = nullptr;
   size_t dlog_cap = 0, feat_cap = 0;
-  int da_T = 128, da_W = 1, da_next = 0;
+  PhaseForm da_F{128, 1, 1, 16, 0};
+  int da_next = 0;
   bool da_tuning = true;
   float da_ms[8] = {};
   // cr_load inputs (capacity-sized)
@@ -576,7 +576,7 @@ extern "C" int cr_init(cr_ctx **out, const cr_system *sys, double pH, const doub
         }
   }
   {
-    // 128 threads until the tuner has timed the shapes
+    // (128 threads per domain until the tuner has timed the forms)
     c->tuning = std::getenv("CRMC_NO_TUNE") == nullptr;
     c->da_tuning = c->tuning;
   }
@@ -598,28 +598,48 @@ extern "C" int cr_init(cr_ctx **out, const cr_system *sys, double pH, const doub
   // scratch region and read the halo beyond the capacity from global memory.
   // The tuner times shapes with either set.  list_capacity / halo_capacity > 0
   // fix the capacities (both sets).
-  S.dcs = sys->list_capacity > 0 ? sys->list_capacity + 2 * P.m : std::max(2 * maxd, maxd + 32) + 2 * P.m;
-  S.dcs = std::min(P.dcap_glob, S.dcs);
-  S.hcs = sys->halo_capacity > 0 ? sys->halo_capacity : std::min(maxh + maxh / 4 + 32, 4096);
-  S.lns = std::min(P.lnmax, S.dcs + 4);
-  while (phase_smem_bytes(S, 512, 1, false) > (size_t)smem_max / 2 && S.dcs > 64) {
-    S.dcs /= 2;
-    S.hcs = std::max(S.hcs / 2, 64);
-    S.lns = std::min(P.lnmax, S.dcs + 4);
+  PhaseCaps &C = S.full;
+  C.dcs = sys->list_capacity > 0 ? sys->list_capacity + 2 * P.m : std::max(2 * maxd, maxd + 32) + 2 * P.m;
+  C.dcs = std::min(P.dcap_glob, C.dcs);
+  C.hcs = sys->halo_capacity > 0 ? sys->halo_capacity : std::min(maxh + maxh / 4 + 32, 4096);
+  C.lns = std::min(P.lnmax, C.dcs + 4);
+  // (the arrays of a domain beyond what an SM has -- a nanoparticle's thousand
+  // sites -- are cut to that; a list or halo in global memory slows its trials
+  // far more than a CTA that has the SM to itself)
+  const PhaseForm largest{512, 1, 1, 16, 0};
+  while (phase_smem_bytes(S, largest, false) > (size_t)smem_max && C.dcs > 64) {
+    C.dcs -= C.dcs / 16;
+    C.hcs = std::max(C.hcs - C.hcs / 16, 64);
+    C.lns = std::min(P.lnmax, C.dcs + 4);
   }
-  if (phase_smem_bytes(S, 512, 1, false) > (size_t)smem_max) { free_ctx(c); return CR_ERR_INVALID_ARG; }
+  const PhaseCaps half = C;
+  if (global && sys->list_capacity <= 0) {
+    // The one domain is the box, whose particle number may grow to the
+    // capacity (a box of acids alone sets its counter-ions free), and a
+    // replica is one CTA: the list takes what an SM has.  (A list sized by the
+    // starting configuration went to global memory once the ions had come:
+    // 500 acids growing to 1,250 particles, 500 trials in each of 128 boxes
+    // 3.21 ms.)
+    C.dcs = std::min(P.dcap_glob, std::max(C.dcs, (int)std::min<int64_t>(sys->capacity, 1 << 16) + 2 * P.m));
+    C.lns = std::min(P.lnmax, C.dcs + 4);
+    while (phase_smem_bytes(S, largest, false) > (size_t)smem_max && C.dcs > half.dcs) {
+      C.dcs = std::max(half.dcs, C.dcs - 64);
+      C.lns = std::min(P.lnmax, C.dcs + 4);
+    }
+  }
+  if (phase_smem_bytes(S, largest, false) > (size_t)smem_max) { free_ctx(c); return CR_ERR_INVALID_ARG; }
   {
     auto pct90 = [](std::vector<int> v) {
       if (v.empty()) return 0;
       std::sort(v.begin(), v.end());
       return v[(size_t)(0.9 * (double)(v.size() - 1))];
     };
-    PhaseShape &Q = c->Sc;
-    Q = S;
-    if (sys->list_capacity <= 0 && sys->halo_capacity <= 0) {
+    PhaseCaps &Q = S.small;
+    Q = half;
+    if (!global && sys->list_capacity <= 0 && sys->halo_capacity <= 0) {
       const int pd = pct90(dsums), ph = pct90(hsums);
-      Q.dcs = std::min(S.dcs, std::max(32, (3 * pd) / 2 + 16) + 2 * P.m);
-      Q.hcs = std::min(S.hcs, ph + ph / 4 + 32);
+      Q.dcs = std::min(C.dcs, std::max(32, (3 * pd) / 2 + 16) + 2 * P.m);
+      Q.hcs = std::min(C.hcs, ph + ph / 4 + 32);
       Q.lns = std::min(P.lnmax, Q.dcs + 4);
     }
   }
@@ -959,55 +979,57 @@ static int grow(TT **p, size_t *cap, size_t n) {
   return CR_OK;
 }
 
-// Online launch-shape tuning (shared by plain and delayed-acceptance sweeps):
-// the first sweeps of unlogged calls time each shape of the set (shapes whose
-// shared memory does not fit are skipped) in TUNE_ROUNDS round-robin passes,
-// and the shape with the shortest of its times is kept: a single pass was
-// swayed by one slow sweep and by the state's drift while the chain starts.
-// For batches whose persistent mode is left to the tuner (pers != null), the
-// candidates are every shape with one launch per colour, then every shape as
-// a persistent sweep; *pers receives the chosen mode.  next counts the timed
-// sweeps; candidate next % tune_count.
-constexpr int TUNE_ROUNDS = 2;
-
+// Online tuning of the launch form (shared by plain and delayed-acceptance
+// sweeps): the first sweeps of unlogged calls time each form that applies in
+// round-robin rounds, and the fastest of the last round is kept.  Earlier
+// rounds only let the state settle: a box that starts without its ions grows
+// for a dozen sweeps, and the shortest time over all rounds then favoured
+// whatever was tried first.  Two rounds; six under the global schedule, which
+// has a third of the forms.  For batches whose persistent mode is left to the
+// tuner (pers != null), the candidates are every form with one launch per
+// colour, then every form as a persistent sweep; *pers receives the chosen
+// mode.  next counts the candidates passed; candidate next % tune_count.
 struct TuneRef {
-  int &T, &W, &next;
+  PhaseForm &F;
+  int &next;
   bool &on;
   float *ms;
-  bool &C;  // the chosen shape uses the compact capacities
+  bool global;             // one domain per replica: one seat, one group
   bool *pers = nullptr;
 };
 
-static int tune_count(const TuneRef &t, bool da) { return phase_shape_count(da) * (t.pers ? 2 : 1); }
-static int tune_total(const TuneRef &t, bool da) { return tune_count(t, da) * TUNE_ROUNDS; }
+static int tune_count(const TuneRef &t, bool da) { return phase_form_count(da) * (t.pers ? 2 : 1); }
+static int tune_total(const TuneRef &t, bool da) { return tune_count(t, da) * (t.global ? 6 : 2); }
 static int tune_cand(const TuneRef &t, bool da) { return t.next % tune_count(t, da); }
 
-static void tune_skip(TuneRef t, const PhaseShape &S, const PhaseShape &Sc, int smem_max, bool da) {
-  const int nshape = phase_shape_count(da);
+// forms that do not apply are passed over: those that do not fit in shared
+// memory; several seats or groups under the global schedule (its one domain
+// takes the CTA, its trials are mostly accepted, and an Ewald trial uses the
+// whole CTA); seats in a persistent sweep (its tasks take whole CTAs)
+static void tune_skip(TuneRef t, const PhaseShape &S, int smem_max, bool da) {
+  const int nform = phase_form_count(da);
   while (t.on && t.next < tune_total(t, da)) {
     const int c = tune_cand(t, da);
-    int t_, r_;
-    phase_shape(c % nshape, &t_, &r_, da);
-    const PhaseShape &Q = phase_shape_compact(c % nshape, da) ? Sc : S;
-    if (phase_smem_bytes(Q, t_, r_, da) <= (size_t)smem_max) break;
+    const PhaseForm &F = phase_form(c % nform, da);
+    const bool whole = F.seats == 1, single = F.seats == 1 && F.groups == 1;
+    if (phase_smem_bytes(S, F, da) <= (size_t)smem_max && (!t.global || single) && (c < nform || whole)) break;
     t.ms[c] = 1e30f;
     t.next++;
   }
 }
 
-static void tune_finish(TuneRef t, float ms, const PhaseShape &S, const PhaseShape &Sc, int smem_max, bool da) {
+static void tune_finish(TuneRef t, float ms, const PhaseShape &S, int smem_max, bool da) {
   const int c = tune_cand(t, da);
-  t.ms[c] = t.next < tune_count(t, da) ? ms : std::min(t.ms[c], ms);
+  t.ms[c] = ms;
   t.next++;
-  tune_skip(t, S, Sc, smem_max, da);
-  const int nshape = phase_shape_count(da);
+  tune_skip(t, S, smem_max, da);
+  const int nform = phase_form_count(da);
   if (t.next == tune_total(t, da)) {
     int best = 0;
     for (int i = 1; i < tune_count(t, da); ++i)
       if (t.ms[i] < t.ms[best]) best = i;
-    phase_shape(best % nshape, &t.T, &t.W, da);
-    t.C = phase_shape_compact(best % nshape, da);
-    if (t.pers) *t.pers = best >= nshape;
+    t.F = phase_form(best % nform, da);
+    if (t.pers) *t.pers = best >= nform;
     t.on = false;
   }
 }
@@ -1039,18 +1061,16 @@ static int sweep_impl(cr_ctx *ctx, uint64_t n_trials, uint64_t seed, cr_sweep_st
   if (log) CR_CUDA(cudaMemcpyAsync(ctx->d_reps, &P, sizeof(SysParams), cudaMemcpyHostToDevice, s));
   const uint64_t n_sweeps = n_trials / (uint64_t)ctx->per_sweep;
   const uint32_t sweep0 = (uint32_t)ctx->sweep;
-  TuneRef tr = da ? TuneRef{ctx->da_T, ctx->da_W, ctx->da_next, ctx->da_tuning, ctx->da_ms, ctx->da_C}
-                  : TuneRef{ctx->T, ctx->W, ctx->tune_next, ctx->tuning, ctx->tune_ms, ctx->C};
+  const bool glob = P.global != 0;
+  TuneRef tr = da ? TuneRef{ctx->da_F, ctx->da_next, ctx->da_tuning, ctx->da_ms, glob}
+                  : TuneRef{ctx->F, ctx->tune_next, ctx->tuning, ctx->tune_ms, glob};
   for (uint64_t sw = 0; sw < n_sweeps; ++sw) {
     const uint32_t swc = (uint32_t)ctx->sweep++;
-    if (!log) tune_skip(tr, ctx->S, ctx->Sc, ctx->smem_max, da);
+    if (!log) tune_skip(tr, ctx->S, ctx->smem_max, da);
     const bool tune = tr.on && !log && tr.next < tune_total(tr, da);
-    int T = tr.T, W = tr.W;
-    const bool compact = tune ? phase_shape_compact(tune_cand(tr, da), da) : tr.C;
-    const PhaseShape &SS = compact ? ctx->Sc : ctx->S;
+    const PhaseForm F = tune ? phase_form(tune_cand(tr, da), da) : tr.F;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (tune) {
-      phase_shape(tune_cand(tr, da), &T, &W, da);
       cudaEventCreate(&e0);
       cudaEventCreate(&e1);
       cudaEventRecord(e0, s);
@@ -1066,7 +1086,7 @@ static int sweep_impl(cr_ctx *ctx, uint64_t n_trials, uint64_t seed, cr_sweep_st
     for (int col = 0; col < P.ncol; ++col) {
       int ti;
       tbegin(ctx, 0, &ti);
-      CR_CUDA(launch_phase(ctx->d_reps, 1, P.nact, SS, T, W, log != nullptr, da, s, swc, sweep0, col, k0, k1));
+      CR_CUDA(launch_phase(ctx->d_reps, 1, P.nact, ctx->S, F, log != nullptr, da, s, swc, sweep0, col, k0, k1));
       tend(ctx, 0, ti);
       ctx->launches_total++;
     }
@@ -1077,7 +1097,7 @@ static int sweep_impl(cr_ctx *ctx, uint64_t n_trials, uint64_t seed, cr_sweep_st
       cudaEventElapsedTime(&ms, e0, e1);
       cudaEventDestroy(e0);
       cudaEventDestroy(e1);
-      tune_finish(tr, ms, ctx->S, ctx->Sc, ctx->smem_max, da);
+      tune_finish(tr, ms, ctx->S, ctx->smem_max, da);
     }
   }
   if (log) {
@@ -1143,11 +1163,8 @@ extern "C" int cr_set_surrogate(cr_ctx *ctx, const cr_mlp *m) {
   // the features use the 5^3 stencil of half-cutoff cells inside the phase's region
   if (P0.global || P0.h != 2 || P0.nc < P0.k + 4 || !std::isfinite(m->b4)) return CR_ERR_INVALID_ARG;
   int smem_ok = 0;
-  for (int i = 0; i < phase_shape_count(true); ++i) {
-    int t, r;
-    phase_shape(i, &t, &r, true);
-    smem_ok |= phase_smem_bytes(ctx->S, t, r, true) <= (size_t)ctx->smem_max;
-  }
+  for (int i = 0; i < phase_form_count(true); ++i)
+    smem_ok |= phase_smem_bytes(ctx->S, phase_form(i, true), true) <= (size_t)ctx->smem_max;
   if (!smem_ok) return CR_ERR_INVALID_ARG;
   // transposed BF16 weights (WT[in][out]) and the biases
   std::vector<uint16_t> w(MLPW_N);
@@ -1669,19 +1686,15 @@ extern "C" int cr_set_launch_shape(cr_ctx *ctx, int32_t threads, int32_t regs) {
     ctx->da_next = 0;
     return CR_OK;
   }
-  int w, wd;
-  const bool plain = phase_shape_named(threads, regs, false, &w), da = phase_shape_named(threads, regs, true, &wd);
+  PhaseForm F, Fd;
+  const bool plain = phase_form_named(threads, regs, false, &F), da = phase_form_named(threads, regs, true, &Fd);
   if (plain) {
-    ctx->T = threads;
-    ctx->W = w;
+    ctx->F = F;
     ctx->regs = regs;
-    ctx->C = false;
     ctx->tuning = false;
   }
   if (da) {  // delayed-acceptance sweeps, where supported
-    ctx->da_T = threads;
-    ctx->da_W = wd;
-    ctx->da_C = false;
+    ctx->da_F = Fd;
     ctx->da_tuning = false;
   }
   return plain || da ? CR_OK : CR_ERR_INVALID_ARG;
@@ -1689,7 +1702,7 @@ extern "C" int cr_set_launch_shape(cr_ctx *ctx, int32_t threads, int32_t regs) {
 
 extern "C" int cr_get_launch_shape(const cr_ctx *ctx, int32_t *threads, int32_t *regs) {
   if (!ctx || !threads || !regs) return CR_ERR_INVALID_ARG;
-  *threads = ctx->T;
+  *threads = ctx->F.threads;
   *regs = ctx->regs;
   return CR_OK;
 }
@@ -1720,21 +1733,23 @@ struct cr_batch {
   cudaStream_t cstream = nullptr;  // capture stream
   cudaGraphExec_t graph = nullptr;
   double g_dt = 0.0, g_gamma = 0.0;
-  int g_T = 0, g_W = 0, g_da = -1;
-  bool g_C = false, g_pers = false, g_fine = false, g_timing = false;
+  PhaseForm g_F{};
+  int g_da = -1;
+  bool g_pers = false, g_fine = false, g_timing = false;
   bool g_ff = false;  // the graph's step evaluates the forces first (a step after a load)
   int64_t g_kernels = 0;                      // kernels per graph launch
   std::vector<std::pair<int, int>> g_pairs;  // phase-kernel event pairs recorded by the graph (timing)
   SysParams *d_reps = nullptr;  // one entry per replica (key_xor = replica index)
-  PhaseShape S{}, Sc{};
-  bool C = false, da_C = false;
+  PhaseShape S{};
   int grid_x = 0, ncol = 8;
-  int T = 128, W = 1, regs = 0;
+  PhaseForm F{128, 1, 1, 16, 0};
+  int regs = 0;
   int smem_max = 0;
   bool tuning = true;
   int tune_next = 0;
   float tune_ms[32] = {};
-  int da_T = 128, da_W = 1, da_next = 0;
+  PhaseForm da_F{128, 1, 1, 16, 0};
+  int da_next = 0;
   bool da_tuning = true;
   float da_ms[16] = {};
   std::vector<SysParams> reps;  // host copy of d_reps
@@ -1835,21 +1850,18 @@ extern "C" int cr_batch_create(cr_batch **out, cr_ctx *const *ctxs, int32_t n) {
     reps[r] = c->P;
     reps[r].key_xor = (uint32_t)r;
     reps[r].log = nullptr;
-    b->S.dcs = std::max(b->S.dcs, c->S.dcs);
-    b->S.hcs = std::max(b->S.hcs, c->S.hcs);
-    b->S.lns = std::max(b->S.lns, c->S.lns);
+    auto grow = [](PhaseCaps &x, const PhaseCaps &y) {
+      x.dcs = std::max(x.dcs, y.dcs);
+      x.hcs = std::max(x.hcs, y.hcs);
+      x.lns = std::max(x.lns, y.lns);
+    };
+    grow(b->S.full, c->S.full);
+    grow(b->S.small, c->S.small);
     b->S.nr3 = std::max(b->S.nr3, c->S.nr3);
     b->S.kc3 = std::max(b->S.kc3, c->S.kc3);
     b->S.chunk = std::max(b->S.chunk, c->S.chunk);
     b->S.ewk = std::max(b->S.ewk, c->S.ewk);
     b->ewald_nk_max = std::max(b->ewald_nk_max, c->P.ewald_nk);
-    b->Sc.dcs = std::max(b->Sc.dcs, c->Sc.dcs);
-    b->Sc.hcs = std::max(b->Sc.hcs, c->Sc.hcs);
-    b->Sc.lns = std::max(b->Sc.lns, c->Sc.lns);
-    b->Sc.nr3 = std::max(b->Sc.nr3, c->Sc.nr3);
-    b->Sc.kc3 = std::max(b->Sc.kc3, c->Sc.kc3);
-    b->Sc.chunk = std::max(b->Sc.chunk, c->Sc.chunk);
-    b->Sc.ewk = std::max(b->Sc.ewk, c->Sc.ewk);
     b->grid_x = std::max(b->grid_x, c->P.nact);
   }
   b->ncol = ctxs[0]->P.ncol;
@@ -1864,7 +1876,7 @@ extern "C" int cr_batch_create(cr_batch **out, cr_ctx *const *ctxs, int32_t n) {
     }
   int smem_max = 0;
   cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctxs[0]->device);
-  if (phase_smem_bytes(b->S, 512, 1, false) > (size_t)smem_max) { delete b; return CR_ERR_INVALID_ARG; }
+  if (phase_smem_bytes(b->S, PhaseForm{512, 1, 1, 16, 0}, false) > (size_t)smem_max) { delete b; return CR_ERR_INVALID_ARG; }
   b->smem_max = smem_max;
   cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, ctxs[0]->device);
   if (cudaMalloc((void **)&b->d_reps, sizeof(SysParams) * n) != cudaSuccess) { delete b; return CR_ERR_NOMEM; }
@@ -1941,7 +1953,7 @@ extern "C" void cr_batch_destroy(cr_batch *b) {
 static int batch_refresh_chem(cr_batch *b);
 
 // one persistent sweep launch of every replica (words zeroed first)
-static int batch_launch_persistent(cr_batch *b, const PhaseShape &SS, int T, int W, bool da, uint32_t swc,
+static int batch_launch_persistent(cr_batch *b, const PhaseForm &F, bool da, uint32_t swc,
                                    uint32_t sweep0, uint32_t k0, uint32_t k1, int withhold = -1,
                                    unsigned long long wait_ns = 2000000000ull, const StepDyn *dyn = nullptr) {
   cr_ctx *c0 = b->ctx[0];
@@ -1963,7 +1975,7 @@ static int batch_launch_persistent(cr_batch *b, const PhaseShape &SS, int T, int
   int ti;
   tbegin(c0, 0, &ti);
   const int sms = b->sms > 0 ? b->sms : 1;
-  CR_CUDA(launch_sweep(b->d_reps, SS, T, W, da, s, swc, sweep0, k0, k1, Q, b->ctas_per_sm * sms, dyn));
+  CR_CUDA(launch_sweep(b->d_reps, b->S, F, da, s, swc, sweep0, k0, k1, Q, b->ctas_per_sm * sms, dyn));
   tend(c0, 0, ti);
   c0->launches_total++;
   return CR_OK;
@@ -1995,11 +2007,12 @@ static int batch_sweep_impl(cr_batch *b, uint64_t n_sweeps, uint64_t seed, bool 
   const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
   const uint32_t sweep0 = (uint32_t)c0->sweep;
   bool &pers_choice = da ? b->da_persistent : b->persistent;
-  TuneRef tr = da ? TuneRef{b->da_T, b->da_W, b->da_next, b->da_tuning, b->da_ms, b->da_C}
-                  : TuneRef{b->T, b->W, b->tune_next, b->tuning, b->tune_ms, b->C};
+  const bool glob = c0->P.global != 0;
+  TuneRef tr = da ? TuneRef{b->da_F, b->da_next, b->da_tuning, b->da_ms, glob}
+                  : TuneRef{b->F, b->tune_next, b->tuning, b->tune_ms, glob};
   if (b->pmode < 0) tr.pers = &pers_choice;
   else pers_choice = b->pmode != 0;
-  const int nshape = phase_shape_count(da);
+  const int nform = phase_form_count(da);
   for (uint64_t sw = 0; sw < n_sweeps; ++sw) {
     const uint32_t swc = (uint32_t)c0->sweep;
     for (cr_ctx *c : b->ctx) {
@@ -2007,17 +2020,14 @@ static int batch_sweep_impl(cr_batch *b, uint64_t n_sweeps, uint64_t seed, bool 
       c->f_valid = false;
       c->fcons_valid = false;
     }
-    tune_skip(tr, b->S, b->Sc, b->smem_max, da);
+    tune_skip(tr, b->S, b->smem_max, da);
     const bool tune = tr.on && tr.next < tune_total(tr, da);
-    int T = tr.T, W = tr.W;
     bool persistent = pers_choice;
     const int cand = tune ? tune_cand(tr, da) : 0;
-    const bool compact = tune ? phase_shape_compact(cand % nshape, da) : tr.C;
-    const PhaseShape &SS = compact ? b->Sc : b->S;
+    const PhaseForm F = tune ? phase_form(cand % nform, da) : tr.F;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (tune) {
-      phase_shape(cand % nshape, &T, &W, da);
-      if (tr.pers) persistent = cand >= nshape;
+      if (tr.pers) persistent = cand >= nform;
       cudaEventCreate(&e0);
       cudaEventCreate(&e1);
       cudaEventRecord(e0, s);
@@ -2031,13 +2041,13 @@ static int batch_sweep_impl(cr_batch *b, uint64_t n_sweeps, uint64_t seed, bool 
       c0->launches_total += 2;
     }
     if (persistent) {
-      const int rc = batch_launch_persistent(b, SS, T, W, da, swc, sweep0, k0, k1);
+      const int rc = batch_launch_persistent(b, F, da, swc, sweep0, k0, k1);
       if (rc != CR_OK) return rc;
     } else {
       for (int col = 0; col < b->ncol; ++col) {
         int ti;
         tbegin(c0, 0, &ti);
-        CR_CUDA(launch_phase(b->d_reps, n, b->grid_x, SS, T, W, false, da, s, swc, sweep0, col, k0, k1));
+        CR_CUDA(launch_phase(b->d_reps, n, b->grid_x, b->S, F, false, da, s, swc, sweep0, col, k0, k1));
         tend(c0, 0, ti);
         c0->launches_total++;
       }
@@ -2049,7 +2059,7 @@ static int batch_sweep_impl(cr_batch *b, uint64_t n_sweeps, uint64_t seed, bool 
       cudaEventElapsedTime(&ms, e0, e1);
       cudaEventDestroy(e0);
       cudaEventDestroy(e1);
-      tune_finish(tr, ms, b->S, b->Sc, b->smem_max, da);
+      tune_finish(tr, ms, b->S, b->smem_max, da);
     }
   }
   return CR_OK;
@@ -2078,17 +2088,12 @@ extern "C" int cr_batch_selftest_wait_timeout(cr_batch *b, int32_t replica, doub
     c->f_valid = false;
     c->fcons_valid = false;
   }
-  int T = b->T, W = b->W;
-  const PhaseShape &SS = b->C ? b->Sc : b->S;
-  if (b->tuning) {  // a shape every context supports
-    T = 128;
-    W = 1;
-  }
+  const PhaseForm F = b->tuning || b->F.seats > 1 ? PhaseForm{128, 1, 1, 16, 0} : b->F;  // (tasks take whole CTAs)
   if (b->order_nc > 0) {
     CR_CUDA(launch_domain_order(b->d_reps, (int)b->ctx.size(), b->ncol, b->order_nact, c0->stream, swc, 1u, 0u));
     c0->launches_total++;
   }
-  const int rc = batch_launch_persistent(b, b->tuning ? b->S : SS, T, W, false, swc, swc, 1u, 0u, replica,
+  const int rc = batch_launch_persistent(b, F, false, swc, swc, 1u, 0u, replica,
                                          (unsigned long long)(timeout_ms * 1e6));
   if (rc != CR_OK) return rc;
   CR_CUDA(cudaStreamSynchronize(c0->stream));
@@ -2199,9 +2204,8 @@ static int batch_capture_cycle(cr_batch *b, double dt, double gamma, bool da, bo
     launches[r] = b->ctx[r]->launches_total;
     fvalid[r] = b->ctx[r]->f_valid ? 1 : 0;
   }
-  const int T = da ? b->da_T : b->T, W = da ? b->da_W : b->W;
-  const bool C = da ? b->da_C : b->C, pers = da ? b->da_persistent : b->persistent;
-  const PhaseShape &SS = C ? b->Sc : b->S;
+  const PhaseForm F = da ? b->da_F : b->F;
+  const bool pers = da ? b->da_persistent : b->persistent;
   const StepDyn *dyn = b->d_dyn;
   int rc = CR_OK;
   while (c0->ev_pool.size() < c0->ev_next + 2 * (size_t)(b->ncol + 2)) {  // no event creation while capturing
@@ -2225,12 +2229,12 @@ static int batch_capture_cycle(cr_batch *b, double dt, double gamma, bool da, bo
     }
     if (rc == CR_OK) {
       if (pers) {
-        rc = batch_launch_persistent(b, SS, T, W, da, 0, 0, 0, 0, -1, 2000000000ull, dyn);
+        rc = batch_launch_persistent(b, F, da, 0, 0, 0, 0, -1, 2000000000ull, dyn);
       } else {
         for (int col = 0; col < b->ncol && rc == CR_OK; ++col) {
           int ti;
           tbegin(c0, 0, &ti);
-          if (launch_phase(b->d_reps, n, b->grid_x, SS, T, W, false, da, s, 0, 0, col, 0, 0, dyn) != cudaSuccess)
+          if (launch_phase(b->d_reps, n, b->grid_x, b->S, F, false, da, s, 0, 0, col, 0, 0, dyn) != cudaSuccess)
             rc = CR_ERR_CUDA;
           tend(c0, 0, ti);
           c0->launches_total++;
@@ -2271,9 +2275,7 @@ static int batch_capture_cycle(cr_batch *b, double dt, double gamma, bool da, bo
   b->g_kernels = kernels;
   b->g_dt = dt;
   b->g_gamma = gamma;
-  b->g_T = T;
-  b->g_W = W;
-  b->g_C = C;
+  b->g_F = F;
   b->g_pers = pers;
   b->g_fine = b->fine;
   b->g_da = da ? 1 : 0;
@@ -2325,11 +2327,11 @@ extern "C" int cr_batch_cycle(cr_batch *b, int32_t n_steps, double dt, double ga
       CR_CUDA(cudaMemcpyAsync(b->d_reps, b->reps.data(), sizeof(SysParams) * b->ctx.size(), cudaMemcpyHostToDevice, s));
   }
   if (!b->d_dyn) CR_CUDA(cudaMalloc((void **)&b->d_dyn, sizeof(StepDyn)));
-  const int T = da ? b->da_T : b->T, W = da ? b->da_W : b->W;
-  const bool C = da ? b->da_C : b->C, pers = da ? b->da_persistent : b->persistent;
+  const PhaseForm F = da ? b->da_F : b->F;
+  const bool pers = da ? b->da_persistent : b->persistent;
   while (step < n_steps) {
     const bool first = ff && step == 0;  // only a call's first step can have stale forces
-    if (!b->graph || b->g_dt != dt || b->g_gamma != gamma || b->g_T != T || b->g_W != W || b->g_C != C ||
+    if (!b->graph || b->g_dt != dt || b->g_gamma != gamma || b->g_F != F ||
         b->g_pers != pers || b->g_fine != b->fine || b->g_da != (da ? 1 : 0) || b->g_timing != c0->timing ||
         b->g_ff != first) {
       if ((rc = batch_capture_cycle(b, dt, gamma, da != 0, first)) != CR_OK) return rc;
@@ -2542,22 +2544,18 @@ extern "C" int cr_batch_set_launch_shape(cr_batch *b, int32_t threads, int32_t r
     return CR_OK;
   }
   if (b->pmode < 0) b->persistent = b->da_persistent = false;  // a fixed shape without a fixed mode: per colour
-  int w, wd;
-  const bool plain = phase_shape_named(threads, regs, false, &w) &&
-                     phase_smem_bytes(b->S, threads, w, false) <= (size_t)b->smem_max;
-  const bool da = phase_shape_named(threads, regs, true, &wd) &&
-                  phase_smem_bytes(b->S, threads, wd, true) <= (size_t)b->smem_max;
+  PhaseForm F, Fd;
+  const bool plain =
+      phase_form_named(threads, regs, false, &F) && phase_smem_bytes(b->S, F, false) <= (size_t)b->smem_max;
+  const bool da =
+      phase_form_named(threads, regs, true, &Fd) && phase_smem_bytes(b->S, Fd, true) <= (size_t)b->smem_max;
   if (plain) {
-    b->T = threads;
-    b->W = w;
+    b->F = F;
     b->regs = regs;
-    b->C = false;
     b->tuning = false;
   }
   if (da) {
-    b->da_T = threads;
-    b->da_W = wd;
-    b->da_C = false;
+    b->da_F = Fd;
     b->da_tuning = false;
   }
   return plain || da ? CR_OK : CR_ERR_INVALID_ARG;
@@ -2565,7 +2563,7 @@ extern "C" int cr_batch_set_launch_shape(cr_batch *b, int32_t threads, int32_t r
 
 extern "C" int cr_batch_get_launch_shape(const cr_batch *b, int32_t *threads, int32_t *regs) {
   if (!b || !threads || !regs) return CR_ERR_INVALID_ARG;
-  *threads = b->T;
+  *threads = b->F.threads;
   *regs = b->regs;
   return CR_OK;
 }

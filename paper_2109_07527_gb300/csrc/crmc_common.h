@@ -139,18 +139,49 @@ constexpr int MLPW_W4 = MLPW_W3 + MLP_H * MLP_H;
 constexpr int MLPW_N = MLPW_W4 + MLP_H;
 constexpr int MLPB_N = 3 * MLP_H + 1;
 
-// Launch-wide shared-memory shape of a phase launch (the same for every CTA;
-// the maximum over the replicas of a batch).
+// Shared-memory capacities of a domain's list, halo and log table: full (the
+// densest domain, with room to grow) or compact (most domains).
+struct PhaseCaps {
+  int dcs;  // domain-list entries held in shared memory
+  int hcs;  // halo particles held in shared memory
+  int lns;  // log-table entries held in shared memory
+};
+
+// Shared-memory shape of a phase launch (the maximum over the replicas of a
+// batch).
 struct PhaseShape {
-  int dcs;     // domain-list entries held in shared memory
-  int hcs;     // halo particles held in shared memory
-  int lns;     // log-table entries held in shared memory
+  PhaseCaps full, small;
   int nr3;     // region cells
   int kc3;     // domain cells
   int chunk;   // trials whose random numbers are drawn at once (min(m, TRIAL_CHUNK))
   int ewk;     // Ewald: kmax + 1 phase factors per axis and changed particle (0 without Ewald)
+};
+
+// Form of a phase launch: threads per CTA; the seats that the CTAs of all but
+// the densest wide16 / 16 of a replica's domains are split into, one domain
+// each; the groups that a CTA working on one domain evaluates trials in; the
+// compact capacities instead of the full ones for a CTA's domain (a seat's are
+// always compact).
+struct PhaseForm {
+  int threads, seats, groups, wide16, compact;
+  bool operator==(const PhaseForm &o) const {
+    return threads == o.threads && seats == o.seats && groups == o.groups && wide16 == o.wide16 && compact == o.compact;
+  }
+  bool operator!=(const PhaseForm &o) const { return !(*this == o); }
+};
+
+// where a domain's arrays lie in shared memory, and their capacities
+struct PhaseLayout {
   static constexpr int N_OFF = 33;
-  unsigned off[N_OFF];  // byte offsets of the CTA's shared arrays (filled for each launch form)
+  unsigned off[N_OFF];
+  int dcs, hcs, lns, chunk, ewk;
+};
+
+// a phase launch's constant parameters
+struct PhaseArgs {
+  PhaseLayout lay[2];  // a CTA's domain; a seat's
+  unsigned seat_bytes;
+  int seats, groups, wide16;
 };
 
 // error bits in *err

@@ -112,17 +112,15 @@ struct LoadJob {
   int n_perm;
 };
 
-// phase kernel shapes (threads, groups that threads are split into); da: the
-// delayed-acceptance set
-size_t phase_smem_bytes(const PhaseShape &S, int threads, int groups, bool da);
-int phase_shape_count(bool da);
-void phase_shape(int i, int *threads, int *groups, bool da);
-bool phase_shape_compact(int i, bool da);  // shape i uses the compact list and halo capacities
-// the shape that a caller's (threads, regs) pair names; false when there is none
-bool phase_shape_named(int threads, int regs, bool da, int *groups);
-cudaError_t launch_phase(const SysParams *d_reps, int n_rep, int grid_x, const PhaseShape &S, int threads, int groups,
-                         bool log, bool da, cudaStream_t s, uint32_t sweep, uint32_t sweep0, int colour,
-                         uint32_t k0, uint32_t k1, const StepDyn *dyn = nullptr);
+// forms of the phase launches; da: the delayed-acceptance set
+size_t phase_smem_bytes(const PhaseShape &S, const PhaseForm &F, bool da);
+int phase_form_count(bool da);
+const PhaseForm &phase_form(int i, bool da);
+// the form that a caller's (threads, regs) pair names; false when there is none
+bool phase_form_named(int threads, int regs, bool da, PhaseForm *F);
+cudaError_t launch_phase(const SysParams *d_reps, int n_rep, int max_nact, const PhaseShape &S, const PhaseForm &F,
+                         bool log, bool da, cudaStream_t s, uint32_t sweep, uint32_t sweep0, int colour, uint32_t k0,
+                         uint32_t k1, const StepDyn *dyn = nullptr);
 // Schedule of a persistent sweep (k_cr_sweep): tasks (colour, replica, rank)
 // claimed in that order; next, done and abort are device words zeroed before
 // every launch.
@@ -139,7 +137,7 @@ struct SweepSched {
   int withhold_rep;       // self-test of the waits: this replica never reports colour 0 (-1: none)
 };
 // one sweep of every replica in one persistent launch; max_ctas > 0 caps the grid
-cudaError_t launch_sweep(const SysParams *d_reps, const PhaseShape &S, int threads, int groups, bool da, cudaStream_t s,
+cudaError_t launch_sweep(const SysParams *d_reps, const PhaseShape &S, const PhaseForm &F, bool da, cudaStream_t s,
                          uint32_t sweep, uint32_t sweep0, uint32_t k0, uint32_t k1, const SweepSched &Q,
                          int max_ctas, const StepDyn *dyn = nullptr);
 // the step counter of a captured cycle (the graph's last node)

@@ -17,7 +17,8 @@
 //      participants (ballot scans of the order); every thread sums its share of
 //      the pair changes -- FP32 Coulomb, FP64 WCA of inserted/deleted ions --
 //      into 64-bit fixed point, exact and therefore independent of the thread
-//      count; warp 0 takes the Metropolis decision and commits the move;
+//      count; warp 0 takes the Metropolis decision and commits the move (or
+//      several groups of threads evaluate consecutive trials side by side);
 //   4. writes the domain's cells back (id-sorted), if a trial was accepted, and
 //      adds its count changes.
 // The move rules are those of Sec. II.C of the paper applied to the domain
@@ -26,6 +27,7 @@
 
 #include <algorithm>
 #include <climits>
+#include <iterator>
 #include <cstdint>
 
 #include "crmc_device.cuh"
@@ -55,23 +57,32 @@ struct Desc {
   int dp, cls, skip;    // WCA presence change, class, list slot (-1 inserted)
 };
 
+// a trial's selection; pres: presence of a before / after, b before / after
+enum Presence { PA_O = 1, PA_N = 2, PB_O = 4, PB_N = 8 };
 struct TrialCtl {
   Desc c[2];
   int nch;    // changed particles needing the energy sweep (0 = decided)
   int flags;  // CR_TRIAL_* bits known before the sweep
   int move;
-  int site, ionA, ionB;  // places in the canonical order (-1 none)
-  unsigned long long id_a, id_b, newid;
+  int placeA, placeB;  // places in the canonical order (-1 none): the site or first ion, the second ion
+  int pres;
   long long ln_ratio_fx, dself_fx;  // 2^-48 fixed point
   float qa_o, qa_n, qb_o, qb_n;  // effective charges of the two changed particles
-  int pa_o, pa_n, pb_o, pb_n;    // presence before / after
-  // delayed acceptance: in-domain cell ranks of a and b, charge and presence
-  // changes, feature group of a (0 ion, 8 site), stage-1 outcome
-  int rka, rkb, dqa, dqb, eta_a, eta_b, cat_a, go;
+  unsigned long long id_a, id_b;  // trial records only
+  // delayed acceptance: in-domain cell ranks of a and b, stage-1 outcome
+  int rka, rkb, go;
   int ewacc;             // Ewald: the trial was accepted (S(k) follows)
   float sur;             // surrogate dE~ (DA)
   long long sur_fx;      // dE~ clamped, 2^-48 fixed point (DA)
 };
+// the charge (0 when absent) of changed particle x (0: a, 1: b) before / after, its presence, and the
+// surrogate's integer changes
+__device__ __forceinline__ bool had(const TrialCtl &C, int x) { return C.pres & (x ? PB_O : PA_O); }
+__device__ __forceinline__ bool has(const TrialCtl &C, int x) { return C.pres & (x ? PB_N : PA_N); }
+__device__ __forceinline__ int q_old(const TrialCtl &C, int x) { return had(C, x) ? __float2int_rn(x ? C.qb_o : C.qa_o) : 0; }
+__device__ __forceinline__ int q_new(const TrialCtl &C, int x) { return has(C, x) ? __float2int_rn(x ? C.qb_n : C.qa_n) : 0; }
+__device__ __forceinline__ int d_charge(const TrialCtl &C, int x) { return q_new(C, x) - q_old(C, x); }
+__device__ __forceinline__ int d_presence(const TrialCtl &C, int x) { return (has(C, x) ? 1 : 0) - (had(C, x) ? 1 : 0); }
 
 // The domain's particles.  A particle keeps its slot of the payload arrays
 // while it lives; `ord` holds the canonical order (in-domain cell rank, then
@@ -96,7 +107,9 @@ constexpr unsigned ORD_SLOT_MASK = (1u << ORD_KIND_SHIFT) - 1u;
 // info word of a free slot: no type, class CR_CLS_NONE, the next free slot + 1
 constexpr int INFO_FREE = 15 | (CR_CLS_NONE << INFO_CLS_SHIFT);
 // a phase's counters beyond the kind counts (misc)
-constexpr int MISC_HW = MISC_N, MISC_FREE = MISC_N + 1, MISC_DIRTY = MISC_N + 2, MISC_TOTAL = MISC_N + 4;
+constexpr int MISC_HW = MISC_N, MISC_FREE = MISC_N + 1, MISC_DIRTY = MISC_N + 2, MISC_RES = MISC_N + 4;
+// and the groups' outcomes of a round, for two rounds in turn
+constexpr int MISC_TOTAL = MISC_RES + 2 * 8;
 
 // FP32 constants of the pair sweep, kept in registers
 struct PairK {
@@ -106,12 +119,16 @@ __device__ __forceinline__ PairK pair_k(const SysParams &P) {
   return PairK{P.Lf, P.halfL, P.rc2, P.alpha, P.c1, P.c2, P.rcf};
 }
 
+// box cell of region coordinate i < nr <= nc along an axis (the domain's k
+// cells from org first, then the h after them, then the h before)
 __device__ __forceinline__ int region_coord(int i, int org, int k, int h, int nr, int nc) {
   int c = (i < k + h) ? org + i : org + i - nr;
-  c %= nc;
-  if (c < 0) c += nc;
-  return c;
+  c += c < 0 ? nc : 0;
+  return c >= nc ? c - nc : c;
 }
+// i / n for 0 <= i < 2^20 with r = 1 / n in FP32 (the half keeps the product
+// away from whole numbers by far more than its rounding)
+__device__ __forceinline__ int div_by(int i, float r) { return (int)(((float)i + 0.5f) * r); }
 
 // Exclusive scan of n ints (shared memory) into pre[0..n] by one warp, each
 // lane a run of consecutive entries
@@ -146,48 +163,34 @@ __device__ __forceinline__ int upper_idx(const int *pre, int n, int j) {
 }
 
 // warp: place of the kth (0-based) entry of a kind in the canonical order, -1
-// if none.  Short lists take one ballot; longer ones eight at a time, so that
-// the loads of 256 entries are in flight together.
-__device__ __forceinline__ int warp_kth(const uint2 *ord, int n, int kind, int kth) {
+// if none.  Long lists are first passed over 256 entries at a time (eight
+// loads in flight, one warp sum); the entry is then found by ballots.  Out of
+// line: one copy of this code serves every selection (the trial loop is bound
+// by instruction fetch).
+__device__ __noinline__ int warp_kth(const uint2 *ord, int n, int kind, int kth) {
   const int lane = threadIdx.x & 31;
-  const unsigned lt = (1u << lane) - 1u;
-  for (int base = 0; base < n; base += 32) {
-    if (n - base > 64) {  // whole 256-entry rounds that end before the kth are skipped together
-      unsigned b[8];
-      int c = 0;
+  int base = 0;
+#pragma unroll 1
+  while (n - base > 64) {
+    int c = 0;
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int j = base + 32 * u + lane;
-        const unsigned e = j < n ? ord[j].x >> ORD_KIND_SHIFT : 15u;
-        b[u] = __ballot_sync(0xffffffffu, e == (unsigned)kind);
-      }
-      int found = -1, before = 0;
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int cu = __popc(b[u]);
-        if (found < 0 && kth < c + cu) {
-          found = u;
-          before = c;
-        }
-        c += cu;
-      }
-      if (found < 0) {
-        kth -= c;
-        base += 224;
-        continue;
-      }
-      unsigned m = 0u;
-#pragma unroll
-      for (int u = 0; u < 8; ++u) m = u == found ? b[u] : m;
-      const unsigned hit = __ballot_sync(0xffffffffu, ((m >> lane) & 1u) && __popc(m & lt) == kth - before);
-      return base + 32 * found + __ffs(hit) - 1;
+    for (int u = 0; u < 8; ++u) {
+      const int j = base + 32 * u + lane;
+      const unsigned e = ord[min(j, n - 1)].x >> ORD_KIND_SHIFT;
+      c += j < n && e == (unsigned)kind ? 1 : 0;
     }
+    c = (int)__reduce_add_sync(0xffffffffu, (unsigned)c);
+    if (kth < c) break;
+    kth -= c;
+    base += 256;
+  }
+#pragma unroll 1
+  for (; base < n; base += 32) {
     const int j = base + lane;
-    const bool m = j < n && (ord[j].x >> ORD_KIND_SHIFT) == (unsigned)kind;
-    const unsigned b = __ballot_sync(0xffffffffu, m);
-    const int c = __popc(b);
+    const unsigned m = __ballot_sync(0xffffffffu, j < n && (ord[j].x >> ORD_KIND_SHIFT) == (unsigned)kind);
+    const int c = __popc(m);
     if (kth < c) {
-      const unsigned hit = __ballot_sync(0xffffffffu, m && __popc(b & lt) == kth);
+      const unsigned hit = __ballot_sync(0xffffffffu, ((m >> lane) & 1u) && __popc(m & ((1u << lane) - 1u)) == kth);
       return base + __ffs(hit) - 1;
     }
     kth -= c;
@@ -197,9 +200,10 @@ __device__ __forceinline__ int warp_kth(const uint2 *ord, int n, int kind, int k
 
 // warp: number of entries with cell rank < r (the ranks ascend); long lists
 // are narrowed 32-fold per round
-__device__ __forceinline__ int warp_lower(const uint2 *ord, int n, int r) {
+__device__ __noinline__ int warp_lower(const uint2 *ord, int n, int r) {
   const int lane = threadIdx.x & 31;
   int base = 0, len = n;
+#pragma unroll 1
   while (len > 32) {
     const int st = (len + 31) >> 5, o = lane * st;
     const int b = __popc(__ballot_sync(0xffffffffu, o < len && (int)ord[base + o].y < r));
@@ -215,6 +219,7 @@ __device__ __forceinline__ int warp_lower(const uint2 *ord, int n, int r) {
 // round from the top down: every load of a round before its stores
 __device__ __forceinline__ void ord_open(uint2 *ord, int n, int p) {
   const int lane = threadIdx.x & 31;
+#pragma unroll 1
   for (int hi = n; hi > p; hi -= 128) {
     const int lo = max(p, hi - 128);
     uint2 x[4];
@@ -233,6 +238,7 @@ __device__ __forceinline__ void ord_open(uint2 *ord, int n, int p) {
 // the bottom up
 __device__ __forceinline__ void ord_close(uint2 *ord, int n, int p) {
   const int lane = threadIdx.x & 31;
+#pragma unroll 1
   for (int lo = p + 1; lo < n; lo += 128) {
     uint2 x[4];
 #pragma unroll
@@ -262,9 +268,10 @@ __device__ __forceinline__ void cc_change_impl(const SysParams &K, const WcaEntr
   double uw[2] = {0.0, 0.0};
   double gs = 0.0;
   bool hit = false;
+#pragma unroll 1
   for (int s = 0; s < 2; ++s) {
-    const bool pres = s ? (t.pa_n && t.pb_n) : (t.pa_o && t.pb_o);
-    if (!pres) continue;
+    const int both = s ? PA_N | PB_N : PA_O | PB_O;
+    if ((t.pres & both) != both) continue;
     const float qa = s ? t.qa_n : t.qa_o, qb = s ? t.qb_n : t.qb_o;
     if (r2 < K.rc2 && qa != 0.0f && qb != 0.0f) {
       const float rinv = rsqrtf(r2);
@@ -279,7 +286,7 @@ __device__ __forceinline__ void cc_change_impl(const SysParams &K, const WcaEntr
       const double r = sqrt(ddx * ddx + ddy * ddy + ddz * ddz);
       if (r < w.wcut_d) {
         const double sv = r - w.del_d;
-        const bool inserted = s == 1 && ((t.pa_n && !t.pa_o) || (t.pb_n && !t.pb_o));
+        const bool inserted = s == 1 && (!(t.pres & PA_O) || !(t.pres & PB_O));  // both are present after
         if (inserted && sv < 0.5 * w.sig_d) {
           ov = 1;
         } else {
@@ -386,10 +393,9 @@ __device__ __forceinline__ int region_of(int r, int dx, int dy, int dz, int k, i
 // one dense layer with ReLU for the two input vectors x[2][n_in] -> y[2][128]:
 // each output is its bias plus one FP32 fused multiply-add per weight, in
 // input order (weights transposed, WT[k][o], so that a warp's loads coalesce)
-template <int T>
 __device__ __forceinline__ void mlp_layer(const uint16_t *__restrict__ WT, const float *__restrict__ b,
-                                          const float *x, int n_in, float *y, int tid) {
-  for (int o = tid; o < 2 * MLP_H; o += T) {
+                                          const float *x, int n_in, float *y, int tid, int n) {
+  for (int o = tid; o < 2 * MLP_H; o += n) {
     const int v = o / MLP_H, i = o % MLP_H;
     const float *xv = x + v * n_in;
     float a = __ldg(&b[i]);
@@ -461,8 +467,8 @@ __device__ __noinline__ PairSum near_pair(const SysParams &P, const WcaEntry &w,
   return out;
 }
 
-// the pair between the two changed particles (one thread per trial; out of
-// line, with its FP64 WCA branch)
+// the pair between the two changed particles when they lie within WCA range
+// of each other (rare; one thread; out of line, with its FP64 branch)
 template <bool WITH_S>
 __device__ __noinline__ PairSum cc_change(const SysParams &P, const TrialCtl &t) {
   PairSum out{0, 0ull, 0};
@@ -488,6 +494,7 @@ template <bool WITH_S>
 __device__ __forceinline__ void queue_flush(const PairK &K, float2 *q, int &qn, long long &acc,
                                             unsigned long long &sacc, int &ov) {
   const int lane = threadIdx.x & 31;
+#pragma unroll 1
   while (qn >= 32) {  // from the end, so that the rest stays where it is
     __syncwarp();
     const float2 e = q[qn - 32 + lane];
@@ -541,6 +548,37 @@ __device__ __forceinline__ SweepPair sweep_pair(const PairK &K, const float *wma
   return p;
 }
 
+// The pair between the two changed particles, as one more queued Coulomb pair:
+// a and b are both present either before the trial or after it, so its change
+// is plus or minus one pair energy, in the same form and rounding as a queued
+// pair's.  Evaluated by one thread of its own it kept the other warps waiting
+// at the trial's barrier.  True when lane 0 of the calling warp queued it;
+// within WCA range it is evaluated here.
+template <bool WITH_S>
+__device__ __forceinline__ bool queue_changed_pair(const SysParams &P, const PairK &K, const float *wr,
+                                                   const TrialCtl &t, float2 *q, long long &acc,
+                                                   unsigned long long &sacc, int &ov) {
+  const Desc &A = t.c[0], &B = t.c[1];
+  const float dx = wrap_diff(B.x, A.x, K.Lf, K.halfL);
+  const float dy = wrap_diff(B.y, A.y, K.Lf, K.halfL);
+  const float dz = wrap_diff(B.z, A.z, K.Lf, K.halfL);
+  const float r2 = dx * dx + dy * dy + dz * dz;
+  const bool after = (t.pres & (PA_N | PB_N)) == (PA_N | PB_N);
+  const float qq = after ? t.qa_n * t.qb_n : -(t.qa_o * t.qb_o);
+  if (r2 < wr[A.cls * 4 + B.cls]) {
+    if ((threadIdx.x & 31) == 0) {
+      const PairSum cc = cc_change<WITH_S>(P, t);
+      acc += cc.acc;
+      sacc += cc.sacc;
+      ov |= cc.ov;
+    }
+    return false;
+  }
+  if (!(r2 < K.rc2) || qq == 0.0f) return false;
+  if ((threadIdx.x & 31) == 0) q[0] = make_float2(r2, P.lBf * qq);
+  return true;
+}
+
 // Both changed particles against one candidate (lane-parallel): two distance
 // tests; the in-range Coulomb pairs of A and B join the warp's queue with one
 // compaction step, and every full 32 queued pairs are evaluated with all
@@ -579,12 +617,26 @@ __device__ __forceinline__ void offer2(const SysParams &P, const PairK &K, const
 }
 
 
-// barrier of a group of G warps (its own named barrier, ids 1 .. 15)
-template <int G>
-__device__ __forceinline__ void group_sync(int group) {
-  if (G == 1) __syncwarp();
-  else asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "r"(32 * G) : "memory");
-}
+// The threads that work on one domain: a whole CTA, or one of its seats.  tid
+// of n; `groups` groups of gn threads each evaluate a trial (several groups
+// only where a domain has the whole CTA; each is then one warp).  Without
+// seats (SEATS false) a domain's barrier is the CTA's.  With seats, seat s has
+// barrier s; a kernel with run-time barrier numbers holds all 16 barriers per
+// CTA, which limits an SM to four CTAs -- no loss for the 256 threads and more
+// of those CTAs, but it halved the residency of 64-thread ones.
+constexpr int MAX_GROUPS = 8;
+template <bool SEATS>
+struct Seat {
+  int tid, n, groups, gn, bar;
+  __device__ __forceinline__ void sync() const {
+    if (SEATS) asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(n) : "memory");
+    else __syncthreads();
+  }
+  __device__ __forceinline__ void group_sync() const {
+    if (gn == 32) __syncwarp();
+    else sync();
+  }
+};
 
 // A CTA's domain, in shared memory (so that the trial loop holds none of it
 // in registers): where it lies, its random-number counters, its list, and the
@@ -597,6 +649,7 @@ struct Dom {
   const int *hpre, *hcell;
   long long log_dom;     // first record of a logged call
   int nhc, hcs;   // halo entries on chip, and their capacity
+  int cpos_at, hcls_at, queue_at;  // byte offsets of cpos, hcls and the queues in the seat's shared memory
   int NH, NR;     // halo entries in all; region cells
   int in_smem, strad, flat, list_cap;
   int org[3], off[3], dd[3], d;
@@ -669,6 +722,11 @@ __device__ __noinline__ void draw_chunk(const SysParams &P, const Dom &D, TrialP
   }
 }
 
+// id of the (first) ion a trial inserts
+__device__ __forceinline__ unsigned long long new_id(uint32_t phi, int d, int m, int kk) {
+  return ((unsigned long long)(phi + 1u) << 32) | (unsigned long long)(2u * ((uint32_t)d * (uint32_t)m + (uint32_t)kk));
+}
+
 // slot of the particle at place i of the canonical order, and a slot's
 // position in [0, L) (w: charge)
 __device__ __forceinline__ int slot_at(const DomList &L, int i) { return (int)(L.ord[i].x & ORD_SLOT_MASK); }
@@ -681,155 +739,104 @@ __device__ __forceinline__ float4 raw_pos(const DomList &L, int s, float Lf) {
 // the move, its participants, the log of the acceptance ratio without the
 // energy, the self-energy change and the two changed particles.  Every lane
 // of the calling warp computes the same values (the list scans are ballots).
-template <bool DA>
+// One path serves the four forms: a is the site, or the first ion of a salt
+// move; b the ion paired with it; a listed particle is the kth of its kind,
+// an inserted one lies at the trial's point.
+template <bool LOG, bool DA>
 __device__ __forceinline__ void select_trial(const SysParams &P, const Dom &D, const int *misc, const TrialPre &q,
                                              int kk, TrialCtl &C) {
-  const DomList L = D.L;
-  const long long *lnt = D.lnt;
-  const int lane = threadIdx.x & 31, d = D.d, m = P.m;
-  const uint32_t phi = D.phi;
+  const int lane = threadIdx.x & 31;
   const int n = misc[0];
   const int mv = pick32(q.w0, 2 * P.n_react);
   const int r = P.react[mv >> 1];
-  const bool fwd = (mv & 1) == 0;
-  int flags = 0, site = -1, ionA = -1, ionB = -1, nch = 0;
-  bool bad = false;
-  long long ln_ratio = 0;
-  const unsigned long long newid = ((unsigned long long)(phi + 1u) << 32) |
-                                   (unsigned long long)(2u * ((uint32_t)d * (uint32_t)m + (uint32_t)kk));
-  unsigned long long id_a = ~0ull, id_b = ~0ull;
-  Desc c0 = {}, c1 = {};
-  float qa_o = 0.f, qa_n = 0.f, qb_o = 0.f, qb_n = 0.f;
-  int pa_o = 0, pa_n = 0, pb_o = 0, pb_n = 0;
-  if (r == R_ACID || r == R_BASE) {
-    const int kn = r == R_ACID ? K_A0 : K_B0, ki = r == R_ACID ? K_A1 : K_B1;
-    const int kx = r == R_ACID ? P.kxp : P.kxm;
-    const float qs = r == R_ACID ? -1.0f : 1.0f;
-    const int n0 = misc[1 + kn], n1 = misc[1 + ki], nx = misc[1 + kx];
-    if (fwd) {
-      if (n0 == 0) flags |= CR_TRIAL_NO_ELIGIBLE;
-      else {
-        site = warp_kth(L.ord, n, kn, pick32(q.w1, n0));
-        if (q.rankA < 0) flags |= CR_TRIAL_EDGE;
-        if (site < 0) { site = 0; bad = true; }
-        const int ss = bad ? 0 : slot_at(L, site);
-        id_a = L.id[ss];
-        id_b = newid;
-        const float4 sp4 = raw_pos(L, ss, P.Lf);
-        const int sinfo = L.info[ss];
-        c0 = Desc{sp4.x, sp4.y, sp4.z, P.lBf * qs, 0, (sinfo >> INFO_CLS_SHIFT) & 3, ss};
-        c1 = Desc{q.ax, q.ay, q.az, P.lBf * (-qs * P.ion_q), 1, P.ion_cls, -1};
-        qa_o = 0.f; qa_n = qs; qb_o = 0.f; qb_n = -qs * P.ion_q;
-        pa_o = pa_n = 1; pb_o = 0; pb_n = 1;
-        nch = 2;
-        ln_ratio = lnt[n0] + P.lnz1_fx - lnt[n1 + 1];
-        ln_ratio -= lnt[nx + 1];
-        ln_ratio += L.lnk[ss];
-      }
-    } else {
-      if (n1 == 0 || nx == 0) flags |= CR_TRIAL_NO_ELIGIBLE;
-      else {
-        site = warp_kth(L.ord, n, ki, pick32(q.w1, n1));
-        ionA = warp_kth(L.ord, n, kx, pick32(q.w2, nx));
-        if (site < 0 || ionA < 0) { site = max(site, 0); ionA = max(ionA, 0); bad = true; }
-        const int ss = bad ? 0 : slot_at(L, site), si = bad ? 0 : slot_at(L, ionA);
-        id_a = L.id[ss];
-        id_b = L.id[si];
-        const float4 sp4 = raw_pos(L, ss, P.Lf), ip4 = raw_pos(L, si, P.Lf);
-        const int sinfo = L.info[ss], iinfo = L.info[si];
-        c0 = Desc{sp4.x, sp4.y, sp4.z, P.lBf * (-qs), 0, (sinfo >> INFO_CLS_SHIFT) & 3, ss};
-        c1 = Desc{ip4.x, ip4.y, ip4.z, P.lBf * (-ip4.w), -1, (iinfo >> INFO_CLS_SHIFT) & 3, si};
-        qa_o = qs; qa_n = 0.f; qb_o = ip4.w; qb_n = 0.f;
-        pa_o = pa_n = 1; pb_o = 1; pb_n = 0;
-        nch = 2;
-        ln_ratio = lnt[n1] - lnt[n0 + 1] - P.lnz1_fx;
-        ln_ratio += lnt[nx];
-        ln_ratio -= L.lnk[ss];
-      }
-    }
+  const bool fwd = (mv & 1) == 0, salt = r == R_SALT;
+  const int kn = r == R_ACID ? K_A0 : K_B0;      // the site's neutral kind; the ionised one follows it
+  const float qs = r == R_ACID ? -1.0f : 1.0f;   // its charge when ionised
+  const bool listA = !salt || !fwd, listB = !fwd;
+  const int kA = salt ? P.kxp : (fwd ? kn : kn + 1), kB = salt || r == R_BASE ? P.kxm : P.kxp;
+  const int nA = misc[1 + kA], nB = misc[1 + kB];
+  int flags = 0, sA = -1, sB = -1, placeA = -1, placeB = -1;
+  if ((listA && nA == 0) || (listB && nB == 0)) {
+    flags = CR_TRIAL_NO_ELIGIBLE;
   } else {
-    const int nxp = misc[1 + P.kxp], nxm = misc[1 + P.kxm];
-    if (fwd) {
-      if (q.rankA < 0 || q.rankB < 0) flags |= CR_TRIAL_EDGE;
-      id_a = newid;
-      id_b = newid + 1u;
-      c0 = Desc{q.ax, q.ay, q.az, P.lBf * P.ion_q, 1, P.ion_cls, -1};
-      c1 = Desc{q.bx, q.by, q.bz, P.lBf * (-P.ion_q), 1, P.ion_cls, -1};
-      qa_o = 0.f; qa_n = P.ion_q; qb_o = 0.f; qb_n = -P.ion_q;
-      pa_o = 0; pa_n = 1; pb_o = 0; pb_n = 1;
-      nch = 2;
-      ln_ratio = 2 * P.lnz1_fx + P.lnsalt_fx;
-      ln_ratio -= lnt[nxp + 1] + lnt[nxm + 1];
-    } else {
-      if (nxp == 0 || nxm == 0) flags |= CR_TRIAL_NO_ELIGIBLE;
-      else {
-        ionA = warp_kth(L.ord, n, P.kxp, pick32(q.w2, nxp));
-        ionB = warp_kth(L.ord, n, P.kxm, pick32(q.w3, nxm));
-        if (ionA < 0 || ionB < 0) { ionA = max(ionA, 0); ionB = max(ionB, 0); bad = true; }
-        const int sa = bad ? 0 : slot_at(L, ionA), sb = bad ? 0 : slot_at(L, ionB);
-        id_a = L.id[sa];
-        id_b = L.id[sb];
-        const float4 a4 = raw_pos(L, sa, P.Lf), b4 = raw_pos(L, sb, P.Lf);
-        c0 = Desc{a4.x, a4.y, a4.z, P.lBf * (-a4.w), -1, (L.info[sa] >> INFO_CLS_SHIFT) & 3, sa};
-        c1 = Desc{b4.x, b4.y, b4.z, P.lBf * (-b4.w), -1, (L.info[sb] >> INFO_CLS_SHIFT) & 3, sb};
-        qa_o = a4.w; qa_n = 0.f; qb_o = b4.w; qb_n = 0.f;
-        pa_o = 1; pa_n = 0; pb_o = 1; pb_n = 0;
-        nch = 2;
-        ln_ratio = -2 * P.lnz1_fx - P.lnsalt_fx;
-        ln_ratio += lnt[nxp] + lnt[nxm];
-      }
+    if (fwd && (q.rankA < 0 || (salt && q.rankB < 0))) flags = CR_TRIAL_EDGE;
+    if (listA) placeA = warp_kth(D.L.ord, n, kA, pick32(salt ? q.w2 : q.w1, nA));
+    if (listB) placeB = warp_kth(D.L.ord, n, kB, pick32(salt ? q.w3 : q.w2, nB));
+    // a failed selection would mean the kind counts and the list disagree:
+    // record it and reject instead of touching memory outside the list
+    if ((listA && placeA < 0) || (listB && placeB < 0)) {
+      flags |= CR_TRIAL_NO_ELIGIBLE;
+      placeA = placeB = -1;
+      if (lane == 0) atomicOr(P.err, ERRB_ARG);
     }
   }
-  // a failed selection would mean the kind counts and the list disagree:
-  // record it and reject instead of touching memory outside the list
-  if (bad) {
-    flags |= CR_TRIAL_NO_ELIGIBLE;
-    if (lane == 0) atomicOr(P.err, ERRB_ARG);
+  Desc c0 = {q.ax, q.ay, q.az, 0.0f, 1, P.ion_cls, -1};
+  Desc c1 = salt ? Desc{q.bx, q.by, q.bz, 0.0f, 1, P.ion_cls, -1} : c0;
+  float qa_o = 0.0f, qa_n = 0.0f, qb_o = 0.0f, qb_n = 0.0f;
+  long long lnk = 0;
+  int rka = q.rankA, rkb = salt ? q.rankB : q.rankA;
+  unsigned long long id_a = ~0ull, id_b = ~0ull;
+  if (placeA >= 0) {
+    sA = slot_at(D.L, placeA);
+    const float4 p = raw_pos(D.L, sA, P.Lf);
+    c0 = Desc{p.x, p.y, p.z, 0.0f, salt ? -1 : 0, (D.L.info[sA] >> INFO_CLS_SHIFT) & 3, sA};
+    qa_o = p.w;
+    lnk = D.L.lnk[sA];
+    if (DA) rka = (int)D.L.ord[placeA].y;
+    if (LOG) id_a = D.L.id[sA];
   }
-  nch = (flags & (CR_TRIAL_NO_ELIGIBLE | CR_TRIAL_EDGE)) ? 0 : nch;
+  if (placeB >= 0) {
+    sB = slot_at(D.L, placeB);
+    const float4 p = raw_pos(D.L, sB, P.Lf);
+    c1 = Desc{p.x, p.y, p.z, 0.0f, -1, (D.L.info[sB] >> INFO_CLS_SHIFT) & 3, sB};
+    qb_o = p.w;
+    if (DA) rkb = (int)D.L.ord[placeB].y;
+    if (LOG) id_b = D.L.id[sB];
+  }
+  if (fwd) {
+    qa_n = salt ? P.ion_q : qs;
+    qb_n = (salt ? -1.0f : -qs) * P.ion_q;
+  }
+  c0.dqlB = P.lBf * (qa_n - qa_o);
+  c1.dqlB = P.lBf * (qb_n - qb_o);
+  const int pres = salt ? (fwd ? PA_N | PB_N : PA_O | PB_O) : (fwd ? PA_O | PA_N | PB_N : PA_O | PA_N | PB_O);
+  // the combinatorial and chemical factor; the counts after a forward move
+  // are one higher, and a reverse move has the inverse form
+  const long long *lnt = D.lnt;
+  const int up = fwd ? 1 : 0;
+  long long ln = P.lnz1_fx - lnt[nB + up];
+  if (salt) ln += P.lnz1_fx + P.lnsalt_fx - lnt[nA + up];
+  else ln += lnk;
+  ln = fwd ? ln : -ln;
+  if (!salt) ln += lnt[nA] - lnt[misc[1 + (fwd ? kn + 1 : kn)] + 1];
   // self-energy change: lB s_self (sum of q_new^2 - q_old^2), an integer multiple
-  const int sq = (pa_n ? (int)(qa_n * qa_n) : 0) - (pa_o ? (int)(qa_o * qa_o) : 0) +
-                 (pb_n ? (int)(qb_n * qb_n) : 0) - (pb_o ? (int)(qb_o * qb_o) : 0);
+  const int sq = (int)(qa_n * qa_n) - (int)(qa_o * qa_o) + (int)(qb_n * qb_n) - (int)(qb_o * qb_o);
   // lane 0 publishes the selection (C lives in shared memory; every lane
   // holds the same values)
-  int rka = 0, rkb = 0;
-  if (DA && nch) {
-    if (r == R_SALT) {
-      rka = fwd ? q.rankA : (int)L.ord[ionA].y;
-      rkb = fwd ? q.rankB : (int)L.ord[ionB].y;
-    } else {
-      rka = (int)L.ord[site].y;
-      rkb = fwd ? q.rankA : (int)L.ord[ionA].y;
-    }
-  }
   if (lane == 0) {
     C.c[0] = c0;
     C.c[1] = c1;
-    C.nch = nch;
+    C.nch = flags & (CR_TRIAL_NO_ELIGIBLE | CR_TRIAL_EDGE) ? 0 : 2;
     C.move = 2 * r + (fwd ? 0 : 1);
     C.flags = flags;
-    C.site = site;
-    C.ionA = ionA;
-    C.ionB = ionB;
-    C.ln_ratio_fx = ln_ratio;
+    C.placeA = placeA;
+    C.placeB = placeB;
+    C.pres = pres;
+    C.ln_ratio_fx = ln;
     C.dself_fx = P.lBself_fx * (long long)sq;
-    C.id_a = id_a;
-    C.id_b = id_b;
-    C.newid = newid;
-    C.sur = 0.0f;
-    C.sur_fx = 0;
     C.qa_o = qa_o; C.qa_n = qa_n; C.qb_o = qb_o; C.qb_n = qb_n;
-    C.pa_o = pa_o; C.pa_n = pa_n; C.pb_o = pb_o; C.pb_n = pb_n;
-    C.rka = rka;
-    C.rkb = rkb;
-    C.dqa = C.dqb = C.eta_a = C.eta_b = C.cat_a = 0;
-    C.go = 1;
+    if (LOG) {  // the ids of a trial without eligible particles stay unused
+      const unsigned long long nid = new_id(D.phi, D.d, P.m, kk);
+      const bool none = flags & CR_TRIAL_NO_ELIGIBLE;
+      C.id_a = listA ? id_a : nid;
+      C.id_b = none || listB ? id_b : (salt ? nid + 1u : nid);
+    }
     if (DA) {
-      C.dqa = (pa_n ? __float2int_rn(qa_n) : 0) - (pa_o ? __float2int_rn(qa_o) : 0);
-      C.dqb = (pb_n ? __float2int_rn(qb_n) : 0) - (pb_o ? __float2int_rn(qb_o) : 0);
-      C.eta_a = pa_n - pa_o;
-      C.eta_b = pb_n - pb_o;
-      C.cat_a = r == R_SALT ? 0 : 8;
+      C.rka = rka;
+      C.rkb = rkb;
+      C.go = 1;
+      C.sur = 0.0f;
+      C.sur_fx = 0;
     }
   }
 }
@@ -847,6 +854,7 @@ __device__ __noinline__ PairSum sweep_rest(const SysParams &P, const TrialCtl &C
   const float4 *lpos = Rg.L.pos;
   const int *linfo = Rg.L.info;
   const int nover = Rg.NH - Rg.nhc, total = nover + (Rg.in_smem ? 0 : nlist);
+#pragma unroll 1
   for (int base = 0; base < total; base += stride) {
     const int u = base + i0;
     float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -879,7 +887,7 @@ __device__ __noinline__ PairSum sweep_rest(const SysParams &P, const TrialCtl &C
 // The pair changes of the two changed particles A and B against the halo and
 // the domain list, summed by a group of threads (thread i0 of `stride`; each
 // thread's part is returned; the warp's queued Coulomb pairs are evaluated at
-// the end).  The pair between A and B is not included.  One loop over the halo
+// the end), and the pair between A and B.  One loop over the halo
 // and the list in shared memory; per 32 candidates it costs two distance tests
 // and one compaction.
 template <bool LOG, bool FLAT>
@@ -890,9 +898,11 @@ __device__ __forceinline__ PairSum sweep_pairs(const PairK &K, const SysParams &
   const SweepPair sp = sweep_pair(K, Rg.wr + 16, C.c[0], C.c[1], Rg.strad);
   PairSum out{0, 0ull, 0};
   int qn = 0;
+  if (i0 < 32 && queue_changed_pair<LOG>(P, K, Rg.wr, C, q, out.acc, out.sacc, out.ov)) qn = 1;
   const int nhc = Rg.nhc, total = nhc + (Rg.in_smem ? nlist : 0);
   const int gap = Rg.hcs - nhc;  // from the on-chip halo to the list's slots
   const int skA = sp.skA >= 0 ? nhc + sp.skA : -1, skB = sp.skB >= 0 ? nhc + sp.skB : -1;
+#pragma unroll 1
   for (int base = 0; base < total; base += stride) {
     const int u = base + i0;
     const bool v = u < total && u != skA && u != skB;
@@ -965,8 +975,8 @@ __device__ __noinline__ void ewald_factors(const SysParams &P, const TrialCtl &C
     f[i] = ew_factor(ew_frac32(x, P.invLd), n);
   }
   if (tid == 0) {
-    dq[0] = (C.pa_n ? C.qa_n : 0.0f) - (C.pa_o ? C.qa_o : 0.0f);
-    dq[1] = (C.pb_n ? C.qb_n : 0.0f) - (C.pb_o ? C.qb_o : 0.0f);
+    dq[0] = (has(C, 0) ? C.qa_n : 0.0f) - (had(C, 0) ? C.qa_o : 0.0f);
+    dq[1] = (has(C, 1) ? C.qb_n : 0.0f) - (had(C, 1) ? C.qb_o : 0.0f);
   }
 }
 
@@ -1039,111 +1049,119 @@ __device__ __noinline__ void ewald_update(const SysParams &P, const float2 *f, c
   }
 }
 
-// payload slot for a new particle: the last one freed, or the next unused one
-__device__ __forceinline__ int slot_take(const DomList &L, int *misc) {
-  const int f = misc[MISC_FREE];
-  if (f > 0) {
-    misc[MISC_FREE] = L.info[f - 1] >> INFO_SITE_SHIFT;
-    return f - 1;
-  }
-  return misc[MISC_HW]++;
-}
-
-// warp: a new ion of cell rank `rank` joins the list (n entries) at place p,
-// after every entry of its cell, as new ids are the largest
-__device__ __forceinline__ void insert_ion(const SysParams &P, const DomList &L, int *misc, int n, int p, int rank,
-                                           float x, float y, float z, float q, const float4 &vel,
-                                           unsigned long long id, int type, int kind, int strad) {
-  ord_open(L.ord, n, p);
-  if ((threadIdx.x & 31) == 0) {
-    const int s = slot_take(L, misc);
-    L.pos[s] = make_float4(frame_x(x, strad, 0, P.halfL, P.Lf), frame_x(y, strad, 1, P.halfL, P.Lf),
-                           frame_x(z, strad, 2, P.halfL, P.Lf), q);
-    L.vel[s] = vel;
-    L.id[s] = id;
-    L.lnk[s] = 0;
-    L.info[s] = type | (P.ion_cls << INFO_CLS_SHIFT);
-    L.ord[p] = make_uint2((unsigned)s | ((unsigned)kind << ORD_KIND_SHIFT), (unsigned)rank);
-  }
-  __syncwarp();
-}
-
-// warp: the particle at place p leaves the list (n entries)
-__device__ __forceinline__ void remove_ion(const DomList &L, int *misc, int n, int p) {
-  if ((threadIdx.x & 31) == 0) {
-    const int s = slot_at(L, p);
-    L.pos[s].w = 0.0f;
-    L.info[s] = INFO_FREE | (misc[MISC_FREE] << INFO_SITE_SHIFT);
-    misc[MISC_FREE] = s + 1;
-  }
-  __syncwarp();
-  ord_close(L.ord, n, p);
-}
-
 // An accepted trial, by one warp: room for the ions an insertion adds -- their
 // cells below the cell capacity and the list below its capacity (else -1 and
-// nothing changes) -- then the site's charge state, the ions inserted or
-// deleted, the kind counts.  Returns the new list size.  Out of line: it runs
-// only for accepted trials and is large.
+// nothing changes) -- then the site's charge state, the ions inserted (after
+// every entry of their cells, as new ids are the largest) or deleted, the kind
+// counts.  Returns the new list size.  Out of line: it runs only for accepted
+// trials.  Lists that fit a warp (n + 2 <= 32) hold their order in the lanes
+// meanwhile.
 __device__ __noinline__ int try_commit(const SysParams &P, const Dom &D, int *misc, const TrialCtl &C,
-                                       const TrialPre &q, const float4 *vel, int n) {
-  const int lane = threadIdx.x & 31, list_cap = D.list_cap, strad = D.strad;
+                                       const TrialPre &q, const float4 *vel, int kk, int n) {
+  const int lane = threadIdx.x & 31;
   const DomList &L = D.L;
   const int r = C.move >> 1;
-  const bool fwd = (C.move & 1) == 0;
-  const float qs = r == R_BASE ? 1.0f : -1.0f;  // charge of an ionised site
-  int pA = 0, pB = 0;
+  const bool fwd = (C.move & 1) == 0, salt = r == R_SALT;
+  const int kn = r == R_ACID ? K_A0 : K_B0;
+  const int nion = salt ? 2 : 1;
+  // the ions of the move: kind of the last one (b); a salt move's first is the cation
+  const int kB = salt || r == R_BASE ? P.kxm : P.kxp;
+  const bool small = n + 2 <= 32;
+  uint2 e = make_uint2(15u << ORD_KIND_SHIFT, 0x7fffffffu);
+  if (small && lane < n) e = L.ord[lane];
+  int at0 = 0, at1 = 0;  // places of the ions inserted
   if (fwd) {
-    const int loA = warp_lower(L.ord, n, q.rankA);
-    pA = warp_lower(L.ord, n, q.rankA + 1);
-    bool full = pA - loA + 1 > P.cap;
-    if (r == R_SALT) {
-      const int loB = warp_lower(L.ord, n, q.rankB);
-      pB = warp_lower(L.ord, n, q.rankB + 1);
-      full = full || pB - loB + 1 + (q.rankB == q.rankA ? 1 : 0) > P.cap;
+    bool full = n + 2 > D.list_cap;
+#pragma unroll 1
+    for (int x = 2 - nion; x < 2; ++x) {
+      const int rk = salt && x ? q.rankB : q.rankA;
+      int below, upto;
+      if (small) {
+        below = __popc(__ballot_sync(FULL, (int)e.y < rk));
+        upto = __popc(__ballot_sync(FULL, (int)e.y <= rk));
+      } else {
+        below = warp_lower(L.ord, n, rk);
+        upto = warp_lower(L.ord, n, rk + 1);
+      }
+      if (x) at1 = upto;
+      else at0 = upto;
+      full = full || upto - below + 1 + (salt && x && q.rankB == q.rankA ? 1 : 0) > P.cap;
     }
-    if (full || n + 2 > list_cap) return -1;
+    if (full) return -1;
+    // the first ion of a salt move lies before the second unless its cell ranks higher
+    if (salt && q.rankA <= q.rankB) at1 += 1;
   }
-  const int move_kind = r == R_SALT || (r == R_ACID) ? P.kxp : P.kxm;  // kind of the first ion
-  if (r != R_SALT) {
-    if (lane == 0) {
-      const int s = slot_at(L, C.site);
-      const int kn = r == R_ACID ? K_A0 : K_B0, ki = kn + 1, dlt = fwd ? 1 : -1;
-      L.info[s] ^= INFO_ION_BIT;
-      L.pos[s].w = fwd ? qs : 0.0f;
-      L.ord[C.site].x = (unsigned)s | ((unsigned)(fwd ? ki : kn) << ORD_KIND_SHIFT);
-      misc[1 + kn] -= dlt;
-      misc[1 + ki] += dlt;
-      misc[1 + move_kind] += dlt;
-    }
+  if (!salt) {  // the site's charge state
+    const int sl = slot_at(L, C.placeA), kd = fwd ? kn + 1 : kn, dlt = fwd ? 1 : -1;
+    const unsigned ne = (unsigned)sl | ((unsigned)kd << ORD_KIND_SHIFT);
     __syncwarp();
+    if (lane == 0) {
+      L.info[sl] ^= INFO_ION_BIT;
+      L.pos[sl].w = C.qa_n;
+      L.ord[C.placeA].x = ne;
+      misc[1 + kn] -= dlt;
+      misc[2 + kn] += dlt;
+    }
+    if (lane == C.placeA) e.x = ne;
+    __syncwarp();
+  }
+  // the ions, one after another: inserted in the order a, b; deleted from the
+  // higher place down
+#pragma unroll 1
+  for (int y = 0; y < nion; ++y) {
+    const bool swap = salt && !fwd && C.placeB < C.placeA;
+    const int x = nion == 1 ? 1 : (fwd || swap ? y : 1 - y);
+    const int kind = x ? kB : P.kxp;
+    const int p = x ? (fwd ? at1 : C.placeB) : (fwd ? at0 : C.placeA);
     if (fwd) {
-      insert_ion(P, L, misc, n, pA, q.rankA, q.ax, q.ay, q.az, -qs * P.ion_q, vel[0], C.newid,
-                 r == R_ACID ? P.txp : P.txm, move_kind, strad);
+      const int f = misc[MISC_FREE];  // the last slot freed, or the next unused one
+      const int sl = f > 0 ? f - 1 : misc[MISC_HW];
+      const bool second = salt && x;
+      const uint2 ne = make_uint2((unsigned)sl | ((unsigned)kind << ORD_KIND_SHIFT),
+                                  (unsigned)(second ? q.rankB : q.rankA));
+      __syncwarp();
+      if (lane == 0) {
+        if (f > 0) misc[MISC_FREE] = L.info[sl] >> INFO_SITE_SHIFT;
+        else misc[MISC_HW] = sl + 1;
+        const float X = second ? q.bx : q.ax, Y = second ? q.by : q.ay, Z = second ? q.bz : q.az;
+        L.pos[sl] = make_float4(frame_x(X, D.strad, 0, P.halfL, P.Lf), frame_x(Y, D.strad, 1, P.halfL, P.Lf),
+                                frame_x(Z, D.strad, 2, P.halfL, P.Lf), x ? C.qb_n : C.qa_n);
+        L.vel[sl] = vel[second ? 1 : 0];
+        L.id[sl] = new_id(D.phi, D.d, P.m, kk) + (second ? 1u : 0u);
+        L.lnk[sl] = 0;
+        L.info[sl] = (kind == P.kxp ? P.txp : P.txm) | (P.ion_cls << INFO_CLS_SHIFT);
+        misc[1 + kind] += 1;
+      }
+      if (small) {
+        const unsigned ex = __shfl_up_sync(FULL, e.x, 1), ey = __shfl_up_sync(FULL, e.y, 1);
+        if (lane > p) e = make_uint2(ex, ey);
+        if (lane == p) e = ne;
+      } else {
+        ord_open(L.ord, n, p);
+        if (lane == 0) L.ord[p] = ne;
+        __syncwarp();
+      }
       n += 1;
     } else {
-      remove_ion(L, misc, n, C.ionA);
+      const int sl = small ? (int)(__shfl_sync(FULL, e.x, p) & ORD_SLOT_MASK) : slot_at(L, p);
+      __syncwarp();
+      if (lane == 0) {
+        L.pos[sl].w = 0.0f;
+        L.info[sl] = INFO_FREE | (misc[MISC_FREE] << INFO_SITE_SHIFT);
+        misc[MISC_FREE] = sl + 1;
+        misc[1 + kind] -= 1;
+      }
+      if (small) {
+        const unsigned ex = __shfl_down_sync(FULL, e.x, 1), ey = __shfl_down_sync(FULL, e.y, 1);
+        if (lane >= p) e = make_uint2(ex, ey);
+      } else {
+        ord_close(L.ord, n, p);
+      }
       n -= 1;
     }
-  } else {
-    if (fwd) {
-      insert_ion(P, L, misc, n, pA, q.rankA, q.ax, q.ay, q.az, P.ion_q, vel[0], C.newid, P.txp, P.kxp, strad);
-      // the first ion lies before the second's place unless its cell ranks higher
-      insert_ion(P, L, misc, n + 1, pB + (q.rankA <= q.rankB ? 1 : 0), q.rankB, q.bx, q.by, q.bz, -P.ion_q, vel[1],
-                 C.newid + 1u, P.txm, P.kxm, strad);
-      n += 2;
-    } else {
-      const int hi = max(C.ionA, C.ionB), lo = min(C.ionA, C.ionB);
-      remove_ion(L, misc, n, hi);
-      remove_ion(L, misc, n - 1, lo);
-      n -= 2;
-    }
-    if (lane == 0) {
-      const int dlt = fwd ? 1 : -1;
-      misc[1 + P.kxp] += dlt;
-      misc[1 + P.kxm] += dlt;
-    }
+    __syncwarp();
   }
+  if (small && lane < n) L.ord[lane] = e;
   if (lane == 0) {
     misc[0] = n;
     misc[MISC_DIRTY] = 1;
@@ -1154,27 +1172,28 @@ __device__ __noinline__ int try_commit(const SysParams &P, const Dom &D, int *mi
 
 }  // namespace
 
-// Shared memory of a phase CTA: the bytes of each array in order (every array
-// starts on a 16-byte boundary); fills S.off and returns the total.
-static size_t phase_layout(PhaseShape &S, int warps, int groups, bool da) {
-  const size_t dcs = S.dcs, chunk = S.chunk, nr3 = S.nr3 + 1, kc3 = S.kc3 + 1;
-  const size_t bytes[PhaseShape::N_OFF] = {
+// Shared memory of a domain's seat: the bytes of each array in order (every
+// array starts on a 16-byte boundary); fills the layout, returns the total.
+static size_t phase_layout(const PhaseCaps &C, const PhaseShape &S, int warps, int cta_warps, int groups, bool da,
+                           PhaseLayout &Y) {
+  const size_t dcs = C.dcs, chunk = S.chunk, nr3 = S.nr3 + 1, kc3 = S.kc3 + 1;
+  const size_t bytes[PhaseLayout::N_OFF] = {
       sizeof(SysParams),
       sizeof(Dom),
-      sizeof(float4) * (S.hcs + dcs),         // halo, then the list's positions
+      sizeof(float4) * (C.hcs + dcs),         // halo, then the list's positions
       sizeof(float4) * dcs,                   // velocities
       sizeof(unsigned long long) * dcs,       // ids
       sizeof(long long) * dcs,                // site constants
       sizeof(int) * dcs,                      // info words
       sizeof(uint2) * dcs,                    // canonical order
-      (size_t)S.hcs,                          // halo classes
-      sizeof(long long) * S.lns,              // log table
+      (size_t)C.hcs,                          // halo classes
+      sizeof(long long) * C.lns,              // log table
       sizeof(TrialPre) * chunk,
       sizeof(float4) * 2 * chunk,             // velocities of inserted ions
       sizeof(TrialCtl) * groups,
-      sizeof(long long) * warps,              // the warps' sums
-      sizeof(unsigned long long) * warps,
-      sizeof(int) * warps,
+      sizeof(long long) * cta_warps,          // the warps' sums
+      sizeof(unsigned long long) * cta_warps,
+      sizeof(int) * cta_warps,
       sizeof(float2) * QCAP * warps,          // queues of Coulomb pairs
       sizeof(int) * MISC_TOTAL,
       sizeof(int) * nr3,                      // halo cells: counts, cells, prefix sums
@@ -1193,10 +1212,18 @@ static size_t phase_layout(PhaseShape &S, int warps, int groups, bool da) {
       da ? sizeof(float) * 2 * MLP_H * groups : 0,
       da ? sizeof(float) * 2 * MLP_H * groups : 0};
   size_t at = 0;
-  for (int i = 0; i < PhaseShape::N_OFF; ++i) {
-    S.off[i] = (unsigned)at;
-    at += (bytes[i] + 15) / 16 * 16;
-  }
+  for (int pass = 0; pass < 2; ++pass)  // first the arrays whose place is the same in both of a launch's layouts
+    for (int i = 0; i < PhaseLayout::N_OFF; ++i) {
+      const bool sized = (i >= 2 && i <= 9) || (i >= 16 && i <= 23 && i != 17);
+      if (sized != (pass == 1)) continue;
+      Y.off[i] = (unsigned)at;
+      at += (bytes[i] + 15) / 16 * 16;
+    }
+  Y.dcs = C.dcs;
+  Y.hcs = C.hcs;
+  Y.lns = C.lns;
+  Y.chunk = S.chunk;
+  Y.ewk = S.ewk;
   return at;
 }
 
@@ -1205,32 +1232,34 @@ static size_t phase_layout(PhaseShape &S, int warps, int groups, bool da) {
 // the colour's launch order.  Every thread of the CTA calls it; smem is the
 // CTA's dynamic shared memory (phase_layout).
 //
-// The CTA is W groups of G warps.
-template <int G, int W, bool LOG, bool DA>
-__device__ __forceinline__ void phase_task(unsigned char *smem, const SysParams *__restrict__ reps,
-                                           const PhaseShape &S, uint32_t sweep, uint32_t sweep0, int colour,
-                                           uint32_t key0, uint32_t key1_base, int rep, int rank) {
-  constexpr int T = 32 * G * W, GT = 32 * G;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int group = W > 1 ? warp / G : 0, gwarp = warp % G, gtid = tid - group * GT;
-
+// Seat threads split into groups: with more than one, the groups take the next
+// trials together, each as if those before it were rejected; the trials up to
+// the first accepted one are then decided exactly as one after another, and
+// the rest are evaluated again on the new state (so the outcomes do not depend
+// on the number).
+template <bool LOG, bool DA, bool SEATS>
+__device__ __forceinline__ void phase_task(unsigned char *smem, const PhaseArgs &A, int which, const Seat<SEATS> seat,
+                                           const SysParams *__restrict__ reps, uint32_t sweep, uint32_t sweep0,
+                                           int colour, uint32_t key0, uint32_t key1_base, int rep, int rank) {
+  const int tid = seat.tid, T = seat.n, GT = seat.gn, lane = tid & 31, warp = tid >> 5;
+  const int group = seat.groups > 1 ? tid / GT : 0, gtid = tid - group * GT, gwarp = gtid >> 5;
   // (the offsets come from the launch's constant parameters)
-#define CRMC_AT(i) (smem + S.off[i])
+#define CRMC_AT(i) (smem + A.lay[0].off[i])
+#define CRMC_SIZED(i) (smem + A.lay[SEATS ? which : 0].off[i])
   SysParams &P = *(SysParams *)CRMC_AT(0);
   Dom &D = *(Dom *)CRMC_AT(1);
-  float4 *cpos = (float4 *)CRMC_AT(2);  // halo [hcs], then the list's positions [dcs]
-  unsigned char *hcls = CRMC_AT(8);
-  long long *lntab_s = (long long *)CRMC_AT(9);
+  float4 *cpos = (float4 *)CRMC_SIZED(2);  // halo [hcs], then the list's positions [dcs]
+  unsigned char *hcls = CRMC_SIZED(8);
+  long long *lntab_s = (long long *)CRMC_SIZED(9);
   TrialPre *tp = (TrialPre *)CRMC_AT(10);
   float4 *tvel = (float4 *)CRMC_AT(11);
   TrialCtl *ctls = (TrialCtl *)CRMC_AT(12);
   long long *red = (long long *)CRMC_AT(13);
   unsigned long long *reds = (unsigned long long *)CRMC_AT(14);
   int *redov = (int *)CRMC_AT(15);
-  float2 *queue = (float2 *)CRMC_AT(16) + warp * QCAP;
   int *misc = (int *)CRMC_AT(17);  // [0] list size, [1 + kind] counts, [MISC_INIT + kind] at start, MISC_HW ...
-  int *hcnt = (int *)CRMC_AT(18), *hcell = (int *)CRMC_AT(19), *hpre = (int *)CRMC_AT(20);
-  int *dcnt = (int *)CRMC_AT(21), *dcell = (int *)CRMC_AT(22), *dpre = (int *)CRMC_AT(23);
+  int *hcnt = (int *)CRMC_SIZED(18), *hcell = (int *)CRMC_SIZED(19), *hpre = (int *)CRMC_SIZED(20);
+  int *dcnt = (int *)CRMC_SIZED(21), *dcell = (int *)CRMC_SIZED(22), *dpre = (int *)CRMC_SIZED(23);
   float2 *ewf = (float2 *)CRMC_AT(24);
   float *ewq = (float *)CRMC_AT(25);
   int *aQi = nullptr, *aQs = nullptr, *aN = nullptr, *dfeat = nullptr;
@@ -1252,7 +1281,7 @@ __device__ __forceinline__ void phase_task(unsigned char *smem, const SysParams 
     for (int i = tid; i < (int)(sizeof(SysParams) / 16); i += T) dst[i] = src[i];
   }
   if (tid < MISC_TOTAL) misc[tid] = 0;
-  __syncthreads();
+  seat.sync();
   if (rank >= P.nact) return;  // uniform over the CTA
   const int bdom = P.order ? P.order[colour * P.nact + rank] : rank;  // active-domain index
   const int k = P.k, h = P.h, nc = P.nc, nr = P.nr, m = P.m;
@@ -1293,30 +1322,33 @@ __device__ __forceinline__ void phase_task(unsigned char *smem, const SysParams 
   // ---- the region's cells and their counts (four cells per thread at a
   // time, so that their loads are in flight together): the domain's own by
   // rank, the halo's by region index (zero at the domain's)
+  const float rnr = 1.0f / (float)nr;
+#pragma unroll 1
   for (int i0 = tid; i0 < NR; i0 += 4 * T) {
     int cl[4], cn[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      const int i = min(i0 + u * T, NR - 1);
-      const int ix = i % nr, iy = (i / nr) % nr, iz = i / (nr * nr);
+      const int i = min(i0 + u * T, NR - 1), iyz = div_by(i, rnr), iz = div_by(iyz, rnr);
+      const int ix = i - iyz * nr, iy = iyz - iz * nr;
       cl[u] = region_coord(ix, org[0], k, h, nr, nc) +
               nc * (region_coord(iy, org[1], k, h, nr, nc) + nc * region_coord(iz, org[2], k, h, nr, nc));
+      // the domain's own cells by rank, the others marked
+      const int r = ix < k && iy < k && iz < k ? ix + k * (iy + k * iz) : -1;
+      cn[u] = P.cnt[cl[u]];
+      cl[u] |= r >= 0 ? 0x80000000 : 0;
+      if (r >= 0 && i0 + u * T < NR) {
+        dcell[r] = cl[u] & 0x7fffffff;
+        hcell[i] = r;
+      }
     }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) cn[u] = P.cnt[cl[u]];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const int i = i0 + u * T;
       if (i >= NR) break;
-      const int ix = i % nr, iy = (i / nr) % nr, iz = i / (nr * nr);
-      const bool own = ix < k && iy < k && iz < k;
+      const bool own = cl[u] < 0;
       hcnt[i] = own ? 0 : cn[u];
-      hcell[i] = cl[u];
-      if (own) {
-        const int r = ix + k * (iy + k * iz);
-        dcnt[r] = cn[u];
-        dcell[r] = cl[u];
-      }
+      if (own) dcnt[hcell[i]] = cn[u];
+      hcell[i] = cl[u] & 0x7fffffff;
     }
   }
   // the WCA pre-check radii
@@ -1324,17 +1356,17 @@ __device__ __forceinline__ void phase_task(unsigned char *smem, const SysParams 
   if (tid < 4)
     D.wr[16 + tid] = fmaxf(fmaxf(wca_radius(P.wca[4 * tid]), wca_radius(P.wca[4 * tid + 1])),
                            fmaxf(wca_radius(P.wca[4 * tid + 2]), wca_radius(P.wca[4 * tid + 3])));
-  __syncthreads();
+  seat.sync();
   if (warp == 0) warp_scan(dcnt, KC, dpre);
   if (warp == (T > 32 ? 1 : 0)) warp_scan(hcnt, NR, hpre);
-  __syncthreads();
+  seat.sync();
   const int ND = dpre[KC], NH = hpre[NR];
-  const int nhc = min(NH, S.hcs);
+  const int nhc = min(NH, A.lay[SEATS ? which : 0].hcs);
   // the list lives in shared memory unless the domain is unusually dense
-  const bool in_smem = ND + 2 * m <= S.dcs;
+  const bool in_smem = ND + 2 * m <= A.lay[SEATS ? which : 0].dcs;
   DomList L;
-  L.pos = cpos + S.hcs; L.vel = (float4 *)CRMC_AT(3); L.id = (unsigned long long *)CRMC_AT(4); L.lnk = (long long *)CRMC_AT(5);
-  L.info = (int *)CRMC_AT(6); L.ord = (uint2 *)CRMC_AT(7);
+  L.pos = cpos + A.lay[SEATS ? which : 0].hcs; L.vel = (float4 *)CRMC_SIZED(3); L.id = (unsigned long long *)CRMC_SIZED(4); L.lnk = (long long *)CRMC_SIZED(5);
+  L.info = (int *)CRMC_SIZED(6); L.ord = (uint2 *)CRMC_SIZED(7);
   if (!in_smem) {
     const size_t o = (size_t)(colour * P.nact + rank) * P.dcap_glob;  // this domain's region of the replica's scratch
     L.pos = P.gs_pos + o; L.vel = P.gs_vel + o; L.id = P.gs_id + o; L.lnk = P.gs_lnk + o;
@@ -1345,20 +1377,23 @@ __device__ __forceinline__ void phase_task(unsigned char *smem, const SysParams 
     }
   }
   const int lnmax_need = min(P.lnmax, ND + 2 * m + 2);
-  const bool ln_in_smem = lnmax_need <= S.lns;
+  const bool ln_in_smem = lnmax_need <= A.lay[SEATS ? which : 0].lns;
   const long long *lnt = ln_in_smem ? lntab_s : P.lntab_fx;
   if (tid == 0) {
     D.L = L;
     D.hpre = hpre;
     D.hcell = hcell;
     D.nhc = nhc;
-    D.hcs = S.hcs;
+    D.cpos_at = (int)A.lay[SEATS ? which : 0].off[2];
+    D.hcls_at = (int)A.lay[SEATS ? which : 0].off[8];
+    D.queue_at = (int)A.lay[SEATS ? which : 0].off[16];
+    D.hcs = A.lay[SEATS ? which : 0].hcs;
     D.NH = NH;
     D.NR = NR;
     D.in_smem = in_smem ? 1 : 0;
     D.strad = strad;
     D.flat = flat ? 1 : 0;
-    D.list_cap = in_smem ? S.dcs : P.dcap_glob;
+    D.list_cap = in_smem ? A.lay[SEATS ? which : 0].dcs : P.dcap_glob;
     D.lnt = lnt;
     D.d = d;
     D.phi = phi;
@@ -1386,7 +1421,7 @@ __device__ __forceinline__ void phase_task(unsigned char *smem, const SysParams 
   }
   if (ln_in_smem)
     for (int i = tid; i < lnmax_need; i += T) lntab_s[i] = P.lntab_fx[i];
-  __syncthreads();
+  seat.sync();
   // ---- the halo (it does not change during the phase)
   for (int j0 = tid; j0 < nhc; j0 += 4 * T) {
     float4 p[4];
@@ -1443,39 +1478,42 @@ __device__ __forceinline__ void phase_task(unsigned char *smem, const SysParams 
       aN[i] = cn;
     }
   }
-  __syncthreads();
+  seat.sync();
   if (tid < N_KIND) misc[MISC_INIT + tid] = misc[1 + tid];
   TrialCtl &ctl = ctls[group];
   // the CTA's statistics: lane l of each group's first warp counts entry l
   unsigned stat = 0u;
 
-  for (int k0 = 0; k0 < P.m; k0 += S.chunk) {
-    const int nchunk = min(S.chunk, P.m - k0);
+  for (int k0 = 0; k0 < P.m; k0 += A.lay[0].chunk) {
+    const int nchunk = min(A.lay[0].chunk, P.m - k0);
     // ---- random numbers of the chunk
     draw_chunk<LOG, DA>(P, D, tp, tvel, k0, nchunk, tid, T);
-    __syncthreads();
+    seat.sync();
 
-    for (int t0 = 0; t0 < nchunk;) {
+    unsigned round = 0u;
+    for (int t0 = 0; t0 < nchunk; round ^= 1u) {
       const int t = t0 + group, kk = k0 + t;
-      const bool mine = W == 1 || t < nchunk;  // uniform over the group
+      const bool mine = t < nchunk;  // uniform over the group
       // ---- the group's first warp: proposal and participants; the selection
       // lives in shared memory across the sweep
-      if (mine && gwarp == 0) select_trial<DA>(P, D, misc, tp[t], kk, ctl);
-      group_sync<G>(group);
+      if (mine && gwarp == 0) select_trial<LOG, DA>(P, D, misc, tp[t], kk, ctl);
+      seat.group_sync();
       // Ewald (global schedule): the changed particles' phase factors
-      const bool ew = !DA && W == 1 && P.ewald_nk > 0 && ctl.nch;
+      const bool ew = !DA && P.ewald_nk > 0 && ctl.nch;  // (one group: the shapes of Ewald systems)
       if (ew) {
-        ewald_factors(P, ctl, ewf, ewq, S.ewk, tid, T);
-        __syncthreads();
+        ewald_factors(P, ctl, ewf, ewq, A.lay[0].ewk, tid, T);
+        seat.sync();
       }
       // ---- delayed acceptance, stage 1: surrogate features and MLP (all of
       // the group's threads), decision in its first warp; a rejection skips
       // the pair sweep
       if (DA && mine && ctl.nch) {
         for (int i = gtid; i < MLP_IN; i += GT) dfeat[i] = 0;
-        group_sync<G>(group);
+        seat.group_sync();
         const int rka = ctl.rka, rkb = ctl.rkb;
-        const int dqa = ctl.dqa, dqb = ctl.dqb, ea = ctl.eta_a, eb = ctl.eta_b;
+        const int dqa = d_charge(ctl, 0), dqb = d_charge(ctl, 1);
+        const int ea = d_presence(ctl, 0), eb = d_presence(ctl, 1);
+        const int cat_a = (ctl.move >> 1) == R_SALT ? 0 : 8;  // feature group of a (0 ion, 8 site)
         for (int it = gtid; it < 250; it += GT) {  // 2 changed particles x 125 stencil cells
           const int sb = it >= 125 ? 1 : 0;
           const int c = it - 125 * sb;
@@ -1490,38 +1528,36 @@ __device__ __forceinline__ void phase_task(unsigned char *smem, const SysParams 
           }
           if (eta != 0 && aN[ri]) atomicAdd(&dfeat[24 * sb + 16 + sh], eta * aN[ri]);
         }
-        group_sync<G>(group);
+        seat.group_sync();
         if (gtid == 0) {  // the changed particles themselves do not count; the a-b pair term
           const TrialCtl &C = ctl;
-          const int qao = __float2int_rn(C.qa_o), qan = __float2int_rn(C.qa_n);
-          const int qbo = __float2int_rn(C.qb_o), qbn = __float2int_rn(C.qb_n);
           for (int sb = 0; sb < 2; ++sb) {
             const int rs = sb ? rkb : rka, dq = sb ? dqb : dqa, eta = sb ? eb : ea;
             for (int x = 0; x < 2; ++x) {
-              if (!(x ? C.pb_o : C.pa_o)) continue;
+              if (!had(C, x)) continue;
               const int sh = shell_ranks(rs, x ? rkb : rka, P.k);
               if (sh < 0) continue;
-              dfeat[24 * sb + (x ? 0 : C.cat_a) + sh] -= dq * (x ? qbo : qao);
+              dfeat[24 * sb + (x ? 0 : cat_a) + sh] -= dq * q_old(C, x);
               dfeat[24 * sb + 16 + sh] -= eta;
             }
           }
           const int sh = shell_ranks(rka, rkb, P.k);
-          if (sh >= 0) dfeat[sh] += (C.pa_n && C.pb_n ? qan * qbn : 0) - (C.pa_o && C.pb_o ? qao * qbo : 0);
+          if (sh >= 0) dfeat[sh] += q_new(C, 0) * q_new(C, 1) - q_old(C, 0) * q_old(C, 1);
         }
-        group_sync<G>(group);
+        seat.group_sync();
         for (int i = gtid; i < MLP_IN; i += GT) {
           const float f = (float)dfeat[i];
           fv[i] = f;
           fv[MLP_IN + i] = -f;
           if (LOG && P.feat_log) P.feat_log[(size_t)(D.log_dom + kk) * MLP_IN + i] = f;
         }
-        group_sync<G>(group);
-        mlp_layer<GT>(P.mlp_w + MLPW_W1, P.mlp_b, fv, MLP_IN, hb0, gtid);
-        group_sync<G>(group);
-        mlp_layer<GT>(P.mlp_w + MLPW_W2, P.mlp_b + MLP_H, hb0, MLP_H, hb1, gtid);
-        group_sync<G>(group);
-        mlp_layer<GT>(P.mlp_w + MLPW_W3, P.mlp_b + 2 * MLP_H, hb1, MLP_H, hb0, gtid);
-        group_sync<G>(group);
+        seat.group_sync();
+        mlp_layer(P.mlp_w + MLPW_W1, P.mlp_b, fv, MLP_IN, hb0, gtid, seat.gn);
+        seat.group_sync();
+        mlp_layer(P.mlp_w + MLPW_W2, P.mlp_b + MLP_H, hb0, MLP_H, hb1, gtid, seat.gn);
+        seat.group_sync();
+        mlp_layer(P.mlp_w + MLPW_W3, P.mlp_b + 2 * MLP_H, hb1, MLP_H, hb0, gtid, seat.gn);
+        seat.group_sync();
         if (gwarp == 0) {
           float y = 0.0f;
           if (lane < 2) {
@@ -1545,7 +1581,7 @@ __device__ __forceinline__ void phase_task(unsigned char *smem, const SysParams 
             ctl.sur_fx = sur_fx;
           }
         }
-        group_sync<G>(group);
+        seat.group_sync();
       } else if (DA && mine && LOG && P.feat_log) {
         for (int i = gtid; i < MLP_IN; i += GT) P.feat_log[(size_t)(D.log_dom + kk) * MLP_IN + i] = 0.0f;
       }
@@ -1556,19 +1592,16 @@ __device__ __forceinline__ void phase_task(unsigned char *smem, const SysParams 
       int ov = 0;
       if (nch) {
         const int nlist = misc[MISC_HW];
-        const PairSum ps = D.flat ? sweep_pairs<LOG, true>(pair_k(P), P, ctl, D, cpos, hcls, nlist, gtid, GT, queue)
-                                  : sweep_general<LOG>(P, ctl, D, cpos, hcls, nlist, gtid, GT, queue);
+        const float4 *cp = (const float4 *)(smem + D.cpos_at);
+        const unsigned char *hc = smem + D.hcls_at;
+        float2 *queue = (float2 *)(smem + D.queue_at) + warp * QCAP;
+        const PairSum ps = D.flat ? sweep_pairs<LOG, true>(pair_k(P), P, ctl, D, cp, hc, nlist, gtid, GT, queue)
+                                  : sweep_general<LOG>(P, ctl, D, cp, hc, nlist, gtid, GT, queue);
         acc = ps.acc;
         sacc = ps.sacc;
         ov = ps.ov;
-        if (gtid == (G > 1 ? 32 : 0)) {  // one thread adds the changed pair itself
-          const PairSum cc = cc_change<LOG>(P, ctl);
-          acc += cc.acc;
-          sacc += cc.sacc;
-          ov |= cc.ov;
-        }
         if (ew) {
-          const PairSum e = ewald_dE<LOG>(P, ewf, ewq, S.ewk, tid, T);
+          const PairSum e = ewald_dE<LOG>(P, ewf, ewq, A.lay[0].ewk, tid, T);
           acc += e.acc;
           sacc += e.sacc;
           ov |= e.ov;
@@ -1576,13 +1609,13 @@ __device__ __forceinline__ void phase_task(unsigned char *smem, const SysParams 
         acc = warp_sum_i64(acc);
         if (LOG) sacc = (unsigned long long)warp_sum_i64((long long)sacc);
         ov = __any_sync(FULL, ov) ? 1 : 0;
-        if (G > 1 && lane == 0) {
+        if (GT > 32 && lane == 0) {
           red[warp] = acc;
           reds[warp] = sacc;
           redov[warp] = ov;
         }
       }
-      if (G > 1) group_sync<G>(group);
+      if (GT > 32) seat.group_sync();
       // ---- the group's first warp: decision
       bool accept = false;
       int flags = 0;
@@ -1599,10 +1632,11 @@ __device__ __forceinline__ void phase_task(unsigned char *smem, const SysParams 
           long long tot = acc;
           unsigned long long stot = sacc;
           int anyov = ov;
-          if (G > 1) {
-            tot = warp_sum_i64(lane < G ? red[warp + lane] : 0ll);
-            if (LOG) stot = (unsigned long long)warp_sum_i64(lane < G ? (long long)reds[warp + lane] : 0ll);
-            anyov = __any_sync(FULL, lane < G && redov[warp + lane]) ? 1 : 0;
+          if (GT > 32) {
+            const int gw = GT >> 5;
+            tot = warp_sum_i64(lane < gw ? red[warp + lane] : 0ll);
+            if (LOG) stot = (unsigned long long)warp_sum_i64(lane < gw ? (long long)reds[warp + lane] : 0ll);
+            anyov = __any_sync(FULL, lane < gw && redov[warp + lane]) ? 1 : 0;
           }
           if (anyov) {
             if (!DA || s1) flags |= CR_TRIAL_OVERLAP;  // DA: only an exact evaluation that decides
@@ -1623,10 +1657,26 @@ __device__ __forceinline__ void phase_task(unsigned char *smem, const SysParams 
           }
         }
       }
+      // ---- with several groups: the trials up to and including the first
+      // accepted one are decided; the later ones were evaluated on a state
+      // that it changes, and are taken up again in the next round
+      bool decided = mine;
+      int done = 1;
+      unsigned won = 0u;
+      if (seat.groups > 1) {
+        int *res = misc + MISC_RES + round * MAX_GROUPS;
+        if (gwarp == 0 && lane == 0) res[group] = accept ? 1 : 0;
+        seat.sync();
+        won = __ballot_sync(FULL, lane < seat.groups && res[lane] != 0);
+        const int first = won ? __ffs(won) - 1 : seat.groups - 1;
+        decided = mine && group <= first;
+        accept = accept && group == first;
+        done = min(first + 1, nchunk - t0);
+      }
       // ---- commit, unless an insertion finds no room (checked before
       // anything changes)
       if (accept) {
-        const int n2 = try_commit(P, D, misc, ctl, tp[t], tvel + 2 * t, misc[0]);
+        const int n2 = try_commit(P, D, misc, ctl, tp[t], tvel + 2 * t, kk, misc[0]);
         if (n2 < 0) {
           accept = false;
           if (lane == 0) atomicOr(P.err, ERRB_CELL_OVERFLOW);
@@ -1636,20 +1686,14 @@ __device__ __forceinline__ void phase_task(unsigned char *smem, const SysParams 
             const TrialCtl &C = ctl;
             for (int x = 0; x < 2; ++x) {
               const int ri = region_of(x ? C.rkb : C.rka, 0, 0, 0, P.k, P.nr);
-              int *aq = (x == 0 && C.cat_a == 8) ? aQs : aQi;
-              if (x ? C.pb_o : C.pa_o) {
-                aq[ri] -= __float2int_rn(x ? C.qb_o : C.qa_o);
-                aN[ri] -= 1;
-              }
-              if (x ? C.pb_n : C.pa_n) {
-                aq[ri] += __float2int_rn(x ? C.qb_n : C.qa_n);
-                aN[ri] += 1;
-              }
+              int *aq = (x == 0 && (C.move >> 1) != R_SALT) ? aQs : aQi;
+              aq[ri] += d_charge(C, x);
+              aN[ri] += d_presence(C, x);
             }
           }
         }
       }
-      if (mine && gwarp == 0) {
+      if (decided && gwarp == 0) {
         const unsigned hit = (1u << ctl.move) | (accept ? 64u << ctl.move : 0u) |
                              (flags & CR_TRIAL_NO_ELIGIBLE ? 1u << 12 : 0u) |
                              (flags & CR_TRIAL_EDGE ? 1u << 13 : 0u) | (flags & CR_TRIAL_OVERLAP ? 1u << 14 : 0u) |
@@ -1679,15 +1723,16 @@ __device__ __forceinline__ void phase_task(unsigned char *smem, const SysParams 
           }
         }
       }
-      t0 += 1;
+      t0 += done;
+      if (won) seat.sync();  // the next selections see the committed state
       if (ew) {
-        __syncthreads();
-        if (ctl.ewacc) ewald_update(P, ewf, ewq, S.ewk, tid, T);
+        seat.sync();
+        if (ctl.ewacc) ewald_update(P, ewf, ewq, A.lay[0].ewk, tid, T);
       }
       // (the other warps wait for the first one's next selection at the
       // group's barrier; what they read of this trial they have read)
     }
-    __syncthreads();  // the chunk's numbers have been read
+    seat.sync();  // the chunk's numbers have been read
   }
   // ---- write the domain back (id-sorted cells), if anything changed, and
   // publish the counts
@@ -1702,7 +1747,7 @@ __device__ __forceinline__ void phase_task(unsigned char *smem, const SysParams 
       dcnt[r] = lo;
       P.cnt[dcell[r]] = lo2 - lo;
     }
-    __syncthreads();
+    seat.sync();
     for (int j = tid; j < n; j += T) {
       const uint2 o = L.ord[j];
       const int sl = (int)(o.x & ORD_SLOT_MASK);
@@ -1720,17 +1765,31 @@ __device__ __forceinline__ void phase_task(unsigned char *smem, const SysParams 
   }
   if (gwarp == 0 && lane < 16 && stat) atomicAdd(&P.stats[lane], (unsigned long long)stat);
 #undef CRMC_AT
+#undef CRMC_SIZED
 }
 
 // ---------------------------------------------------------------------------
-// the phase kernel: one CTA per active domain of one colour, of W groups of G
-// warps (G == 1, W == 1: one warp, no block barriers)
+// the phase kernel.  Of a replica's domains (densest first) the first
+// A.wide16 / 16 have a CTA each; the others share CTAs, one domain per seat of
+// blockDim / A.seats threads.  Thread counts are run-time values, so that every
+// seat runs the same code.
+//
+// What bounds it: one domain's chain of trials, each some 200 + instructions
+// that one warp fetches and runs once (4.0 of the 13.5 cycles between a warp's
+// instructions wait for instructions, 3.6 at barriers; issue active 24 %).
+// With one CTA of 64 threads per domain the densest domain of a colour, coils
+// of a chain with 60 and more beads, lasted as long as two waves of the others.
+// Seats give it four times the threads and the shared memory of four, from the
+// same launch.  13 polyelectrolyte boxes (125 domains a colour each): a sweep
+// 1.03 ms with 64 threads per domain; 0.79 ms with 1/16 of the domains on 256
+// threads and the rest on seats of 64, of which 0.17 ms came from shorter code
+// in the trial loop (one path for the four move forms, loops not unrolled);
+// 64 ragged single chains 0.80 -> 0.55 ms.  A box alone (125 domains for 152
+// SMs) runs fastest with 256 threads for every domain.
 // ---------------------------------------------------------------------------
-constexpr int min_ctas(int T) { return T <= 32 ? 16 : (T <= 64 ? 8 : (T <= 128 ? 4 : (T <= 256 ? 2 : 1))); }
-
-template <int G, int W, bool LOG, bool DA>
-__global__ void __launch_bounds__(32 * G * W, min_ctas(32 * G * W))
-    k_cr_phase(const SysParams *__restrict__ reps, const __grid_constant__ PhaseShape S, uint32_t sweep,
+template <bool LOG, bool DA, bool SEATS>
+__global__ void __launch_bounds__(512, 1)
+    k_cr_phase(const SysParams *__restrict__ reps, const __grid_constant__ PhaseArgs A, uint32_t sweep,
                uint32_t sweep0, int colour, uint32_t key0, uint32_t key1_base, const StepDyn *dyn) {
   extern __shared__ __align__(16) unsigned char smem[];
   if (dyn) {  // a captured cycle: this step's sweep counter and key
@@ -1739,8 +1798,20 @@ __global__ void __launch_bounds__(32 * G * W, min_ctas(32 * G * W))
     key0 = (uint32_t)seed;
     key1_base = (uint32_t)(seed >> 32);
   }
-  phase_task<G, W, LOG, DA>(smem, reps, S, sweep, sweep0, colour, key0, key1_base, (int)blockIdx.x,
-                            (int)blockIdx.y);
+  const int rep = (int)blockIdx.x, y = (int)blockIdx.y, T = (int)blockDim.x;
+  int rank = y, which = 0, base = 0;
+  Seat<SEATS> seat{(int)threadIdx.x, T, A.groups, T / A.groups, 0};
+  if (SEATS) {
+    const int wide = (reps[rep].nact * A.wide16 + 15) >> 4;
+    if (y >= wide) {  // one of the CTA's seats
+      const int n = T / A.seats, at = (int)threadIdx.x / n;
+      rank = wide + (y - wide) * A.seats + at;
+      seat = Seat<SEATS>{(int)threadIdx.x - at * n, n, 1, n, at};
+      which = 1;
+      base = at * (int)A.seat_bytes;
+    }
+  }
+  phase_task<LOG, DA, SEATS>(smem + base, A, which, seat, reps, sweep, sweep0, colour, key0, key1_base, rep, rank);
 }
 
 // ---------------------------------------------------------------------------
@@ -1799,9 +1870,9 @@ __device__ __forceinline__ bool wait_at_least(const unsigned *p, unsigned need, 
   return true;
 }
 
-template <int G, int W, bool DA>
-__global__ void __launch_bounds__(32 * G * W, min_ctas(32 * G * W))
-    k_cr_sweep(const SysParams *__restrict__ reps, const __grid_constant__ PhaseShape S, uint32_t sweep,
+template <bool DA>
+__global__ void __launch_bounds__(512, 1)
+    k_cr_sweep(const SysParams *__restrict__ reps, const __grid_constant__ PhaseArgs A, uint32_t sweep,
                uint32_t sweep0, uint32_t key0, uint32_t key1_base, SweepSched Q, const StepDyn *dyn) {
   extern __shared__ __align__(16) unsigned char smem[];
   if (dyn) {  // a captured cycle: this step's sweep counter and key
@@ -1863,7 +1934,8 @@ __global__ void __launch_bounds__(32 * G * W, min_ctas(32 * G * W))
     int r = 0;
     while (Q.rep_first[r + 1] <= q) ++r;
     if (s_run)
-      phase_task<G, W, false, DA>(smem, reps, S, sweep, sweep0, c, key0, key1_base, r, q - Q.rep_first[r]);
+      phase_task<false, DA, false>(smem, A, 0, Seat<false>{(int)threadIdx.x, (int)blockDim.x, A.groups, (int)blockDim.x / A.groups, 0},
+                            reps, sweep, sweep0, c, key0, key1_base, r, q - Q.rep_first[r]);
     __syncthreads();  // the task's stores are done, its shared memory is free
     if (threadIdx.x == 0 && !(r == Q.withhold_rep && c == 0)) {
       __threadfence();
@@ -1873,27 +1945,43 @@ __global__ void __launch_bounds__(32 * G * W, min_ctas(32 * G * W))
   }
 }
 
-template <int G, int W, bool DA>
-static cudaError_t launch_sweep_t(const SysParams *d_reps, PhaseShape S, cudaStream_t s, uint32_t sweep,
-                                  uint32_t sweep0, uint32_t k0, uint32_t k1, const SweepSched &Q, int max_ctas,
-                                  const StepDyn *dyn) {
-  constexpr int T = 32 * G * W;
+// the launch's constant parameters: layouts of a CTA's domain and of a seat's
+static PhaseArgs phase_args(const PhaseShape &S, const PhaseForm &F, bool da, size_t *smem) {
+  PhaseArgs A{};
+  A.seats = F.seats;
+  A.groups = F.groups;
+  A.wide16 = F.wide16;
+  const int warps = F.threads / 32;
+  const size_t wide = phase_layout(F.compact ? S.small : S.full, S, warps, warps, F.groups, da, A.lay[0]);
+  size_t narrow = 0;
+  if (F.seats > 1) narrow = phase_layout(S.small, S, warps / F.seats, warps, 1, da, A.lay[1]);
+  A.seat_bytes = (unsigned)narrow;
+  *smem = std::max(wide, narrow * (size_t)F.seats);
+  return A;
+}
+
+size_t phase_smem_bytes(const PhaseShape &S, const PhaseForm &F, bool da) {
+  size_t b = 0;
+  phase_args(S, F, da, &b);
+  return b;
+}
+
+template <bool DA>
+static cudaError_t launch_sweep_t(const SysParams *d_reps, const PhaseShape &S, const PhaseForm &F, cudaStream_t s,
+                                  uint32_t sweep, uint32_t sweep0, uint32_t k0, uint32_t k1, const SweepSched &Q,
+                                  int max_ctas, const StepDyn *dyn) {
   static size_t attr_bytes = 0;
-  static int per_sm = 0;
-  static size_t per_sm_bytes = ~(size_t)0;
-  const size_t smem = phase_layout(S, T / 32, W, DA);
+  size_t smem = 0;
+  const PhaseArgs A = phase_args(S, F, DA, &smem);
   if (smem > attr_bytes) {
-    cudaError_t e = cudaFuncSetAttribute(k_cr_sweep<G, W, DA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k_cr_sweep<DA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     attr_bytes = smem;
   }
-  if (smem != per_sm_bytes) {  // resident CTAs per SM at this shared-memory size
-    int nb = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_cr_sweep<G, W, DA>, T, smem);
-    if (e != cudaSuccess) return e;
-    per_sm = std::max(nb, 1);
-    per_sm_bytes = smem;
-  }
+  int per_sm = 0;  // resident CTAs per SM at this block and shared-memory size
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cr_sweep<DA>, F.threads, smem);
+  if (e != cudaSuccess) return e;
+  per_sm = std::max(per_sm, 1);
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -1901,28 +1989,15 @@ static cudaError_t launch_sweep_t(const SysParams *d_reps, PhaseShape S, cudaStr
   int grid = std::min(total, per_sm * std::max(sms, 1));
   if (max_ctas > 0) grid = std::min(grid, max_ctas);
   if (grid <= 0) return cudaSuccess;
-  k_cr_sweep<G, W, DA><<<grid, T, smem, s>>>(d_reps, S, sweep, sweep0, k0, k1, Q, dyn);
+  k_cr_sweep<DA><<<grid, F.threads, smem, s>>>(d_reps, A, sweep, sweep0, k0, k1, Q, dyn);
   return cudaGetLastError();
 }
 
-// the instantiated shapes: X(threads, groups), for plain and delayed-acceptance sweeps
-#define CRMC_SHAPES(X) X(32, 1) X(64, 1) X(128, 1) X(256, 1) X(512, 1)
-#define CRMC_SHAPES_DA(X) X(128, 1) X(256, 1) X(512, 1)
-
-cudaError_t launch_sweep(const SysParams *d_reps, const PhaseShape &S, int threads, int groups, bool da, cudaStream_t s,
-                         uint32_t sweep, uint32_t sweep0, uint32_t k0, uint32_t k1, const SweepSched &Q,
-                         int max_ctas, const StepDyn *dyn) {
-#define CRMC_SW(TT, WW, DD)             \
-  if (da == DD && threads == TT && groups == WW) \
-    return launch_sweep_t<TT / 32 / WW, WW, DD>(d_reps, S, s, sweep, sweep0, k0, k1, Q, max_ctas, dyn);
-#define CRMC_SW_PLAIN(TT, WW) CRMC_SW(TT, WW, false)
-#define CRMC_SW_DA(TT, WW) CRMC_SW(TT, WW, true)
-  CRMC_SHAPES(CRMC_SW_PLAIN)
-  CRMC_SHAPES_DA(CRMC_SW_DA)
-#undef CRMC_SW
-#undef CRMC_SW_PLAIN
-#undef CRMC_SW_DA
-  return cudaErrorInvalidValue;
+cudaError_t launch_sweep(const SysParams *d_reps, const PhaseShape &S, const PhaseForm &F, bool da, cudaStream_t s,
+                         uint32_t sweep, uint32_t sweep0, uint32_t k0, uint32_t k1, const SweepSched &Q, int max_ctas,
+                         const StepDyn *dyn) {
+  return da ? launch_sweep_t<true>(d_reps, S, F, s, sweep, sweep0, k0, k1, Q, max_ctas, dyn)
+            : launch_sweep_t<false>(d_reps, S, F, s, sweep, sweep0, k0, k1, Q, max_ctas, dyn);
 }
 
 // ---------------------------------------------------------------------------
@@ -2086,71 +2161,67 @@ cudaError_t launch_ewald_sk(const SysParams *d_reps, int n_rep, int max_nk, cuda
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
-size_t phase_smem_bytes(const PhaseShape &S, int threads, int groups, bool da) {
-  PhaseShape Q = S;
-  return phase_layout(Q, threads / 32, groups, da);
-}
-
-template <int G, int W, bool LOG, bool DA>
-static cudaError_t launch_phase_t(const SysParams *d_reps, int n_rep, int grid_x, PhaseShape S, cudaStream_t s,
-                                  uint32_t sweep, uint32_t sweep0, int colour, uint32_t k0, uint32_t k1,
-                                  const StepDyn *dyn) {
-  constexpr int T = 32 * G * W;
+template <bool LOG, bool DA, bool SEATS>
+static cudaError_t launch_phase_t(const SysParams *d_reps, int n_rep, int max_nact, const PhaseShape &S,
+                                  const PhaseForm &F, cudaStream_t s, uint32_t sweep, uint32_t sweep0, int colour,
+                                  uint32_t k0, uint32_t k1, const StepDyn *dyn) {
   static size_t attr_bytes = 0;
-  const size_t smem = phase_layout(S, T / 32, W, DA);
+  size_t smem = 0;
+  const PhaseArgs A = phase_args(S, F, DA, &smem);
   if (smem > attr_bytes) {
     cudaError_t e =
-        cudaFuncSetAttribute(k_cr_phase<G, W, LOG, DA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(k_cr_phase<LOG, DA, SEATS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     attr_bytes = smem;
   }
-  k_cr_phase<G, W, LOG, DA><<<dim3(n_rep, grid_x), T, smem, s>>>(d_reps, S, sweep, sweep0, colour, k0, k1, dyn);
+  int gy = max_nact;  // CTAs of the replica with the most domains (no fewer for any smaller one)
+  if (SEATS) {
+    const int wide = (max_nact * F.wide16 + 15) >> 4;
+    gy = wide + (max_nact - wide + F.seats - 1) / F.seats;
+  }
+  k_cr_phase<LOG, DA, SEATS>
+      <<<dim3(n_rep, gy), F.threads, smem, s>>>(d_reps, A, sweep, sweep0, colour, k0, k1, dyn);
   return cudaGetLastError();
 }
 
-// variants the autotuner picks from: (threads per CTA, groups, compact).
-// Compact variants size the shared-memory list and halo for most domains
-// rather than the densest (denser ones spill to global memory), so that more
-// CTAs fit on an SM.
-static const int kShapes[][3] = {{32, 1, 0},  {64, 1, 0}, {128, 1, 0}, {256, 1, 0}, {512, 1, 0},
-                                 {32, 1, 1},  {64, 1, 1}, {128, 1, 1}, {256, 1, 1}};
-
-// shapes with a delayed-acceptance variant (the surrogate runs on >= 128 threads)
-static const int kShapesDA[][3] = {{128, 1, 0}, {256, 1, 0}, {512, 1, 0}, {128, 1, 1}, {256, 1, 1}};
-
-int phase_shape_count(bool da) {
-  return da ? (int)(sizeof(kShapesDA) / sizeof(kShapesDA[0])) : (int)(sizeof(kShapes) / sizeof(kShapes[0]));
+cudaError_t launch_phase(const SysParams *d_reps, int n_rep, int max_nact, const PhaseShape &S, const PhaseForm &F,
+                         bool log, bool da, cudaStream_t s, uint32_t sweep, uint32_t sweep0, int colour, uint32_t k0,
+                         uint32_t k1, const StepDyn *dyn) {
+  // (a logged sweep takes the form without its seats: the records do not depend on it)
+  const PhaseForm G = log && F.seats > 1 ? PhaseForm{128, 1, 1, 16, 0} : F;
+#define CRMC_CASE(LL, DD, SS)                 \
+  if (log == LL && da == DD && (G.seats > 1) == SS) \
+    return launch_phase_t<LL, DD, SS>(d_reps, n_rep, max_nact, S, G, s, sweep, sweep0, colour, k0, k1, dyn);
+  CRMC_CASE(false, false, false)
+  CRMC_CASE(false, false, true)
+  CRMC_CASE(true, false, false)
+  CRMC_CASE(false, true, false)
+  CRMC_CASE(false, true, true)
+  CRMC_CASE(true, true, false)
+#undef CRMC_CASE
+  return cudaErrorInvalidValue;
 }
-void phase_shape(int i, int *threads, int *groups, bool da) {
-  *threads = da ? kShapesDA[i][0] : kShapes[i][0];
-  *groups = da ? kShapesDA[i][1] : kShapes[i][1];
-}
-bool phase_shape_compact(int i, bool da) { return (da ? kShapesDA[i][2] : kShapes[i][2]) != 0; }
 
-bool phase_shape_named(int threads, int regs, bool da, int *groups) {
-  *groups = 1;
+// Forms the autotuner picks from.  Compact forms size the shared-memory list
+// and halo for most domains rather than the densest (denser ones spill to
+// global memory), so that more CTAs fit on an SM; forms with seats give the
+// densest domains a CTA each.
+static const PhaseForm kForms[] = {
+    // threads, seats (of 64 or 128 threads), groups (of 32), wide16, compact
+    {64, 1, 1, 16, 1},  {128, 1, 1, 16, 0}, {256, 1, 1, 16, 0}, {512, 1, 1, 16, 0}, {128, 1, 4, 16, 0}, {256, 1, 8, 16, 0},
+    {128, 2, 1, 2, 0},  {256, 4, 1, 1, 0},  {256, 4, 1, 2, 0},  {256, 4, 1, 4, 0},  {256, 2, 1, 2, 0},  {512, 4, 1, 4, 0}};
+// forms with a delayed-acceptance variant (the surrogate runs on >= 128 threads)
+static const PhaseForm kFormsDA[] = {
+    {128, 1, 1, 16, 0}, {256, 1, 1, 16, 0}, {512, 1, 1, 16, 0}, {128, 1, 1, 16, 1}, {256, 1, 1, 16, 1}};
+
+int phase_form_count(bool da) { return da ? (int)std::size(kFormsDA) : (int)std::size(kForms); }
+const PhaseForm &phase_form(int i, bool da) { return da ? kFormsDA[i] : kForms[i]; }
+
+bool phase_form_named(int threads, int regs, bool da, PhaseForm *F) {
+  *F = PhaseForm{threads, 1, 1, 16, 0};
   if (regs != 0) return !da && ((threads == 128 && regs == 4) || (threads == 256 && regs == 2) || (threads == 512 && regs == 1));
   if (da) return threads == 128 || threads == 256 || threads == 512;
   return threads == 32 || threads == 64 || threads == 128 || threads == 256 || threads == 512;
-}
-
-cudaError_t launch_phase(const SysParams *d_reps, int n_rep, int grid_x, const PhaseShape &S, int threads, int groups,
-                         bool log, bool da, cudaStream_t s, uint32_t sweep, uint32_t sweep0, int colour,
-                         uint32_t k0, uint32_t k1, const StepDyn *dyn) {
-#define CRMC_CASE(TT, WW, DD)                                                                                   \
-  if (da == DD && threads == TT && groups == WW)                                                                \
-    return log ? launch_phase_t<TT / 32 / WW, WW, true, DD>(d_reps, n_rep, grid_x, S, s, sweep, sweep0, colour, \
-                                                            k0, k1, dyn)                                        \
-               : launch_phase_t<TT / 32 / WW, WW, false, DD>(d_reps, n_rep, grid_x, S, s, sweep, sweep0, colour, \
-                                                             k0, k1, dyn);
-#define CRMC_CASE_PLAIN(TT, WW) CRMC_CASE(TT, WW, false)
-#define CRMC_CASE_DA(TT, WW) CRMC_CASE(TT, WW, true)
-  CRMC_SHAPES(CRMC_CASE_PLAIN)
-  CRMC_SHAPES_DA(CRMC_CASE_DA)
-#undef CRMC_CASE
-#undef CRMC_CASE_PLAIN
-#undef CRMC_CASE_DA
-  return cudaErrorInvalidValue;
 }
 
 }  // namespace crmc
