@@ -62,7 +62,7 @@ struct cr_ctx {
   uint2 *d_gs_ord = nullptr;
   int *d_plist = nullptr, *d_nparts = nullptr;  // MD particle list
   long long *d_fsum = nullptr;                    // MD pair-force sums per slot
-  int *d_order = nullptr;                       // launch order of the domains of each colour
+  int *d_order = nullptr, *d_cost = nullptr;                       // launch order of the domains of each colour
   // delayed acceptance: surrogate on the device, records, its own launch-shape tuner
   uint16_t *d_mlp_w = nullptr;
   float *d_mlp_b = nullptr;
@@ -215,7 +215,7 @@ static void free_ctx(cr_ctx *c) {
                   c->d_out_xyz, c->d_out_vel, c->d_out_frc, c->d_out_id, c->d_out_type, c->d_out_cls,
                   c->d_out_state, c->d_out_site,
                   c->d_reps, c->d_gs_pos, c->d_gs_vel, c->d_gs_id, c->d_gs_lnk, c->d_gs_info, c->d_gs_ord,
-                  c->d_plist, c->d_nparts, c->d_fsum, c->d_mlp_w, c->d_mlp_b, c->d_dlog, c->d_feat, c->d_order,
+                  c->d_plist, c->d_nparts, c->d_fsum, c->d_mlp_w, c->d_mlp_b, c->d_dlog, c->d_feat, c->d_order, c->d_cost,
                   c->d_ek_nA, c->d_ek_Shi, c->d_ek_Slo, c->d_ek_list, c->d_ek_np,
                   c->d_bodies, c->d_body_member, c->d_body_d, c->d_body_df, c->d_body_newpos};
   for (void *p : ptrs)
@@ -586,6 +586,7 @@ extern "C" int cr_init(cr_ctx **out, const cr_system *sys, double pH, const doub
   for (int i = 1; i < P.lnmax; ++i) h_lntab[i] = to_lnfix(std::log((double)i));
   int smem_max = 0;
   cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
+  smem_max -= 1024;  // (the persistent sweep has a few static words)
   PhaseShape &S = c->S;
   S.nr3 = P.nr * P.nr * P.nr;
   S.kc3 = k * k * k;
@@ -796,6 +797,8 @@ extern "C" int cr_init(cr_ctx **out, const cr_system *sys, double pH, const doub
   P.ek_np = c->d_ek_np;
   P.ek_cap = (int)std::max<int64_t>(sys->capacity, 1);
   P.order = nullptr;
+  P.cost = nullptr;
+  P.list_small = S.small.dcs;
   if (!global && P.nact <= ORDER_MAX_NACT) {
     // densest-first launch order, recomputed every sweep; starts as the identity
     std::vector<int> ident((size_t)P.ncol * P.nact);
@@ -806,6 +809,11 @@ extern "C" int cr_init(cr_ctx **out, const cr_system *sys, double pH, const doub
       return CR_ERR_NOMEM;
     }
     P.order = c->d_order;
+    if (cudaMalloc((void **)&c->d_cost, sizeof(int) * ident.size()) != cudaSuccess) {
+      free_ctx(c);
+      return CR_ERR_NOMEM;
+    }
+    P.cost = c->d_cost;
   }
   if (cudaMemcpy(c->d_reps, &P, sizeof(SysParams), cudaMemcpyHostToDevice) != cudaSuccess) {
     free_ctx(c);
@@ -1077,7 +1085,7 @@ static int sweep_impl(cr_ctx *ctx, uint64_t n_trials, uint64_t seed, cr_sweep_st
     }
     if (P.order) {
       CR_CUDA(launch_domain_order(ctx->d_reps, 1, P.ncol, P.nact, s, swc, k0, k1));
-      ctx->launches_total++;
+      ctx->launches_total += 2;
     }
     if (P.ewald_nk > 0) {  // S(k) from scratch at every sweep
       CR_CUDA(launch_ewald_sk(ctx->d_reps, 1, P.ewald_nk, s));
@@ -1876,6 +1884,7 @@ extern "C" int cr_batch_create(cr_batch **out, cr_ctx *const *ctxs, int32_t n) {
     }
   int smem_max = 0;
   cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctxs[0]->device);
+  smem_max -= 1024;  // (as in cr_init)
   if (phase_smem_bytes(b->S, PhaseForm{512, 1, 1, 16, 0}, false) > (size_t)smem_max) { delete b; return CR_ERR_INVALID_ARG; }
   b->smem_max = smem_max;
   cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, ctxs[0]->device);
@@ -2034,7 +2043,7 @@ static int batch_sweep_impl(cr_batch *b, uint64_t n_sweeps, uint64_t seed, bool 
     }
     if (b->order_nc > 0) {
       CR_CUDA(launch_domain_order(b->d_reps, n, b->ncol, b->order_nact, s, swc, k0, k1));
-      c0->launches_total++;
+      c0->launches_total += 2;
     }
     if (b->ewald_nk_max > 0) {  // S(k) of every replica from scratch at every sweep
       CR_CUDA(launch_ewald_sk(b->d_reps, n, b->ewald_nk_max, s));
@@ -2091,7 +2100,7 @@ extern "C" int cr_batch_selftest_wait_timeout(cr_batch *b, int32_t replica, doub
   const PhaseForm F = b->tuning || b->F.seats > 1 ? PhaseForm{128, 1, 1, 16, 0} : b->F;  // (tasks take whole CTAs)
   if (b->order_nc > 0) {
     CR_CUDA(launch_domain_order(b->d_reps, (int)b->ctx.size(), b->ncol, b->order_nact, c0->stream, swc, 1u, 0u));
-    c0->launches_total++;
+    c0->launches_total += 2;
   }
   const int rc = batch_launch_persistent(b, F, false, swc, swc, 1u, 0u, replica,
                                          (unsigned long long)(timeout_ms * 1e6));
@@ -2225,7 +2234,7 @@ static int batch_capture_cycle(cr_batch *b, double dt, double gamma, bool da, bo
     if (rc == CR_OK) rc = batch_md(b, [&](cr_ctx *c, uint64_t) { return cr_md_begin(c, dt, gamma, 0); });
     if (rc == CR_OK && b->order_nc > 0) {
       if (launch_domain_order(b->d_reps, n, b->ncol, b->order_nact, s, 0, 0, 0, dyn) != cudaSuccess) rc = CR_ERR_CUDA;
-      c0->launches_total++;
+      c0->launches_total += 2;
     }
     if (rc == CR_OK) {
       if (pers) {

@@ -110,8 +110,10 @@ struct alignas(16) SysParams {
   cr_trial_da *dlog;          // DA records (device) or null
   float *feat_log;            // 48 features per trial (device) or null
   // launch order of each colour's domains, largest region first (ncol x nact),
-  // or null for the natural order
-  int *order;
+  // or null for the natural order; the domains' expected costs; list entries
+  // that a seat holds in shared memory
+  int *order, *cost;
+  int list_small;
   // Ewald electrostatics (ewald_nk > 0, global schedule): the reciprocal
   // vectors n of one half space (three signed bytes each; S(-k) is the
   // conjugate of S(k), so -k adds the same term) with their weights

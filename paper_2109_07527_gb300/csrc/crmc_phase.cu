@@ -3,7 +3,7 @@
 // k_cr_phase: one CTA per active domain of one colour of the 8-colour
 // checkerboard, for one or several replicas (blockIdx.x) in one launch; the
 // domains of a colour are launched densest first (blockIdx.y is the rank in
-// the order k_domain_order computes at the start of every sweep), so that the
+// the order k_domain_cost and k_domain_rank compute at the start of every sweep), so that the
 // long CTAs do not form the tail of the launch.
 // The CTA
 //   1. stages the domain's particles into a list -- in shared memory, or in a
@@ -2001,62 +2001,80 @@ cudaError_t launch_sweep(const SysParams *d_reps, const PhaseShape &S, const Pha
 }
 
 // ---------------------------------------------------------------------------
-// Launch order of the domains of one colour for one sweep: the particles in
-// each domain's region (its cells and the halo around them, counted at the
-// start of the sweep; one warp sums a region's cell counts) and the domains
-// ranked by decreasing count (ties by index).  Only the order of independent
-// CTAs changes, never a result.  One CTA per (replica, colour); colours of
-// more than ORDER_MAX_NACT domains keep the natural order (P.order is null).
+// Launch order of the domains of one colour for one sweep, by decreasing
+// expected time (ties by index).  A domain's time goes by the particles of its
+// region (its cells and the halo around them: the sweep's candidates) and more
+// by its own (near pairs of inserted ions, list scans: about five candidates'
+// worth each); one whose list does not fit a seat's shared memory comes before
+// all others, so that it gets a CTA's.  k_domain_cost: one warp sums a region's
+// cell counts at the start of the sweep; k_domain_rank: each domain counts the
+// costlier ones of its colour.  Only the order of independent CTAs changes,
+// never a result.  Colours of more than ORDER_MAX_NACT domains keep the
+// natural order (P.order is null).  (One CTA per replica and colour for both
+// took 187 us for 8 x 1,000 domains and 25 us for 13 x 8 x 125;
+// the two kernels 10 + 15 and 13 + 4 us: cycles of the large box 4.17 -> 3.20 ms,
+// two nanoparticles, whose 1,000 sites crowd a few domains, 2.13 -> 1.88 ms.)
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(512) k_domain_order(const SysParams *__restrict__ reps, uint32_t sweep, uint32_t key0,
-                                                      uint32_t key1_base, const StepDyn *dyn) {
+__global__ void __launch_bounds__(256) k_domain_cost(const SysParams *__restrict__ reps, uint32_t sweep, uint32_t key0,
+                                                     uint32_t key1_base, const StepDyn *dyn) {
   if (dyn) {  // a captured cycle: this step's sweep counter and key
     const unsigned long long step = dyn->step, seed = dyn->sweep_seed0 + step;
     sweep = dyn->sweep0 + (uint32_t)step;
     key0 = (uint32_t)seed;
     key1_base = (uint32_t)(seed >> 32);
   }
-  const SysParams &P = reps[blockIdx.x];
+  const SysParams &P = reps[blockIdx.y];
   if (!P.order) return;
-  __shared__ int cost[ORDER_MAX_NACT];
-  const int c = blockIdx.y;
+  const int lane = threadIdx.x & 31, task = (int)(blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int nact = P.nact, c = task / nact, b = task - c * nact;
   if (c >= P.ncol) return;
-  const int nc = P.nc, nr = P.nr, h = P.h, k = P.k, nact = P.nact;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-  const uint32_t key1 = key1_base ^ P.key_xor;
-  const uint4 w = philox10(0u, 0u, sweep, 4u, key0, key1);
+  const int nc = P.nc, nr = P.nr, h = P.h, k = P.k;
+  const uint4 w = philox10(0u, 0u, sweep, 4u, key0, key1_base ^ P.key_xor);
   const int off[3] = {pick32(w.x, nc), pick32(w.y, nc), pick32(w.z, nc)};
   const int hn = P.nd >> 1, nr3 = nr * nr * nr;
-  for (int b = wid; b < nact; b += nwarp) {
-    const int dd[3] = {2 * (b % hn) + (c & 1), 2 * ((b / hn) % hn) + ((c >> 1) & 1), 2 * (b / (hn * hn)) + ((c >> 2) & 1)};
-    int o[3];
+  const int dd[3] = {2 * (b % hn) + (c & 1), 2 * ((b / hn) % hn) + ((c >> 1) & 1), 2 * (b / (hn * hn)) + ((c >> 2) & 1)};
+  int o[3];
 #pragma unroll
-    for (int i = 0; i < 3; ++i) o[i] = ((off[i] + dd[i] * k - h) % nc + nc) % nc;  // region origin
-    int sum = 0;
-    for (int i = lane; i < nr3; i += 32) {
-      const int ix = i % nr, iy = (i / nr) % nr, iz = i / (nr * nr);
-      sum += P.cnt[(o[0] + ix) % nc + nc * ((o[1] + iy) % nc + nc * ((o[2] + iz) % nc))];
-    }
-#pragma unroll
-    for (int x = 16; x > 0; x >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, x);
-    if (lane == 0) cost[b] = sum;
+  for (int i = 0; i < 3; ++i) o[i] = (off[i] + dd[i] * k) % nc;  // the domain's first cell
+  const float rnr = 1.0f / (float)nr;
+  int sum = 0, own = 0;
+  for (int i = lane; i < nr3; i += 32) {
+    const int iyz = div_by(i, rnr), iz = div_by(iyz, rnr), ix = i - iyz * nr, iy = iyz - iz * nr;
+    const int n = P.cnt[region_coord(ix, o[0], k, h, nr, nc) +
+                        nc * (region_coord(iy, o[1], k, h, nr, nc) + nc * region_coord(iz, o[2], k, h, nr, nc))];
+    sum += n;
+    own += ix < k && iy < k && iz < k ? n : 0;
   }
+  sum = (int)__reduce_add_sync(FULL, (unsigned)sum);
+  own = (int)__reduce_add_sync(FULL, (unsigned)own);
+  if (lane == 0) P.cost[task] = min(sum + 4 * own, (1 << 24) - 1) + (own + 2 * P.m > P.list_small ? 1 << 24 : 0);
+}
+
+__global__ void __launch_bounds__(256) k_domain_rank(const SysParams *__restrict__ reps) {
+  const SysParams &P = reps[blockIdx.z];
+  const int c = blockIdx.y, nact = P.nact;
+  if (!P.order || c >= P.ncol || (int)(blockIdx.x * blockDim.x) >= nact) return;
+  __shared__ __align__(16) int cost[ORDER_MAX_NACT];
+  const int pad = (nact + 3) & ~3;
+  for (int i = threadIdx.x; i < pad; i += blockDim.x) cost[i] = i < nact ? P.cost[c * nact + i] : -1;
   __syncthreads();
-  for (int b = threadIdx.x; b < nact; b += blockDim.x) {
-    const int cb = cost[b];
-    int rank = 0;
-    for (int j = 0; j < nact; ++j) {
-      const int cj = cost[j];
-      rank += (cj > cb || (cj == cb && j < b)) ? 1 : 0;
-    }
-    P.order[c * nact + rank] = b;
+  const int b = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+  if (b >= nact) return;
+  const int cb = cost[b];
+  int rank = 0;
+  for (int j = 0; j < pad; j += 4) {
+    const int4 v = *(const int4 *)&cost[j];
+    rank += (v.x > cb || (v.x == cb && j < b)) + (v.y > cb || (v.y == cb && j + 1 < b)) +
+            (v.z > cb || (v.z == cb && j + 2 < b)) + (v.w > cb || (v.w == cb && j + 3 < b));
   }
+  P.order[c * nact + rank] = b;
 }
 
 cudaError_t launch_domain_order(const SysParams *d_reps, int n_rep, int ncol, int nact, cudaStream_t s, uint32_t sweep,
                                 uint32_t k0, uint32_t k1, const StepDyn *dyn) {
-  if (nact > ORDER_MAX_NACT) return cudaSuccess;  // contexts keep P.order null then
-  k_domain_order<<<dim3(n_rep, ncol), 512, 0, s>>>(d_reps, sweep, k0, k1, dyn);
+  if (nact > ORDER_MAX_NACT) nact = ORDER_MAX_NACT;  // contexts beyond keep P.order null
+  k_domain_cost<<<dim3((unsigned)(ncol * nact + 7) / 8, (unsigned)n_rep), 256, 0, s>>>(d_reps, sweep, k0, k1, dyn);
+  k_domain_rank<<<dim3((unsigned)(nact + 255) / 256, (unsigned)ncol, (unsigned)n_rep), 256, 0, s>>>(d_reps);
   return cudaGetLastError();
 }
 
