@@ -1174,13 +1174,14 @@ extern "C" int cr_set_surrogate(cr_ctx *ctx, const cr_mlp *m) {
   for (int i = 0; i < phase_form_count(true); ++i)
     smem_ok |= phase_smem_bytes(ctx->S, phase_form(i, true), true) <= (size_t)ctx->smem_max;
   if (!smem_ok) return CR_ERR_INVALID_ARG;
-  // transposed BF16 weights (WT[in][out]) and the biases
+  // the BF16 weights in blocks of eight inputs of one output (mlp_layer), and the biases
   std::vector<uint16_t> w(MLPW_N);
+  auto at = [](int o, int k) { return ((k >> 3) * MLP_H + o) * 8 + (k & 7); };
   for (int o = 0; o < MLP_H; ++o) {
-    for (int k = 0; k < MLP_IN; ++k) w[MLPW_W1 + k * MLP_H + o] = m->W1[o * MLP_IN + k];
+    for (int k = 0; k < MLP_IN; ++k) w[MLPW_W1 + at(o, k)] = m->W1[o * MLP_IN + k];
     for (int k = 0; k < MLP_H; ++k) {
-      w[MLPW_W2 + k * MLP_H + o] = m->W2[o * MLP_H + k];
-      w[MLPW_W3 + k * MLP_H + o] = m->W3[o * MLP_H + k];
+      w[MLPW_W2 + at(o, k)] = m->W2[o * MLP_H + k];
+      w[MLPW_W3 + at(o, k)] = m->W3[o * MLP_H + k];
     }
     w[MLPW_W4 + o] = m->w4[o];
   }

@@ -103,8 +103,8 @@ struct alignas(16) SysParams {
   int *err;                   // error bits
   cr_trial *log;              // trial records (device) or null
   long long per_sweep;        // trials per sweep (log indexing)
-  // delayed acceptance: surrogate weights (BF16, transposed: W1T [48][128],
-  // W2T, W3T [128][128], w4 [128]), biases (b1, b2, b3, b4), records
+  // delayed acceptance: surrogate weights (BF16; W1, W2, W3 in blocks of eight
+  // inputs of one output, w4 [128]), biases (b1, b2, b3, b4), records
   const uint16_t *mlp_w;
   const float *mlp_b;
   cr_trial_da *dlog;          // DA records (device) or null
