@@ -82,7 +82,7 @@ struct cr_ctx {
   float *d_in_frc = nullptr;
   // cr_state: id ordering on the device and the output arrays in the
   // caller's layouts (capacity-sized), one copy each to the caller
-  int *d_present = nullptr;
+  int *d_present = nullptr, *d_chunk = nullptr;  // marks of input ids; their chunks' counts, then prefix sums
   int ion_lo_bits = 32;  // the low words of inserted ids stay below 2^ion_lo_bits
   unsigned long long *d_ion_key = nullptr, *d_ion_key2 = nullptr;
   int *d_ion_val = nullptr, *d_ion_val2 = nullptr, *d_ion_rank = nullptr;
@@ -198,6 +198,9 @@ extern "C" const char *cr_strerror(int code) {
   }
 }
 
+// chunks of n input ids in a state read
+static size_t state_chunks(int n) { return (size_t)std::max((n + STATE_CHUNK - 1) / STATE_CHUNK, 1); }
+
 static void free_ctx(cr_ctx *c) {
   if (!c) return;
   if (c->bound) {  // the caller's buffers stay with the caller
@@ -211,7 +214,7 @@ static void free_ctx(cr_ctx *c) {
                   c->d_frc, c->d_frc2, c->d_fcons, c->d_pid, c->d_pid2, c->d_stats, c->d_lnK, c->d_lntab,
                   c->d_counts, c->d_perm, c->d_bond_off, c->d_bond_nbr, c->d_log,
                   c->d_in_xyz, c->d_in_vel, c->d_init_type, c->d_in_type, c->d_in_cls, c->d_site_map, c->d_in_state,
-                  c->d_in_id, c->d_in_frc, c->d_present, c->d_ion_key, c->d_ion_key2, c->d_ion_val, c->d_ion_val2, c->d_ion_rank, c->d_sort_tmp,
+                  c->d_in_id, c->d_in_frc, c->d_present, c->d_chunk, c->d_ion_key, c->d_ion_key2, c->d_ion_val, c->d_ion_val2, c->d_ion_rank, c->d_sort_tmp,
                   c->d_out_xyz, c->d_out_vel, c->d_out_frc, c->d_out_id, c->d_out_type, c->d_out_cls,
                   c->d_out_state, c->d_out_site,
                   c->d_reps, c->d_gs_pos, c->d_gs_vel, c->d_gs_id, c->d_gs_lnk, c->d_gs_info, c->d_gs_ord,
@@ -685,6 +688,7 @@ extern "C" int cr_init(cr_ctx **out, const cr_system *sys, double pH, const doub
   {
     const size_t cp = (size_t)std::max(sys->capacity, 1);
     ALLOC(c->d_present, (size_t)std::max(n, 1));
+    ALLOC(c->d_chunk, 2 * state_chunks(n));
     ALLOC(c->d_ion_key, cp);
     ALLOC(c->d_ion_val, cp);
     ALLOC(c->d_ion_rank, cp);
@@ -760,6 +764,7 @@ extern "C" int cr_init(cr_ctx **out, const cr_system *sys, double pH, const doub
   c->d_err = (int *)(c->d_counts + N_KIND + 1);
   cudaMemset(c->d_counts, 0, sizeof(long long) * (N_KIND + 2));
   cudaMemset(c->d_present, 0, sizeof(int) * (size_t)std::max(n, 1));
+  cudaMemset(c->d_chunk, 0, sizeof(int) * 2 * state_chunks(n));
   COPY(c->d_counts, kinds, (size_t)N_KIND);
   if (n > 0) COPY(c->d_site_map, site_of.data(), (size_t)n);
   if (n > 0) COPY(c->d_init_type, sys->type, (size_t)n);
@@ -1465,6 +1470,8 @@ static int state_begin(cr_ctx *ctx, const cr_state_view *out, cudaStream_t s, St
   B.cap = (int)ctx->capacity;
   B.lo_bits = ctx->ion_lo_bits;
   B.present = ctx->d_present;
+  B.chunk = ctx->d_chunk;
+  B.chunk_base = ctx->d_chunk + state_chunks(ctx->n_input);
   B.n_ions = ctx->d_counter;
   B.ion_key = ctx->d_ion_key;
   B.ion_key_alt = ctx->d_ion_key2;
@@ -1517,6 +1524,7 @@ static int state_arrays(cr_ctx *ctx, cr_state_view *out, cudaStream_t s, const S
     rc = CR_ERR_CUDA;
   if (rc != CR_OK) {  // clear the marks for the next read
     CR_CUDA(cudaMemsetAsync(ctx->d_present, 0, sizeof(int) * (size_t)std::max(ctx->n_input, 1), s));
+    CR_CUDA(cudaMemsetAsync(ctx->d_chunk, 0, sizeof(int) * state_chunks(ctx->n_input), s));
     CR_CUDA(cudaMemsetAsync(ctx->d_counter, 0, sizeof(int), s));
     return rc;
   }
@@ -2418,10 +2426,11 @@ extern "C" int cr_batch_state_packed(cr_batch *b, cr_batch_packed *p) {
   if (!b || !p || !p->n) return CR_ERR_INVALID_ARG;
   const size_t R = b->ctx.size();
   int64_t capmax = 0;
-  int max_slots = 0;
+  int max_cells = 0, max_input = 0;
   for (cr_ctx *c : b->ctx) {
     capmax = std::max<int64_t>(capmax, c->capacity);
-    max_slots = std::max(max_slots, c->P.ncell * c->P.cap);
+    max_cells = std::max(max_cells, c->P.ncell);
+    max_input = std::max(max_input, c->n_input);
   }
   if (p->stride < capmax) return CR_ERR_INVALID_ARG;
   const int64_t S = p->stride;
@@ -2455,6 +2464,8 @@ extern "C" int cr_batch_state_packed(cr_batch *b, cr_batch_packed *p) {
     B.cap = (int)c->capacity;
     B.lo_bits = c->ion_lo_bits;
     B.present = c->d_present;
+    B.chunk = c->d_chunk;
+    B.chunk_base = c->d_chunk + state_chunks(c->n_input);
     B.n_ions = c->d_counter;
     B.ion_key = c->d_ion_key;
     B.ion_val = c->d_ion_val;
@@ -2471,8 +2482,8 @@ extern "C" int cr_batch_state_packed(cr_batch *b, cr_batch_packed *p) {
     B.state = p->state ? (zs ? zs : b->d_pk_state) + r * S : nullptr;
   }
   CR_CUDA(cudaMemcpyAsync(b->d_sbufs, b->h_sbufs, R * sizeof(StateBufs), cudaMemcpyHostToDevice, s));
-  CR_CUDA(launch_state_batch(b->d_reps, b->d_sbufs, (int)R, max_slots, (int)capmax, b->d_nout, b->d_errout, s));
-  b->ctx[0]->launches_total += 3;
+  CR_CUDA(launch_state_batch(b->d_reps, b->d_sbufs, (int)R, max_cells, max_input, (int)capmax, b->d_nout, b->d_errout, s));
+  b->ctx[0]->launches_total += 5;
   CR_CUDA(cudaMemcpyAsync(b->h_nout, b->d_nout, R * sizeof(long long), cudaMemcpyDeviceToHost, s));
   int *herr = (int *)(b->h_nout + R);
   CR_CUDA(cudaMemcpyAsync(herr, b->d_errout, R * sizeof(int), cudaMemcpyDeviceToHost, s));

@@ -73,15 +73,17 @@ struct RebuildBufs {
 
 // the configuration read back in id order (crmc_state.cu); output arrays
 // that are null are not written
-constexpr int STATE_BLOCK_SORT_MAX = 16384;  // ions ranked by tile counting; more: device-wide sort
+constexpr int STATE_BLOCK_SORT_MAX = 16384;  // ions ranked by sorted tiles; more: device-wide sort
+constexpr int STATE_CHUNK = 1024;             // input ids per chunk
 struct StateBufs {
   int n_input, cap;               // input ids are 0..n_input-1; ion list capacity
   int lo_bits;                    // the low words of ion ids stay below 2^lo_bits
   int *present;                   // [n_input] slot + 1 of each input id, 0 absent
+  int *chunk, *chunk_base;        // present ids of each chunk of STATE_CHUNK, and before it
   int *n_ions;                    // number of inserted ions found
   unsigned long long *ion_key, *ion_key_alt;  // [cap] ion sort keys (the alternates for the device-wide sort)
   int *ion_val, *ion_val_alt;                 // [cap] their slots
-  int *ion_rank;                              // [cap] rank of each ion among the ion ids
+  int *ion_rank;                              // [cap] slot of each rank among the ion ids
   void *sort_tmp;                 // device-wide sort scratch (capacities above STATE_BLOCK_SORT_MAX)
   size_t sort_tmp_bytes;
   const float4 *vel_src, *frc_src;  // velocities; forces (null: zeros)
@@ -169,11 +171,11 @@ cudaError_t launch_state_mark(const SysParams &P, const StateBufs &B, cudaStream
 cudaError_t launch_state_order(const SysParams &P, const StateBufs &B, int n_present, int n_ions, int end_bit,
                                cudaStream_t s, int *launches);
 size_t state_sort_temp_bytes(int cap);
-// every replica of a batch in two launches (marks, ordering), the counts read
+// every replica of a batch in five launches (marks, ranks, ordering), the counts read
 // on the device; n_out[r] = particles of replica r, -1 when its read needs the
 // per-context path; err_out[r] its error word
-cudaError_t launch_state_batch(const SysParams *d_reps, const StateBufs *d_bufs, int n_rep, int max_slots,
-                               int max_cap, long long *d_n_out, int *d_err_out, cudaStream_t s);
+cudaError_t launch_state_batch(const SysParams *d_reps, const StateBufs *d_bufs, int n_rep, int max_cells,
+                               int max_input, int max_cap, long long *d_n_out, int *d_err_out, cudaStream_t s);
 // Ewald: S(k) of every replica of a batch from scratch (the occupied slots
 // listed, then one thread per reciprocal vector); max_nk: the largest
 // number of reciprocal vectors over the replicas
