@@ -1894,7 +1894,16 @@ extern "C" int cr_batch_create(cr_batch **out, cr_ctx *const *ctxs, int32_t n) {
   int smem_max = 0;
   cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctxs[0]->device);
   smem_max -= 1024;  // (as in cr_init)
-  if (phase_smem_bytes(b->S, PhaseForm{512, 1, 1, 16, 0}, false) > (size_t)smem_max) { delete b; return CR_ERR_INVALID_ARG; }
+  // (each replica's list and halo fit an SM; the largest list of one beside the largest region or reciprocal
+  // sum of another may not: cut as in cr_init, what does not fit goes to global memory)
+  const PhaseForm largest{512, 1, 1, 16, 0};
+  while (phase_smem_bytes(b->S, largest, false) > (size_t)smem_max && b->S.full.dcs > 64) {
+    PhaseCaps &C = b->S.full;
+    C.dcs -= C.dcs / 16;
+    C.hcs = std::max(C.hcs - C.hcs / 16, 64);
+    C.lns = std::min(C.lns, C.dcs + 4);
+  }
+  if (phase_smem_bytes(b->S, largest, false) > (size_t)smem_max) { delete b; return CR_ERR_INVALID_ARG; }
   b->smem_max = smem_max;
   cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, ctxs[0]->device);
   if (cudaMalloc((void **)&b->d_reps, sizeof(SysParams) * n) != cudaSuccess) { delete b; return CR_ERR_NOMEM; }
