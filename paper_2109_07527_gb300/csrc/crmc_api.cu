@@ -1415,32 +1415,10 @@ extern "C" int cr_md_begin(cr_ctx *ctx, double dt, double gamma, uint64_t seed) 
   return CR_OK;
 }
 
-// cr_md_end's force evaluation; in a captured cycle (dyn) the key and the
-// evaluation counter come from the step parameters in device memory
-static int md_end_impl(cr_ctx *ctx, double dt, double gamma, uint64_t seed, const StepDyn *dyn, unsigned rep,
-                       int eval_off = 0) {
-  MdParams M = md_params(ctx, 2, dt, gamma, seed);
-  M.dyn = dyn;
-  M.rep = rep;
-  M.eval_off = eval_off;
-  return md_force_eval(ctx, M);
-}
-
-// the force evaluation that opens a captured step whose forces are stale (as
-// cr_md_begin does it call by call: Langevin terms, no kick), counters from dyn
-static int md_first_impl(cr_ctx *ctx, double dt, double gamma, const StepDyn *dyn, unsigned rep) {
-  MdParams M = md_params(ctx, 1, dt, gamma, 0);
-  M.dyn = dyn;
-  M.rep = rep;
-  const int rc = md_force_eval(ctx, M);
-  if (rc == CR_OK) ctx->f_valid = true;  // the captured md_begin then only kicks and drifts
-  return rc;
-}
-
 extern "C" int cr_md_end(cr_ctx *ctx, double dt, double gamma, uint64_t seed) {
   if (!ctx || !(dt > 0.0) || !(gamma >= 0.0)) return CR_ERR_INVALID_ARG;
   int rc;
-  if ((rc = md_end_impl(ctx, dt, gamma, seed, nullptr, 0)) != CR_OK) return rc;
+  if ((rc = md_force_eval(ctx, md_params(ctx, 2, dt, gamma, seed))) != CR_OK) return rc;
   ctx->md_eval++;
   ctx->f_valid = true;
   ctx->fcons_valid = false;
@@ -1789,6 +1767,12 @@ struct cr_batch {
   int8_t *d_pk_state = nullptr;
   bool holds_refs = false;  // the contexts' batch_refs count this batch
   int ewald_nk_max = 0;     // largest number of Ewald reciprocal vectors over the replicas
+  // batched MD steps: per-replica parameters on the device (for md_dt, md_gamma) and the
+  // lengths of the replicas' particle lists
+  MdJob *d_md = nullptr;
+  int *d_nparts = nullptr;
+  MdBatchShape md_shape{};
+  double md_dt = 0.0, md_gamma = 0.0;
 };
 
 // The device address of caller memory the GPU can access directly (device
@@ -1966,6 +1950,8 @@ extern "C" void cr_batch_destroy(cr_batch *b) {
     b->ctx[0]->ev_reserved = 0;
   }
   if (b->d_dyn) cudaFree(b->d_dyn);
+  if (b->d_md) cudaFree(b->d_md);
+  if (b->d_nparts) cudaFree(b->d_nparts);
   if (b->cstream) cudaStreamDestroy(b->cstream);
   free_packed_staging(b);
   void *dp[] = {b->d_sbufs, b->d_jobs, b->d_nout, b->d_errout};
@@ -2161,15 +2147,105 @@ static int batch_md(cr_batch *b, Fn fn) {
   return rc;
 }
 
+// One launch per step of an MD call serves every replica, where their force
+// states and evaluation counters agree (they do unless a program stepped
+// some replicas by themselves); otherwise batch_md runs the calls side by side.
+static bool batch_md_together(const cr_batch *b) {
+  const cr_ctx *c0 = b->ctx[0];
+  for (const cr_ctx *c : b->ctx)
+    if (c->f_valid != c0->f_valid || c->md_eval != c0->md_eval) return false;
+  return b->ctx.size() <= 65535;  // (the grid's last dimension)
+}
+
+// the replicas' MD parameters for this step and friction, on the device
+static int batch_md_jobs(cr_batch *b, double dt, double gamma) {
+  cudaStream_t s = b->ctx[0]->stream;
+  const size_t n = b->ctx.size();
+  if (b->md_dt == dt && b->md_gamma == gamma) return CR_OK;  // (dt > 0: 0 before the first)
+  if (!b->d_nparts) {  // first MD step of the batch
+    CR_CUDA(cudaMalloc((void **)&b->d_nparts, sizeof(int) * n));
+    for (const cr_ctx *c : b->ctx) md_batch_shape(c->P, (int)c->capacity, &b->md_shape);
+  }
+  if (!b->d_md) CR_CUDA(cudaMalloc((void **)&b->d_md, sizeof(MdJob) * n));
+  std::vector<MdJob> jobs(n);
+  for (size_t r = 0; r < n; ++r) {
+    cr_ctx *c = b->ctx[r];
+    MdParams &M = jobs[r].M;
+    M = md_params(c, 2, dt, gamma, 0);
+    M.fsum = c->d_fsum;
+    M.plist = c->d_plist;
+    M.n_particles = b->d_nparts + r;
+    M.max_particles = (int)c->capacity;
+    jobs[r].B = RebuildBufs{c->d_cnt2, c->d_pos2, c->d_pid2, c->d_info2, c->d_vel2, c->d_frc2, c->d_vel, c->d_frc};
+  }
+  // (a pageable source: staged before the call returns)
+  CR_CUDA(cudaMemcpyAsync(b->d_md, jobs.data(), sizeof(MdJob) * n, cudaMemcpyHostToDevice, s));
+  b->md_dt = dt;
+  b->md_gamma = gamma;
+  return CR_OK;
+}
+
+// one force evaluation of every replica (mode, seed and counters as in
+// md_force_eval; with dyn they come from the captured step's parameters)
+static int batch_md_forces(cr_batch *b, int mode, uint64_t seed, const StepDyn *dyn = nullptr, int eval_off = 0) {
+  cr_ctx *c0 = b->ctx[0];
+  const int n = (int)b->ctx.size();
+  if (b->ewald_nk_max > 0) {
+    CR_CUDA(launch_ewald_sk(b->d_reps, n, b->ewald_nk_max, c0->stream));
+    c0->launches_total += 3;  // occupied slots, S(k), reciprocal forces
+  }
+  const MdCall Q{(uint32_t)seed, (uint32_t)(seed >> 32), c0->md_eval, mode, dyn, eval_off};
+  CR_CUDA(launch_md_forces_batch(b->d_reps, b->d_md, n, b->md_shape, b->d_nparts, Q, c0->stream));
+  c0->launches_total += 2 + __builtin_popcount((unsigned)b->md_shape.variants);  // list, finish, pair forces
+  for (cr_ctx *c : b->ctx) {
+    c->md_eval++;
+    c->f_valid = true;
+    c->fcons_valid = false;
+  }
+  return CR_OK;
+}
+
+// half kick, drift and cell rebuild of every replica, after the forces if they are stale
+static int batch_md_drift(cr_batch *b, uint64_t seed) {
+  cr_ctx *c0 = b->ctx[0];
+  if (!c0->f_valid) {
+    const int rc = batch_md_forces(b, 1, seed);
+    if (rc != CR_OK) return rc;
+  }
+  CR_CUDA(launch_kick_drift_rebuild_batch(b->d_reps, b->d_md, (int)b->ctx.size(), b->md_shape.cells, c0->stream));
+  c0->launches_total += 2;
+  for (cr_ctx *c : b->ctx) {
+    c->stream = c0->stream;
+    c->f_valid = false;  // positions moved: the closing kick needs new forces
+    c->fcons_valid = false;
+  }
+  return CR_OK;
+}
+
 extern "C" int cr_batch_md_step(cr_batch *b, int32_t n_steps, double dt, double gamma, uint64_t seed) {
+  if (b && n_steps > 0 && dt > 0.0 && gamma >= 0.0 && batch_md_together(b)) {
+    int rc = batch_md_jobs(b, dt, gamma);
+    for (int st = 0; st < n_steps && rc == CR_OK; ++st) {
+      if ((rc = batch_md_drift(b, seed)) == CR_OK) rc = batch_md_forces(b, 2, seed);
+    }
+    return rc;
+  }
   return batch_md(b, [&](cr_ctx *c, uint64_t r) { return cr_md_step(c, n_steps, dt, gamma, seed ^ (r << 32)); });
 }
 
 extern "C" int cr_batch_md_begin(cr_batch *b, double dt, double gamma, uint64_t seed) {
+  if (b && dt > 0.0 && gamma >= 0.0 && batch_md_together(b)) {
+    const int rc = batch_md_jobs(b, dt, gamma);
+    return rc != CR_OK ? rc : batch_md_drift(b, seed);
+  }
   return batch_md(b, [&](cr_ctx *c, uint64_t r) { return cr_md_begin(c, dt, gamma, seed ^ (r << 32)); });
 }
 
 extern "C" int cr_batch_md_end(cr_batch *b, double dt, double gamma, uint64_t seed) {
+  if (b && dt > 0.0 && gamma >= 0.0 && batch_md_together(b)) {
+    const int rc = batch_md_jobs(b, dt, gamma);
+    return rc != CR_OK ? rc : batch_md_forces(b, 2, seed);
+  }
   return batch_md(b, [&](cr_ctx *c, uint64_t r) { return cr_md_end(c, dt, gamma, seed ^ (r << 32)); });
 }
 
@@ -2248,8 +2324,8 @@ static int batch_capture_cycle(cr_batch *b, double dt, double gamma, bool da, bo
     return CR_ERR_CUDA;
   }
   {
-    if (ff) rc = batch_md(b, [&](cr_ctx *c, uint64_t r) { return md_first_impl(c, dt, gamma, dyn, (unsigned)r); });
-    if (rc == CR_OK) rc = batch_md(b, [&](cr_ctx *c, uint64_t) { return cr_md_begin(c, dt, gamma, 0); });
+    if (ff) rc = batch_md_forces(b, 1, 0, dyn);
+    if (rc == CR_OK) rc = batch_md_drift(b, 0);  // (the forces are valid)
     if (rc == CR_OK && b->order_nc > 0) {
       if (launch_domain_order(b->d_reps, n, b->ncol, b->order_nact, s, 0, 0, 0, dyn) != cudaSuccess) rc = CR_ERR_CUDA;
       c0->launches_total += 2;
@@ -2268,10 +2344,7 @@ static int batch_capture_cycle(cr_batch *b, double dt, double gamma, bool da, bo
         }
       }
     }
-    if (rc == CR_OK)
-      rc = batch_md(b, [&](cr_ctx *c, uint64_t r) {
-        return md_end_impl(c, dt, gamma, 0, dyn, (unsigned)r, ff ? 1 : 0);
-      });
+    if (rc == CR_OK) rc = batch_md_forces(b, 2, 0, dyn, ff ? 1 : 0);
     if (rc == CR_OK && launch_step_advance(b->d_dyn, s) != cudaSuccess) rc = CR_ERR_CUDA;
     c0->launches_total++;
   }
@@ -2354,6 +2427,7 @@ extern "C" int cr_batch_cycle(cr_batch *b, int32_t n_steps, double dt, double ga
       CR_CUDA(cudaMemcpyAsync(b->d_reps, b->reps.data(), sizeof(SysParams) * b->ctx.size(), cudaMemcpyHostToDevice, s));
   }
   if (!b->d_dyn) CR_CUDA(cudaMalloc((void **)&b->d_dyn, sizeof(StepDyn)));
+  if ((rc = batch_md_jobs(b, dt, gamma)) != CR_OK) return rc;
   const PhaseForm F = da ? b->da_F : b->F;
   const bool pers = da ? b->da_persistent : b->persistent;
   while (step < n_steps) {

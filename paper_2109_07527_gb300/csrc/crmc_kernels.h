@@ -106,6 +106,24 @@ struct LoadBufs {
   const float *frc;              // [3n] integrator forces (a restore), or null: zero
 };
 
+// one replica's MD step in a batched launch, and what changes from call to
+// call: the seed's words (the replica's index goes into the high one), the
+// evaluation counter, the mode, or dyn for a captured cycle
+struct MdJob {
+  MdParams M;
+  RebuildBufs B;
+};
+struct MdCall {
+  uint32_t key0, key1, eval;
+  int mode;
+  const StepDyn *dyn;
+  int eval_off;
+};
+// the largest counts over a batch's replicas, and the force variants they take
+struct MdBatchShape {
+  int cells, particles, ewald_particles, variants;
+};
+
 // one replica's load in a batched load
 struct LoadJob {
   LoadBufs I;
@@ -156,6 +174,13 @@ cudaError_t launch_md_forces(const SysParams &P, const MdParams &M, int *plist, 
 // the per-cell id sort back into the primary arrays
 cudaError_t launch_kick_drift_rebuild(const SysParams &P, const MdParams &M, const RebuildBufs &B, int *perm_slot,
                                       int n_perm, cudaStream_t s);
+// the same for every replica of a batch, one launch per step; n_particles: the
+// jobs' list lengths, contiguous (S(k) of each Ewald replica is current)
+void md_batch_shape(const SysParams &P, int max_particles, MdBatchShape *S);
+cudaError_t launch_md_forces_batch(const SysParams *d_reps, const MdJob *d_jobs, int n_rep, const MdBatchShape &S,
+                                   int *n_particles, const MdCall &C, cudaStream_t s);
+cudaError_t launch_kick_drift_rebuild_batch(const SysParams *d_reps, const MdJob *d_jobs, int n_rep, int max_cells,
+                                            cudaStream_t s);
 cudaError_t launch_load(const SysParams &P, const LoadBufs &I, const RebuildBufs &B, int *perm_slot, int n_perm,
                         cudaStream_t s);
 // loads of every replica of a batch (counts zeroed, scatter, cell sort,

@@ -3,6 +3,7 @@
 // check kernel (sm_103a).
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 
 #include "crmc_device.cuh"
@@ -18,45 +19,62 @@ namespace crmc {
 // ---------------------------------------------------------------------------
 constexpr float FFIX_INV = 1.0f / 16777216.0f;
 
+// what the pair terms need of SysParams, and the class pairs' WCA constants in
+// shared memory (eps, sig, del, squared cutoff; -1 when off)
+struct PairConsts {
+  float L, halfL, rc2, alpha, lB, c2;
+  const float4 *wca;
+};
+__device__ __forceinline__ float4 wca_consts(const WcaEntry &w) {
+  return make_float4(w.eps, w.sig, w.del, w.on ? w.wcut2 : -1.0f);
+}
+
 // FLAT: i and j are given in the stencil's flat frame (md_frame), where the
 // plain difference is the minimum-image one bit for bit
-// The pair's force on i in 2^-24 fixed point (zero out of range).  The terms
-// are odd in (i, j): exchanging the particles negates dx, dy, dz exactly and
-// leaves r^2 and g unchanged (charges are 0 or +-1, the WCA table is
-// symmetric), and fix24 rounds symmetrically, so the force on j is exactly
-// the negated value.
+// The pair's force on i in units of 2^-23 (zero out of range): fix24 gives
+// multiples of 2^-23, twice the rounded integer v 2^23, one conversion while
+// that fits an int.  The terms are odd in (i, j): exchanging the particles
+// negates dx, dy, dz exactly and leaves r^2 and g unchanged (charges are 0 or
+// +-1, the WCA table is symmetric), and the conversion rounds symmetrically,
+// so the force on j is exactly the negated value.
 template <bool FLAT = false>
-__device__ __forceinline__ void force_pair(const SysParams &P, float xi, float yi, float zi, float qi, int ci,
+__device__ __forceinline__ void force_pair(const PairConsts &K, float xi, float yi, float zi, float qi, int ci,
                                            float xj, float yj, float zj, float qj, int cj, long long &fx,
                                            long long &fy, long long &fz) {
-  const float dx = FLAT ? xi - xj : wrap_diff(xi, xj, P.Lf, P.halfL);
-  const float dy = FLAT ? yi - yj : wrap_diff(yi, yj, P.Lf, P.halfL);
-  const float dz = FLAT ? zi - zj : wrap_diff(zi, zj, P.Lf, P.halfL);
+  const float dx = FLAT ? xi - xj : wrap_diff(xi, xj, K.L, K.halfL);
+  const float dy = FLAT ? yi - yj : wrap_diff(yi, yj, K.L, K.halfL);
+  const float dz = FLAT ? zi - zj : wrap_diff(zi, zj, K.L, K.halfL);
   const float r2 = dx * dx + dy * dy + dz * dz;
-  const WcaEntry &w = P.wca[ci * 4 + cj];
-  const bool coul = r2 < P.rc2 && qi != 0.0f && qj != 0.0f;
-  const bool wca = w.on && r2 < w.wcut2;
+  const float4 w = K.wca[ci * 4 + cj];
+  const bool coul = r2 < K.rc2 && qi != 0.0f && qj != 0.0f;
+  const bool wca = r2 < w.w;
   if (!coul && !wca) return;
   const float rinv = rsqrtf(r2);
   float g = 0.0f;  // force / r along (ri - rj), positive = repulsive
   if (coul) {
     const float r = r2 * rinv;
-    const float ar = P.alpha * r;
-    g = P.lBf * qi * qj * (erfcf(ar) * rinv * rinv + 1.1283791670955126f * P.alpha * __expf(-ar * ar) * rinv - P.c2) * rinv;
+    const float ar = K.alpha * r;
+    g = K.lB * qi * qj * (erfcf(ar) * rinv * rinv + 1.1283791670955126f * K.alpha * __expf(-ar * ar) * rinv - K.c2) * rinv;
   }
   if (wca) {
-    const float s = r2 * rinv - w.del;
+    const float s = r2 * rinv - w.z;
     const float is = __fdividef(1.0f, s);
-    const float t = w.sig * is;
+    const float t = w.y * is;
     const float t2 = t * t;
     const float t6 = t2 * t2 * t2;
-    g += 24.0f * w.eps * (2.0f * t6 * t6 - t6) * is * rinv;
+    g += 24.0f * w.x * (2.0f * t6 * t6 - t6) * is * rinv;
   }
-  fx += fix24(g * dx);
-  fy += fix24(g * dy);
-  fz += fix24(g * dz);
+  const float vx = g * dx, vy = g * dy, vz = g * dz;
+  if (fmaxf(fmaxf(fabsf(vx), fabsf(vy)), fabsf(vz)) < 128.0f) {
+    fx = __float2int_rn(vx * 8388608.0f);
+    fy = __float2int_rn(vy * 8388608.0f);
+    fz = __float2int_rn(vz * 8388608.0f);
+  } else {
+    fx = fix24(vx) >> 1;
+    fy = fix24(vy) >> 1;
+    fz = fix24(vz) >> 1;
+  }
 }
-
 
 // FENE bonds, Langevin and the store of the total force, for one particle
 // (lane 0 of its warp)
@@ -133,7 +151,7 @@ __device__ __forceinline__ int wrap_cell(int c, int nc) { return c < 0 ? c + nc 
 __device__ __forceinline__ float md_frame(float x, bool s, float halfL, float L) { return s && x >= halfL ? x - L : x; }
 
 // compact list of occupied slots; one atomic per warp of 32 cells
-__global__ void k_plist(SysParams P, int *plist, int *n_out, int max_out, long long *fsum) {
+__device__ __forceinline__ void list_particles(const SysParams &P, int *plist, int *n_out, int max_out, long long *fsum) {
   const int c = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
   const int n = c < P.ncell ? P.cnt[c] : 0;
   int x = n;
@@ -157,6 +175,13 @@ __global__ void k_plist(SysParams P, int *plist, int *n_out, int max_out, long l
       fsum[3 * (c * P.cap + s) + 2] = 0;
     }
 }
+__global__ void k_plist(SysParams P, int *plist, int *n_out, int max_out, long long *fsum) {
+  list_particles(P, plist, n_out, max_out, fsum);
+}
+__global__ void k_plist_batch(const SysParams *__restrict__ reps, const MdJob *__restrict__ jobs) {
+  const MdParams &M = jobs[blockIdx.y].M;
+  list_particles(reps[blockIdx.y], const_cast<int *>(M.plist), const_cast<int *>(M.n_particles), M.max_particles, M.fsum);
+}
 
 // MD forces: one warp per particle.  The candidates of the (2h+1)^3 stencil of
 // neighbour cells (cell side >= rc/h) are numbered consecutively over the
@@ -174,160 +199,193 @@ __global__ void k_plist(SysParams P, int *plist, int *n_out, int max_out, long l
 // goes into j's fixed-point sums by 64-bit integer atomics (exact and
 // order-free, so the sums equal those of evaluating the pair from both ends).
 template <bool SPLIT, bool FLAT>
-__device__ __forceinline__ void md_pair(const SysParams &P, const MdParams &M, int g2, float xi, float yi, float zi,
-                                        float qi, int clsi, bool sx, bool sy, bool sz, long long &fx, long long &fy,
-                                        long long &fz) {
-  const float4 pj = P.pos[g2];
+__device__ __forceinline__ void md_pair(const PairConsts &K, const float4 *pos, const int *info, long long *fsum, int g2,
+                                        float xi, float yi, float zi, float qi, int clsi, bool sx, bool sy, bool sz,
+                                        long long &fx, long long &fy, long long &fz) {
+  const float4 pj = pos[g2];
   long long vx = 0, vy = 0, vz = 0;
-  force_pair<FLAT>(P, xi, yi, zi, qi, clsi, FLAT ? md_frame(pj.x, sx, P.halfL, P.Lf) : pj.x,
-                   FLAT ? md_frame(pj.y, sy, P.halfL, P.Lf) : pj.y, FLAT ? md_frame(pj.z, sz, P.halfL, P.Lf) : pj.z,
-                   pj.w, (P.info[g2] >> INFO_CLS_SHIFT) & 3, vx, vy, vz);
+  force_pair<FLAT>(K, xi, yi, zi, qi, clsi, FLAT ? md_frame(pj.x, sx, K.halfL, K.L) : pj.x,
+                   FLAT ? md_frame(pj.y, sy, K.halfL, K.L) : pj.y, FLAT ? md_frame(pj.z, sz, K.halfL, K.L) : pj.z,
+                   pj.w, (info[g2] >> INFO_CLS_SHIFT) & 3, vx, vy, vz);
   fx += vx;
   fy += vy;
   fz += vz;
   if (SPLIT && (vx | vy | vz) != 0) {
-    unsigned long long *d = reinterpret_cast<unsigned long long *>(M.fsum) + 3 * g2;
-    atomicAdd(d, (unsigned long long)(-vx));
-    atomicAdd(d + 1, (unsigned long long)(-vy));
-    atomicAdd(d + 2, (unsigned long long)(-vz));
+    unsigned long long *d = reinterpret_cast<unsigned long long *>(fsum) + 3 * g2;
+    atomicAdd(d, (unsigned long long)(-2 * vx));
+    atomicAdd(d + 1, (unsigned long long)(-2 * vy));
+    atomicAdd(d + 2, (unsigned long long)(-2 * vz));
   }
 }
 
 template <int NBC, bool SPLIT, bool FLAT = false>  // NBC: 2h+1 when the box has at least that many cells per dimension, else 0
-__global__ void __launch_bounds__(MD_THREADS) k_md_forces(SysParams P, MdParams M) {
+__device__ __forceinline__ void list_forces(const SysParams &P, const MdParams &M) {
+  __shared__ float4 wca_s[16];
   __shared__ int queue[MD_NW][MD_QCAP];
   __shared__ int cpre[MD_NW][MD_CPL * 32 + 1];  // exclusive prefix of the stencil cells' counts
   __shared__ int cbs[MD_NW][MD_CPL * 32];       // first slot of each stencil cell
   __shared__ int startcell[MD_NW][32];          // per round: the cell that starts at each candidate position
   const int lane = threadIdx.x & 31;
   const int wl = threadIdx.x >> 5;
-  const int w = blockIdx.x * MD_NW + wl;
-  if (w >= *M.n_particles || w >= M.max_particles) return;  // whole warp
+  const int n_list = min(*M.n_particles, M.max_particles);
+  if ((int)blockIdx.x * MD_NW >= n_list) return;  // whole CTA
+  if (threadIdx.x < 16) wca_s[threadIdx.x] = wca_consts(P.wca[threadIdx.x]);
+  __syncthreads();
   const int nc = P.nc, h = P.h, cap = P.cap;
-  const int gi = M.plist[w];
-  const float4 pi = P.pos[gi];
-  const int clsi = (P.info[gi] >> INFO_CLS_SHIFT) & 3;
-  const int cell = gi / cap;
-  const int cx = cell % nc, cy = (cell / nc) % nc, cz = cell / (nc * nc);
-  const int nb = NBC > 0 ? NBC : min(2 * h + 1, nc);
-  const bool all = NBC == 0 && nb == nc;  // every cell of the dimension, once
-  const int nb3 = nb * nb * nb;
-  const bool sx = FLAT && (cx < h || cx + h >= nc), sy = FLAT && (cy < h || cy + h >= nc),
-             sz = FLAT && (cz < h || cz + h >= nc);
-  const float xi = FLAT ? md_frame(pi.x, sx, P.halfL, P.Lf) : pi.x, yi = FLAT ? md_frame(pi.y, sy, P.halfL, P.Lf) : pi.y,
-              zi = FLAT ? md_frame(pi.z, sz, P.halfL, P.Lf) : pi.z;
-  // stencil cell o = lane + 32 t: its first slot and count; the candidates of
-  // all cells are then numbered consecutively (exclusive prefix over o)
-  int run = 0;
-  int lpre[MD_CPL], lcnt[MD_CPL];  // this lane's cells: first candidate number and count
-#pragma unroll
-  for (int t = 0; t < MD_CPL; ++t) {
-    const int o = lane + 32 * t;
-    int n = 0, base = 0;
-    // SPLIT over a 5^3 stencil (at least 5 cells per dimension, so no two
-    // offsets name the same cell): only the upper half of the offsets, the
-    // own cell (o = 62) with its higher slots; the partner's warp finds the
-    // pair through the opposite offset otherwise
-    if (o < nb3 && !(SPLIT && NBC == 5 && o < HALF5)) {
-      const int ox = o % nb, oy = (o / nb) % nb, oz = o / (nb * nb);
-      const int jx = all ? ox : wrap_cell(cx + ox - h, nc);
-      const int jy = all ? oy : wrap_cell(cy + oy - h, nc);
-      const int jz = all ? oz : wrap_cell(cz + oz - h, nc);
-      const int jc = jx + nc * (jy + nc * jz);
-      base = jc * cap;
-      n = P.cnt[jc];
-      if (FLAT && n > 0) {  // a cell whose box lies beyond the interaction reach holds no partner
-        const float x0 = (float)(cx + ox - h) * P.af, y0 = (float)(cy + oy - h) * P.af,
-                    z0 = (float)(cz + oz - h) * P.af;
-        const float ex = fmaxf(0.0f, fmaxf(x0 - pi.x, pi.x - (x0 + P.af)));
-        const float ey = fmaxf(0.0f, fmaxf(y0 - pi.y, pi.y - (y0 + P.af)));
-        const float ez = fmaxf(0.0f, fmaxf(z0 - pi.z, pi.z - (z0 + P.af)));
-        if (ex * ex + ey * ey + ez * ez > M.reach2) n = 0;
-      }
-    }
-    int x = n;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, x, d);
-      if (lane >= d) x += y;
-    }
-    cpre[wl][o] = run + x - n;
-    cbs[wl][o] = base;
-    lpre[t] = run + x - n;
-    lcnt[t] = n;
-    run += __shfl_sync(0xffffffffu, x, 31);
-  }
-  if (lane == 0) cpre[wl][MD_CPL * 32] = run;
-  __syncwarp();
-  const int total = run;
-  int *q = queue[wl];
-  const int *pre = cpre[wl];
-  int qn = 0;
-  long long fx = 0, fy = 0, fz = 0;
-  int carry = 0;  // the cell that runs on past the previous round's last candidate
-  for (int c0 = 0; c0 < total; c0 += 32) {
-    const int c = c0 + lane;
-    // cell of candidate c: the last non-empty cell that starts at or before
-    // it; each lane marks where its own cells start inside this round
-    unsigned mk = 0u;
+  const PairConsts K{P.Lf, P.halfL, P.rc2, P.alpha, P.lBf, P.c2, wca_s};
+  const float4 *pos = P.pos;
+  const int *info = P.info, *cnt = P.cnt;
+  const float af = P.af, reach2 = M.reach2;
+  for (int w = blockIdx.x * MD_NW + wl; w < n_list; w += gridDim.x * MD_NW) {  // (whole warps)
+    const int gi = M.plist[w];
+    const float4 pi = pos[gi];
+    const int clsi = (info[gi] >> INFO_CLS_SHIFT) & 3;
+    const int cell = gi / cap;
+    const int cx = cell % nc, cy = (cell / nc) % nc, cz = cell / (nc * nc);
+    const int nb = NBC > 0 ? NBC : min(2 * h + 1, nc);
+    const bool all = NBC == 0 && nb == nc;  // every cell of the dimension, once
+    const int nb3 = nb * nb * nb;
+    const bool sx = FLAT && (cx < h || cx + h >= nc), sy = FLAT && (cy < h || cy + h >= nc),
+               sz = FLAT && (cz < h || cz + h >= nc);
+    const float xi = FLAT ? md_frame(pi.x, sx, K.halfL, K.L) : pi.x, yi = FLAT ? md_frame(pi.y, sy, K.halfL, K.L) : pi.y,
+                zi = FLAT ? md_frame(pi.z, sz, K.halfL, K.L) : pi.z;
+    // stencil cell o = lane + 32 t: its first slot and count; the candidates of
+    // all cells are then numbered consecutively (exclusive prefix over o)
+    int run = 0;
+    int lpre[MD_CPL], lcnt[MD_CPL];  // this lane's cells: first candidate number and count
 #pragma unroll
     for (int t = 0; t < MD_CPL; ++t) {
-      const int st = lpre[t] - c0;
-      if (lcnt[t] > 0 && st >= 0 && st < 32) {
-        mk |= 1u << st;
-        startcell[wl][st] = lane + 32 * t;
+      const int o = lane + 32 * t;
+      int n = 0, base = 0;
+      // SPLIT over a 5^3 stencil (at least 5 cells per dimension, so no two
+      // offsets name the same cell): only the upper half of the offsets, the
+      // own cell (o = 62) with its higher slots; the partner's warp finds the
+      // pair through the opposite offset otherwise
+      if (o < nb3 && !(SPLIT && NBC == 5 && o < HALF5)) {
+        const int ox = o % nb, oy = (o / nb) % nb, oz = o / (nb * nb);
+        const int jx = all ? ox : wrap_cell(cx + ox - h, nc);
+        const int jy = all ? oy : wrap_cell(cy + oy - h, nc);
+        const int jz = all ? oz : wrap_cell(cz + oz - h, nc);
+        const int jc = jx + nc * (jy + nc * jz);
+        base = jc * cap;
+        n = cnt[jc];
+        if (FLAT && n > 0) {  // a cell whose box lies beyond the interaction reach holds no partner
+          const float x0 = (float)(cx + ox - h) * af, y0 = (float)(cy + oy - h) * af,
+                      z0 = (float)(cz + oz - h) * af;
+          const float ex = fmaxf(0.0f, fmaxf(x0 - pi.x, pi.x - (x0 + af)));
+          const float ey = fmaxf(0.0f, fmaxf(y0 - pi.y, pi.y - (y0 + af)));
+          const float ez = fmaxf(0.0f, fmaxf(z0 - pi.z, pi.z - (z0 + af)));
+          if (ex * ex + ey * ey + ez * ez > reach2) n = 0;
+        }
+      }
+      int x = n;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, d);
+        if (lane >= d) x += y;
+      }
+      cpre[wl][o] = run + x - n;
+      cbs[wl][o] = base;
+      lpre[t] = run + x - n;
+      lcnt[t] = n;
+      run += __shfl_sync(0xffffffffu, x, 31);
+    }
+    if (lane == 0) cpre[wl][MD_CPL * 32] = run;
+    __syncwarp();
+    const int total = run;
+    int *q = queue[wl];
+    const int *pre = cpre[wl];
+    int qn = 0;
+    long long fx = 0, fy = 0, fz = 0;
+    int carry = 0;  // the cell that runs on past the previous round's last candidate
+    for (int c0 = 0; c0 < total; c0 += 32) {
+      const int c = c0 + lane;
+      // cell of candidate c: the last non-empty cell that starts at or before
+      // it; each lane marks where its own cells start inside this round
+      unsigned mk = 0u;
+#pragma unroll
+      for (int t = 0; t < MD_CPL; ++t) {
+        const int st = lpre[t] - c0;
+        if (lcnt[t] > 0 && st >= 0 && st < 32) {
+          mk |= 1u << st;
+          startcell[wl][st] = lane + 32 * t;
+        }
+      }
+      mk = __reduce_or_sync(0xffffffffu, mk);
+      __syncwarp();
+      const unsigned upto = mk & (0xffffffffu >> (31 - lane));
+      const int cell_o = upto ? startcell[wl][31 - __clz(upto)] : carry;
+      carry = __shfl_sync(0xffffffffu, cell_o, 31);
+      __syncwarp();
+      bool in = false;
+      int gj = -1;
+      if (c < total) {
+        gj = cbs[wl][cell_o] + (c - pre[cell_o]);
+        // SPLIT: each pair once (the upper half of a 5^3 stencil and the higher
+        // slots of the own cell; otherwise every pair from its lower slot)
+        if (SPLIT ? ((NBC == 5 && cell_o != HALF5) || gj > gi) : gj != gi) {
+          const float4 pj = pos[gj];
+          const int cj = (info[gj] >> INFO_CLS_SHIFT) & 3;
+          const float dx = FLAT ? xi - md_frame(pj.x, sx, K.halfL, K.L) : wrap_diff(pi.x, pj.x, K.L, K.halfL);
+          const float dy = FLAT ? yi - md_frame(pj.y, sy, K.halfL, K.L) : wrap_diff(pi.y, pj.y, K.L, K.halfL);
+          const float dz = FLAT ? zi - md_frame(pj.z, sz, K.halfL, K.L) : wrap_diff(pi.z, pj.z, K.L, K.halfL);
+          const float r2 = dx * dx + dy * dy + dz * dz;
+          in = (r2 < K.rc2 && pi.w != 0.0f && pj.w != 0.0f) || r2 < wca_s[clsi * 4 + cj].w;
+        }
+      }
+      const unsigned m = __ballot_sync(0xffffffffu, in);
+      if (in) q[qn + __popc(m & ((1u << lane) - 1u))] = gj;
+      qn += __popc(m);
+      if (qn >= 32) {
+        __syncwarp();
+        md_pair<SPLIT, FLAT>(K, pos, info, M.fsum, q[lane], xi, yi, zi, pi.w, clsi, sx, sy, sz, fx, fy, fz);
+        const int rest = qn - 32;
+        int keep = 0;
+        if (lane < rest) keep = q[32 + lane];
+        __syncwarp();
+        if (lane < rest) q[lane] = keep;
+        __syncwarp();
+        qn = rest;
       }
     }
-    mk = __reduce_or_sync(0xffffffffu, mk);
     __syncwarp();
-    const unsigned upto = mk & (0xffffffffu >> (31 - lane));
-    const int cell_o = upto ? startcell[wl][31 - __clz(upto)] : carry;
-    carry = __shfl_sync(0xffffffffu, cell_o, 31);
-    __syncwarp();
-    bool in = false;
-    int gj = -1;
-    if (c < total) {
-      gj = cbs[wl][cell_o] + (c - pre[cell_o]);
-      // SPLIT: each pair once (the upper half of a 5^3 stencil and the higher
-      // slots of the own cell; otherwise every pair from its lower slot)
-      if (SPLIT ? ((NBC == 5 && cell_o != HALF5) || gj > gi) : gj != gi) {
-        const float4 pj = P.pos[gj];
-        const int cj = (P.info[gj] >> INFO_CLS_SHIFT) & 3;
-        const float dx = FLAT ? xi - md_frame(pj.x, sx, P.halfL, P.Lf) : wrap_diff(pi.x, pj.x, P.Lf, P.halfL);
-        const float dy = FLAT ? yi - md_frame(pj.y, sy, P.halfL, P.Lf) : wrap_diff(pi.y, pj.y, P.Lf, P.halfL);
-        const float dz = FLAT ? zi - md_frame(pj.z, sz, P.halfL, P.Lf) : wrap_diff(pi.z, pj.z, P.Lf, P.halfL);
-        const float r2 = dx * dx + dy * dy + dz * dz;
-        const WcaEntry &wc = P.wca[clsi * 4 + cj];
-        in = (r2 < P.rc2 && pi.w != 0.0f && pj.w != 0.0f) || (wc.on && r2 < wc.wcut2);
-      }
+    if (lane < qn) md_pair<SPLIT, FLAT>(K, pos, info, M.fsum, q[lane], xi, yi, zi, pi.w, clsi, sx, sy, sz, fx, fy, fz);
+    fx = warp_sum_i64(fx);
+    fy = warp_sum_i64(fy);
+    fz = warp_sum_i64(fz);
+    if (SPLIT) {  // this particle's own pairs join what its partners added
+      if (lane < 3)
+        atomicAdd(reinterpret_cast<unsigned long long *>(M.fsum) + 3 * gi + lane,
+                  (unsigned long long)(2 * (lane == 0 ? fx : (lane == 1 ? fy : fz))));
+    } else if (lane == 0) {
+      finish_particle(P, M, gi, pi, 2 * fx, 2 * fy, 2 * fz);
     }
-    const unsigned m = __ballot_sync(0xffffffffu, in);
-    if (in) q[qn + __popc(m & ((1u << lane) - 1u))] = gj;
-    qn += __popc(m);
-    if (qn >= 32) {
-      __syncwarp();
-      md_pair<SPLIT, FLAT>(P, M, q[lane], xi, yi, zi, pi.w, clsi, sx, sy, sz, fx, fy, fz);
-      const int rest = qn - 32;
-      int keep = 0;
-      if (lane < rest) keep = q[32 + lane];
-      __syncwarp();
-      if (lane < rest) q[lane] = keep;
-      __syncwarp();
-      qn = rest;
-    }
+    __syncwarp();  // the warp's shared memory is used again
   }
-  __syncwarp();
-  if (lane < qn) md_pair<SPLIT, FLAT>(P, M, q[lane], xi, yi, zi, pi.w, clsi, sx, sy, sz, fx, fy, fz);
-  fx = warp_sum_i64(fx);
-  fy = warp_sum_i64(fy);
-  fz = warp_sum_i64(fz);
-  if (SPLIT) {  // this particle's own pairs join what its partners added
-    if (lane < 3)
-      atomicAdd(reinterpret_cast<unsigned long long *>(M.fsum) + 3 * gi + lane,
-                (unsigned long long)(lane == 0 ? fx : (lane == 1 ? fy : fz)));
-  } else if (lane == 0) {
-    finish_particle(P, M, gi, pi, fx, fy, fz);
-  }
+}
+
+template <int NBC, bool SPLIT, bool FLAT = false>
+__global__ void __launch_bounds__(MD_THREADS) k_md_forces(SysParams P, MdParams M) {
+  list_forces<NBC, SPLIT, FLAT>(P, M);
+}
+
+// Batched MD steps: one launch per step for all replicas (blockIdx.y), where
+// each had its own on a stream of its own: nine launches and six event calls
+// per cycle and replica under Ewald, more host time than the kernels took
+// (64 electrolytes, two cycles with an MD step each: 16.2 -> 13.8 ms; captured,
+// 13 polyelectrolyte boxes 5.15 -> 5.03 ms, 64 chains 3.43 -> 3.33 ms, four
+// cycles and a read).  A replica runs the variant that a context of its own
+// would; a launch per variant present, the others' CTAs leave at once.
+__device__ __forceinline__ bool flat_stencil(const SysParams &P) {  // narrower than 0.4 L
+  return 2.5f * (float)(2 * P.h + 1) * P.af < P.Lf;
+}
+template <int NBC, bool FLAT>
+__global__ void __launch_bounds__(MD_THREADS) k_md_forces_batch(const SysParams *__restrict__ reps,
+                                                                const MdJob *__restrict__ jobs) {
+  const SysParams &P = reps[blockIdx.y];
+  const int nbc = P.h == 2 && P.nc >= 5 ? 5 : (P.h == 1 && P.nc >= 3 ? 3 : 0);
+  if (nbc != NBC || (NBC == 5 && flat_stencil(P) != FLAT)) return;  // another launch's replica
+  list_forces<NBC, true, FLAT>(P, jobs[blockIdx.y].M);
 }
 
 // FENE bonds, Langevin and the store of every particle's force (and the
@@ -338,18 +396,65 @@ __global__ void k_md_finish(SysParams P, MdParams M) {
   const int gi = M.plist[w];
   finish_particle(P, M, gi, P.pos[gi], M.fsum[3 * gi], M.fsum[3 * gi + 1], M.fsum[3 * gi + 2]);
 }
+__global__ void __launch_bounds__(256) k_md_finish_batch(const SysParams *__restrict__ reps,
+                                                         const MdJob *__restrict__ jobs, MdCall C) {
+  const int w = blockIdx.x * blockDim.x + threadIdx.x;
+  const MdParams &J = jobs[blockIdx.y].M;
+  if (w >= *J.n_particles || w >= J.max_particles) return;
+  MdParams M = J;
+  M.mode = C.mode;
+  M.key0 = C.key0;
+  M.key1 = C.key1 ^ blockIdx.y;
+  M.eval = C.eval;
+  M.dyn = C.dyn;
+  M.rep = blockIdx.y;
+  M.eval_off = C.eval_off;
+  const int gi = M.plist[w];
+  finish_particle(reps[blockIdx.y], M, gi, reps[blockIdx.y].pos[gi], M.fsum[3 * gi], M.fsum[3 * gi + 1],
+                  M.fsum[3 * gi + 2]);
+}
+
+// The particles of 32 consecutive cells, numbered over the cells and dealt to
+// the CTA's threads: f(cell, place in the cell, the cell's count).  A thread
+// per slot (19 in 20 empty in the polyelectrolyte solution) and, for the sort,
+// a warp per cell of 1.4 particles took 9.1 + 11.9 us per replica; so dealt,
+// 13 replicas take 22 + 24 us together (cold caches).
+constexpr int CELL_GROUP = 32;
+constexpr int CELL_THREADS = 256;  // at most
+static inline unsigned cell_groups(int ncell) { return (unsigned)((ncell + CELL_GROUP - 1) / CELL_GROUP); }
+// one system: 256 threads, so that dense cells (a nanoparticle's shell) are
+// done early; many: 64, about what 32 cells hold
+static inline unsigned cell_threads(unsigned groups) { return groups < 8 * 152 ? 256u : 64u; }
+template <typename F>
+__device__ __forceinline__ void for_cell_particles(int n, F f) {
+  const int lane = threadIdx.x & 31, c0 = blockIdx.x * CELL_GROUP;
+  int pre = n;  // n: the count of cell c0 + lane
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, pre, o);
+    if (lane >= o) pre += y;
+  }
+  const int total = __shfl_sync(0xffffffffu, pre, 31);
+  pre -= n;
+  for (int e0 = threadIdx.x - lane; e0 < total; e0 += (int)blockDim.x) {
+    const int e = e0 + lane;
+    int l = 0;  // the last cell that starts at or before e (empty ones share their start with the next)
+#pragma unroll
+    for (int s = 16; s > 0; s >>= 1)
+      if (__shfl_sync(0xffffffffu, pre, l + s) <= e) l += s;
+    const int first = __shfl_sync(0xffffffffu, pre, l), cn = __shfl_sync(0xffffffffu, n, l);
+    if (e < total) f(c0 + l, e - first, cn);
+  }
+}
 
 // v += dt/2 f; x += dt v; wrap into [0, L); the particle goes straight into
-// its new cell of the scratch arrays (unordered; k_rebuild_sort orders them)
-__global__ void k_md_kick_drift_scatter(SysParams P, MdParams M, RebuildBufs B) {
-  const int g = blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= P.ncell * P.cap) return;
-  const int c = g / P.cap;
-  if (g - c * P.cap >= P.cnt[c]) return;
+// its new cell of the scratch arrays (unordered; the rebuild orders them)
+__device__ __forceinline__ void kick_drift_scatter(const SysParams &P, const MdParams &M, const RebuildBufs &B, int g) {
   float4 v = M.vel[g];
   const float4 f = M.fout[g];
   const float4 p = P.pos[g];
   const unsigned long long id = P.pid[g];
+  const int info = P.info[g];
   const int mb = (M.n_bodies > 0 && id < (unsigned long long)M.n_perm) ? M.body_member[id] : -1;
   float x[3];
   if (mb >= 0) {  // a rigid body's member: placed by its body (k_body_drift)
@@ -380,55 +485,59 @@ __global__ void k_md_kick_drift_scatter(SysParams P, MdParams M, RebuildBufs B) 
   const int o = cell * P.cap + s;
   B.pos[o] = make_float4(x[0], x[1], x[2], p.w);
   B.pid[o] = id;
-  B.info[o] = P.info[g];
+  B.info[o] = info;
   B.vel[o] = v;
   B.frc[o] = f;
 }
 
-// rebuild: one warp per cell sorts the cell by id into the primary arrays
-__device__ __forceinline__ void rebuild_sort_cell(const SysParams &P, const RebuildBufs &B, int *perm_slot, int n_perm,
-                                                  int warp) {
-  const int lane = threadIdx.x & 31;
-  if (warp >= P.ncell) return;
-  const int c = warp;
-  const int n = min(B.cnt[c], P.cap);
-  const int base = c * P.cap;
-  if (n <= 32) {  // the cell's ids in the lanes, ranks by shuffles
-    const unsigned long long id = lane < n ? B.pid[base + lane] : ~0ull;
+__device__ __forceinline__ void kick_drift_cells(const SysParams &P, const MdParams &M, const RebuildBufs &B) {
+  const int c = blockIdx.x * CELL_GROUP + (threadIdx.x & 31);
+  for_cell_particles(c < P.ncell ? P.cnt[c] : 0,
+                     [&](int cell, int s, int) { kick_drift_scatter(P, M, B, cell * P.cap + s); });
+}
+__global__ void __launch_bounds__(CELL_THREADS) k_md_kick_drift_scatter(SysParams P, MdParams M, RebuildBufs B) {
+  kick_drift_cells(P, M, B);
+}
+__global__ void __launch_bounds__(CELL_THREADS) k_md_kick_drift_scatter_batch(const SysParams *__restrict__ reps,
+                                                                              const MdJob *__restrict__ jobs) {
+  kick_drift_cells(reps[blockIdx.y], jobs[blockIdx.y].M, jobs[blockIdx.y].B);
+}
+
+// rebuild: the particles of 32 cells sorted by id within each cell into the
+// primary arrays, a thread per particle (its rank: the smaller ids of its cell)
+__device__ __forceinline__ void rebuild_sort_cells(const SysParams &P, const RebuildBufs &B, int *perm_slot, int n_perm) {
+  const int c = blockIdx.x * CELL_GROUP + (threadIdx.x & 31);
+  const int n = c < P.ncell ? min(B.cnt[c], P.cap) : 0;
+  for_cell_particles(n, [&](int cell, int s, int cn) {
+    const int base = cell * P.cap, src = base + s;
+    const unsigned long long id = B.pid[src];
+    const float4 p = B.pos[src], v = B.vel[src], f = B.frc[src];
+    const int info = B.info[src];
     int rank = 0;
-    for (int o = 0; o < n; ++o) rank += __shfl_sync(0xffffffffu, id, o) < id ? 1 : 0;
-    if (lane < n) {
-      const int dst = base + rank;
-      P.pos[dst] = B.pos[base + lane];
-      P.pid[dst] = id;
-      P.info[dst] = B.info[base + lane];
-      B.vel_src[dst] = B.vel[base + lane];
-      B.frc_src[dst] = B.frc[base + lane];
-      if (id < (unsigned long long)n_perm) perm_slot[id] = dst;
-    }
-  } else {
-    for (int e = lane; e < n; e += 32) {
-      const unsigned long long id = B.pid[base + e];
-      int rank = 0;
-      for (int o = 0; o < n; ++o) rank += B.pid[base + o] < id;
-      const int dst = base + rank;
-      P.pos[dst] = B.pos[base + e];
-      P.pid[dst] = id;
-      P.info[dst] = B.info[base + e];
-      B.vel_src[dst] = B.vel[base + e];
-      B.frc_src[dst] = B.frc[base + e];
-      if (id < (unsigned long long)n_perm) perm_slot[id] = dst;
-    }
-  }
-  __syncwarp();
-  if (lane == 0) {
+#pragma unroll 4
+    for (int o = 0; o < cn; ++o) rank += B.pid[base + o] < id ? 1 : 0;
+    const int dst = base + rank;
+    P.pos[dst] = p;
+    P.pid[dst] = id;
+    P.info[dst] = info;
+    B.vel_src[dst] = v;
+    B.frc_src[dst] = f;
+    if (id < (unsigned long long)n_perm) perm_slot[id] = dst;
+  });
+  __syncthreads();  // every warp has read the counts
+  if (threadIdx.x < CELL_GROUP && c < P.ncell) {
     P.cnt[c] = n;
     B.cnt[c] = 0;
   }
 }
 
-__global__ void k_rebuild_sort(SysParams P, RebuildBufs B, int *perm_slot, int n_perm) {
-  rebuild_sort_cell(P, B, perm_slot, n_perm, (blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+__global__ void __launch_bounds__(CELL_THREADS) k_rebuild_sort(SysParams P, RebuildBufs B, int *perm_slot, int n_perm) {
+  rebuild_sort_cells(P, B, perm_slot, n_perm);
+}
+__global__ void __launch_bounds__(CELL_THREADS) k_md_rebuild_sort_batch(const SysParams *__restrict__ reps,
+                                                                        const MdJob *__restrict__ jobs) {
+  const MdJob &J = jobs[blockIdx.y];
+  rebuild_sort_cells(reps[blockIdx.y], J.B, const_cast<int *>(J.M.perm_slot), J.M.n_perm);
 }
 
 // the loaded configuration must be neutral (kind counts of the load)
@@ -497,9 +606,9 @@ __global__ void k_load_scatter_batch(const SysParams *__restrict__ reps, const L
   const LoadJob &J = jobs[blockIdx.y];
   load_particle(reps[blockIdx.y], J.I, J.B, blockIdx.x * blockDim.x + threadIdx.x);
 }
-__global__ void k_rebuild_sort_batch(const SysParams *__restrict__ reps, const LoadJob *__restrict__ jobs) {
+__global__ void __launch_bounds__(CELL_THREADS) k_rebuild_sort_batch(const SysParams *__restrict__ reps, const LoadJob *__restrict__ jobs) {
   const LoadJob &J = jobs[blockIdx.y];
-  rebuild_sort_cell(reps[blockIdx.y], J.B, J.perm_slot, J.n_perm, (blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+  rebuild_sort_cells(reps[blockIdx.y], J.B, J.perm_slot, J.n_perm);
 }
 __global__ void k_load_neutral_batch(const SysParams *__restrict__ reps) {
   if (threadIdx.x != 0) return;
@@ -945,7 +1054,7 @@ __device__ __forceinline__ float2 ewf_mul(float2 a, float2 b) {
   return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 
-__global__ void __launch_bounds__(EWF_THREADS) k_ewald_forces(SysParams P, MdParams M) {
+__device__ __forceinline__ void ewald_forces(const SysParams &P, const MdParams &M) {
   __shared__ float2 f[3 * EWF_K1];
   __shared__ float part[EWF_THREADS / 32][3];
   const int w = blockIdx.x, t = threadIdx.x, lane = t & 31, wl = t >> 5;
@@ -999,6 +1108,12 @@ __global__ void __launch_bounds__(EWF_THREADS) k_ewald_forces(SysParams P, MdPar
   }
 }
 
+__global__ void __launch_bounds__(EWF_THREADS) k_ewald_forces(SysParams P, MdParams M) { ewald_forces(P, M); }
+__global__ void __launch_bounds__(EWF_THREADS) k_ewald_forces_batch(const SysParams *__restrict__ reps,
+                                                                    const MdJob *__restrict__ jobs) {
+  if (reps[blockIdx.y].ewald_nk > 0) ewald_forces(reps[blockIdx.y], jobs[blockIdx.y].M);
+}
+
 cudaError_t launch_step_advance(StepDyn *dyn, cudaStream_t s) {
   k_step_advance<<<1, 32, 0, s>>>(dyn);
   return cudaGetLastError();
@@ -1032,19 +1147,54 @@ cudaError_t launch_md_forces(const SysParams &P, const MdParams &M, int *plist, 
   return cudaGetLastError();
 }
 
+cudaError_t launch_md_forces_batch(const SysParams *d_reps, const MdJob *d_jobs, int n_rep, const MdBatchShape &S,
+                                   int *n_particles, const MdCall &C, cudaStream_t s) {
+  const cudaError_t e = cudaMemsetAsync(n_particles, 0, sizeof(int) * (size_t)n_rep, s);
+  if (e != cudaSuccess) return e;
+  k_plist_batch<<<dim3((unsigned)((S.cells + 255) / 256), (unsigned)n_rep), 256, 0, s>>>(d_reps, d_jobs);
+  // (eight times the CTAs that 152 SMs hold, over the replicas: the capacities allow for several times
+  // the particles there are, and 64 replicas' empty CTAs cost more than the loop)
+  const unsigned share = (unsigned)std::max(8 * 8 * 152 / n_rep, 32);
+  const dim3 grid(std::min((unsigned)((S.particles + MD_NW - 1) / MD_NW), share), (unsigned)n_rep);
+  if (S.variants & 1) k_md_forces_batch<5, true><<<grid, MD_THREADS, 0, s>>>(d_reps, d_jobs);
+  if (S.variants & 2) k_md_forces_batch<5, false><<<grid, MD_THREADS, 0, s>>>(d_reps, d_jobs);
+  if (S.variants & 4) k_md_forces_batch<3, false><<<grid, MD_THREADS, 0, s>>>(d_reps, d_jobs);
+  if (S.variants & 8) k_md_forces_batch<0, false><<<grid, MD_THREADS, 0, s>>>(d_reps, d_jobs);
+  if (S.ewald_particles > 0)
+    k_ewald_forces_batch<<<dim3((unsigned)S.ewald_particles, (unsigned)n_rep), EWF_THREADS, 0, s>>>(d_reps, d_jobs);
+  k_md_finish_batch<<<dim3((unsigned)((S.particles + 255) / 256), (unsigned)n_rep), 256, 0, s>>>(d_reps, d_jobs, C);
+  return cudaGetLastError();
+}
+
+void md_batch_shape(const SysParams &P, int max_particles, MdBatchShape *S) {
+  const bool flat = 2.5f * (float)(2 * P.h + 1) * P.af < P.Lf;  // (flat_stencil)
+  S->variants |= P.h == 2 && P.nc >= 5 ? (flat ? 1 : 2) : (P.h == 1 && P.nc >= 3 ? 4 : 8);
+  S->cells = std::max(S->cells, P.ncell);
+  S->particles = std::max(S->particles, max_particles);
+  if (P.ewald_nk > 0) S->ewald_particles = std::max(S->ewald_particles, max_particles);
+}
+
 cudaError_t launch_kick_drift_rebuild(const SysParams &P, const MdParams &M, const RebuildBufs &B, int *perm_slot,
                                       int n_perm, cudaStream_t s) {
-  const int n = P.ncell * P.cap;
   if (M.n_bodies > 0) k_body_drift<<<M.n_bodies, RB_THREADS, 0, s>>>(P, M);
-  k_md_kick_drift_scatter<<<(n + 255) / 256, 256, 0, s>>>(P, M, B);
-  k_rebuild_sort<<<(P.ncell * 32 + 255) / 256, 256, 0, s>>>(P, B, perm_slot, n_perm);
+  k_md_kick_drift_scatter<<<cell_groups(P.ncell), cell_threads(cell_groups(P.ncell)), 0, s>>>(P, M, B);
+  k_rebuild_sort<<<cell_groups(P.ncell), cell_threads(cell_groups(P.ncell)), 0, s>>>(P, B, perm_slot, n_perm);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_kick_drift_rebuild_batch(const SysParams *d_reps, const MdJob *d_jobs, int n_rep, int max_cells,
+                                            cudaStream_t s) {
+  const dim3 grid(cell_groups(max_cells), (unsigned)n_rep);
+  const unsigned threads = cell_threads(grid.x * grid.y);
+  k_md_kick_drift_scatter_batch<<<grid, threads, 0, s>>>(d_reps, d_jobs);
+  k_md_rebuild_sort_batch<<<grid, threads, 0, s>>>(d_reps, d_jobs);
   return cudaGetLastError();
 }
 
 cudaError_t launch_load(const SysParams &P, const LoadBufs &I, const RebuildBufs &B, int *perm_slot, int n_perm,
                         cudaStream_t s) {
   if (I.n > 0) k_load_scatter<<<(I.n + 255) / 256, 256, 0, s>>>(P, I, B);
-  k_rebuild_sort<<<(P.ncell * 32 + 255) / 256, 256, 0, s>>>(P, B, perm_slot, n_perm);
+  k_rebuild_sort<<<cell_groups(P.ncell), cell_threads(cell_groups(P.ncell)), 0, s>>>(P, B, perm_slot, n_perm);
   k_load_neutral<<<1, 32, 0, s>>>(P);
   return cudaGetLastError();
 }
@@ -1053,7 +1203,7 @@ cudaError_t launch_load_batch(const SysParams *d_reps, const LoadJob *d_jobs, in
                               cudaStream_t s) {
   k_load_zero_batch<<<n_rep, 32, 0, s>>>(d_reps);
   if (max_n > 0) k_load_scatter_batch<<<dim3((max_n + 255) / 256, n_rep), 256, 0, s>>>(d_reps, d_jobs);
-  k_rebuild_sort_batch<<<dim3((max_cells * 32 + 255) / 256, n_rep), 256, 0, s>>>(d_reps, d_jobs);
+  k_rebuild_sort_batch<<<dim3(cell_groups(max_cells), n_rep), cell_threads(cell_groups(max_cells) * n_rep), 0, s>>>(d_reps, d_jobs);
   k_load_neutral_batch<<<n_rep, 32, 0, s>>>(d_reps);
   return cudaGetLastError();
 }
