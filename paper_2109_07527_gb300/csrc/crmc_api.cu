@@ -121,7 +121,10 @@ struct cr_ctx {
   int64_t launches[2] = {0, 0};
   int64_t launches_total = 0;
   // Ewald electrostatics: reciprocal vectors, weights, structure factor
-  int2 *d_ek_nA = nullptr;
+  float *d_ek_A = nullptr;
+  int4 *d_ek_z = nullptr, *d_ek_vec = nullptr;
+  int2 *d_ek_item = nullptr;
+  int *d_ek_col = nullptr;
   float2 *d_ek_Shi = nullptr, *d_ek_Slo = nullptr;
   int *d_ek_list = nullptr, *d_ek_np = nullptr;
   // caller-owned slot arrays (cr_bind_device_buffers) and batch membership
@@ -219,7 +222,7 @@ static void free_ctx(cr_ctx *c) {
                   c->d_out_state, c->d_out_site,
                   c->d_reps, c->d_gs_pos, c->d_gs_vel, c->d_gs_id, c->d_gs_lnk, c->d_gs_info, c->d_gs_ord,
                   c->d_plist, c->d_nparts, c->d_fsum, c->d_mlp_w, c->d_mlp_b, c->d_dlog, c->d_feat, c->d_order, c->d_cost,
-                  c->d_ek_nA, c->d_ek_Shi, c->d_ek_Slo, c->d_ek_list, c->d_ek_np,
+                  c->d_ek_A, c->d_ek_z, c->d_ek_vec, c->d_ek_item, c->d_ek_col, c->d_ek_Shi, c->d_ek_Slo, c->d_ek_list, c->d_ek_np,
                   c->d_bodies, c->d_body_member, c->d_body_d, c->d_body_df, c->d_body_newpos};
   for (void *p : ptrs)
     if (p) cudaFree(p);
@@ -401,7 +404,10 @@ extern "C" int cr_init(cr_ctx **out, const cr_system *sys, double pH, const doub
   P.lB_self = sys->dsf_self ? lB * (-(erc / (2.0 * rc) + alpha / std::sqrt(M_PI))) : 0.0;
   // Ewald electrostatics (global schedule only): the real-space term without
   // the DSF shift, the Ewald self term, the reciprocal vectors and weights
-  std::vector<int2> ek_nA;
+  std::vector<float> ek_A;
+  std::vector<int4> ek_z, ek_vec;
+  std::vector<int2> ek_item;
+  std::vector<int> ek_col;
   if (sys->ewald_kmax < 0 || sys->ewald_kmax > 32) { free_ctx(c); return CR_ERR_INVALID_ARG; }
   if (sys->ewald_kmax > 0) {
     if (!global) { free_ctx(c); return CR_ERR_INVALID_ARG; }
@@ -410,9 +416,43 @@ extern "C" int cr_init(cr_ctx **out, const cr_system *sys, double pH, const doub
     P.lB_self = lB * (-alpha / std::sqrt(M_PI));
     const int km = sys->ewald_kmax;
     const double V = L * L * L, kf = 2.0 * M_PI / L;
+    // columns of one half space, (0, 0) first, then the longest first
+    struct Column { int nx, ny, top; };
+    std::vector<Column> cols;
+    for (int ny = -km; ny <= km; ++ny)
+      for (int nx = 0; nx <= km; ++nx) {
+        const int r2 = km * km - nx * nx - ny * ny;
+        if (r2 < 0 || (nx == 0 && ny < 0)) continue;
+        int top = (int)std::sqrt((double)r2);
+        while (top * top > r2) --top;
+        while ((top + 1) * (top + 1) <= r2) ++top;
+        cols.push_back(Column{nx, ny, top});
+      }
+    std::stable_sort(cols.begin(), cols.end(), [](const Column &x, const Column &y) {
+      const bool x0 = x.nx == 0 && x.ny == 0, y0 = y.nx == 0 && y.ny == 0;
+      return x0 != y0 ? x0 : x.top > y.top;
+    });
+    ek_z.assign((size_t)km + 4, make_int4(0, 0, 0, 0));
+    int place = 0;
+    for (int sign = 0; sign < 2; ++sign) {
+      for (int z = sign; z <= km; ++z) {
+        int reach = 0;
+        while (reach < (int)cols.size() && cols[reach].top >= z) ++reach;
+        ek_z[z].x = reach;
+        (sign ? ek_z[z].z : ek_z[z].y) = place;
+        place += reach;
+      }
+      if (sign == 0) P.ewald_plus = place;
+    }
+    ek_A.assign((size_t)place, 0.0f);
+    for (const Column &c : cols) ek_col.push_back((c.nx & 255) | ((c.ny & 255) << 8));
+    for (int z0 = 0; z0 <= km; z0 += 4)
+      for (int c = 0; c < ek_z[z0].x; ++c) ek_item.push_back(make_int2(ek_col[c] | (z0 / 4) << 16, c));
+    std::vector<int> col_of((size_t)(km + 1) * (2 * km + 1), -1);
+    for (size_t c = 0; c < cols.size(); ++c) col_of[cols[c].nx * (2 * km + 1) + cols[c].ny + km] = (int)c;
     for (int nz = -km; nz <= km; ++nz)
       for (int ny = -km; ny <= km; ++ny)
-        for (int nx = -km; nx <= km; ++nx) {
+        for (int nx = 0; nx <= km; ++nx) {
           const int n2 = nx * nx + ny * ny + nz * nz;
           if (!(n2 > 0 && n2 <= km * km)) continue;
           // one half space: -k contributes the same term (S(-k) = conj S(k))
@@ -421,11 +461,16 @@ extern "C" int cr_init(cr_ctx **out, const cr_system *sys, double pH, const doub
           const float A = (float)(2.0 * 2.0 * M_PI * lB / V * std::exp(-k2 / (4.0 * alpha * alpha)) / k2);
           int Ab;
           std::memcpy(&Ab, &A, sizeof Ab);
-          ek_nA.push_back(make_int2((nx & 255) | ((ny & 255) << 8) | ((nz & 255) << 16), Ab));
+          const int4 &z = ek_z[std::abs(nz)];
+          const int at = (nz < 0 ? z.z : z.y) + col_of[nx * (2 * km + 1) + ny + km];
+          ek_A[at] = A;
+          ek_vec.push_back(make_int4((nx & 255) | ((ny & 255) << 8) | ((nz & 255) << 16), Ab, at, 0));
         }
   }
   P.ewald_kmax = sys->ewald_kmax;
-  P.ewald_nk = (int)ek_nA.size();
+  P.ewald_nk = (int)ek_A.size();
+  P.ewald_items = (int)ek_item.size();
+  P.ewald_vec = (int)ek_vec.size();
   P.invLd = 1.0 / L;
   for (int i = 0; i < 4; ++i)  // a pair potential: the class-pair table is symmetric
     for (int j = 0; j < i; ++j)
@@ -730,7 +775,11 @@ extern "C" int cr_init(cr_ctx **out, const cr_system *sys, double pH, const doub
   ALLOC(c->d_nparts, 1);
   ALLOC(c->d_fsum, 3 * (size_t)P.ncell * (size_t)P.cap);  // per slot: both ends of each pair add to it
   if (P.ewald_nk > 0) {
-    ALLOC(c->d_ek_nA, (size_t)P.ewald_nk);
+    ALLOC(c->d_ek_A, ek_A.size());
+    ALLOC(c->d_ek_z, ek_z.size());
+    ALLOC(c->d_ek_vec, ek_vec.size());
+    ALLOC(c->d_ek_item, ek_item.size());
+    ALLOC(c->d_ek_col, ek_col.size());
     ALLOC(c->d_ek_Shi, (size_t)P.ewald_nk);
     ALLOC(c->d_ek_Slo, (size_t)P.ewald_nk);
     ALLOC(c->d_ek_list, (size_t)std::max(sys->capacity, 1));
@@ -769,7 +818,11 @@ extern "C" int cr_init(cr_ctx **out, const cr_system *sys, double pH, const doub
   if (n > 0) COPY(c->d_site_map, site_of.data(), (size_t)n);
   if (n > 0) COPY(c->d_init_type, sys->type, (size_t)n);
   if (P.ewald_nk > 0) {
-    COPY(c->d_ek_nA, ek_nA.data(), ek_nA.size());
+    COPY(c->d_ek_A, ek_A.data(), ek_A.size());
+    COPY(c->d_ek_z, ek_z.data(), ek_z.size());
+    COPY(c->d_ek_vec, ek_vec.data(), ek_vec.size());
+    COPY(c->d_ek_item, ek_item.data(), ek_item.size());
+    COPY(c->d_ek_col, ek_col.data(), ek_col.size());
   }
 #undef COPY
   cudaMemset(c->d_cnt2, 0, sizeof(int) * P.ncell);
@@ -795,7 +848,11 @@ extern "C" int cr_init(cr_ctx **out, const cr_system *sys, double pH, const doub
   P.gs_lnk = c->d_gs_lnk;
   P.gs_info = c->d_gs_info;
   P.gs_ord = c->d_gs_ord;
-  P.ek_nA = c->d_ek_nA;
+  P.ek_A = c->d_ek_A;
+  P.ek_z = c->d_ek_z;
+  P.ek_vec = c->d_ek_vec;
+  P.ek_item = c->d_ek_item;
+  P.ek_col = c->d_ek_col;
   P.ek_Shi = c->d_ek_Shi;
   P.ek_Slo = c->d_ek_Slo;
   P.ek_list = c->d_ek_list;
@@ -1093,7 +1150,7 @@ static int sweep_impl(cr_ctx *ctx, uint64_t n_trials, uint64_t seed, cr_sweep_st
       ctx->launches_total += 2;
     }
     if (P.ewald_nk > 0) {  // S(k) from scratch at every sweep
-      CR_CUDA(launch_ewald_sk(ctx->d_reps, 1, P.ewald_nk, s));
+      CR_CUDA(launch_ewald_sk(ctx->d_reps, 1, P.ewald_items, P.ewald_plus, s));
       ctx->launches_total += 2;
     }
     for (int col = 0; col < P.ncol; ++col) {
@@ -1358,7 +1415,7 @@ static int md_force_eval(cr_ctx *ctx, const MdParams &M) {
   MdParams Q = M;
   Q.fsum = ctx->d_fsum;
   if (ctx->P.ewald_nk > 0) {  // S(k) of the current positions for the reciprocal forces
-    CR_CUDA(launch_ewald_sk(ctx->d_reps, 1, ctx->P.ewald_nk, ctx->stream));
+    CR_CUDA(launch_ewald_sk(ctx->d_reps, 1, ctx->P.ewald_items, ctx->P.ewald_plus, ctx->stream));
     ctx->launches_total += 3;  // occupied slots, S(k), reciprocal forces
   }
   CR_CUDA(launch_md_forces(ctx->P, Q, ctx->d_plist, ctx->d_nparts, (int)ctx->capacity, ctx->stream));
@@ -1766,7 +1823,7 @@ struct cr_batch {
   int *d_pk_type = nullptr, *d_pk_cls = nullptr;
   int8_t *d_pk_state = nullptr;
   bool holds_refs = false;  // the contexts' batch_refs count this batch
-  int ewald_nk_max = 0;     // largest number of Ewald reciprocal vectors over the replicas
+  int ewald_items = 0, ewald_plus = 0;  // largest numbers of Ewald items and nz >= 0 places over the replicas
   // batched MD steps: per-replica parameters on the device (for md_dt, md_gamma) and the
   // lengths of the replicas' particle lists
   MdJob *d_md = nullptr;
@@ -1862,7 +1919,8 @@ extern "C" int cr_batch_create(cr_batch **out, cr_ctx *const *ctxs, int32_t n) {
     b->S.kc3 = std::max(b->S.kc3, c->S.kc3);
     b->S.chunk = std::max(b->S.chunk, c->S.chunk);
     b->S.ewk = std::max(b->S.ewk, c->S.ewk);
-    b->ewald_nk_max = std::max(b->ewald_nk_max, c->P.ewald_nk);
+    b->ewald_items = std::max(b->ewald_items, c->P.ewald_items);
+    b->ewald_plus = std::max(b->ewald_plus, c->P.ewald_plus);
     b->grid_x = std::max(b->grid_x, c->P.nact);
   }
   b->ncol = ctxs[0]->P.ncol;
@@ -2049,8 +2107,8 @@ static int batch_sweep_impl(cr_batch *b, uint64_t n_sweeps, uint64_t seed, bool 
       CR_CUDA(launch_domain_order(b->d_reps, n, b->ncol, b->order_nact, s, swc, k0, k1));
       c0->launches_total += 2;
     }
-    if (b->ewald_nk_max > 0) {  // S(k) of every replica from scratch at every sweep
-      CR_CUDA(launch_ewald_sk(b->d_reps, n, b->ewald_nk_max, s));
+    if (b->ewald_items > 0) {  // S(k) of every replica from scratch at every sweep
+      CR_CUDA(launch_ewald_sk(b->d_reps, n, b->ewald_items, b->ewald_plus, s));
       c0->launches_total += 2;
     }
     if (persistent) {
@@ -2190,8 +2248,8 @@ static int batch_md_jobs(cr_batch *b, double dt, double gamma) {
 static int batch_md_forces(cr_batch *b, int mode, uint64_t seed, const StepDyn *dyn = nullptr, int eval_off = 0) {
   cr_ctx *c0 = b->ctx[0];
   const int n = (int)b->ctx.size();
-  if (b->ewald_nk_max > 0) {
-    CR_CUDA(launch_ewald_sk(b->d_reps, n, b->ewald_nk_max, c0->stream));
+  if (b->ewald_items > 0) {
+    CR_CUDA(launch_ewald_sk(b->d_reps, n, b->ewald_items, b->ewald_plus, c0->stream));
     c0->launches_total += 3;  // occupied slots, S(k), reciprocal forces
   }
   const MdCall Q{(uint32_t)seed, (uint32_t)(seed >> 32), c0->md_eval, mode, dyn, eval_off};

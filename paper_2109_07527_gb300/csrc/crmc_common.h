@@ -115,13 +115,26 @@ struct alignas(16) SysParams {
   int *order, *cost;
   int list_small;
   // Ewald electrostatics (ewald_nk > 0, global schedule): the reciprocal
-  // vectors n of one half space (three signed bytes each; S(-k) is the
-  // conjugate of S(k), so -k adds the same term) with their weights
-  // 2 A_k = 2 (2 pi lB / V) exp(-k^2 / (4 alpha^2)) / k^2 (FP32), and S(k) of
-  // the state as an unevaluated sum hi + lo of two FP32 complex numbers
-  // (about 48 bits; the trials read hi)
+  // vectors n of one half space (S(-k) is the conjugate of S(k), so -k adds
+  // the same term) with their weights 2 A_k = 2 (2 pi lB / V)
+  // exp(-k^2 / (4 alpha^2)) / k^2 (FP32), and S(k) of the state as an
+  // unevaluated sum hi + lo of two FP32 complex numbers (about 48 bits; the
+  // trials read hi).  Storage: columns of equal (nx, ny), the longest first
+  // (so that those reaching nz are the first ones), in slices nz = 0 .. kmax,
+  // then -1 .. -kmax; of column (0, 0) only nz > 0 belongs to the half space,
+  // its other places have weight 0.  An item is four consecutive |nz| of a
+  // column: a thread forms the column's factor e_x e_y once for up to eight
+  // vectors, and |nz| is uniform over a warp.
   int ewald_nk, ewald_kmax;
-  const int2 *ek_nA;  // (n code, weight bits) of each reciprocal vector
+  int ewald_plus, ewald_items;  // places with nz >= 0; items
+  const float *ek_A;            // [ewald_nk] weights
+  const int4 *ek_z;             // [kmax + 4] of |nz|: columns that reach it, the slices' first places (+, -)
+  const int *ek_col;            // nx | ny << 8 of each column
+  const int2 *ek_item;          // nx | ny << 8 | (|nz| / 4) << 16, column
+  // every vector in the order of nz, ny, nx: n code (three signed bytes),
+  // weight bits, place
+  int ewald_vec;
+  const int4 *ek_vec;
   float2 *ek_Shi, *ek_Slo;
   double invLd;  // 1 / L in FP64
   int *ek_list, *ek_np;  // occupied slots (the structure-factor kernel's particle list) and their number

@@ -1025,9 +1025,9 @@ __global__ void __launch_bounds__(RB_THREADS) k_body_drift(SysParams P, MdParams
 // space of k with the doubled weights A' (the vectors the CR-MC trials use),
 // F_j = 2 q_j sum_k A'_k k Im(S(k)^* exp(i k.r_j)), Im(...) = C sin - D cos,
 // S = C + i D of the current positions (k_ewald_sk runs just before).  One
-// CTA of 256 threads per particle of the force kernel's list (a particle's
-// sum spans thousands of vectors: eight warps keep the SM busy where one warp
-// per particle left it waiting on latencies); the axis factors
+// CTA of 256 threads per four particles of the force kernel's list, which
+// share each vector's loads and decoding (one particle per CTA re-read 24
+// bytes and re-decoded them for 20 flops); the axis factors
 // exp(i 2 pi n x / L), n <= kmax, from the coordinate's 0.32 fixed-point
 // fraction (an exact phase reduction); each thread sums every 256th vector in
 // order, the warps by a fixed butterfly, the eight warp sums in warp order;
@@ -1036,6 +1036,7 @@ __global__ void __launch_bounds__(RB_THREADS) k_body_drift(SysParams P, MdParams
 // ---------------------------------------------------------------------------
 constexpr int EWF_THREADS = 256;
 constexpr int EWF_K1 = 33;  // kmax + 1 for kmax <= 32
+constexpr int EWF_P = 4;    // particles per CTA
 
 __device__ __forceinline__ float2 ewf_factor(float x, double invL, int n) {
   const uint32_t U = (uint32_t)(unsigned long long)llrint((double)x * invL * 4294967296.0);
@@ -1045,66 +1046,70 @@ __device__ __forceinline__ float2 ewf_factor(float x, double invL, int n) {
   return make_float2(cs, sn);
 }
 
-__device__ __forceinline__ float2 ewf_get(const float2 *f, int n) {
-  const float2 v = f[n < 0 ? -n : n];
-  return make_float2(v.x, n < 0 ? -v.y : v.y);
-}
-
 __device__ __forceinline__ float2 ewf_mul(float2 a, float2 b) {
   return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 
 __device__ __forceinline__ void ewald_forces(const SysParams &P, const MdParams &M) {
-  __shared__ float2 f[3 * EWF_K1];
-  __shared__ float part[EWF_THREADS / 32][3];
-  const int w = blockIdx.x, t = threadIdx.x, lane = t & 31, wl = t >> 5;
-  if (w >= *M.n_particles || w >= M.max_particles) return;  // whole CTA
-  const int gi = M.plist[w];
-  const float4 p = P.pos[gi];
-  if (p.w == 0.0f) return;
+  __shared__ float2 f[EWF_P][3 * EWF_K1];
+  __shared__ float part[EWF_P][EWF_THREADS / 32][3];
+  const int w0 = blockIdx.x * EWF_P, t = threadIdx.x, lane = t & 31, wl = t >> 5, np = min(*M.n_particles, M.max_particles);
+  if (w0 >= np) return;  // whole CTA
   const int ewk = P.ewald_kmax + 1;
-  for (int i = t; i < 3 * ewk; i += EWF_THREADS) {
-    const int ax = i / ewk, n = i - ax * ewk;
-    f[i] = ewf_factor(ax == 0 ? p.x : (ax == 1 ? p.y : p.z), P.invLd, n);
+  float q[EWF_P];
+#pragma unroll
+  for (int p = 0; p < EWF_P; ++p) q[p] = w0 + p < np ? P.pos[M.plist[w0 + p]].w : 0.0f;
+  for (int i = t; i < EWF_P * 3 * ewk; i += EWF_THREADS) {
+    const int p = i / (3 * ewk), ax = i / ewk - 3 * p, n = i % ewk;
+    if (w0 + p >= np) break;
+    const float4 r = P.pos[M.plist[w0 + p]];
+    f[p][ax * EWF_K1 + n] = ewf_factor(ax == 0 ? r.x : (ax == 1 ? r.y : r.z), P.invLd, n);
   }
   __syncthreads();
-  float gx = 0.0f, gy = 0.0f, gz = 0.0f;
-#pragma unroll 4
-  for (int i = t; i < P.ewald_nk; i += EWF_THREADS) {
-    const int2 v = P.ek_nA[i];
-    const float2 hi = P.ek_Shi[i], lo = P.ek_Slo[i];
+  float gx[EWF_P], gy[EWF_P], gz[EWF_P];
+#pragma unroll
+  for (int p = 0; p < EWF_P; ++p) gx[p] = gy[p] = gz[p] = 0.0f;
+#pragma unroll 2
+  for (int i = t; i < P.ewald_vec; i += EWF_THREADS) {
+    const int4 v = P.ek_vec[i];
+    const float2 hi = P.ek_Shi[v.z], lo = P.ek_Slo[v.z];
     const int nx = (int)(signed char)(v.x & 255), ny = (int)(signed char)((v.x >> 8) & 255),
               nz = (int)(signed char)((v.x >> 16) & 255);
-    const float C = hi.x + lo.x, D = hi.y + lo.y;
-    const float2 e = ewf_mul(ewf_mul(ewf_get(f, nx), ewf_get(f + ewk, ny)), ewf_get(f + 2 * ewk, nz));
-    const float g = __int_as_float(v.y) * (C * e.y - D * e.x);
-    gx += g * (float)nx;
-    gy += g * (float)ny;
-    gz += g * (float)nz;
+    const int iy = EWF_K1 + abs(ny), iz = 2 * EWF_K1 + abs(nz);  // (nx >= 0)
+    const float C = hi.x + lo.x, D = hi.y + lo.y, A = __int_as_float(v.y);
+#pragma unroll
+    for (int p = 0; p < EWF_P; ++p) {
+      if (q[p] == 0.0f) continue;
+      const float2 ey = f[p][iy], ez = f[p][iz];
+      const float2 e = ewf_mul(ewf_mul(f[p][nx], make_float2(ey.x, ny < 0 ? -ey.y : ey.y)),
+                               make_float2(ez.x, nz < 0 ? -ez.y : ez.y));
+      const float g = A * (C * e.y - D * e.x);
+      gx[p] += g * (float)nx;
+      gy[p] += g * (float)ny;
+      gz[p] += g * (float)nz;
+    }
   }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    gx += __shfl_xor_sync(0xffffffffu, gx, o);
-    gy += __shfl_xor_sync(0xffffffffu, gy, o);
-    gz += __shfl_xor_sync(0xffffffffu, gz, o);
-  }
-  if (lane == 0) {
-    part[wl][0] = gx;
-    part[wl][1] = gy;
-    part[wl][2] = gz;
+  for (int p = 0; p < EWF_P; ++p) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      gx[p] += __shfl_xor_sync(0xffffffffu, gx[p], o);
+      gy[p] += __shfl_xor_sync(0xffffffffu, gy[p], o);
+      gz[p] += __shfl_xor_sync(0xffffffffu, gz[p], o);
+    }
+    if (lane == 0) {
+      part[p][wl][0] = gx[p];
+      part[p][wl][1] = gy[p];
+      part[p][wl][2] = gz[p];
+    }
   }
   __syncthreads();
-  if (t == 0) {
-    float sx = 0.0f, sy = 0.0f, sz = 0.0f;
-    for (int k = 0; k < EWF_THREADS / 32; ++k) {
-      sx += part[k][0];
-      sy += part[k][1];
-      sz += part[k][2];
-    }
-    const float s = 2.0f * p.w * (float)(6.283185307179586 * P.invLd);
-    M.fsum[3 * gi] += fix24(s * sx);
-    M.fsum[3 * gi + 1] += fix24(s * sy);
-    M.fsum[3 * gi + 2] += fix24(s * sz);
+  if (t < EWF_P * 3 && w0 + t / 3 < np) {
+    const int p = t / 3, ax = t - 3 * p, gi = M.plist[w0 + p];
+    float sum = 0.0f;
+    for (int k = 0; k < EWF_THREADS / 32; ++k) sum += part[p][k][ax];
+    const float s = 2.0f * P.pos[gi].w * (float)(6.283185307179586 * P.invLd);
+    M.fsum[3 * gi + ax] += fix24(s * sum);
   }
 }
 
@@ -1136,7 +1141,7 @@ cudaError_t launch_md_forces(const SysParams &P, const MdParams &M, int *plist, 
     else if (P.h == 1 && P.nc >= 3) k_md_forces<3, true><<<grid, MD_THREADS, 0, s>>>(P, Q);
     else k_md_forces<0, true><<<grid, MD_THREADS, 0, s>>>(P, Q);
     if (P.ewald_nk > 0)  // S(k) of these positions is current (launch_ewald_sk before this call)
-      k_ewald_forces<<<(unsigned)max_particles, EWF_THREADS, 0, s>>>(P, Q);
+      k_ewald_forces<<<(unsigned)((max_particles + EWF_P - 1) / EWF_P), EWF_THREADS, 0, s>>>(P, Q);
     k_md_finish<<<(unsigned)((max_particles + 255) / 256), 256, 0, s>>>(P, Q);
   } else {
     if (P.h == 2 && P.nc >= 5) k_md_forces<5, false><<<grid, MD_THREADS, 0, s>>>(P, Q);
@@ -1161,7 +1166,7 @@ cudaError_t launch_md_forces_batch(const SysParams *d_reps, const MdJob *d_jobs,
   if (S.variants & 4) k_md_forces_batch<3, false><<<grid, MD_THREADS, 0, s>>>(d_reps, d_jobs);
   if (S.variants & 8) k_md_forces_batch<0, false><<<grid, MD_THREADS, 0, s>>>(d_reps, d_jobs);
   if (S.ewald_particles > 0)
-    k_ewald_forces_batch<<<dim3((unsigned)S.ewald_particles, (unsigned)n_rep), EWF_THREADS, 0, s>>>(d_reps, d_jobs);
+    k_ewald_forces_batch<<<dim3((unsigned)((S.ewald_particles + EWF_P - 1) / EWF_P), (unsigned)n_rep), EWF_THREADS, 0, s>>>(d_reps, d_jobs);
   k_md_finish_batch<<<dim3((unsigned)((S.particles + 255) / 256), (unsigned)n_rep), 256, 0, s>>>(d_reps, d_jobs, C);
   return cudaGetLastError();
 }

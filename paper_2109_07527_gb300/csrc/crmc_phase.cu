@@ -1017,44 +1017,63 @@ __device__ __noinline__ void ewald_factors(const SysParams &P, const TrialCtl &C
   }
 }
 
-// dS(k) of the trial for the reciprocal vector of code `code`
-__device__ __forceinline__ float2 ewald_dS(const float2 *f, const float *dq, int ewk, int code) {
+// the two changed particles' factors of an item's column, and dS(k) of the
+// trial for nz = +-|nz| from them
+struct EwColumn {
+  float2 a, b;  // e_x e_y of the changed particles
+};
+__device__ __forceinline__ EwColumn ew_column(const float2 *f, int ewk, int code) {
   int nx, ny, nz;
   ew_decode(code, nx, ny, nz);
-  const float2 ea = ew_cmul(ew_cmul(ew_axis(f, nx), ew_axis(f + ewk, ny)), ew_axis(f + 2 * ewk, nz));
-  const float2 eb = ew_cmul(ew_cmul(ew_axis(f + 3 * ewk, nx), ew_axis(f + 4 * ewk, ny)), ew_axis(f + 5 * ewk, nz));
+  return EwColumn{ew_cmul(ew_axis(f, nx), ew_axis(f + ewk, ny)), ew_cmul(ew_axis(f + 3 * ewk, nx), ew_axis(f + 4 * ewk, ny))};
+}
+__device__ __forceinline__ float2 ewald_dS(const EwColumn &c, float2 za, float2 zb, const float *dq) {
+  const float2 ea = ew_cmul(c.a, za);
+  const float2 eb = ew_cmul(c.b, zb);
   return make_float2(dq[0] * ea.x + dq[1] * eb.x, dq[0] * ea.y + dq[1] * eb.y);
 }
+__device__ __forceinline__ float2 ew_conj(float2 v) { return make_float2(v.x, -v.y); }
 
 // this thread's share of the reciprocal energy change, into 2^-32 fixed point
-// (vectors tid, tid + T, ...; four loaded ahead at a time)
+// (items tid, tid + T, ...; an item's vectors loaded ahead; sums of integers,
+// so the order of the vectors does not matter)
 template <bool WITH_S>
 __device__ __noinline__ PairSum ewald_dE(const SysParams &P, const float2 *f, const float *dq, int ewk, int tid,
                                          int T) {
   PairSum out{0, 0ull, 0};
-  const int nk = P.ewald_nk;
-  const int2 *nA = P.ek_nA;
+  const float *A = P.ek_A;
   const float2 *S32 = P.ek_Shi;
-  for (int i0 = tid; i0 < nk; i0 += 4 * T) {
-    int2 v[4];
-    float2 sv[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int i = i0 + u * T;
-      v[u] = i < nk ? nA[i] : make_int2(0, 0);
-      sv[u] = i < nk ? S32[i] : make_float2(0.0f, 0.0f);
+  const int4 *zt = P.ek_z;
+  auto add = [&](float w, float2 s, float2 d) {
+    const float term = w * (2.0f * (s.x * d.x + s.y * d.y) + (d.x * d.x + d.y * d.y));
+    if (!(fabsf(term) < BIG_TERM)) {
+      out.ov = 1;
+    } else {
+      out.acc += fix32(term);
+      if (WITH_S) out.sacc += (unsigned long long)fix32(fabsf(term));
     }
+  };
+  for (int it = tid; it < P.ewald_items; it += T) {
+    const int2 item = P.ek_item[it];
+    const int z0 = item.x >> 16 << 2;
+    float w[8];
+    float2 sv[8];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      if (i0 + u * T >= nk) continue;
-      const float2 d = ewald_dS(f, dq, ewk, v[u].x);
-      const float term = __int_as_float(v[u].y) * (2.0f * (sv[u].x * d.x + sv[u].y * d.y) + (d.x * d.x + d.y * d.y));
-      if (!(fabsf(term) < BIG_TERM)) {
-        out.ov = 1;
-      } else {
-        out.acc += fix32(term);
-        if (WITH_S) out.sacc += (unsigned long long)fix32(fabsf(term));
-      }
+    for (int k = 0; k < 4; ++k) {
+      const int4 z = zt[z0 + k];
+      const bool in = item.y < z.x, neg = in && z0 + k > 0;
+      w[2 * k] = in ? A[z.y + item.y] : 0.0f;
+      sv[2 * k] = in ? S32[z.y + item.y] : make_float2(0.0f, 0.0f);
+      w[2 * k + 1] = neg ? A[z.z + item.y] : 0.0f;
+      sv[2 * k + 1] = neg ? S32[z.z + item.y] : make_float2(0.0f, 0.0f);
+    }
+    const EwColumn c = ew_column(f, ewk, item.x);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (z0 + k >= ewk) break;
+      const float2 za = f[2 * ewk + z0 + k], zb = f[5 * ewk + z0 + k];
+      add(w[2 * k], sv[2 * k], ewald_dS(c, za, zb, dq));
+      add(w[2 * k + 1], sv[2 * k + 1], ewald_dS(c, ew_conj(za), ew_conj(zb), dq));
     }
   }
   return out;
@@ -1073,16 +1092,28 @@ __device__ __forceinline__ void ew_add2(float &hi, float &lo, float d) {
 }
 
 // an accepted trial: S(k) += dS(k) for this thread's reciprocal vectors (the
-// same vectors ewald_dE gave it)
+// same items ewald_dE gave it)
 __device__ __noinline__ void ewald_update(const SysParams &P, const float2 *f, const float *dq, int ewk, int tid,
                                           int T) {
-  for (int i = tid; i < P.ewald_nk; i += T) {
-    const float2 d = ewald_dS(f, dq, ewk, P.ek_nA[i].x);
+  auto add = [&](int i, float2 d) {
     float2 hi = P.ek_Shi[i], lo = P.ek_Slo[i];
     ew_add2(hi.x, lo.x, d.x);
     ew_add2(hi.y, lo.y, d.y);
     P.ek_Shi[i] = hi;
     P.ek_Slo[i] = lo;
+  };
+  for (int it = tid; it < P.ewald_items; it += T) {
+    const int2 item = P.ek_item[it];
+    const int z0 = item.x >> 16 << 2;
+    const EwColumn c = ew_column(f, ewk, item.x);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int4 z = P.ek_z[z0 + k];
+      if (item.y >= z.x) break;  // (a column reaches every |nz| below its last)
+      const float2 za = f[2 * ewk + z0 + k], zb = f[5 * ewk + z0 + k];
+      add(z.y + item.y, ewald_dS(c, za, zb, dq));
+      if (z0 + k > 0) add(z.z + item.y, ewald_dS(c, ew_conj(za), ew_conj(zb), dq));
+    }
   }
 }
 
@@ -2118,10 +2149,10 @@ cudaError_t launch_domain_order(const SysParams *d_reps, int n_rep, int ncol, in
 // ---------------------------------------------------------------------------
 // Ewald structure factor S(k) = sum_j q_j exp(i k.r_j) of every replica from
 // scratch (at every sweep): k_ewald_list lists each replica's occupied slots
-// (one CTA per replica, cells in order), k_ewald_sk gives each reciprocal
-// vector a thread, the particles in tiles of 32 whose axis factors the CTA
-// computes together in shared memory (FP32 products summed per tile, tiles
-// summed in FP64).
+// (one CTA per replica, cells in order), k_ewald_sk gives each item (up to
+// eight reciprocal vectors) a thread, the particles in tiles of 32 whose axis
+// factors the CTA computes together in shared memory (FP32 products summed
+// per tile, tiles summed in FP64).
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_ewald_list(const SysParams *__restrict__ reps) {
   const SysParams &P = reps[blockIdx.x];
@@ -2158,19 +2189,44 @@ __global__ void __launch_bounds__(256) k_ewald_list(const SysParams *__restrict_
 
 constexpr int EW_TILE = 32;
 constexpr int EW_KMAX = 32;
+constexpr int EW_THREADS = 128;
 
-__global__ void __launch_bounds__(256) k_ewald_sk(const SysParams *__restrict__ reps) {
+// FP32 pipes and shared-memory reads bound it: a thread per vector took three
+// factors from shared memory and two complex products for every particle, an
+// item's thread forms e_x e_y once for up to eight vectors and reads each e_z,
+// which is uniform over the warp, once for +nz and -nz (64 boxes of 1,150
+// particles, |n| <= 16, 8,578 vectors: 0.28 ms per 16 boxes before, 0.49 ms per
+// 64 now).  ZS: |nz| per thread, 4 (an item) or, where fewer than two CTAs of
+// items per SM exist (a single box has 10), 1.
+template <int ZS>
+__global__ void __launch_bounds__(EW_THREADS) k_ewald_sk(const SysParams *__restrict__ reps) {
   const SysParams &P = reps[blockIdx.y];
-  const int nk = P.ewald_nk;
-  if (nk <= 0 || (int)blockIdx.x * 256 >= nk) return;  // uniform over the CTA
-  __shared__ float2 fac[EW_TILE][3][EW_KMAX + 1];
+  const int n_work = ZS == 4 ? P.ewald_items : P.ewald_plus;
+  if (P.ewald_nk <= 0 || (int)blockIdx.x * EW_THREADS >= n_work) return;  // uniform over the CTA
+  __shared__ float2 fac[EW_TILE][3][EW_KMAX + 4];
   __shared__ float qt[EW_TILE];
   __shared__ uint32_t ut[EW_TILE][3];
   const int ewk = P.ewald_kmax + 1, np = *P.ek_np;
-  const int i = (int)blockIdx.x * 256 + (int)threadIdx.x;
-  int nx = 0, ny = 0, nz = 0;
-  if (i < nk) ew_decode(P.ek_nA[i].x, nx, ny, nz);
-  double re = 0.0, im = 0.0;
+  const int i = (int)blockIdx.x * EW_THREADS + (int)threadIdx.x;
+  const bool mine = i < n_work;
+  int col = 0, z0 = 0, code = 0;
+  if (mine) {
+    if (ZS == 4) {
+      const int2 item = P.ek_item[i];
+      code = item.x;
+      col = item.y;
+      z0 = item.x >> 16 << 2;
+    } else {
+      while (z0 + 1 < ewk && P.ek_z[z0 + 1].y <= i) ++z0;
+      col = i - P.ek_z[z0].y;
+      code = P.ek_col[col];
+    }
+  }
+  int nx, ny, nz;
+  ew_decode(code, nx, ny, nz);
+  double re[2 * ZS], im[2 * ZS];
+#pragma unroll
+  for (int k = 0; k < 2 * ZS; ++k) re[k] = im[k] = 0.0;
   for (int t0 = 0; t0 < np; t0 += EW_TILE) {
     const int nt = min(EW_TILE, np - t0);
     if (threadIdx.x < 3 * nt) {  // the tile's coordinates as 0.32 fixed-point fractions of L
@@ -2180,36 +2236,57 @@ __global__ void __launch_bounds__(256) k_ewald_sk(const SysParams *__restrict__ 
       if (ax == 0) qt[p] = r.w;
     }
     __syncthreads();
-    for (int v = threadIdx.x; v < nt * 3 * ewk; v += 256) {
+    for (int v = threadIdx.x; v < nt * 3 * ewk; v += EW_THREADS) {
       const int p = v / (3 * ewk), ax = (v / ewk) % 3, n = v % ewk;
-      fac[p][ax][n] = ew_factor(ut[p][ax], n);
+      if (qt[p] != 0.0f) fac[p][ax][n] = ew_factor(ut[p][ax], n);
     }
     __syncthreads();
-    if (i < nk) {
-      float tr = 0.0f, ti = 0.0f;
+    if (mine) {
+      float tr[2 * ZS], ti[2 * ZS];
+#pragma unroll
+      for (int k = 0; k < 2 * ZS; ++k) tr[k] = ti[k] = 0.0f;
       for (int p = 0; p < nt; ++p) {
         const float q = qt[p];
         if (q == 0.0f) continue;
-        const float2 e = ew_cmul(ew_cmul(ew_axis(fac[p][0], nx), ew_axis(fac[p][1], ny)), ew_axis(fac[p][2], nz));
-        tr += q * e.x;
-        ti += q * e.y;
+        const float2 xy = ew_cmul(ew_axis(fac[p][0], nx), ew_axis(fac[p][1], ny));
+#pragma unroll
+        for (int k = 0; k < ZS; ++k) {  // (places beyond kmax hold no factor and are not stored)
+          const float2 ez = fac[p][2][z0 + k];
+          const float2 ep = ew_cmul(xy, ez), em = ew_cmul(xy, ew_conj(ez));
+          tr[2 * k] += q * ep.x;
+          ti[2 * k] += q * ep.y;
+          tr[2 * k + 1] += q * em.x;
+          ti[2 * k + 1] += q * em.y;
+        }
       }
-      re += (double)tr;
-      im += (double)ti;
+#pragma unroll
+      for (int k = 0; k < 2 * ZS; ++k) {
+        re[k] += (double)tr[k];
+        im[k] += (double)ti[k];
+      }
     }
     __syncthreads();
   }
-  if (i < nk) {
-    const float hr = (float)re, hm = (float)im;
-    P.ek_Shi[i] = make_float2(hr, hm);
-    P.ek_Slo[i] = make_float2((float)(re - (double)hr), (float)(im - (double)hm));
+  if (!mine) return;
+#pragma unroll
+  for (int k = 0; k < 2 * ZS; ++k) {
+    const int4 z = P.ek_z[z0 + k / 2];
+    if (col >= z.x || ((k & 1) && z0 + k / 2 == 0)) continue;
+    const int o = col + ((k & 1) ? z.z : z.y);
+    const float hr = (float)re[k], hm = (float)im[k];
+    P.ek_Shi[o] = make_float2(hr, hm);
+    P.ek_Slo[o] = make_float2((float)(re[k] - (double)hr), (float)(im[k] - (double)hm));
   }
 }
 
-cudaError_t launch_ewald_sk(const SysParams *d_reps, int n_rep, int max_nk, cudaStream_t s) {
-  if (n_rep <= 0 || max_nk <= 0) return cudaSuccess;
+cudaError_t launch_ewald_sk(const SysParams *d_reps, int n_rep, int max_items, int max_plus, cudaStream_t s) {
+  if (n_rep <= 0 || max_items <= 0) return cudaSuccess;
   k_ewald_list<<<n_rep, 256, 0, s>>>(d_reps);
-  k_ewald_sk<<<dim3((unsigned)((max_nk + 255) / 256), (unsigned)n_rep), 256, 0, s>>>(d_reps);
+  const unsigned g4 = (unsigned)((max_items + EW_THREADS - 1) / EW_THREADS);
+  if ((long long)g4 * n_rep >= 2 * 152)
+    k_ewald_sk<4><<<dim3(g4, (unsigned)n_rep), EW_THREADS, 0, s>>>(d_reps);
+  else
+    k_ewald_sk<1><<<dim3((unsigned)((max_plus + EW_THREADS - 1) / EW_THREADS), (unsigned)n_rep), EW_THREADS, 0, s>>>(d_reps);
   return cudaGetLastError();
 }
 
