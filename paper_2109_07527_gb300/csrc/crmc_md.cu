@@ -218,7 +218,7 @@ __device__ __forceinline__ void md_pair(const PairConsts &K, const float4 *pos, 
   }
 }
 
-template <int NBC, bool SPLIT, bool FLAT = false>  // NBC: 2h+1 when the box has at least that many cells per dimension, else 0
+template <int NBC, bool SPLIT, bool FLAT, bool LOOP>  // NBC: 2h+1 when the box has at least that many cells per dimension, else 0; LOOP: more particles than warps
 __device__ __forceinline__ void list_forces(const SysParams &P, const MdParams &M) {
   __shared__ float4 wca_s[16];
   __shared__ int queue[MD_NW][MD_QCAP];
@@ -360,13 +360,14 @@ __device__ __forceinline__ void list_forces(const SysParams &P, const MdParams &
     } else if (lane == 0) {
       finish_particle(P, M, gi, pi, 2 * fx, 2 * fy, 2 * fz);
     }
+    if (!LOOP) break;
     __syncwarp();  // the warp's shared memory is used again
   }
 }
 
 template <int NBC, bool SPLIT, bool FLAT = false>
 __global__ void __launch_bounds__(MD_THREADS) k_md_forces(SysParams P, MdParams M) {
-  list_forces<NBC, SPLIT, FLAT>(P, M);
+  list_forces<NBC, SPLIT, FLAT, false>(P, M);
 }
 
 // Batched MD steps: one launch per step for all replicas (blockIdx.y), where
@@ -385,7 +386,7 @@ __global__ void __launch_bounds__(MD_THREADS) k_md_forces_batch(const SysParams 
   const SysParams &P = reps[blockIdx.y];
   const int nbc = P.h == 2 && P.nc >= 5 ? 5 : (P.h == 1 && P.nc >= 3 ? 3 : 0);
   if (nbc != NBC || (NBC == 5 && flat_stencil(P) != FLAT)) return;  // another launch's replica
-  list_forces<NBC, true, FLAT>(P, jobs[blockIdx.y].M);
+  list_forces<NBC, true, FLAT, true>(P, jobs[blockIdx.y].M);
 }
 
 // FENE bonds, Langevin and the store of every particle's force (and the

@@ -198,7 +198,8 @@ __device__ __forceinline__ void emit(const SysParams &P, const StateBufs &B, int
 // unmarked: a present id's place is the number of present ids before it --
 // those of the chunks before and, by ballots and a scan of the warps' counts,
 // of its own -- so that consecutive threads write consecutive entries.
-__device__ __forceinline__ void order_inputs(const SysParams &P, const StateBufs &B, int c) {
+// all: every input id is present, so the chunks before are full.
+__device__ __forceinline__ void order_inputs(const SysParams &P, const StateBufs &B, int c, bool all) {
   __shared__ int part[ORDER_THREADS / 32];
   const int t = threadIdx.x, lane = t & 31, w = t >> 5, i = c * ORDER_THREADS + t;
   const int g = i < B.n_input ? B.present[i] - 1 : -1;
@@ -216,9 +217,10 @@ __device__ __forceinline__ void order_inputs(const SysParams &P, const StateBufs
   }
   __syncthreads();
   if (g >= 0) {
-    emit(P, B, g, B.chunk_base[c] + (w > 0 ? part[w - 1] : 0) + __popc(bal & ((1u << lane) - 1u)));
+    emit(P, B, g, (all ? c * ORDER_THREADS : B.chunk_base[c]) + (w > 0 ? part[w - 1] : 0) + __popc(bal & ((1u << lane) - 1u)));
     B.present[i] = 0;
   }
+  if (t == 0) B.chunk[c] = 0;
 }
 
 // CTA x < input_chunks: a chunk of the input ids; the others 1024 ions each,
@@ -226,7 +228,7 @@ __device__ __forceinline__ void order_inputs(const SysParams &P, const StateBufs
 __device__ __forceinline__ void order_cta(const SysParams &P, const StateBufs &B, int input_chunks, int n_present,
                                           int n_ions, const int *slot) {
   if ((int)blockIdx.x < input_chunks) {
-    if ((int)blockIdx.x * ORDER_THREADS < B.n_input) order_inputs(P, B, blockIdx.x);
+    if ((int)blockIdx.x * ORDER_THREADS < B.n_input) order_inputs(P, B, blockIdx.x, n_present == B.n_input);
     return;
   }
   const int r = ((int)blockIdx.x - input_chunks) * ORDER_THREADS + (int)threadIdx.x;
@@ -299,12 +301,17 @@ size_t state_sort_temp_bytes(int cap) {
 
 cudaError_t launch_state_order(const SysParams &P, const StateBufs &B, int n_present, int n_ions, int end_bit,
                                cudaStream_t s, int *launches) {
-  int n_launch = 2;
+  int n_launch = 1;
   const int *slot = B.ion_rank;
   const bool wide = n_ions > STATE_BLOCK_SORT_MAX;
-  // (the chunks' prefix sums come from the sort kernel's last CTA, also without ions)
+  // (the chunks' prefix sums come from the sort kernel's last CTA, also without
+  // ions; a configuration as it was given -- no ion inserted, no id gone -- needs
+  // neither, and the launch would cost a small read 5 of 70 us)
   const unsigned nt = wide ? 0u : (unsigned)((n_ions + RANK_TILE - 1) / RANK_TILE);
-  k_ion_sort<<<nt + 1, RANK_TILE, 0, s>>>(B, wide ? 0 : n_ions);
+  if (n_ions > 0 || n_present != B.n_input) {
+    k_ion_sort<<<nt + 1, RANK_TILE, 0, s>>>(B, wide ? 0 : n_ions);
+    ++n_launch;
+  }
   if (wide) {  // many ions: device-wide radix sort
     if (!B.sort_tmp || !B.ion_key_alt || !B.ion_val_alt) return cudaErrorInvalidValue;
     cub::DoubleBuffer<unsigned long long> k(B.ion_key, B.ion_key_alt);
@@ -314,7 +321,9 @@ cudaError_t launch_state_order(const SysParams &P, const StateBufs &B, int n_pre
     if (e != cudaSuccess) return e;
     slot = v.Current();
     n_launch += (end_bit + 7) / 8 + 2;  // histogram, scan and one pass per 8 bits
-  } else if (n_ions > 0) {
+  } else if (nt == 1) {  // one tile: its order is the ranks'
+    slot = B.ion_val;
+  } else if (nt > 1) {
     k_ion_rank<<<nt, RANK_TILE, 0, s>>>(B, n_ions);
     ++n_launch;
   }
