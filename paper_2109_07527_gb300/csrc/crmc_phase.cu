@@ -849,7 +849,9 @@ __device__ __forceinline__ void select_trial(const SysParams &P, const Dom &D, c
   // self-energy change: lB s_self (sum of q_new^2 - q_old^2), an integer multiple
   const int sq = (int)(qa_n * qa_n) - (int)(qa_o * qa_o) + (int)(qb_n * qb_n) - (int)(qb_o * qb_o);
   // lane 0 publishes the selection (C lives in shared memory; every lane
-  // holds the same values)
+  // holds the same values), once every lane has read the previous trial's: a
+  // forward salt move scans no list, so nothing else lets the warp meet here
+  __syncwarp();
   if (lane == 0) {
     C.c[0] = c0;
     C.c[1] = c1;
