@@ -111,6 +111,19 @@ __device__ __forceinline__ double wrap_diff_d(float a, float b, double L, double
   return d;
 }
 
+// FP64 squared distance and WCA energy at s = r - delta (gs: the terms'
+// magnitudes), rounded alike wherever they are inlined
+__device__ __forceinline__ double dist2_d(double dx, double dy, double dz) {
+  return __fma_rn(dz, dz, __fma_rn(dy, dy, __dmul_rn(dx, dx)));
+}
+__device__ __forceinline__ double wca_energy_d(const WcaEntry &w, double s, double &gs) {
+  const double t = w.sig_d / s;
+  const double t2 = __dmul_rn(t, t);
+  const double t6 = __dmul_rn(__dmul_rn(t2, t2), t2);
+  gs = __dmul_rn(w.eps_d, __fma_rn(__dmul_rn(4.0, t6), t6, __fma_rn(4.0, t6, 1.0)));
+  return __fma_rn(__dmul_rn(4.0, w.eps_d), __fma_rn(t6, t6, -t6), w.eps_d);
+}
+
 // WCA change of an inserted (dp > 0) or deleted (dp < 0) particle against a
 // bystander, in FP64 from the exact float positions: the steep (sigma/s)^12
 // would amplify FP32 distance rounding twelvefold.  Returns the change and
@@ -121,18 +134,14 @@ __device__ __forceinline__ bool wca_change_d(const WcaEntry &w, int dp, float cx
                                              int &ov) {
   const double dx = wrap_diff_d(xj, cx, L, halfL), dy = wrap_diff_d(yj, cy, L, halfL),
                dz = wrap_diff_d(zj, cz, L, halfL);
-  const double r = sqrt(dx * dx + dy * dy + dz * dz);
+  const double r = sqrt(dist2_d(dx, dy, dz));
   if (!(r < w.wcut_d)) return false;
   const double s = r - w.del_d;
   if (dp > 0 && s < 0.5 * w.sig_d) {
     ov = 1;
     return false;
   }
-  const double t = w.sig_d / s;
-  const double t2 = t * t;
-  const double t6 = t2 * t2 * t2;
-  du = (double)dp * (4.0 * w.eps_d * (t6 * t6 - t6) + w.eps_d);
-  gs = w.eps_d * (4.0 * t6 * t6 + 4.0 * t6 + 1.0);
+  du = __dmul_rn((double)dp, wca_energy_d(w, s, gs));
   return true;
 }
 

@@ -252,17 +252,46 @@ __device__ __forceinline__ void ord_close(uint2 *ord, int n, int p) {
   }
 }
 
+// The rounding of a pair's terms, the same in every copy of the code that
+// evaluates one (the compiler otherwise picks the products it fuses anew for
+// each place a function is inlined at): a pair counts the same whether its
+// candidate comes from shared or global memory, in whichever form of the launch
+// and in logged sweeps.  Left to the compiler, the two differed in the last bit
+// of a distance, and about one trial in 10^8 was decided by where its domain's
+// list lay.  The flat frame and the general one add the squares in another
+// order; a box has regions of one of them only, and each order is the one that
+// chains saved with earlier versions were run with.
+template <bool FLAT>
+__device__ __forceinline__ float pair_r2(float dx, float dy, float dz) {
+  return __fmaf_rn(dz, dz, FLAT ? __fmaf_rn(dy, dy, __fmul_rn(dx, dx)) : __fmaf_rn(dx, dx, __fmul_rn(dy, dy)));
+}
+// shifted Coulomb energy of unit charges at lB = 1: ef = erfc(alpha r), r = r2 rinv
+struct PairPhi {
+  float ef, r, rinv;
+};
+__device__ __forceinline__ PairPhi pair_phi(float r2, float alpha) {
+  const float rinv = rsqrtf(r2);
+  const float r = __fmul_rn(r2, rinv);
+  return PairPhi{erfcf(__fmul_rn(alpha, r)), r, rinv};
+}
+__device__ __forceinline__ float phi_value(const PairPhi &p, float c1, float c2, float rcf) {
+  return __fmaf_rn(c2, __fsub_rn(p.r, rcf), __fmaf_rn(p.ef, p.rinv, -c1));
+}
+__device__ __forceinline__ float phi_gross(const PairPhi &p, float c1, float c2, float rcf) {  // sum of the terms' magnitudes
+  return __fmaf_rn(c2, fabsf(__fsub_rn(p.r, rcf)), __fmaf_rn(p.ef, p.rinv, c1));
+}
+
 // pair change between the two changed particles: u_new - u_old, Coulomb in
 // FP32 and WCA in FP64, into fixed point (without a WCA term the FP64 sum
 // reduces to the FP32 change, taken directly)
-template <bool WITH_S>
+template <bool WITH_S, bool FLAT>
 __device__ __forceinline__ void cc_change_impl(const SysParams &K, const WcaEntry *wca, const TrialCtl &t, long long &acc,
                                                unsigned long long &sacc, int &ov) {
   const Desc &A = t.c[0], &B = t.c[1];
   const float dx = wrap_diff(B.x, A.x, K.Lf, K.halfL);
   const float dy = wrap_diff(B.y, A.y, K.Lf, K.halfL);
   const float dz = wrap_diff(B.z, A.z, K.Lf, K.halfL);
-  const float r2 = dx * dx + dy * dy + dz * dz;
+  const float r2 = pair_r2<FLAT>(dx, dy, dz);
   const WcaEntry &w = wca[A.cls * 4 + B.cls];
   float uc[2] = {0.0f, 0.0f};
   double uw[2] = {0.0, 0.0};
@@ -274,33 +303,30 @@ __device__ __forceinline__ void cc_change_impl(const SysParams &K, const WcaEntr
     if ((t.pres & both) != both) continue;
     const float qa = s ? t.qa_n : t.qa_o, qb = s ? t.qb_n : t.qb_o;
     if (r2 < K.rc2 && qa != 0.0f && qb != 0.0f) {
-      const float rinv = rsqrtf(r2);
-      const float r = r2 * rinv;
-      const float e = erfcf(K.alpha * r) * rinv;
-      uc[s] = K.lBf * qa * qb * (e - K.c1 + K.c2 * (r - K.rcf));
-      if (WITH_S) gs += (double)(fabsf(K.lBf * qa * qb) * (e + K.c1 + K.c2 * fabsf(r - K.rcf)));
+      const PairPhi p = pair_phi(r2, K.alpha);
+      const float qq = __fmul_rn(K.lBf, __fmul_rn(qa, qb));
+      uc[s] = __fmul_rn(qq, phi_value(p, K.c1, K.c2, K.rcf));
+      if (WITH_S) gs += (double)__fmul_rn(fabsf(qq), phi_gross(p, K.c1, K.c2, K.rcf));
     }
     if (w.on && r2 < 1.0001f * w.wcut2) {
       const double ddx = wrap_diff_d(B.x, A.x, K.Ld, K.halfLd), ddy = wrap_diff_d(B.y, A.y, K.Ld, K.halfLd),
                    ddz = wrap_diff_d(B.z, A.z, K.Ld, K.halfLd);
-      const double r = sqrt(ddx * ddx + ddy * ddy + ddz * ddz);
+      const double r = sqrt(dist2_d(ddx, ddy, ddz));
       if (r < w.wcut_d) {
         const double sv = r - w.del_d;
         const bool inserted = s == 1 && (!(t.pres & PA_O) || !(t.pres & PB_O));  // both are present after
         if (inserted && sv < 0.5 * w.sig_d) {
           ov = 1;
         } else {
-          const double tt = w.sig_d / sv;
-          const double t2 = tt * tt;
-          const double t6 = t2 * t2 * t2;
-          uw[s] = 4.0 * w.eps_d * (t6 * t6 - t6) + w.eps_d;
-          if (WITH_S) gs += w.eps_d * (4.0 * t6 * t6 + 4.0 * t6 + 1.0);
+          double g = 0.0;
+          uw[s] = wca_energy_d(w, sv, g);
+          if (WITH_S) gs += g;
           hit = true;
         }
       }
     }
   }
-  const float dc = uc[1] - uc[0];
+  const float dc = __fsub_rn(uc[1], uc[0]);
   if (!hit) {  // dw = 0: |dc| < 2^20 decides, fix32(dc) is the sum
     if (dc != 0.0f) {
       if (!(fabsf(dc) < BIG_TERM)) {
@@ -317,7 +343,7 @@ __device__ __forceinline__ void cc_change_impl(const SysParams &K, const WcaEntr
     if (!(fabs((double)dc + dw) < (double)BIG_TERM)) {
       ov = 1;
     } else {
-      acc += fix32(dc) + __double2ll_rn(dw * (double)FIX_SCALE);
+      acc += fix32(dc) + __double2ll_rn(__dmul_rn(dw, (double)FIX_SCALE));
       if (WITH_S) sacc += (unsigned long long)__double2ll_rn(fmin(gs, (double)BIG_TERM) * (double)FIX_SCALE);
     }
   }
@@ -446,15 +472,13 @@ __device__ __noinline__ void mlp_layer(const uint4 *__restrict__ W, const float 
 template <bool WITH_S>
 __device__ __forceinline__ void coul_eval(const PairK &K, float r2, float qp, long long &acc,
                                           unsigned long long &sacc, int &ov) {
-  const float rinv = rsqrtf(r2);
-  const float r = r2 * rinv;
-  const float e = erfcf(K.alpha * r) * rinv;
-  const float du = qp * (e - K.c1 + K.c2 * (r - K.rcf));
+  const PairPhi p = pair_phi(r2, K.alpha);
+  const float du = __fmul_rn(qp, phi_value(p, K.c1, K.c2, K.rcf));
   if (!(fabsf(du) < BIG_TERM)) {
     ov = 1;
   } else {
     acc += fix32(du);
-    if (WITH_S) sacc += (unsigned long long)fix32(fminf(fabsf(qp) * (e + K.c1 + K.c2 * fabsf(r - K.rcf)), BIG_TERM));
+    if (WITH_S) sacc += (unsigned long long)fix32(fminf(__fmul_rn(fabsf(qp), phi_gross(p, K.c1, K.c2, K.rcf)), BIG_TERM));
   }
 }
 
@@ -475,11 +499,10 @@ __device__ __noinline__ PairSum near_pair(const SysParams &P, const WcaEntry &w,
   float du = 0.0f, gs = 0.0f;
   const bool any = r2 < P.rc2 && cdq != 0.0f && qj != 0.0f;
   if (any) {
-    const float rinv = rsqrtf(r2);
-    const float r = r2 * rinv;
-    const float e = erfcf(P.alpha * r) * rinv;
-    du = cdq * qj * (e - P.c1 + P.c2 * (r - P.rcf));
-    if (WITH_S) gs = fabsf(cdq * qj) * (e + P.c1 + P.c2 * fabsf(r - P.rcf));
+    const PairPhi p = pair_phi(r2, P.alpha);
+    const float qq = __fmul_rn(cdq, qj);
+    du = __fmul_rn(qq, phi_value(p, P.c1, P.c2, P.rcf));
+    if (WITH_S) gs = __fmul_rn(fabsf(qq), phi_gross(p, P.c1, P.c2, P.rcf));
   }
   double du_w = 0.0, gs_w = 0.0;
   int ovw = 0;
@@ -491,7 +514,7 @@ __device__ __noinline__ PairSum near_pair(const SysParams &P, const WcaEntry &w,
       out.ov = 1;
     } else {
       if (any) out.acc += fix32(du);
-      out.acc += __double2ll_rn(du_w * (double)FIX_SCALE);
+      out.acc += __double2ll_rn(__dmul_rn(du_w, (double)FIX_SCALE));
       if (WITH_S) out.sacc += (unsigned long long)__double2ll_rn(fmin((double)gs + gs_w, (double)BIG_TERM) * (double)FIX_SCALE);
     }
   } else if (any) {  // beyond the WCA cutoff after all: Coulomb only
@@ -506,10 +529,10 @@ __device__ __noinline__ PairSum near_pair(const SysParams &P, const WcaEntry &w,
 
 // the pair between the two changed particles when they lie within WCA range
 // of each other (rare; one thread; out of line, with its FP64 branch)
-template <bool WITH_S>
+template <bool WITH_S, bool FLAT>
 __device__ __noinline__ PairSum cc_change(const SysParams &P, const TrialCtl &t) {
   PairSum out{0, 0ull, 0};
-  cc_change_impl<WITH_S>(P, P.wca, t, out.acc, out.sacc, out.ov);
+  cc_change_impl<WITH_S, FLAT>(P, P.wca, t, out.acc, out.sacc, out.ov);
   return out;
 }
 
@@ -591,7 +614,7 @@ __device__ __forceinline__ SweepPair sweep_pair(const PairK &K, const float *wma
 // pair's.  Evaluated by one thread of its own it kept the other warps waiting
 // at the trial's barrier.  True when lane 0 of the calling warp queued it;
 // within WCA range it is evaluated here.
-template <bool WITH_S>
+template <bool WITH_S, bool FLAT>
 __device__ __forceinline__ bool queue_changed_pair(const SysParams &P, const PairK &K, const float *wr,
                                                    const TrialCtl &t, float2 *q, long long &acc,
                                                    unsigned long long &sacc, int &ov) {
@@ -599,12 +622,12 @@ __device__ __forceinline__ bool queue_changed_pair(const SysParams &P, const Pai
   const float dx = wrap_diff(B.x, A.x, K.Lf, K.halfL);
   const float dy = wrap_diff(B.y, A.y, K.Lf, K.halfL);
   const float dz = wrap_diff(B.z, A.z, K.Lf, K.halfL);
-  const float r2 = dx * dx + dy * dy + dz * dz;
+  const float r2 = pair_r2<FLAT>(dx, dy, dz);
   const bool after = (t.pres & (PA_N | PB_N)) == (PA_N | PB_N);
-  const float qq = after ? t.qa_n * t.qb_n : -(t.qa_o * t.qb_o);
+  const float qq = after ? __fmul_rn(t.qa_n, t.qb_n) : -__fmul_rn(t.qa_o, t.qb_o);
   if (r2 < wr[A.cls * 4 + B.cls]) {
     if ((threadIdx.x & 31) == 0) {
-      const PairSum cc = cc_change<WITH_S>(P, t);
+      const PairSum cc = cc_change<WITH_S, FLAT>(P, t);
       acc += cc.acc;
       sacc += cc.sacc;
       ov |= cc.ov;
@@ -612,7 +635,7 @@ __device__ __forceinline__ bool queue_changed_pair(const SysParams &P, const Pai
     return false;
   }
   if (!(r2 < K.rc2) || qq == 0.0f) return false;
-  if ((threadIdx.x & 31) == 0) q[0] = make_float2(r2, P.lBf * qq);
+  if ((threadIdx.x & 31) == 0) q[0] = make_float2(r2, __fmul_rn(P.lBf, qq));
   return true;
 }
 
@@ -635,7 +658,7 @@ __device__ __forceinline__ void offer2(const SysParams &P, const PairK &K, const
     ax = wrap_diff(xj, p.ax, K.Lf, K.halfL); ay = wrap_diff(yj, p.ay, K.Lf, K.halfL); az = wrap_diff(zj, p.az, K.Lf, K.halfL);
     bx = wrap_diff(xj, p.bx, K.Lf, K.halfL); by = wrap_diff(yj, p.by, K.Lf, K.halfL); bz = wrap_diff(zj, p.bz, K.Lf, K.halfL);
   }
-  const float rA = ax * ax + ay * ay + az * az, rB = bx * bx + by * by + bz * bz;
+  const float rA = pair_r2<FLAT>(ax, ay, az), rB = pair_r2<FLAT>(bx, by, bz);
   const bool charged = valid && qj != 0.0f;
   bool inA = charged && rA < p.rcA, inB = charged && rB < p.rcB;
   if (valid && (rA < p.wmA || rB < p.wmB)) {
@@ -647,8 +670,8 @@ __device__ __forceinline__ void offer2(const SysParams &P, const PairK &K, const
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   const int nA = __popc(mA);
-  if (inA) q[qn + __popc(mA & lt)] = make_float2(rA, p.qA * qj);
-  if (inB) q[qn + nA + __popc(mB & lt)] = make_float2(rB, p.qB * qj);
+  if (inA) q[qn + __popc(mA & lt)] = make_float2(rA, __fmul_rn(p.qA, qj));
+  if (inB) q[qn + nA + __popc(mB & lt)] = make_float2(rB, __fmul_rn(p.qB, qj));
   qn += nA + __popc(mB);
   if (qn >= 32) queue_flush<WITH_S>(K, q, qn, acc, sacc, ov);
 }
@@ -937,7 +960,7 @@ __device__ __forceinline__ PairSum sweep_pairs(const PairK &K, const SysParams &
   const SweepPair sp = sweep_pair(K, Rg.wr + 16, C.c[0], C.c[1], Rg.strad);
   PairSum out{0, 0ull, 0};
   int qn = 0;
-  if (i0 < 32 && queue_changed_pair<LOG>(P, K, Rg.wr, C, q, out.acc, out.sacc, out.ov)) qn = 1;
+  if (i0 < 32 && queue_changed_pair<LOG, FLAT>(P, K, Rg.wr, C, q, out.acc, out.sacc, out.ov)) qn = 1;
   const int nhc = Rg.nhc, total = nhc + (Rg.in_smem ? nlist : 0);
   const int gap = Rg.hcs - nhc;  // from the on-chip halo to the list's slots
   const int skA = sp.skA >= 0 ? nhc + sp.skA : -1, skB = sp.skB >= 0 ? nhc + sp.skB : -1;
