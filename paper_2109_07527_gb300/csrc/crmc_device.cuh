@@ -145,6 +145,13 @@ __device__ __forceinline__ bool wca_change_d(const WcaEntry &w, int dp, float cx
   return true;
 }
 
+// complex product and the sum of two products with the fused products fixed,
+// so that every copy of the Ewald sums rounds alike
+__device__ __forceinline__ float sum2(float a, float b, float c, float d) { return __fmaf_rn(a, b, __fmul_rn(c, d)); }
+__device__ __forceinline__ float2 cmul(float2 a, float2 b) {
+  return make_float2(sum2(a.x, b.x, -a.y, b.y), sum2(a.x, b.y, a.y, b.x));
+}
+
 // int64 sum over the warp (mod 2^64, exact), result in every lane: v = a 2^42
 // + b 2^21 + c with b, c in [0, 2^21) and a in [-2^21, 2^21), each part
 // summed by one 32-bit warp reduction (partial sums below 2^26 in magnitude)

@@ -1047,10 +1047,6 @@ __device__ __forceinline__ float2 ewf_factor(float x, double invL, int n) {
   return make_float2(cs, sn);
 }
 
-__device__ __forceinline__ float2 ewf_mul(float2 a, float2 b) {
-  return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
-}
-
 __device__ __forceinline__ void ewald_forces(const SysParams &P, const MdParams &M) {
   __shared__ float2 f[EWF_P][3 * EWF_K1];
   __shared__ float part[EWF_P][EWF_THREADS / 32][3];
@@ -1082,12 +1078,12 @@ __device__ __forceinline__ void ewald_forces(const SysParams &P, const MdParams 
     for (int p = 0; p < EWF_P; ++p) {
       if (q[p] == 0.0f) continue;
       const float2 ey = f[p][iy], ez = f[p][iz];
-      const float2 e = ewf_mul(ewf_mul(f[p][nx], make_float2(ey.x, ny < 0 ? -ey.y : ey.y)),
-                               make_float2(ez.x, nz < 0 ? -ez.y : ez.y));
-      const float g = A * (C * e.y - D * e.x);
-      gx[p] += g * (float)nx;
-      gy[p] += g * (float)ny;
-      gz[p] += g * (float)nz;
+      const float2 e = cmul(cmul(make_float2(ey.x, ny < 0 ? -ey.y : ey.y), f[p][nx]),
+                            make_float2(ez.x, nz < 0 ? -ez.y : ez.y));
+      const float g = __fmul_rn(A, sum2(C, e.y, -D, e.x));
+      gx[p] = __fmaf_rn(g, (float)nx, gx[p]);
+      gy[p] = __fmaf_rn(g, (float)ny, gy[p]);
+      gz[p] = __fmaf_rn(g, (float)nz, gz[p]);
     }
   }
 #pragma unroll
@@ -1110,7 +1106,7 @@ __device__ __forceinline__ void ewald_forces(const SysParams &P, const MdParams 
     float sum = 0.0f;
     for (int k = 0; k < EWF_THREADS / 32; ++k) sum += part[p][k][ax];
     const float s = 2.0f * P.pos[gi].w * (float)(6.283185307179586 * P.invLd);
-    M.fsum[3 * gi + ax] += fix24(s * sum);
+    M.fsum[3 * gi + ax] += fix24(__fmul_rn(s, sum));
   }
 }
 

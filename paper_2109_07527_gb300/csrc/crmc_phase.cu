@@ -1003,7 +1003,10 @@ __device__ __noinline__ PairSum sweep_general(const SysParams &P, const TrialCtl
 // phase exp(i 2 pi n u), u = x / L, is reduced exactly in integers: U = u in
 // 0.32 fixed point (FP64), n U mod 2^32 is the fraction of n u; FP32 sincospi
 // of that fraction gives the factor.  A reciprocal vector's factor is the
-// product of its three axes' factors (the conjugate for negative n).
+// product of its three axes' factors (the conjugate for negative n), y and x
+// first (ew_xy).  The sums' fused products are fixed: contexts and batches,
+// items and slices, logged and unlogged trials add the same bits, those of the
+// sums before the vectors went by columns.
 __device__ __forceinline__ uint32_t ew_frac32(float x, double invL) {
   return (uint32_t)(unsigned long long)llrint((double)x * invL * 4294967296.0);
 }
@@ -1013,13 +1016,11 @@ __device__ __forceinline__ float2 ew_factor(uint32_t U, int n) {
   sincospif((float)t * (2.0f / 4294967296.0f), &sn, &cs);
   return make_float2(cs, sn);
 }
-__device__ __forceinline__ float2 ew_cmul(float2 a, float2 b) {
-  return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
-}
 __device__ __forceinline__ float2 ew_axis(const float2 *f, int n) {
   const float2 v = f[n < 0 ? -n : n];
   return make_float2(v.x, n < 0 ? -v.y : v.y);
 }
+__device__ __forceinline__ float2 ew_xy(float2 ex, float2 ey) { return cmul(ey, ex); }
 __device__ __forceinline__ void ew_decode(int code, int &nx, int &ny, int &nz) {
   nx = (int)(signed char)(code & 255);
   ny = (int)(signed char)((code >> 8) & 255);
@@ -1050,12 +1051,12 @@ struct EwColumn {
 __device__ __forceinline__ EwColumn ew_column(const float2 *f, int ewk, int code) {
   int nx, ny, nz;
   ew_decode(code, nx, ny, nz);
-  return EwColumn{ew_cmul(ew_axis(f, nx), ew_axis(f + ewk, ny)), ew_cmul(ew_axis(f + 3 * ewk, nx), ew_axis(f + 4 * ewk, ny))};
+  return EwColumn{ew_xy(ew_axis(f, nx), ew_axis(f + ewk, ny)), ew_xy(ew_axis(f + 3 * ewk, nx), ew_axis(f + 4 * ewk, ny))};
 }
 __device__ __forceinline__ float2 ewald_dS(const EwColumn &c, float2 za, float2 zb, const float *dq) {
-  const float2 ea = ew_cmul(c.a, za);
-  const float2 eb = ew_cmul(c.b, zb);
-  return make_float2(dq[0] * ea.x + dq[1] * eb.x, dq[0] * ea.y + dq[1] * eb.y);
+  const float2 ea = cmul(c.a, za);
+  const float2 eb = cmul(c.b, zb);
+  return make_float2(sum2(dq[0], ea.x, dq[1], eb.x), sum2(dq[0], ea.y, dq[1], eb.y));
 }
 __device__ __forceinline__ float2 ew_conj(float2 v) { return make_float2(v.x, -v.y); }
 
@@ -1070,7 +1071,7 @@ __device__ __noinline__ PairSum ewald_dE(const SysParams &P, const float2 *f, co
   const float2 *S32 = P.ek_Shi;
   const int4 *zt = P.ek_z;
   auto add = [&](float w, float2 s, float2 d) {
-    const float term = w * (2.0f * (s.x * d.x + s.y * d.y) + (d.x * d.x + d.y * d.y));
+    const float term = __fmul_rn(w, __fmaf_rn(2.0f, sum2(s.x, d.x, s.y, d.y), sum2(d.x, d.x, d.y, d.y)));
     if (!(fabsf(term) < BIG_TERM)) {
       out.ov = 1;
     } else {
@@ -2273,15 +2274,15 @@ __global__ void __launch_bounds__(EW_THREADS) k_ewald_sk(const SysParams *__rest
       for (int p = 0; p < nt; ++p) {
         const float q = qt[p];
         if (q == 0.0f) continue;
-        const float2 xy = ew_cmul(ew_axis(fac[p][0], nx), ew_axis(fac[p][1], ny));
+        const float2 xy = ew_xy(ew_axis(fac[p][0], nx), ew_axis(fac[p][1], ny));
 #pragma unroll
         for (int k = 0; k < ZS; ++k) {  // (places beyond kmax hold no factor and are not stored)
           const float2 ez = fac[p][2][z0 + k];
-          const float2 ep = ew_cmul(xy, ez), em = ew_cmul(xy, ew_conj(ez));
-          tr[2 * k] += q * ep.x;
-          ti[2 * k] += q * ep.y;
-          tr[2 * k + 1] += q * em.x;
-          ti[2 * k + 1] += q * em.y;
+          const float2 ep = cmul(xy, ez), em = cmul(xy, ew_conj(ez));
+          tr[2 * k] = __fmaf_rn(q, ep.x, tr[2 * k]);
+          ti[2 * k] = __fmaf_rn(q, ep.y, ti[2 * k]);
+          tr[2 * k + 1] = __fmaf_rn(q, em.x, tr[2 * k + 1]);
+          ti[2 * k + 1] = __fmaf_rn(q, em.y, ti[2 * k + 1]);
         }
       }
 #pragma unroll

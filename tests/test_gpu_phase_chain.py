@@ -3,13 +3,17 @@
   * the statistics of unlogged sweeps are those of the trials' records, also
     where consecutive selections scan no list (a box of salt moves);
   * a trial's energy has the same bits wherever the domain's list and halo lie
-    (shared or global memory), and logged sweeps give the unlogged chain.
+    (shared or global memory), and logged sweeps give the unlogged chain;
+  * the Ewald sums keep the bits they had before the reciprocal vectors went by
+    columns, and one box's slices give what a batch's items give.
 """
+import zlib
+
 import numpy as np
 import pytest
 
 from paper_2109_07527_gb300 import workloads as W
-from test_gpu_forms import _ions
+from test_gpu_forms import _electrolyte, _ions
 
 pytestmark = pytest.mark.gpu
 
@@ -76,3 +80,42 @@ def test_logged_sweeps_give_the_unlogged_chain(crmc, kw):
         assert np.array_equal(x[key], y[key]), key
     a.close()
     c.close()
+
+
+def test_ewald_sums_keep_their_rounding(crmc):
+    """Checksums of energies and forces from the version that gave each reciprocal vector a thread (249 particles,
+    about 1,500 vectors): sums of float products, so one product fused otherwise shows."""
+    w = W.weak_acid_electrolyte(n_acid=150, L=30.0, pH=7.0, pKa=6.5, pIS=1.5, rc=12.0, seed=3, trials_per_domain=40,
+                                alpha=0.3)
+    w.params["ewald_kmax"] = 9
+    g = crmc.Context(w)
+    log = np.concatenate([g.sweep(40, 100 + k, log=True)["log"] for k in range(4)])
+    assert zlib.crc32(np.ascontiguousarray(log["dE"]).tobytes()) == 0x95a45c54
+    g.close()
+    g = crmc.Context(w)
+    g.sweep(400, 1)
+    g.sweep(40, 2, log=True)
+    g.md_forces()
+    force = g.state()["force"]
+    assert force.shape == (249, 3) and zlib.crc32(np.ascontiguousarray(force).tobytes()) == 0x58c73e94
+    g.close()
+
+
+def test_many_ewald_boxes_equal_single_ones(crmc):
+    """64 boxes of 16 reciprocal vectors per axis go by items of a column, well past two CTAs of items per SM; a box
+    alone goes by slices."""
+    make = lambda r: _electrolyte(20.0, 16, 10 + r, acids=12)
+    b = crmc.Batch([crmc.Context(make(r)) for r in range(64)])
+    b.md_begin(0.005, 1.0, 7)
+    b.sweep(2, 50)
+    b.md_end(0.005, 1.0, 7)
+    for r in (0, 31, 63):
+        g = crmc.Context(make(r))
+        g.md_begin(0.005, 1.0, 7 ^ (r << 32))
+        g.sweep(g.trials_per_sweep * 2, 50 ^ (r << 32))
+        g.md_end(0.005, 1.0, 7 ^ (r << 32))
+        x, y = b.contexts[r].state(), g.state()
+        for key in ("id", "xyz", "vel", "state"):
+            assert np.array_equal(x[key], y[key]), (r, key)
+        g.close()
+    b.close()
