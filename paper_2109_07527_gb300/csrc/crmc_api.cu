@@ -35,7 +35,7 @@ struct cr_ctx {
   int tune_next = 0;     // sweeps timed so far
   bool tuning = true;
   float tune_ms[16] = {};
-  PhaseShape S{};  // shared-memory capacities
+  PhaseShape S{}, S_da{};  // shared-memory capacities; those of delayed-acceptance sweeps
   SysParams *d_reps = nullptr;  // device copy of P (the phase kernel reads it)
   int64_t per_sweep = 0;
   // sizes
@@ -199,6 +199,22 @@ extern "C" const char *cr_strerror(int code) {
     case CR_ERR_NO_DEVICE: return "no CUDA device";
     default: return "unknown error";
   }
+}
+
+// S for delayed-acceptance sweeps: the region's aggregates and the surrogate's
+// layers lie beside the list and halo, which are cut until the largest form fits
+// (what is cut off goes to global memory)
+static PhaseShape da_shape(PhaseShape S, size_t smem_max) {
+  for (int compact = 0; compact < 2; ++compact) {
+    PhaseCaps &C = compact ? S.small : S.full;
+    const PhaseForm largest{512, 1, 1, 16, compact};
+    while (phase_smem_bytes(S, largest, true) > smem_max && (C.dcs > 64 || C.hcs > 64)) {
+      C.dcs = std::max(C.dcs - std::max(C.dcs / 16, 1), std::min(C.dcs, 64));
+      C.hcs = std::max(C.hcs - std::max(C.hcs / 16, 1), std::min(C.hcs, 64));
+      C.lns = std::min(C.lns, C.dcs + 4);
+    }
+  }
+  return S;
 }
 
 // chunks of n input ids in a state read
@@ -693,6 +709,7 @@ extern "C" int cr_init(cr_ctx **out, const cr_system *sys, double pH, const doub
     }
   }
   c->smem_max = smem_max;
+  c->S_da = da_shape(S, (size_t)smem_max);
   P.per_sweep = c->per_sweep;
   P.key_xor = 0u;
 
@@ -1132,11 +1149,12 @@ static int sweep_impl(cr_ctx *ctx, uint64_t n_trials, uint64_t seed, cr_sweep_st
   const uint64_t n_sweeps = n_trials / (uint64_t)ctx->per_sweep;
   const uint32_t sweep0 = (uint32_t)ctx->sweep;
   const bool glob = P.global != 0;
+  const PhaseShape &S = da ? ctx->S_da : ctx->S;
   TuneRef tr = da ? TuneRef{ctx->da_F, ctx->da_next, ctx->da_tuning, ctx->da_ms, glob}
                   : TuneRef{ctx->F, ctx->tune_next, ctx->tuning, ctx->tune_ms, glob};
   for (uint64_t sw = 0; sw < n_sweeps; ++sw) {
     const uint32_t swc = (uint32_t)ctx->sweep++;
-    if (!log) tune_skip(tr, ctx->S, ctx->smem_max, da);
+    if (!log) tune_skip(tr, S, ctx->smem_max, da);
     const bool tune = tr.on && !log && tr.next < tune_total(tr, da);
     const PhaseForm F = tune ? phase_form(tune_cand(tr, da), da) : tr.F;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -1156,7 +1174,7 @@ static int sweep_impl(cr_ctx *ctx, uint64_t n_trials, uint64_t seed, cr_sweep_st
     for (int col = 0; col < P.ncol; ++col) {
       int ti;
       tbegin(ctx, 0, &ti);
-      CR_CUDA(launch_phase(ctx->d_reps, 1, P.nact, ctx->S, F, log != nullptr, da, s, swc, sweep0, col, k0, k1));
+      CR_CUDA(launch_phase(ctx->d_reps, 1, P.nact, S, F, log != nullptr, da, s, swc, sweep0, col, k0, k1));
       tend(ctx, 0, ti);
       ctx->launches_total++;
     }
@@ -1167,7 +1185,7 @@ static int sweep_impl(cr_ctx *ctx, uint64_t n_trials, uint64_t seed, cr_sweep_st
       cudaEventElapsedTime(&ms, e0, e1);
       cudaEventDestroy(e0);
       cudaEventDestroy(e1);
-      tune_finish(tr, ms, ctx->S, ctx->smem_max, da);
+      tune_finish(tr, ms, S, ctx->smem_max, da);
     }
   }
   if (log) {
@@ -1234,7 +1252,7 @@ extern "C" int cr_set_surrogate(cr_ctx *ctx, const cr_mlp *m) {
   if (P0.global || P0.h != 2 || P0.nc < P0.k + 4 || !std::isfinite(m->b4)) return CR_ERR_INVALID_ARG;
   int smem_ok = 0;
   for (int i = 0; i < phase_form_count(true); ++i)
-    smem_ok |= phase_smem_bytes(ctx->S, phase_form(i, true), true) <= (size_t)ctx->smem_max;
+    smem_ok |= phase_smem_bytes(ctx->S_da, phase_form(i, true), true) <= (size_t)ctx->smem_max;
   if (!smem_ok) return CR_ERR_INVALID_ARG;
   // the BF16 weights in blocks of eight inputs of one output (mlp_layer), and the biases
   std::vector<uint16_t> w(MLPW_N);
@@ -1739,7 +1757,10 @@ extern "C" int cr_set_launch_shape(cr_ctx *ctx, int32_t threads, int32_t regs) {
     return CR_OK;
   }
   PhaseForm F, Fd;
-  const bool plain = phase_form_named(threads, regs, false, &F), da = phase_form_named(threads, regs, true, &Fd);
+  const bool plain =
+      phase_form_named(threads, regs, false, &F) && phase_smem_bytes(ctx->S, F, false) <= (size_t)ctx->smem_max;
+  const bool da =
+      phase_form_named(threads, regs, true, &Fd) && phase_smem_bytes(ctx->S_da, Fd, true) <= (size_t)ctx->smem_max;
   if (plain) {
     ctx->F = F;
     ctx->regs = regs;
@@ -1792,7 +1813,7 @@ struct cr_batch {
   int64_t g_kernels = 0;                      // kernels per graph launch
   std::vector<std::pair<int, int>> g_pairs;  // phase-kernel event pairs recorded by the graph (timing)
   SysParams *d_reps = nullptr;  // one entry per replica (key_xor = replica index)
-  PhaseShape S{};
+  PhaseShape S{}, S_da{};
   int grid_x = 0, ncol = 8;
   PhaseForm F{128, 1, 1, 16, 0};
   int regs = 0;
@@ -1947,6 +1968,7 @@ extern "C" int cr_batch_create(cr_batch **out, cr_ctx *const *ctxs, int32_t n) {
   }
   if (phase_smem_bytes(b->S, largest, false) > (size_t)smem_max) { delete b; return CR_ERR_INVALID_ARG; }
   b->smem_max = smem_max;
+  b->S_da = da_shape(b->S, (size_t)smem_max);
   cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, ctxs[0]->device);
   if (cudaMalloc((void **)&b->d_reps, sizeof(SysParams) * n) != cudaSuccess) { delete b; return CR_ERR_NOMEM; }
   if (cudaMemcpy(b->d_reps, reps.data(), sizeof(SysParams) * n, cudaMemcpyHostToDevice) != cudaSuccess) {
@@ -2046,7 +2068,7 @@ static int batch_launch_persistent(cr_batch *b, const PhaseForm &F, bool da, uin
   int ti;
   tbegin(c0, 0, &ti);
   const int sms = b->sms > 0 ? b->sms : 1;
-  CR_CUDA(launch_sweep(b->d_reps, b->S, F, da, s, swc, sweep0, k0, k1, Q, b->ctas_per_sm * sms, dyn));
+  CR_CUDA(launch_sweep(b->d_reps, da ? b->S_da : b->S, F, da, s, swc, sweep0, k0, k1, Q, b->ctas_per_sm * sms, dyn));
   tend(c0, 0, ti);
   c0->launches_total++;
   return CR_OK;
@@ -2084,6 +2106,7 @@ static int batch_sweep_impl(cr_batch *b, uint64_t n_sweeps, uint64_t seed, bool 
   if (b->pmode < 0) tr.pers = &pers_choice;
   else pers_choice = b->pmode != 0;
   const int nform = phase_form_count(da);
+  const PhaseShape &S = da ? b->S_da : b->S;
   for (uint64_t sw = 0; sw < n_sweeps; ++sw) {
     const uint32_t swc = (uint32_t)c0->sweep;
     for (cr_ctx *c : b->ctx) {
@@ -2091,7 +2114,7 @@ static int batch_sweep_impl(cr_batch *b, uint64_t n_sweeps, uint64_t seed, bool 
       c->f_valid = false;
       c->fcons_valid = false;
     }
-    tune_skip(tr, b->S, b->smem_max, da);
+    tune_skip(tr, S, b->smem_max, da);
     const bool tune = tr.on && tr.next < tune_total(tr, da);
     bool persistent = pers_choice;
     const int cand = tune ? tune_cand(tr, da) : 0;
@@ -2118,7 +2141,7 @@ static int batch_sweep_impl(cr_batch *b, uint64_t n_sweeps, uint64_t seed, bool 
       for (int col = 0; col < b->ncol; ++col) {
         int ti;
         tbegin(c0, 0, &ti);
-        CR_CUDA(launch_phase(b->d_reps, n, b->grid_x, b->S, F, false, da, s, swc, sweep0, col, k0, k1));
+        CR_CUDA(launch_phase(b->d_reps, n, b->grid_x, S, F, false, da, s, swc, sweep0, col, k0, k1));
         tend(c0, 0, ti);
         c0->launches_total++;
       }
@@ -2130,7 +2153,7 @@ static int batch_sweep_impl(cr_batch *b, uint64_t n_sweeps, uint64_t seed, bool 
       cudaEventElapsedTime(&ms, e0, e1);
       cudaEventDestroy(e0);
       cudaEventDestroy(e1);
-      tune_finish(tr, ms, b->S, b->smem_max, da);
+      tune_finish(tr, ms, S, b->smem_max, da);
     }
   }
   return CR_OK;
@@ -2395,7 +2418,8 @@ static int batch_capture_cycle(cr_batch *b, double dt, double gamma, bool da, bo
         for (int col = 0; col < b->ncol && rc == CR_OK; ++col) {
           int ti;
           tbegin(c0, 0, &ti);
-          if (launch_phase(b->d_reps, n, b->grid_x, b->S, F, false, da, s, 0, 0, col, 0, 0, dyn) != cudaSuccess)
+          if (launch_phase(b->d_reps, n, b->grid_x, da ? b->S_da : b->S, F, false, da, s, 0, 0, col, 0, 0, dyn) !=
+              cudaSuccess)
             rc = CR_ERR_CUDA;
           tend(c0, 0, ti);
           c0->launches_total++;
@@ -2710,7 +2734,7 @@ extern "C" int cr_batch_set_launch_shape(cr_batch *b, int32_t threads, int32_t r
   const bool plain =
       phase_form_named(threads, regs, false, &F) && phase_smem_bytes(b->S, F, false) <= (size_t)b->smem_max;
   const bool da =
-      phase_form_named(threads, regs, true, &Fd) && phase_smem_bytes(b->S, Fd, true) <= (size_t)b->smem_max;
+      phase_form_named(threads, regs, true, &Fd) && phase_smem_bytes(b->S_da, Fd, true) <= (size_t)b->smem_max;
   if (plain) {
     b->F = F;
     b->regs = regs;

@@ -5,7 +5,8 @@
   * a trial's energy has the same bits wherever the domain's list and halo lie
     (shared or global memory), and logged sweeps give the unlogged chain;
   * the Ewald sums keep the bits they had before the reciprocal vectors went by
-    columns, and one box's slices give what a batch's items give.
+    columns, and one box's slices give what a batch's items give;
+  * a surrogate runs beside lists that take all of an SM's shared memory.
 """
 import zlib
 
@@ -119,3 +120,38 @@ def test_many_ewald_boxes_equal_single_ones(crmc):
             assert np.array_equal(x[key], y[key]), (r, key)
         g.close()
     b.close()
+
+
+@pytest.mark.parametrize("threads", [0, 128, 512])
+def test_surrogates_run_beside_lists_as_large_as_an_sm(crmc, threads):
+    """Every form of a delayed-acceptance sweep fits, logged or not, fixed or tuned, in contexts and in batches (by
+    colour and persistent), and gives the chain of small lists."""
+    w = W.config2(seed=9, scale=0.5)
+    mlp = W.random_mlp(seed=4, gain=0.7, out_gain=0.3)
+
+    def make(**kw):
+        g = crmc.Context(w, cell_capacity=512, **kw)
+        g.set_surrogate(mlp)
+        if threads:
+            g.set_launch_shape(threads, 0)
+        return g
+
+    large = dict(list_capacity=3091, halo_capacity=64)  # (what 512 threads without a surrogate leave)
+    a, ref = make(**large), make()
+    n = a.trials_per_sweep * 2
+    r = [g.sweep_da(n, 5, log=True)["log"] for g in (a, ref)]
+    assert r[0].tobytes() == r[1].tobytes()
+    for g in (a, ref):
+        g.sweep_da(n * 6, 6)
+    for mode in (0, 1):
+        b = crmc.Batch([make(**large)])
+        b.set_persistent(mode)
+        if threads:
+            b.set_launch_shape(threads, 0)
+        b.sweep_da(2, 5)
+        b.sweep_da(12, 6)
+        for c in b.contexts + [a]:
+            x, y = c.state(), ref.state()
+            for key in ("id", "xyz", "vel", "state"):
+                assert np.array_equal(x[key], y[key]), key
+        b.close()
