@@ -187,7 +187,7 @@ struct PhaseForm {
 
 // where a domain's arrays lie in shared memory, and their capacities
 struct PhaseLayout {
-  static constexpr int N_OFF = 33;
+  static constexpr int N_OFF = 32;
   unsigned off[N_OFF];
   int dcs, hcs, lns, chunk, ewk;
 };

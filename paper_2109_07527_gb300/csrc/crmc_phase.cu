@@ -131,8 +131,9 @@ __device__ __forceinline__ int region_coord(int i, int org, int k, int h, int nr
 __device__ __forceinline__ int div_by(int i, float r) { return (int)(((float)i + 0.5f) * r); }
 
 // Exclusive scan of n ints (shared memory) into pre[0..n] by one warp, each
-// lane a run of consecutive entries
-__device__ __forceinline__ void warp_scan(const int *vals, int n, int *pre) {
+// lane a run of consecutive entries.  SWAP: what pre held goes into vals.
+template <bool SWAP>
+__device__ __forceinline__ void warp_scan(int *vals, int n, int *pre) {
   const int lane = threadIdx.x & 31;
   const int per = (n + 31) >> 5;
   const int lo = min(n, lane * per), hi = min(n, lo + per);
@@ -146,8 +147,10 @@ __device__ __forceinline__ void warp_scan(const int *vals, int n, int *pre) {
   }
   int run = x - s;
   for (int i = lo; i < hi; ++i) {
+    const int v = vals[i];
+    if (SWAP) vals[i] = pre[i];
     pre[i] = run;
-    run += vals[i];
+    run += v;
   }
   if (lane == 31) pre[n] = x;
 }
@@ -1293,8 +1296,7 @@ static size_t phase_layout(const PhaseCaps &C, const PhaseShape &S, int warps, i
       sizeof(int) * nr3,                      // halo cells: counts, cells, prefix sums
       sizeof(int) * nr3,
       sizeof(int) * nr3,
-      sizeof(int) * kc3,                      // domain cells: counts, cells, prefix sums
-      sizeof(int) * kc3,
+      sizeof(int) * kc3,                      // domain cells: counts, then the cells; prefix sums
       sizeof(int) * kc3,
       sizeof(float2) * 6 * S.ewk,             // Ewald: axis factors, charge changes
       sizeof(float) * 4,
@@ -1308,7 +1310,7 @@ static size_t phase_layout(const PhaseCaps &C, const PhaseShape &S, int warps, i
   size_t at = 0;
   for (int pass = 0; pass < 2; ++pass)  // first the arrays whose place is the same in both of a launch's layouts
     for (int i = 0; i < PhaseLayout::N_OFF; ++i) {
-      const bool sized = (i >= 2 && i <= 9) || (i >= 16 && i <= 23 && i != 17);
+      const bool sized = (i >= 2 && i <= 9) || (i >= 16 && i <= 22 && i != 17);
       if (sized != (pass == 1)) continue;
       Y.off[i] = (unsigned)at;
       at += (bytes[i] + 15) / 16 * 16;
@@ -1353,19 +1355,19 @@ __device__ __forceinline__ void phase_task(unsigned char *smem, const PhaseArgs 
   int *redov = (int *)CRMC_AT(15);
   int *misc = (int *)CRMC_AT(17);  // [0] list size, [1 + kind] counts, [MISC_INIT + kind] at start, MISC_HW ...
   int *hcnt = (int *)CRMC_SIZED(18), *hcell = (int *)CRMC_SIZED(19), *hpre = (int *)CRMC_SIZED(20);
-  int *dcnt = (int *)CRMC_SIZED(21), *dcell = (int *)CRMC_SIZED(22), *dpre = (int *)CRMC_SIZED(23);
-  float2 *ewf = (float2 *)CRMC_AT(24);
-  float *ewq = (float *)CRMC_AT(25);
+  int *dcnt = (int *)CRMC_SIZED(21), *dpre = (int *)CRMC_SIZED(22);
+  float2 *ewf = (float2 *)CRMC_AT(23);
+  float *ewq = (float *)CRMC_AT(24);
   int *aQi = nullptr, *aQs = nullptr, *aN = nullptr, *dfeat = nullptr;
   float *fv = nullptr, *hb0 = nullptr, *hb1 = nullptr;
   if (DA) {
-    aQi = (int *)CRMC_AT(26);
-    aQs = (int *)CRMC_AT(27);
-    aN = (int *)CRMC_AT(28);
-    dfeat = (int *)CRMC_AT(29) + group * MLP_IN;
-    fv = (float *)CRMC_AT(30) + group * 2 * MLP_IN;
-    hb0 = (float *)CRMC_AT(31) + group * 2 * MLP_H;
-    hb1 = (float *)CRMC_AT(32) + group * 2 * MLP_H;
+    aQi = (int *)CRMC_AT(25);
+    aQs = (int *)CRMC_AT(26);
+    aN = (int *)CRMC_AT(27);
+    dfeat = (int *)CRMC_AT(28) + group * MLP_IN;
+    fv = (float *)CRMC_AT(29) + group * 2 * MLP_IN;
+    hb0 = (float *)CRMC_AT(30) + group * 2 * MLP_H;
+    hb1 = (float *)CRMC_AT(31) + group * 2 * MLP_H;
   }
 
   {
@@ -1415,7 +1417,8 @@ __device__ __forceinline__ void phase_task(unsigned char *smem, const PhaseArgs 
 
   // ---- the region's cells and their counts (four cells per thread at a
   // time, so that their loads are in flight together): the domain's own by
-  // rank, the halo's by region index (zero at the domain's)
+  // rank (the cells where their prefix sums will be), the halo's by region
+  // index (zero at the domain's)
   const float rnr = 1.0f / (float)nr;
 #pragma unroll 1
   for (int i0 = tid; i0 < NR; i0 += 4 * T) {
@@ -1431,7 +1434,7 @@ __device__ __forceinline__ void phase_task(unsigned char *smem, const PhaseArgs 
       cn[u] = P.cnt[cl[u]];
       cl[u] |= r >= 0 ? 0x80000000 : 0;
       if (r >= 0 && i0 + u * T < NR) {
-        dcell[r] = cl[u] & 0x7fffffff;
+        dpre[r] = cl[u] & 0x7fffffff;
         hcell[i] = r;
       }
     }
@@ -1451,9 +1454,10 @@ __device__ __forceinline__ void phase_task(unsigned char *smem, const PhaseArgs 
     D.wr[16 + tid] = fmaxf(fmaxf(wca_radius(P.wca[4 * tid]), wca_radius(P.wca[4 * tid + 1])),
                            fmaxf(wca_radius(P.wca[4 * tid + 2]), wca_radius(P.wca[4 * tid + 3])));
   seat.sync();
-  if (warp == 0) warp_scan(dcnt, KC, dpre);
-  if (warp == (T > 32 ? 1 : 0)) warp_scan(hcnt, NR, hpre);
+  if (warp == 0) warp_scan<true>(dcnt, KC, dpre);
+  if (warp == (T > 32 ? 1 : 0)) warp_scan<false>(hcnt, NR, hpre);
   seat.sync();
+  int *dcell = dcnt;  // the domain's cells, from here on
   const int ND = dpre[KC], NH = hpre[NR];
   const int nhc = min(NH, A.lay[SEATS ? which : 0].hcs);
   // the list lives in shared memory unless the domain is unusually dense
@@ -1510,7 +1514,7 @@ __device__ __forceinline__ void phase_task(unsigned char *smem, const PhaseArgs 
     for (int q = 0; q < n; ++q) *(int *)&cpos[j0 + q] = g + q;
   }
   for (int r = tid; r < KC; r += T) {
-    const int j0 = dpre[r], n = dcnt[r], g = dcell[r] * P.cap;
+    const int j0 = dpre[r], n = dpre[r + 1] - j0, g = dcell[r] * P.cap;
     for (int q = 0; q < n; ++q) L.ord[j0 + q] = make_uint2((unsigned)(g + q), (unsigned)r);
   }
   if (ln_in_smem)
@@ -1838,14 +1842,15 @@ __device__ __forceinline__ void phase_task(unsigned char *smem, const PhaseArgs 
       while (lo < hi) { const int mid = (lo + hi) >> 1; if ((int)L.ord[mid].y < r) lo = mid + 1; else hi = mid; }
       int lo2 = lo, hi2 = n;  // first entry with rank > r
       while (lo2 < hi2) { const int mid = (lo2 + hi2) >> 1; if ((int)L.ord[mid].y <= r) lo2 = mid + 1; else hi2 = mid; }
-      dcnt[r] = lo;
-      P.cnt[dcell[r]] = lo2 - lo;
+      const int cell = dcell[r];
+      dcell[r] = cell * P.cap - lo;  // from a place in the list to the slot
+      P.cnt[cell] = lo2 - lo;
     }
     seat.sync();
     for (int j = tid; j < n; j += T) {
       const uint2 o = L.ord[j];
       const int sl = (int)(o.x & ORD_SLOT_MASK);
-      const int g = dcell[o.y] * P.cap + (j - dcnt[o.y]);
+      const int g = dcell[o.y] + j;
       const unsigned long long id = L.id[sl];
       P.pos[g] = raw_pos(L, sl, P.Lf);
       P.vel[g] = L.vel[sl];

@@ -6,7 +6,8 @@
     (shared or global memory), and logged sweeps give the unlogged chain;
   * the Ewald sums keep the bits they had before the reciprocal vectors went by
     columns, and one box's slices give what a batch's items give;
-  * a surrogate runs beside lists that take all of an SM's shared memory.
+  * a surrogate runs beside lists that take all of an SM's shared memory;
+  * domains of as many cells as ever fitted are accepted.
 """
 import zlib
 
@@ -14,6 +15,7 @@ import numpy as np
 import pytest
 
 from paper_2109_07527_gb300 import workloads as W
+from parity_util import compare_logs, compare_states
 from test_gpu_forms import _electrolyte, _ions
 
 pytestmark = pytest.mark.gpu
@@ -155,3 +157,15 @@ def test_surrogates_run_beside_lists_as_large_as_an_sm(crmc, threads):
             for key in ("id", "xyz", "vel", "state"):
                 assert np.array_equal(x[key], y[key]), key
         b.close()
+
+
+@pytest.mark.parametrize("cells,per_rc,L,rc", [(19, 2, 57.2, 3.0), (20, 1, 80.5, 2.0)])
+def test_domains_of_many_cells(crmc, cells, per_rc, L, rc):
+    """The cell tables of 6,859 and 8,000 cells and their halos take nine tenths of an SM's shared memory."""
+    w = _ions(400, L, rc, 6, cells_per_rc=per_rc)
+    g = crmc.Context(w, domain_cells=cells)
+    assert g.info["nc"] == 2 * cells
+    n = g.trials_per_sweep * 6
+    o, lo, ties = compare_logs(w, g.sweep(n, 8, log=True)["log"], n, 8, dict(domain_cells=cells))
+    compare_states(g, o, w.n_sites)
+    g.close()
