@@ -1845,12 +1845,11 @@ struct cr_batch {
   int8_t *d_pk_state = nullptr;
   bool holds_refs = false;  // the contexts' batch_refs count this batch
   int ewald_items = 0, ewald_plus = 0;  // largest numbers of Ewald items and nz >= 0 places over the replicas
-  // batched MD steps: per-replica parameters on the device (for md_dt, md_gamma) and the
-  // lengths of the replicas' particle lists
+  // batched MD steps: per-replica parameters on the device and the lengths of
+  // the replicas' particle lists
   MdJob *d_md = nullptr;
   int *d_nparts = nullptr;
   MdBatchShape md_shape{};
-  double md_dt = 0.0, md_gamma = 0.0;
 };
 
 // The device address of caller memory the GPU can access directly (device
@@ -2000,6 +1999,26 @@ extern "C" int cr_batch_create(cr_batch **out, cr_ctx *const *ctxs, int32_t n) {
     if (cudaMalloc((void **)&b->d_rep_first, sizeof(int) * 2 * (n + 1)) != cudaSuccess ||
         cudaMalloc((void **)&b->d_words, sizeof(unsigned) * b->words) != cudaSuccess ||
         cudaMemcpy(b->d_rep_first, first.data(), sizeof(int) * 2 * (n + 1), cudaMemcpyHostToDevice) != cudaSuccess) {
+      cr_batch_destroy(b);
+      return CR_ERR_NOMEM;
+    }
+  }
+  {  // batched MD steps (a context's arrays stay where they are while it is in a batch)
+    std::vector<MdJob> jobs(n);
+    bool ok = cudaMalloc((void **)&b->d_nparts, sizeof(int) * n) == cudaSuccess &&
+              cudaMalloc((void **)&b->d_md, sizeof(MdJob) * n) == cudaSuccess;
+    for (int r = 0; r < n && ok; ++r) {
+      cr_ctx *c = ctxs[r];
+      md_batch_shape(c->P, (int)c->capacity, &b->md_shape);
+      MdParams &M = jobs[r].M;
+      M = md_params(c, 2, 0.0, 0.0, 0);
+      M.fsum = c->d_fsum;
+      M.plist = c->d_plist;
+      M.n_particles = b->d_nparts + r;
+      M.max_particles = (int)c->capacity;
+      jobs[r].B = RebuildBufs{c->d_cnt2, c->d_pos2, c->d_pid2, c->d_info2, c->d_vel2, c->d_frc2, c->d_vel, c->d_frc};
+    }
+    if (!ok || cudaMemcpy(b->d_md, jobs.data(), sizeof(MdJob) * n, cudaMemcpyHostToDevice) != cudaSuccess) {
       cr_batch_destroy(b);
       return CR_ERR_NOMEM;
     }
@@ -2238,44 +2257,18 @@ static bool batch_md_together(const cr_batch *b) {
   return b->ctx.size() <= 65535;  // (the grid's last dimension)
 }
 
-// the replicas' MD parameters for this step and friction, on the device
-static int batch_md_jobs(cr_batch *b, double dt, double gamma) {
-  cudaStream_t s = b->ctx[0]->stream;
-  const size_t n = b->ctx.size();
-  if (b->md_dt == dt && b->md_gamma == gamma) return CR_OK;  // (dt > 0: 0 before the first)
-  if (!b->d_nparts) {  // first MD step of the batch
-    CR_CUDA(cudaMalloc((void **)&b->d_nparts, sizeof(int) * n));
-    for (const cr_ctx *c : b->ctx) md_batch_shape(c->P, (int)c->capacity, &b->md_shape);
-  }
-  if (!b->d_md) CR_CUDA(cudaMalloc((void **)&b->d_md, sizeof(MdJob) * n));
-  std::vector<MdJob> jobs(n);
-  for (size_t r = 0; r < n; ++r) {
-    cr_ctx *c = b->ctx[r];
-    MdParams &M = jobs[r].M;
-    M = md_params(c, 2, dt, gamma, 0);
-    M.fsum = c->d_fsum;
-    M.plist = c->d_plist;
-    M.n_particles = b->d_nparts + r;
-    M.max_particles = (int)c->capacity;
-    jobs[r].B = RebuildBufs{c->d_cnt2, c->d_pos2, c->d_pid2, c->d_info2, c->d_vel2, c->d_frc2, c->d_vel, c->d_frc};
-  }
-  // (a pageable source: staged before the call returns)
-  CR_CUDA(cudaMemcpyAsync(b->d_md, jobs.data(), sizeof(MdJob) * n, cudaMemcpyHostToDevice, s));
-  b->md_dt = dt;
-  b->md_gamma = gamma;
-  return CR_OK;
-}
-
 // one force evaluation of every replica (mode, seed and counters as in
 // md_force_eval; with dyn they come from the captured step's parameters)
-static int batch_md_forces(cr_batch *b, int mode, uint64_t seed, const StepDyn *dyn = nullptr, int eval_off = 0) {
+static int batch_md_forces(cr_batch *b, int mode, double dt, double gamma, uint64_t seed, const StepDyn *dyn = nullptr,
+                           int eval_off = 0) {
   cr_ctx *c0 = b->ctx[0];
   const int n = (int)b->ctx.size();
   if (b->ewald_items > 0) {
     CR_CUDA(launch_ewald_sk(b->d_reps, n, b->ewald_items, b->ewald_plus, c0->stream));
     c0->launches_total += 3;  // occupied slots, S(k), reciprocal forces
   }
-  const MdCall Q{(uint32_t)seed, (uint32_t)(seed >> 32), c0->md_eval, mode, dyn, eval_off};
+  const MdParams M = md_params(c0, mode, dt, gamma, seed);
+  const MdCall Q{M.dt, M.gamma, M.amp, M.key0, M.key1, M.eval, mode, dyn, eval_off};
   CR_CUDA(launch_md_forces_batch(b->d_reps, b->d_md, n, b->md_shape, b->d_nparts, Q, c0->stream));
   c0->launches_total += 2 + __builtin_popcount((unsigned)b->md_shape.variants);  // list, finish, pair forces
   for (cr_ctx *c : b->ctx) {
@@ -2287,13 +2280,14 @@ static int batch_md_forces(cr_batch *b, int mode, uint64_t seed, const StepDyn *
 }
 
 // half kick, drift and cell rebuild of every replica, after the forces if they are stale
-static int batch_md_drift(cr_batch *b, uint64_t seed) {
+static int batch_md_drift(cr_batch *b, double dt, double gamma, uint64_t seed) {
   cr_ctx *c0 = b->ctx[0];
   if (!c0->f_valid) {
-    const int rc = batch_md_forces(b, 1, seed);
+    const int rc = batch_md_forces(b, 1, dt, gamma, seed);
     if (rc != CR_OK) return rc;
   }
-  CR_CUDA(launch_kick_drift_rebuild_batch(b->d_reps, b->d_md, (int)b->ctx.size(), b->md_shape.cells, c0->stream));
+  CR_CUDA(launch_kick_drift_rebuild_batch(b->d_reps, b->d_md, (int)b->ctx.size(), b->md_shape.cells, (float)dt,
+                                          c0->stream));
   c0->launches_total += 2;
   for (cr_ctx *c : b->ctx) {
     c->stream = c0->stream;
@@ -2305,28 +2299,21 @@ static int batch_md_drift(cr_batch *b, uint64_t seed) {
 
 extern "C" int cr_batch_md_step(cr_batch *b, int32_t n_steps, double dt, double gamma, uint64_t seed) {
   if (b && n_steps > 0 && dt > 0.0 && gamma >= 0.0 && batch_md_together(b)) {
-    int rc = batch_md_jobs(b, dt, gamma);
-    for (int st = 0; st < n_steps && rc == CR_OK; ++st) {
-      if ((rc = batch_md_drift(b, seed)) == CR_OK) rc = batch_md_forces(b, 2, seed);
-    }
+    int rc = CR_OK;
+    for (int st = 0; st < n_steps && rc == CR_OK; ++st)
+      if ((rc = batch_md_drift(b, dt, gamma, seed)) == CR_OK) rc = batch_md_forces(b, 2, dt, gamma, seed);
     return rc;
   }
   return batch_md(b, [&](cr_ctx *c, uint64_t r) { return cr_md_step(c, n_steps, dt, gamma, seed ^ (r << 32)); });
 }
 
 extern "C" int cr_batch_md_begin(cr_batch *b, double dt, double gamma, uint64_t seed) {
-  if (b && dt > 0.0 && gamma >= 0.0 && batch_md_together(b)) {
-    const int rc = batch_md_jobs(b, dt, gamma);
-    return rc != CR_OK ? rc : batch_md_drift(b, seed);
-  }
+  if (b && dt > 0.0 && gamma >= 0.0 && batch_md_together(b)) return batch_md_drift(b, dt, gamma, seed);
   return batch_md(b, [&](cr_ctx *c, uint64_t r) { return cr_md_begin(c, dt, gamma, seed ^ (r << 32)); });
 }
 
 extern "C" int cr_batch_md_end(cr_batch *b, double dt, double gamma, uint64_t seed) {
-  if (b && dt > 0.0 && gamma >= 0.0 && batch_md_together(b)) {
-    const int rc = batch_md_jobs(b, dt, gamma);
-    return rc != CR_OK ? rc : batch_md_forces(b, 2, seed);
-  }
+  if (b && dt > 0.0 && gamma >= 0.0 && batch_md_together(b)) return batch_md_forces(b, 2, dt, gamma, seed);
   return batch_md(b, [&](cr_ctx *c, uint64_t r) { return cr_md_end(c, dt, gamma, seed ^ (r << 32)); });
 }
 
@@ -2405,8 +2392,8 @@ static int batch_capture_cycle(cr_batch *b, double dt, double gamma, bool da, bo
     return CR_ERR_CUDA;
   }
   {
-    if (ff) rc = batch_md_forces(b, 1, 0, dyn);
-    if (rc == CR_OK) rc = batch_md_drift(b, 0);  // (the forces are valid)
+    if (ff) rc = batch_md_forces(b, 1, dt, gamma, 0, dyn);
+    if (rc == CR_OK) rc = batch_md_drift(b, dt, gamma, 0);  // (the forces are valid)
     if (rc == CR_OK && b->order_nc > 0) {
       if (launch_domain_order(b->d_reps, n, b->ncol, b->order_nact, s, 0, 0, 0, dyn) != cudaSuccess) rc = CR_ERR_CUDA;
       c0->launches_total += 2;
@@ -2426,7 +2413,7 @@ static int batch_capture_cycle(cr_batch *b, double dt, double gamma, bool da, bo
         }
       }
     }
-    if (rc == CR_OK) rc = batch_md_forces(b, 2, 0, dyn, ff ? 1 : 0);
+    if (rc == CR_OK) rc = batch_md_forces(b, 2, dt, gamma, 0, dyn, ff ? 1 : 0);
     if (rc == CR_OK && launch_step_advance(b->d_dyn, s) != cudaSuccess) rc = CR_ERR_CUDA;
     c0->launches_total++;
   }
@@ -2509,7 +2496,6 @@ extern "C" int cr_batch_cycle(cr_batch *b, int32_t n_steps, double dt, double ga
       CR_CUDA(cudaMemcpyAsync(b->d_reps, b->reps.data(), sizeof(SysParams) * b->ctx.size(), cudaMemcpyHostToDevice, s));
   }
   if (!b->d_dyn) CR_CUDA(cudaMalloc((void **)&b->d_dyn, sizeof(StepDyn)));
-  if ((rc = batch_md_jobs(b, dt, gamma)) != CR_OK) return rc;
   const PhaseForm F = da ? b->da_F : b->F;
   const bool pers = da ? b->da_persistent : b->persistent;
   while (step < n_steps) {

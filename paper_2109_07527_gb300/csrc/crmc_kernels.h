@@ -106,14 +106,17 @@ struct LoadBufs {
   const float *frc;              // [3n] integrator forces (a restore), or null: zero
 };
 
-// one replica's MD step in a batched launch, and what changes from call to
-// call: the seed's words (the replica's index goes into the high one), the
-// evaluation counter, the mode, or dyn for a captured cycle
+// one replica's MD step in a batched launch (the same for the batch's life),
+// and what changes from call to call, given by value so that a launch can stand
+// in a caller's stream capture: the step and friction, the seed's words (the
+// replica's index goes into the high one), the evaluation counter, the mode, or
+// dyn for a captured cycle
 struct MdJob {
   MdParams M;
   RebuildBufs B;
 };
 struct MdCall {
+  float dt, gamma, amp;
   uint32_t key0, key1, eval;
   int mode;
   const StepDyn *dyn;
@@ -180,7 +183,7 @@ void md_batch_shape(const SysParams &P, int max_particles, MdBatchShape *S);
 cudaError_t launch_md_forces_batch(const SysParams *d_reps, const MdJob *d_jobs, int n_rep, const MdBatchShape &S,
                                    int *n_particles, const MdCall &C, cudaStream_t s);
 cudaError_t launch_kick_drift_rebuild_batch(const SysParams *d_reps, const MdJob *d_jobs, int n_rep, int max_cells,
-                                            cudaStream_t s);
+                                            float dt, cudaStream_t s);
 cudaError_t launch_load(const SysParams &P, const LoadBufs &I, const RebuildBufs &B, int *perm_slot, int n_perm,
                         cudaStream_t s);
 // loads of every replica of a batch (counts zeroed, scatter, cell sort,

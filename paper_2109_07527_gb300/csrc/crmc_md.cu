@@ -403,6 +403,9 @@ __global__ void __launch_bounds__(256) k_md_finish_batch(const SysParams *__rest
   const MdParams &J = jobs[blockIdx.y].M;
   if (w >= *J.n_particles || w >= J.max_particles) return;
   MdParams M = J;
+  M.dt = C.dt;
+  M.gamma = C.gamma;
+  M.amp = C.amp;
   M.mode = C.mode;
   M.key0 = C.key0;
   M.key1 = C.key1 ^ blockIdx.y;
@@ -450,7 +453,8 @@ __device__ __forceinline__ void for_cell_particles(int n, F f) {
 
 // v += dt/2 f; x += dt v; wrap into [0, L); the particle goes straight into
 // its new cell of the scratch arrays (unordered; the rebuild orders them)
-__device__ __forceinline__ void kick_drift_scatter(const SysParams &P, const MdParams &M, const RebuildBufs &B, int g) {
+__device__ __forceinline__ void kick_drift_scatter(const SysParams &P, const MdParams &M, float dt, const RebuildBufs &B,
+                                                   int g) {
   float4 v = M.vel[g];
   const float4 f = M.fout[g];
   const float4 p = P.pos[g];
@@ -464,12 +468,12 @@ __device__ __forceinline__ void kick_drift_scatter(const SysParams &P, const MdP
     x[1] = q.y;
     x[2] = q.z;
   } else {
-    v.x += 0.5f * M.dt * f.x;
-    v.y += 0.5f * M.dt * f.y;
-    v.z += 0.5f * M.dt * f.z;
-    x[0] = p.x + M.dt * v.x;
-    x[1] = p.y + M.dt * v.y;
-    x[2] = p.z + M.dt * v.z;
+    v.x += 0.5f * dt * f.x;
+    v.y += 0.5f * dt * f.y;
+    v.z += 0.5f * dt * f.z;
+    x[0] = p.x + dt * v.x;
+    x[1] = p.y + dt * v.y;
+    x[2] = p.z + dt * v.z;
     for (int i = 0; i < 3; ++i) {
       x[i] -= P.Lf * floorf(x[i] * P.invL);
       if (x[i] >= P.Lf) x[i] -= P.Lf;
@@ -491,17 +495,17 @@ __device__ __forceinline__ void kick_drift_scatter(const SysParams &P, const MdP
   B.frc[o] = f;
 }
 
-__device__ __forceinline__ void kick_drift_cells(const SysParams &P, const MdParams &M, const RebuildBufs &B) {
+__device__ __forceinline__ void kick_drift_cells(const SysParams &P, const MdParams &M, float dt, const RebuildBufs &B) {
   const int c = blockIdx.x * CELL_GROUP + (threadIdx.x & 31);
   for_cell_particles(c < P.ncell ? P.cnt[c] : 0,
-                     [&](int cell, int s, int) { kick_drift_scatter(P, M, B, cell * P.cap + s); });
+                     [&](int cell, int s, int) { kick_drift_scatter(P, M, dt, B, cell * P.cap + s); });
 }
 __global__ void __launch_bounds__(CELL_THREADS) k_md_kick_drift_scatter(SysParams P, MdParams M, RebuildBufs B) {
-  kick_drift_cells(P, M, B);
+  kick_drift_cells(P, M, M.dt, B);
 }
 __global__ void __launch_bounds__(CELL_THREADS) k_md_kick_drift_scatter_batch(const SysParams *__restrict__ reps,
-                                                                              const MdJob *__restrict__ jobs) {
-  kick_drift_cells(reps[blockIdx.y], jobs[blockIdx.y].M, jobs[blockIdx.y].B);
+                                                                              const MdJob *__restrict__ jobs, float dt) {
+  kick_drift_cells(reps[blockIdx.y], jobs[blockIdx.y].M, dt, jobs[blockIdx.y].B);
 }
 
 // rebuild: the particles of 32 cells sorted by id within each cell into the
@@ -1185,10 +1189,10 @@ cudaError_t launch_kick_drift_rebuild(const SysParams &P, const MdParams &M, con
 }
 
 cudaError_t launch_kick_drift_rebuild_batch(const SysParams *d_reps, const MdJob *d_jobs, int n_rep, int max_cells,
-                                            cudaStream_t s) {
+                                            float dt, cudaStream_t s) {
   const dim3 grid(cell_groups(max_cells), (unsigned)n_rep);
   const unsigned threads = cell_threads(grid.x * grid.y);
-  k_md_kick_drift_scatter_batch<<<grid, threads, 0, s>>>(d_reps, d_jobs);
+  k_md_kick_drift_scatter_batch<<<grid, threads, 0, s>>>(d_reps, d_jobs, dt);
   k_md_rebuild_sort_batch<<<grid, threads, 0, s>>>(d_reps, d_jobs);
   return cudaGetLastError();
 }
