@@ -2272,6 +2272,7 @@ static int batch_md_forces(cr_batch *b, int mode, double dt, double gamma, uint6
   CR_CUDA(launch_md_forces_batch(b->d_reps, b->d_md, n, b->md_shape, b->d_nparts, Q, c0->stream));
   c0->launches_total += 2 + __builtin_popcount((unsigned)b->md_shape.variants);  // list, finish, pair forces
   for (cr_ctx *c : b->ctx) {
+    c->stream = c0->stream;  // what follows on a replica of its own follows the launch
     c->md_eval++;
     c->f_valid = true;
     c->fcons_valid = false;

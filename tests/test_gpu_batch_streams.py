@@ -1,4 +1,5 @@
-"""Batched MD steps on the caller's streams: the calls can stand in a caller's own
+"""Batched MD steps on the caller's streams: work on one replica follows a batch
+call on the stream that the call used, and the calls can stand in a caller's own
 stream capture, with the step and friction that they were given."""
 import ctypes as C
 
@@ -29,6 +30,27 @@ def _same(a, c):
         sx, sy = x.state(), y.state()
         for k in KEYS:
             assert np.array_equal(sx[k], sy[k]), k
+
+
+def test_a_replica_follows_the_stream_of_the_last_batch_call(crmc):
+    """The first replica's stream changes between the two halves of a step; the second's velocities are read while
+    the closing half waits on the new stream behind 50 ms of other work."""
+    first, second = torch.cuda.Stream(), torch.cuda.Stream()
+    a, ref = _batch(crmc, first), _batch(crmc)
+    for b in (a, ref):
+        b.md_step(1, 0.005, 1.0, 3)
+        b.md_begin(0.005, 1.0, 4)
+    torch.cuda.synchronize()
+    crmc._lib().cr_set_stream(a.contexts[0]._h, C.c_void_p(second.cuda_stream))
+    with torch.cuda.stream(second):
+        torch.cuda._sleep(100_000_000)
+    a.md_end(0.005, 1.0, 4)
+    ref.md_end(0.005, 1.0, 4)
+    x, y = a.contexts[1].state(), ref.contexts[1].state()
+    for k in KEYS:
+        assert np.array_equal(x[k], y[k]), k
+    a.close()
+    ref.close()
 
 
 @pytest.mark.parametrize("warm", [False, True])
