@@ -19,6 +19,7 @@
 #include "crmc.h"
 #include "crmc_common.h"
 #include "crmc_kernels.h"
+#include "crmc_tune.h"
 
 using namespace crmc;
 
@@ -32,9 +33,7 @@ struct cr_ctx {
   PhaseForm F{128, 1, 1, 16, 0};
   int regs = 0;
   int smem_max = 0;
-  int tune_next = 0;     // sweeps timed so far
-  bool tuning = true;
-  float tune_ms[16] = {};
+  FormTuner tune;
   PhaseShape S{}, S_da{};  // shared-memory capacities; those of delayed-acceptance sweeps
   SysParams *d_reps = nullptr;  // device copy of P (the phase kernel reads it)
   int64_t per_sweep = 0;
@@ -71,9 +70,7 @@ struct cr_ctx {
   float *d_feat = nullptr;
   size_t dlog_cap = 0, feat_cap = 0;
   PhaseForm da_F{128, 1, 1, 16, 0};
-  int da_next = 0;
-  bool da_tuning = true;
-  float da_ms[8] = {};
+  FormTuner da_tune;
   // cr_load inputs (capacity-sized)
   float *d_in_xyz = nullptr, *d_in_vel = nullptr;
   int *d_in_type = nullptr, *d_in_cls = nullptr, *d_site_map = nullptr;
@@ -641,8 +638,7 @@ extern "C" int cr_init(cr_ctx **out, const cr_system *sys, double pH, const doub
   }
   {
     // (128 threads per domain until the tuner has timed the forms)
-    c->tuning = std::getenv("CRMC_NO_TUNE") == nullptr;
-    c->da_tuning = c->tuning;
+    c->tune.on = c->da_tune.on = std::getenv("CRMC_NO_TUNE") == nullptr;
   }
   P.lnmax = std::max(2 * k * k * k * cap, (int)std::min<long long>((long long)sys->capacity, 1 << 20)) + 2 * P.m + 4;
   std::vector<long long> h_lntab(P.lnmax);
@@ -1066,59 +1062,25 @@ static int grow(TT **p, size_t *cap, size_t n) {
   return CR_OK;
 }
 
-// Online tuning of the launch form (shared by plain and delayed-acceptance
-// sweeps): the first sweeps of unlogged calls time each form that applies in
-// round-robin rounds, and the fastest of the last round is kept.  Earlier
-// rounds only let the state settle: a box that starts without its ions grows
-// for a dozen sweeps, and the shortest time over all rounds then favoured
-// whatever was tried first.  Two rounds; six under the global schedule, which
-// has a third of the forms.  For batches whose persistent mode is left to the
-// tuner (pers != null), the candidates are every form with one launch per
-// colour, then every form as a persistent sweep; *pers receives the chosen
-// mode.  next counts the candidates passed; candidate next % tune_count.
-struct TuneRef {
-  PhaseForm &F;
-  int &next;
-  bool &on;
-  float *ms;
-  bool global;             // one domain per replica: one seat, one group
-  bool *pers = nullptr;
-};
-
-static int tune_count(const TuneRef &t, bool da) { return phase_form_count(da) * (t.pers ? 2 : 1); }
-static int tune_total(const TuneRef &t, bool da) { return tune_count(t, da) * (t.global ? 6 : 2); }
-static int tune_cand(const TuneRef &t, bool da) { return t.next % tune_count(t, da); }
-
-// forms that do not apply are passed over: those that do not fit in shared
-// memory; several seats or groups under the global schedule (its one domain
-// takes the CTA, its trials are mostly accepted, and an Ewald trial uses the
-// whole CTA); seats in a persistent sweep (its tasks take whole CTAs)
-static void tune_skip(TuneRef t, const PhaseShape &S, int smem_max, bool da) {
+// Online tuning of the launch form (FormTuner; shared by plain and
+// delayed-acceptance sweeps): unlogged sweeps time the forms that apply.  For
+// batches whose persistent mode is left to the tuner, the candidates are every
+// form with one launch per colour, then every form as a persistent sweep.
+// Forms that do not apply: those that do not fit in shared memory; several
+// seats or groups under the global schedule (its one domain takes the CTA, its
+// trials are mostly accepted, and an Ewald trial uses the whole CTA); seats in
+// a persistent sweep (its tasks take whole CTAs).
+static void tune_begin(FormTuner &t, const PhaseShape &S, int smem_max, bool da, bool global, bool by_colour,
+                       bool persistent) {
+  std::vector<int> cand;
   const int nform = phase_form_count(da);
-  while (t.on && t.next < tune_total(t, da)) {
-    const int c = tune_cand(t, da);
+  for (int c = by_colour ? 0 : nform; c < (persistent ? 2 : 1) * nform; ++c) {
     const PhaseForm &F = phase_form(c % nform, da);
-    const bool whole = F.seats == 1, single = F.seats == 1 && F.groups == 1;
-    if (phase_smem_bytes(S, F, da) <= (size_t)smem_max && (!t.global || single) && (c < nform || whole)) break;
-    t.ms[c] = 1e30f;
-    t.next++;
+    const bool whole = F.seats == 1, single = whole && F.groups == 1;
+    if (phase_smem_bytes(S, F, da) <= (size_t)smem_max && (!global || single) && (c < nform || whole))
+      cand.push_back(c);
   }
-}
-
-static void tune_finish(TuneRef t, float ms, const PhaseShape &S, int smem_max, bool da) {
-  const int c = tune_cand(t, da);
-  t.ms[c] = ms;
-  t.next++;
-  tune_skip(t, S, smem_max, da);
-  const int nform = phase_form_count(da);
-  if (t.next == tune_total(t, da)) {
-    int best = 0;
-    for (int i = 1; i < tune_count(t, da); ++i)
-      if (t.ms[i] < t.ms[best]) best = i;
-    t.F = phase_form(best % nform, da);
-    if (t.pers) *t.pers = best >= nform;
-    t.on = false;
-  }
+  t.begin(cand, global);
 }
 
 static int sweep_impl(cr_ctx *ctx, uint64_t n_trials, uint64_t seed, cr_sweep_stats *stats, cr_trial *log,
@@ -1148,15 +1110,14 @@ static int sweep_impl(cr_ctx *ctx, uint64_t n_trials, uint64_t seed, cr_sweep_st
   if (log) CR_CUDA(cudaMemcpyAsync(ctx->d_reps, &P, sizeof(SysParams), cudaMemcpyHostToDevice, s));
   const uint64_t n_sweeps = n_trials / (uint64_t)ctx->per_sweep;
   const uint32_t sweep0 = (uint32_t)ctx->sweep;
-  const bool glob = P.global != 0;
   const PhaseShape &S = da ? ctx->S_da : ctx->S;
-  TuneRef tr = da ? TuneRef{ctx->da_F, ctx->da_next, ctx->da_tuning, ctx->da_ms, glob}
-                  : TuneRef{ctx->F, ctx->tune_next, ctx->tuning, ctx->tune_ms, glob};
+  PhaseForm &form = da ? ctx->da_F : ctx->F;
+  FormTuner &tuner = da ? ctx->da_tune : ctx->tune;
   for (uint64_t sw = 0; sw < n_sweeps; ++sw) {
     const uint32_t swc = (uint32_t)ctx->sweep++;
-    if (!log) tune_skip(tr, S, ctx->smem_max, da);
-    const bool tune = tr.on && !log && tr.next < tune_total(tr, da);
-    const PhaseForm F = tune ? phase_form(tune_cand(tr, da), da) : tr.F;
+    if (!log && tuner.on && !tuner.begun()) tune_begin(tuner, S, ctx->smem_max, da, P.global != 0, true, false);
+    const bool tune = tuner.on && !log;
+    const PhaseForm F = tune ? phase_form(tuner.current(), da) : form;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (tune) {
       cudaEventCreate(&e0);
@@ -1185,7 +1146,7 @@ static int sweep_impl(cr_ctx *ctx, uint64_t n_trials, uint64_t seed, cr_sweep_st
       cudaEventElapsedTime(&ms, e0, e1);
       cudaEventDestroy(e0);
       cudaEventDestroy(e1);
-      tune_finish(tr, ms, S, ctx->smem_max, da);
+      if (tuner.record(ms)) form = phase_form(tuner.current(), da);
     }
   }
   if (log) {
@@ -1749,11 +1710,9 @@ extern "C" int cr_get_timing(cr_ctx *ctx, double *ms, int64_t *launches, int64_t
 extern "C" int cr_set_launch_shape(cr_ctx *ctx, int32_t threads, int32_t regs) {
   if (!ctx) return CR_ERR_INVALID_ARG;
   if (threads == 0) {  // re-enable tuning
-    ctx->tuning = true;
-    ctx->tune_next = 0;
+    ctx->tune.restart();
+    ctx->da_tune.restart();
     ctx->regs = 0;
-    ctx->da_tuning = true;
-    ctx->da_next = 0;
     return CR_OK;
   }
   PhaseForm F, Fd;
@@ -1764,11 +1723,11 @@ extern "C" int cr_set_launch_shape(cr_ctx *ctx, int32_t threads, int32_t regs) {
   if (plain) {
     ctx->F = F;
     ctx->regs = regs;
-    ctx->tuning = false;
+    ctx->tune.on = false;
   }
   if (da) {  // delayed-acceptance sweeps, where supported
     ctx->da_F = Fd;
-    ctx->da_tuning = false;
+    ctx->da_tune.on = false;
   }
   return plain || da ? CR_OK : CR_ERR_INVALID_ARG;
 }
@@ -1818,13 +1777,8 @@ struct cr_batch {
   PhaseForm F{128, 1, 1, 16, 0};
   int regs = 0;
   int smem_max = 0;
-  bool tuning = true;
-  int tune_next = 0;
-  float tune_ms[32] = {};
   PhaseForm da_F{128, 1, 1, 16, 0};
-  int da_next = 0;
-  bool da_tuning = true;
-  float da_ms[16] = {};
+  FormTuner tune, da_tune;
   std::vector<SysParams> reps;  // host copy of d_reps
   cudaStream_t stream = nullptr;  // the contexts' shared stream (destroy does not touch the contexts)
   int order_nc = 0, order_nact = 0;  // largest box and colour among replicas with a launch order (0: none)
@@ -1945,8 +1899,7 @@ extern "C" int cr_batch_create(cr_batch **out, cr_ctx *const *ctxs, int32_t n) {
   }
   b->ncol = ctxs[0]->P.ncol;
   b->stream = ctxs[0]->stream;
-  b->tuning = std::getenv("CRMC_NO_TUNE") == nullptr;
-  b->da_tuning = b->tuning;
+  b->tune.on = b->da_tune.on = std::getenv("CRMC_NO_TUNE") == nullptr;
   b->reps = reps;
   for (int r = 0; r < n; ++r)
     if (reps[r].order) {
@@ -2119,11 +2072,9 @@ static int batch_sweep_impl(cr_batch *b, uint64_t n_sweeps, uint64_t seed, bool 
   const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
   const uint32_t sweep0 = (uint32_t)c0->sweep;
   bool &pers_choice = da ? b->da_persistent : b->persistent;
-  const bool glob = c0->P.global != 0;
-  TuneRef tr = da ? TuneRef{b->da_F, b->da_next, b->da_tuning, b->da_ms, glob}
-                  : TuneRef{b->F, b->tune_next, b->tuning, b->tune_ms, glob};
-  if (b->pmode < 0) tr.pers = &pers_choice;
-  else pers_choice = b->pmode != 0;
+  PhaseForm &form = da ? b->da_F : b->F;
+  FormTuner &tuner = da ? b->da_tune : b->tune;
+  if (b->pmode >= 0) pers_choice = b->pmode != 0;
   const int nform = phase_form_count(da);
   const PhaseShape &S = da ? b->S_da : b->S;
   for (uint64_t sw = 0; sw < n_sweeps; ++sw) {
@@ -2133,14 +2084,15 @@ static int batch_sweep_impl(cr_batch *b, uint64_t n_sweeps, uint64_t seed, bool 
       c->f_valid = false;
       c->fcons_valid = false;
     }
-    tune_skip(tr, S, b->smem_max, da);
-    const bool tune = tr.on && tr.next < tune_total(tr, da);
+    if (tuner.on && !tuner.begun())
+      tune_begin(tuner, S, b->smem_max, da, c0->P.global != 0, b->pmode <= 0, b->pmode != 0);
+    const bool tune = tuner.on;
     bool persistent = pers_choice;
-    const int cand = tune ? tune_cand(tr, da) : 0;
-    const PhaseForm F = tune ? phase_form(cand % nform, da) : tr.F;
+    const int cand = tune ? tuner.current() : 0;
+    const PhaseForm F = tune ? phase_form(cand % nform, da) : form;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (tune) {
-      if (tr.pers) persistent = cand >= nform;
+      if (b->pmode < 0) persistent = cand >= nform;
       cudaEventCreate(&e0);
       cudaEventCreate(&e1);
       cudaEventRecord(e0, s);
@@ -2172,7 +2124,10 @@ static int batch_sweep_impl(cr_batch *b, uint64_t n_sweeps, uint64_t seed, bool 
       cudaEventElapsedTime(&ms, e0, e1);
       cudaEventDestroy(e0);
       cudaEventDestroy(e1);
-      tune_finish(tr, ms, S, b->smem_max, da);
+      if (tuner.record(ms)) {
+        form = phase_form(tuner.current() % nform, da);
+        if (b->pmode < 0) pers_choice = tuner.current() >= nform;
+      }
     }
   }
   return CR_OK;
@@ -2201,7 +2156,7 @@ extern "C" int cr_batch_selftest_wait_timeout(cr_batch *b, int32_t replica, doub
     c->f_valid = false;
     c->fcons_valid = false;
   }
-  const PhaseForm F = b->tuning || b->F.seats > 1 ? PhaseForm{128, 1, 1, 16, 0} : b->F;  // (tasks take whole CTAs)
+  const PhaseForm F = b->tune.on || b->F.seats > 1 ? PhaseForm{128, 1, 1, 16, 0} : b->F;  // (tasks take whole CTAs)
   if (b->order_nc > 0) {
     CR_CUDA(launch_domain_order(b->d_reps, (int)b->ctx.size(), b->ncol, b->order_nact, c0->stream, swc, 1u, 0u));
     c0->launches_total += 2;
@@ -2468,7 +2423,7 @@ extern "C" int cr_batch_cycle(cr_batch *b, int32_t n_steps, double dt, double ga
   // of a completed step, the graph that evaluates them first when none does
   // (a step after a load); otherwise steps run call by call
   auto graphable = [&](bool forces) {
-    if (da ? b->da_tuning : b->tuning) return false;
+    if (da ? b->da_tune.on : b->tune.on) return false;
     for (cr_ctx *c : b->ctx)
       if (c->f_valid != forces || c->md_eval != c0->md_eval || c->sweep != c0->sweep || c->stream != s) return false;
     return true;
@@ -2711,9 +2666,9 @@ extern "C" int cr_batch_load_packed(cr_batch *b, const cr_batch_packed *p) {
 extern "C" int cr_batch_set_launch_shape(cr_batch *b, int32_t threads, int32_t regs) {
   if (!b) return CR_ERR_INVALID_ARG;
   if (threads == 0) {  // re-enable tuning
-    b->tuning = b->da_tuning = true;
+    b->tune.restart();
+    b->da_tune.restart();
     b->regs = 0;
-    b->tune_next = b->da_next = 0;
     return CR_OK;
   }
   if (b->pmode < 0) b->persistent = b->da_persistent = false;  // a fixed shape without a fixed mode: per colour
@@ -2725,11 +2680,11 @@ extern "C" int cr_batch_set_launch_shape(cr_batch *b, int32_t threads, int32_t r
   if (plain) {
     b->F = F;
     b->regs = regs;
-    b->tuning = false;
+    b->tune.on = false;
   }
   if (da) {
     b->da_F = Fd;
-    b->da_tuning = false;
+    b->da_tune.on = false;
   }
   return plain || da ? CR_OK : CR_ERR_INVALID_ARG;
 }
