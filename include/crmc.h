@@ -418,7 +418,13 @@ int cr_restore(cr_ctx *ctx, int32_t n, const float *xyz, const float *vel, const
 /* Launch shape of the colour-phase kernel: threads per domain.  Supported
  * pairs: (32|64|128|256|512, 0); (128, 4), (256, 2) and (512, 1), which name
  * halo particles held in registers per thread, run the shape of that many
- * threads (every shape keeps its halo in shared memory).
+ * threads (every shape keeps its halo in shared memory); and the pairs that
+ * cr_get_launch_shape gives for the forms of the launch that the tuner chooses
+ * among: seats | groups << 4 | compact << 8 | wide << 12, the domains that
+ * share a CTA, the groups of threads that evaluate trials side by side, 1 for
+ * compact capacities, and the sixteenths of the domains that have a CTA each
+ * beside shared ones (16: all).  A pair read back can be set again, e.g. to
+ * keep a form across contexts.
  * By default the first unlogged sweeps time the forms of the launch that apply
  * (threads per domain, one or several domains or trials per CTA, full or
  * compact shared-memory capacities), one per sweep: all once, then the fastest

@@ -28,8 +28,8 @@ struct cr_ctx {
   cudaStream_t stream = nullptr;
   SysParams P{};
   // launch form of the phase kernel, chosen by timing real sweeps (the chain
-  // does not depend on it: the energy sums are exact fixed point); regs: as
-  // given to cr_set_launch_shape
+  // does not depend on it: the energy sums are exact fixed point); regs: the
+  // second value of the pair that names it
   PhaseForm F{128, 1, 1, 16, 0};
   int regs = 0;
   int smem_max = 0;
@@ -1146,7 +1146,10 @@ static int sweep_impl(cr_ctx *ctx, uint64_t n_trials, uint64_t seed, cr_sweep_st
       cudaEventElapsedTime(&ms, e0, e1);
       cudaEventDestroy(e0);
       cudaEventDestroy(e1);
-      if (tuner.record(ms)) form = phase_form(tuner.current(), da);
+      if (tuner.record(ms)) {
+        form = phase_form(tuner.current(), da);
+        if (!da) ctx->regs = phase_form_code(form);
+      }
     }
   }
   if (log) {
@@ -2126,6 +2129,7 @@ static int batch_sweep_impl(cr_batch *b, uint64_t n_sweeps, uint64_t seed, bool 
       cudaEventDestroy(e1);
       if (tuner.record(ms)) {
         form = phase_form(tuner.current() % nform, da);
+        if (!da) b->regs = phase_form_code(form);
         if (b->pmode < 0) pers_choice = tuner.current() >= nform;
       }
     }

@@ -141,6 +141,7 @@ int phase_form_count(bool da);
 const PhaseForm &phase_form(int i, bool da);
 // the form that a caller's (threads, regs) pair names; false when there is none
 bool phase_form_named(int threads, int regs, bool da, PhaseForm *F);
+int phase_form_code(const PhaseForm &F);  // the regs that name F
 cudaError_t launch_phase(const SysParams *d_reps, int n_rep, int max_nact, const PhaseShape &S, const PhaseForm &F,
                          bool log, bool da, cudaStream_t s, uint32_t sweep, uint32_t sweep0, int colour, uint32_t k0,
                          uint32_t k1, const StepDyn *dyn = nullptr);

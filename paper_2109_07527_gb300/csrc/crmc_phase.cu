@@ -2380,7 +2380,21 @@ static const PhaseForm kFormsDA[] = {
 int phase_form_count(bool da) { return da ? (int)std::size(kFormsDA) : (int)std::size(kForms); }
 const PhaseForm &phase_form(int i, bool da) { return da ? kFormsDA[i] : kForms[i]; }
 
+// the second value of the pair that names a form: 0 for whole CTAs with the
+// full capacities; the other forms' values lie above 16
+int phase_form_code(const PhaseForm &F) {
+  if (F == PhaseForm{F.threads, 1, 1, 16, 0}) return 0;
+  return F.seats | F.groups << 4 | F.compact << 8 | F.wide16 << 12;
+}
+
 bool phase_form_named(int threads, int regs, bool da, PhaseForm *F) {
+  if (regs >= 16) {
+    for (int i = 0; i < phase_form_count(da); ++i) {
+      *F = phase_form(i, da);
+      if (F->threads == threads && phase_form_code(*F) == regs) return true;
+    }
+    return false;
+  }
   *F = PhaseForm{threads, 1, 1, 16, 0};
   if (regs != 0) return !da && ((threads == 128 && regs == 4) || (threads == 256 && regs == 2) || (threads == 512 && regs == 1));
   if (da) return threads == 128 || threads == 256 || threads == 512;

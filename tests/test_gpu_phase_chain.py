@@ -7,7 +7,9 @@
   * the Ewald sums keep the bits they had before the reciprocal vectors went by
     columns, and one box's slices give what a batch's items give;
   * a surrogate runs beside lists that take all of an SM's shared memory;
-  * domains of as many cells as ever fitted are accepted.
+  * domains of as many cells as ever fitted are accepted;
+  * every form of the launch can be named, and gives one chain, with lists and
+    halos on chip and in global memory; a form read back can be set again.
 """
 import zlib
 
@@ -169,3 +171,62 @@ def test_domains_of_many_cells(crmc, cells, per_rc, L, rc):
     o, lo, ties = compare_logs(w, g.sweep(n, 8, log=True)["log"], n, 8, dict(domain_cells=cells))
     compare_states(g, o, w.n_sites)
     g.close()
+
+
+def _code(seats, groups, wide, compact):
+    """The second value of a form's pair (cr_set_launch_shape)."""
+    return seats | groups << 4 | compact << 8 | wide << 12
+
+
+# the forms that the tuner chooses among, beyond whole CTAs with the full capacities
+FORMS = [(64, _code(1, 1, 16, 1)), (128, _code(1, 4, 16, 0)), (256, _code(1, 8, 16, 0)), (128, _code(2, 1, 2, 0)),
+         (256, _code(4, 1, 1, 0)), (256, _code(4, 1, 2, 0)), (256, _code(4, 1, 4, 0)), (256, _code(2, 1, 2, 0)),
+         (512, _code(4, 1, 4, 0))]
+BOXES = [lambda: W.config2(seed=21, pH=6.0), lambda: W.config4(seed=4, n_rep=1, hi=300)[0],
+         lambda: _ions(2400, 40.0, 10.0, 8, clump=0.3)]  # flat; small; lists of 30 to 500 entries
+
+
+@pytest.fixture(scope="module")
+def chains(crmc):
+    """The boxes' states after eight sweeps of 128 threads per domain."""
+    out = []
+    for box in BOXES:
+        g = crmc.Context(box())
+        g.set_launch_shape(128, 0)
+        g.sweep(g.trials_per_sweep * 8, 3)
+        out.append(g.state())
+        g.close()
+    return out
+
+
+@pytest.mark.parametrize("kw", [{}] + CAPACITIES)
+@pytest.mark.parametrize("threads,regs", FORMS + [(32, 0), (512, 0)])
+def test_every_form_gives_one_chain(crmc, chains, threads, regs, kw):
+    for box, ref in zip(BOXES, chains):
+        g = crmc.Context(box(), **kw)
+        g.set_launch_shape(threads, regs)
+        assert g.launch_shape() == (threads, regs)
+        g.sweep(g.trials_per_sweep * 8, 3)
+        s = g.state()
+        for key in ("id", "xyz", "vel", "state"):
+            assert np.array_equal(s[key], ref[key]), key
+        g.close()
+
+
+def test_a_tuned_form_can_be_read_and_set_again(crmc):
+    g, c = [crmc.Context(W.config2(seed=21, scale=0.5)) for _ in range(2)]
+    b = crmc.Batch([c])
+    for x, k in ((g, g.trials_per_sweep * 30), (b, 60)):
+        x.sweep(k, 1)
+        shape = x.launch_shape()
+        assert shape in FORMS + [(t, 0) for t in (128, 256, 512)]
+        x.set_launch_shape(128, 4)
+        assert x.launch_shape() == (128, 4)
+        x.set_launch_shape(*shape)
+        assert x.launch_shape() == shape
+    for bad in ((256, 17), (64, _code(4, 1, 2, 0)), (128, -1), (96, 0)):
+        with pytest.raises(crmc.CrError):
+            g.set_launch_shape(*bad)
+        with pytest.raises(crmc.CrError):
+            b.set_launch_shape(*bad)
+    b.close()
