@@ -427,12 +427,13 @@ int cr_restore(cr_ctx *ctx, int32_t n, const float *xyz, const float *vel, const
  * keep a form across contexts.
  * By default the first unlogged sweeps time the forms of the launch that apply
  * (threads per domain, one or several domains or trials per CTA, full or
- * compact shared-memory capacities), one per sweep: all once, then the fastest
- * third three times; the form with the shortest of the latter times is kept
- * (under the global schedule every form six times, the last three counted).
- * The trial outcomes never depend on the form (a pair's terms round alike
- * everywhere, their sums are exact fixed point).  cr_set_launch_shape(ctx, 0, 0) restarts the tuning; an unsupported
- * pair gives CR_ERR_INVALID_ARG. */
+ * compact shared-memory capacities), one per sweep; three later sweeps are each
+ * run in every form of the fastest third (four at most), from the same state,
+ * and the fastest on these is kept (after 2 n sweeps of n forms, 3 n under the global
+ * schedule).  The trial outcomes never depend on the form (a pair's terms round
+ * alike everywhere, their sums are exact fixed point).
+ * cr_set_launch_shape(ctx, 0, 0) restarts the tuning; an unsupported pair gives
+ * CR_ERR_INVALID_ARG. */
 int cr_set_launch_shape(cr_ctx *ctx, int32_t threads, int32_t regs);
 int cr_get_launch_shape(const cr_ctx *ctx, int32_t *threads, int32_t *regs);
 

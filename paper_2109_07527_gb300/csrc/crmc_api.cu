@@ -46,7 +46,7 @@ struct cr_ctx {
          *d_frc2 = nullptr, *d_fcons = nullptr;
   unsigned long long *d_pid = nullptr, *d_pid2 = nullptr, *d_stats = nullptr;
   long long *d_lnK = nullptr, *d_lntab = nullptr;
-  long long *d_counts = nullptr;
+  long long *d_counts = nullptr, *d_kept = nullptr;  // (d_kept: kind counts and statistics of keep_state)
   int *d_perm = nullptr, *d_bond_off = nullptr, *d_bond_nbr = nullptr;
   // d_counts holds N_KIND + 2 words: [0, N_KIND) kind counts, [N_KIND] ions found by cr_state
   // (an int), [N_KIND + 1] the error word (an int), read back with one copy
@@ -228,7 +228,7 @@ static void free_ctx(cr_ctx *c) {
   }
   void *ptrs[] = {c->d_cnt, c->d_cnt2, c->d_info, c->d_info2, c->d_pos, c->d_pos2, c->d_vel, c->d_vel2,
                   c->d_frc, c->d_frc2, c->d_fcons, c->d_pid, c->d_pid2, c->d_stats, c->d_lnK, c->d_lntab,
-                  c->d_counts, c->d_perm, c->d_bond_off, c->d_bond_nbr, c->d_log,
+                  c->d_counts, c->d_kept, c->d_perm, c->d_bond_off, c->d_bond_nbr, c->d_log,
                   c->d_in_xyz, c->d_in_vel, c->d_init_type, c->d_in_type, c->d_in_cls, c->d_site_map, c->d_in_state,
                   c->d_in_id, c->d_in_frc, c->d_present, c->d_chunk, c->d_ion_key, c->d_ion_key2, c->d_ion_val, c->d_ion_val2, c->d_ion_rank, c->d_sort_tmp,
                   c->d_out_xyz, c->d_out_vel, c->d_out_frc, c->d_out_id, c->d_out_type, c->d_out_cls,
@@ -733,6 +733,7 @@ extern "C" int cr_init(cr_ctx **out, const cr_system *sys, double pH, const doub
   ALLOC(c->d_lnK, std::max<size_t>(lnK.size(), 1));
   ALLOC(c->d_lntab, P.lnmax);
   ALLOC(c->d_counts, N_KIND + 2);
+  ALLOC(c->d_kept, N_KIND + 16);
   ALLOC(c->d_perm, std::max(n, 1));
   ALLOC(c->d_bond_off, n + 1);
   ALLOC(c->d_bond_nbr, std::max(2 * nb, 1));
@@ -1083,6 +1084,61 @@ static void tune_begin(FormTuner &t, const PhaseShape &S, int smem_max, bool da,
   t.begin(cand, global);
 }
 
+// a context's configuration into the rebuild's scratch arrays (unused by a
+// sweep), back from them, or the scratch cell counts left zero again.  The
+// slots of permanent particles need no copy: a sweep writes, and does not read, them.
+enum class Keep { SAVE, RESTORE, DROP };
+static cudaError_t keep_state(cr_ctx *c, Keep what, cudaStream_t s) {
+  const size_t cells = (size_t)c->P.ncell, slots = cells * (size_t)c->P.cap;
+  if (what == Keep::DROP) return cudaMemsetAsync(c->d_cnt2, 0, sizeof(int) * cells, s);
+  struct Pair {
+    void *now, *kept;
+    size_t bytes;
+  } const pairs[] = {{c->d_cnt, c->d_cnt2, sizeof(int) * cells},
+                     {c->d_pos, c->d_pos2, sizeof(float4) * slots},
+                     {c->d_vel, c->d_vel2, sizeof(float4) * slots},
+                     {c->d_pid, c->d_pid2, sizeof(unsigned long long) * slots},
+                     {c->d_info, c->d_info2, sizeof(int) * slots},
+                     {c->d_counts, c->d_kept, sizeof(long long) * N_KIND},
+                     {c->d_stats, c->d_kept + N_KIND, sizeof(unsigned long long) * 16}};
+  for (const Pair &p : pairs) {
+    const bool save = what == Keep::SAVE;
+    const cudaError_t e =
+        cudaMemcpyAsync(save ? p.kept : p.now, save ? p.now : p.kept, p.bytes, cudaMemcpyDeviceToDevice, s);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+// A timed sweep of the tuner: run(form, last) queues the sweep in one form,
+// keep(what) applies keep_state to every context of the call.
+template <typename Run, typename KeepAll>
+static int timed_sweep(FormTuner &t, cudaStream_t s, Run run, KeepAll keep) {
+  cudaEvent_t e0 = nullptr, e1 = nullptr;
+  cudaError_t e = cudaEventCreate(&e0);
+  if (e == cudaSuccess) e = cudaEventCreate(&e1);
+  int rc = CR_OK;
+  const int n = t.forms();
+  if (e == cudaSuccess && n > 1) e = keep(Keep::SAVE);
+  for (int i = 0; i < n && e == cudaSuccess && rc == CR_OK; ++i) {
+    if (i > 0) e = keep(Keep::RESTORE);
+    if (e == cudaSuccess) e = cudaEventRecord(e0, s);
+    if (e == cudaSuccess) rc = run(t.form(i), i == n - 1);
+    if (e == cudaSuccess && rc == CR_OK) e = cudaEventRecord(e1, s);
+    if (e == cudaSuccess && rc == CR_OK) e = cudaEventSynchronize(e1);
+    float ms = 0.0f;
+    if (e == cudaSuccess && rc == CR_OK) e = cudaEventElapsedTime(&ms, e0, e1);
+    t.time(i, ms);
+  }
+  const cudaError_t d = n > 1 ? keep(Keep::DROP) : cudaSuccess;
+  if (e0) cudaEventDestroy(e0);
+  if (e1) cudaEventDestroy(e1);
+  if (rc != CR_OK) return rc;
+  CR_CUDA(e);
+  CR_CUDA(d);
+  return CR_OK;
+}
+
 static int sweep_impl(cr_ctx *ctx, uint64_t n_trials, uint64_t seed, cr_sweep_stats *stats, cr_trial *log,
                       bool da = false, cr_trial_da *dlog = nullptr, float *feat = nullptr) {
   if (!ctx) return CR_ERR_INVALID_ARG;
@@ -1115,41 +1171,44 @@ static int sweep_impl(cr_ctx *ctx, uint64_t n_trials, uint64_t seed, cr_sweep_st
   FormTuner &tuner = da ? ctx->da_tune : ctx->tune;
   for (uint64_t sw = 0; sw < n_sweeps; ++sw) {
     const uint32_t swc = (uint32_t)ctx->sweep++;
-    if (!log && tuner.on && !tuner.begun()) tune_begin(tuner, S, ctx->smem_max, da, P.global != 0, true, false);
-    const bool tune = tuner.on && !log;
-    const PhaseForm F = tune ? phase_form(tuner.current(), da) : form;
-    cudaEvent_t e0 = nullptr, e1 = nullptr;
-    if (tune) {
-      cudaEventCreate(&e0);
-      cudaEventCreate(&e1);
-      cudaEventRecord(e0, s);
-    }
-    if (P.order) {
-      CR_CUDA(launch_domain_order(ctx->d_reps, 1, P.ncol, P.nact, s, swc, k0, k1));
-      ctx->launches_total += 2;
-    }
-    if (P.ewald_nk > 0) {  // S(k) from scratch at every sweep
-      CR_CUDA(launch_ewald_sk(ctx->d_reps, 1, P.ewald_items, P.ewald_plus, s));
-      ctx->launches_total += 2;
-    }
-    for (int col = 0; col < P.ncol; ++col) {
-      int ti;
-      tbegin(ctx, 0, &ti);
-      CR_CUDA(launch_phase(ctx->d_reps, 1, P.nact, S, F, log != nullptr, da, s, swc, sweep0, col, k0, k1));
-      tend(ctx, 0, ti);
-      ctx->launches_total++;
-    }
-    if (tune) {
-      cudaEventRecord(e1, s);
-      cudaEventSynchronize(e1);
-      float ms = 0.0f;
-      cudaEventElapsedTime(&ms, e0, e1);
-      cudaEventDestroy(e0);
-      cudaEventDestroy(e1);
-      if (tuner.record(ms)) {
-        form = phase_form(tuner.current(), da);
-        if (!da) ctx->regs = phase_form_code(form);
+    auto run = [&](const PhaseForm &F) -> int {
+      if (P.order) {
+        CR_CUDA(launch_domain_order(ctx->d_reps, 1, P.ncol, P.nact, s, swc, k0, k1));
+        ctx->launches_total += 2;
       }
+      if (P.ewald_nk > 0) {  // S(k) from scratch at every sweep
+        CR_CUDA(launch_ewald_sk(ctx->d_reps, 1, P.ewald_items, P.ewald_plus, s));
+        ctx->launches_total += 2;
+      }
+      for (int col = 0; col < P.ncol; ++col) {
+        int ti;
+        tbegin(ctx, 0, &ti);
+        CR_CUDA(launch_phase(ctx->d_reps, 1, P.nact, S, F, log != nullptr, da, s, swc, sweep0, col, k0, k1));
+        tend(ctx, 0, ti);
+        ctx->launches_total++;
+      }
+      return CR_OK;
+    };
+    int rc;
+    if (!log && tuner.on && !tuner.begun()) tune_begin(tuner, S, ctx->smem_max, da, P.global != 0, true, false);
+    const bool tune = !log && tuner.on;
+    if (tune && tuner.forms() > 0) {
+      const bool timing = ctx->timing;
+      rc = timed_sweep(
+          tuner, s,
+          [&](int c, bool last) {
+            ctx->timing = timing && last;
+            return run(phase_form(c, da));
+          },
+          [&](Keep what) { return keep_state(ctx, what, s); });
+      ctx->timing = timing;
+    } else {
+      rc = run(form);
+    }
+    if (rc != CR_OK) return rc;
+    if (tune) {
+      form = phase_form(tuner.pass(), da);
+      if (!da) ctx->regs = phase_form_code(form);
     }
   }
   if (log) {
@@ -2087,31 +2146,16 @@ static int batch_sweep_impl(cr_batch *b, uint64_t n_sweeps, uint64_t seed, bool 
       c->f_valid = false;
       c->fcons_valid = false;
     }
-    if (tuner.on && !tuner.begun())
-      tune_begin(tuner, S, b->smem_max, da, c0->P.global != 0, b->pmode <= 0, b->pmode != 0);
-    const bool tune = tuner.on;
-    bool persistent = pers_choice;
-    const int cand = tune ? tuner.current() : 0;
-    const PhaseForm F = tune ? phase_form(cand % nform, da) : form;
-    cudaEvent_t e0 = nullptr, e1 = nullptr;
-    if (tune) {
-      if (b->pmode < 0) persistent = cand >= nform;
-      cudaEventCreate(&e0);
-      cudaEventCreate(&e1);
-      cudaEventRecord(e0, s);
-    }
-    if (b->order_nc > 0) {
-      CR_CUDA(launch_domain_order(b->d_reps, n, b->ncol, b->order_nact, s, swc, k0, k1));
-      c0->launches_total += 2;
-    }
-    if (b->ewald_items > 0) {  // S(k) of every replica from scratch at every sweep
-      CR_CUDA(launch_ewald_sk(b->d_reps, n, b->ewald_items, b->ewald_plus, s));
-      c0->launches_total += 2;
-    }
-    if (persistent) {
-      const int rc = batch_launch_persistent(b, F, da, swc, sweep0, k0, k1);
-      if (rc != CR_OK) return rc;
-    } else {
+    auto run = [&](const PhaseForm &F, bool persistent) -> int {
+      if (b->order_nc > 0) {
+        CR_CUDA(launch_domain_order(b->d_reps, n, b->ncol, b->order_nact, s, swc, k0, k1));
+        c0->launches_total += 2;
+      }
+      if (b->ewald_items > 0) {  // S(k) of every replica from scratch at every sweep
+        CR_CUDA(launch_ewald_sk(b->d_reps, n, b->ewald_items, b->ewald_plus, s));
+        c0->launches_total += 2;
+      }
+      if (persistent) return batch_launch_persistent(b, F, da, swc, sweep0, k0, k1);
       for (int col = 0; col < b->ncol; ++col) {
         int ti;
         tbegin(c0, 0, &ti);
@@ -2119,19 +2163,36 @@ static int batch_sweep_impl(cr_batch *b, uint64_t n_sweeps, uint64_t seed, bool 
         tend(c0, 0, ti);
         c0->launches_total++;
       }
+      return CR_OK;
+    };
+    int rc;
+    if (tuner.on && !tuner.begun())
+      tune_begin(tuner, S, b->smem_max, da, c0->P.global != 0, b->pmode <= 0, b->pmode != 0);
+    const bool tune = tuner.on;
+    if (tune && tuner.forms() > 0) {
+      const bool timing = c0->timing;
+      rc = timed_sweep(
+          tuner, s,
+          [&](int c, bool last) {
+            c0->timing = timing && last;
+            return run(phase_form(c % nform, da), b->pmode < 0 ? c >= nform : pers_choice);
+          },
+          [&](Keep what) {
+            cudaError_t e = cudaSuccess;
+            for (cr_ctx *c : b->ctx)
+              if (e == cudaSuccess) e = keep_state(c, what, s);
+            return e;
+          });
+      c0->timing = timing;
+    } else {
+      rc = run(form, pers_choice);
     }
+    if (rc != CR_OK) return rc;
     if (tune) {
-      cudaEventRecord(e1, s);
-      cudaEventSynchronize(e1);
-      float ms = 0.0f;
-      cudaEventElapsedTime(&ms, e0, e1);
-      cudaEventDestroy(e0);
-      cudaEventDestroy(e1);
-      if (tuner.record(ms)) {
-        form = phase_form(tuner.current() % nform, da);
-        if (!da) b->regs = phase_form_code(form);
-        if (b->pmode < 0) pers_choice = tuner.current() >= nform;
-      }
+      const int choice = tuner.pass();
+      form = phase_form(choice % nform, da);
+      if (!da) b->regs = phase_form_code(form);
+      if (b->pmode < 0) pers_choice = choice >= nform;
     }
   }
   return CR_OK;
