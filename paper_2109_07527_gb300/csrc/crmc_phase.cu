@@ -1303,10 +1303,10 @@ static size_t phase_layout(const PhaseCaps &C, const PhaseShape &S, int warps, i
       da ? sizeof(int) * nr3 : 0,             // DA: region cell aggregates (ion charge, site charge, particles)
       da ? sizeof(int) * nr3 : 0,
       da ? sizeof(int) * nr3 : 0,
-      da ? sizeof(int) * MLP_IN * groups : 0,  // per group: feature bins, surrogate layers
-      da ? sizeof(float) * 2 * MLP_IN * groups : 0,
-      da ? sizeof(float) * 2 * MLP_H * groups : 0,
-      da ? sizeof(float) * 2 * MLP_H * groups : 0};
+      da ? sizeof(int) * MLP_IN : 0,          // feature bins, surrogate layers
+      da ? sizeof(float) * 2 * MLP_IN : 0,
+      da ? sizeof(float) * 2 * MLP_H : 0,
+      da ? sizeof(float) * 2 * MLP_H : 0};
   size_t at = 0;
   for (int pass = 0; pass < 2; ++pass)  // first the arrays whose place is the same in both of a launch's layouts
     for (int i = 0; i < PhaseLayout::N_OFF; ++i) {
@@ -1364,10 +1364,10 @@ __device__ __forceinline__ void phase_task(unsigned char *smem, const PhaseArgs 
     aQi = (int *)CRMC_AT(25);
     aQs = (int *)CRMC_AT(26);
     aN = (int *)CRMC_AT(27);
-    dfeat = (int *)CRMC_AT(28) + group * MLP_IN;
-    fv = (float *)CRMC_AT(29) + group * 2 * MLP_IN;
-    hb0 = (float *)CRMC_AT(30) + group * 2 * MLP_H;
-    hb1 = (float *)CRMC_AT(31) + group * 2 * MLP_H;
+    dfeat = (int *)CRMC_AT(28);
+    fv = (float *)CRMC_AT(29);
+    hb0 = (float *)CRMC_AT(30);
+    hb1 = (float *)CRMC_AT(31);
   }
 
   {
@@ -1602,9 +1602,9 @@ __device__ __forceinline__ void phase_task(unsigned char *smem, const PhaseArgs 
         ewald_factors(P, ctl, ewf, ewq, A.lay[0].ewk, tid, T);
         seat.sync();
       }
-      // ---- delayed acceptance, stage 1: surrogate features and MLP (all of
-      // the group's threads), decision in its first warp; a rejection skips
-      // the pair sweep
+      // ---- delayed acceptance (one group, no seats: its forms), stage 1:
+      // surrogate features and MLP (all threads), decision in the first warp; a
+      // rejection skips the pair sweep
       if (DA && mine && ctl.nch) {
         for (int i = gtid; i < MLP_IN; i += GT) dfeat[i] = 0;
         seat.group_sync();
@@ -2359,7 +2359,6 @@ cudaError_t launch_phase(const SysParams *d_reps, int n_rep, int max_nact, const
   CRMC_CASE(false, false, true)
   CRMC_CASE(true, false, false)
   CRMC_CASE(false, true, false)
-  CRMC_CASE(false, true, true)
   CRMC_CASE(true, true, false)
 #undef CRMC_CASE
   return cudaErrorInvalidValue;

@@ -235,7 +235,7 @@ __device__ __forceinline__ void order_cta(const SysParams &P, const StateBufs &B
   if (r < n_ions) emit(P, B, slot[r], n_present + r);
 }
 
-// (counts from the host; the ion counter is cleared by a copy node after it)
+// (counts from the host, which has read the ion counter)
 __global__ void __launch_bounds__(ORDER_THREADS) k_state_order(SysParams P, StateBufs B, int input_chunks,
                                                                int n_present, int n_ions, const int *slot) {
   if (blockIdx.x == 0 && threadIdx.x == 0) *B.n_ions = 0;  // the count came to the host as n_ions
