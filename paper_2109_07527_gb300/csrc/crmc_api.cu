@@ -121,8 +121,8 @@ struct cr_ctx {
   float *d_ek_A = nullptr;
   int4 *d_ek_z = nullptr, *d_ek_vec = nullptr;
   int2 *d_ek_item = nullptr;
-  int *d_ek_col = nullptr;
-  float2 *d_ek_Shi = nullptr, *d_ek_Slo = nullptr;
+  int *d_ek_place = nullptr;
+  float2 *d_ek_Shi = nullptr, *d_ek_Slo = nullptr, *d_ek_Sf = nullptr;
   int *d_ek_list = nullptr, *d_ek_np = nullptr;
   // caller-owned slot arrays (cr_bind_device_buffers) and batch membership
   bool bound = false;
@@ -235,7 +235,7 @@ static void free_ctx(cr_ctx *c) {
                   c->d_out_state, c->d_out_site,
                   c->d_reps, c->d_gs_pos, c->d_gs_vel, c->d_gs_id, c->d_gs_lnk, c->d_gs_info, c->d_gs_ord,
                   c->d_plist, c->d_nparts, c->d_fsum, c->d_mlp_w, c->d_mlp_b, c->d_dlog, c->d_feat, c->d_order, c->d_cost,
-                  c->d_ek_A, c->d_ek_z, c->d_ek_vec, c->d_ek_item, c->d_ek_col, c->d_ek_Shi, c->d_ek_Slo, c->d_ek_list, c->d_ek_np,
+                  c->d_ek_A, c->d_ek_z, c->d_ek_vec, c->d_ek_item, c->d_ek_place, c->d_ek_Shi, c->d_ek_Slo, c->d_ek_Sf, c->d_ek_list, c->d_ek_np,
                   c->d_bodies, c->d_body_member, c->d_body_d, c->d_body_df, c->d_body_newpos};
   for (void *p : ptrs)
     if (p) cudaFree(p);
@@ -420,7 +420,7 @@ extern "C" int cr_init(cr_ctx **out, const cr_system *sys, double pH, const doub
   std::vector<float> ek_A;
   std::vector<int4> ek_z, ek_vec;
   std::vector<int2> ek_item;
-  std::vector<int> ek_col;
+  std::vector<int> ek_col, ek_place;
   if (sys->ewald_kmax < 0 || sys->ewald_kmax > 32) { free_ctx(c); return CR_ERR_INVALID_ARG; }
   if (sys->ewald_kmax > 0) {
     if (!global) { free_ctx(c); return CR_ERR_INVALID_ARG; }
@@ -455,9 +455,9 @@ extern "C" int cr_init(cr_ctx **out, const cr_system *sys, double pH, const doub
         (sign ? ek_z[z].z : ek_z[z].y) = place;
         place += reach;
       }
-      if (sign == 0) P.ewald_plus = place;
     }
     ek_A.assign((size_t)place, 0.0f);
+    ek_place.assign((size_t)place, -1);
     for (const Column &c : cols) ek_col.push_back((c.nx & 255) | ((c.ny & 255) << 8));
     for (int z0 = 0; z0 <= km; z0 += 4)
       for (int c = 0; c < ek_z[z0].x; ++c) ek_item.push_back(make_int2(ek_col[c] | (z0 / 4) << 16, c));
@@ -477,6 +477,7 @@ extern "C" int cr_init(cr_ctx **out, const cr_system *sys, double pH, const doub
           const int4 &z = ek_z[std::abs(nz)];
           const int at = (nz < 0 ? z.z : z.y) + col_of[nx * (2 * km + 1) + ny + km];
           ek_A[at] = A;
+          ek_place[at] = (int)ek_vec.size();
           ek_vec.push_back(make_int4((nx & 255) | ((ny & 255) << 8) | ((nz & 255) << 16), Ab, at, 0));
         }
   }
@@ -654,10 +655,10 @@ extern "C" int cr_init(cr_ctx **out, const cr_system *sys, double pH, const doub
   S.ewk = P.ewald_nk > 0 ? P.ewald_kmax + 1 : 0;
   // Shared-memory list and halo capacities: the densest domain of the
   // starting configuration with room for growth, and its densest halo.  The
-  // compact set (Sc) is sized for the 90th percentile instead, so that more
+  // compact set (S.small) is sized for the 90th percentile instead, so that more
   // CTAs fit on an SM; denser domains then keep their list in a global
   // scratch region and read the halo beyond the capacity from global memory.
-  // The tuner times shapes with either set.  list_capacity / halo_capacity > 0
+  // The tuner times forms with either set.  list_capacity / halo_capacity > 0
   // fix the capacities (both sets).
   PhaseCaps &C = S.full;
   C.dcs = sys->list_capacity > 0 ? sys->list_capacity + 2 * P.m : std::max(2 * maxd, maxd + 32) + 2 * P.m;
@@ -793,9 +794,10 @@ extern "C" int cr_init(cr_ctx **out, const cr_system *sys, double pH, const doub
     ALLOC(c->d_ek_z, ek_z.size());
     ALLOC(c->d_ek_vec, ek_vec.size());
     ALLOC(c->d_ek_item, ek_item.size());
-    ALLOC(c->d_ek_col, ek_col.size());
     ALLOC(c->d_ek_Shi, (size_t)P.ewald_nk);
     ALLOC(c->d_ek_Slo, (size_t)P.ewald_nk);
+    ALLOC(c->d_ek_Sf, ek_vec.size());
+    ALLOC(c->d_ek_place, ek_place.size());
     ALLOC(c->d_ek_list, (size_t)std::max(sys->capacity, 1));
     ALLOC(c->d_ek_np, 1);
   }
@@ -835,8 +837,11 @@ extern "C" int cr_init(cr_ctx **out, const cr_system *sys, double pH, const doub
     COPY(c->d_ek_A, ek_A.data(), ek_A.size());
     COPY(c->d_ek_z, ek_z.data(), ek_z.size());
     COPY(c->d_ek_vec, ek_vec.data(), ek_vec.size());
+    COPY(c->d_ek_place, ek_place.data(), ek_place.size());
+    // (places outside the half space are not always written; their weight is 0)
+    cudaMemset(c->d_ek_Shi, 0, sizeof(float2) * (size_t)P.ewald_nk);
+    cudaMemset(c->d_ek_Slo, 0, sizeof(float2) * (size_t)P.ewald_nk);
     COPY(c->d_ek_item, ek_item.data(), ek_item.size());
-    COPY(c->d_ek_col, ek_col.data(), ek_col.size());
   }
 #undef COPY
   cudaMemset(c->d_cnt2, 0, sizeof(int) * P.ncell);
@@ -865,8 +870,9 @@ extern "C" int cr_init(cr_ctx **out, const cr_system *sys, double pH, const doub
   P.ek_A = c->d_ek_A;
   P.ek_z = c->d_ek_z;
   P.ek_vec = c->d_ek_vec;
+  P.ek_place = c->d_ek_place;
+  P.ek_Sf = c->d_ek_Sf;
   P.ek_item = c->d_ek_item;
-  P.ek_col = c->d_ek_col;
   P.ek_Shi = c->d_ek_Shi;
   P.ek_Slo = c->d_ek_Slo;
   P.ek_list = c->d_ek_list;
@@ -1177,7 +1183,7 @@ static int sweep_impl(cr_ctx *ctx, uint64_t n_trials, uint64_t seed, cr_sweep_st
         ctx->launches_total += 2;
       }
       if (P.ewald_nk > 0) {  // S(k) from scratch at every sweep
-        CR_CUDA(launch_ewald_sk(ctx->d_reps, 1, P.ewald_items, P.ewald_plus, s));
+        CR_CUDA(launch_ewald_sk(ctx->d_reps, 1, P.ewald_items, P.ewald_vec, s));
         ctx->launches_total += 2;
       }
       for (int col = 0; col < P.ncol; ++col) {
@@ -1456,7 +1462,7 @@ static int md_force_eval(cr_ctx *ctx, const MdParams &M) {
   MdParams Q = M;
   Q.fsum = ctx->d_fsum;
   if (ctx->P.ewald_nk > 0) {  // S(k) of the current positions for the reciprocal forces
-    CR_CUDA(launch_ewald_sk(ctx->d_reps, 1, ctx->P.ewald_items, ctx->P.ewald_plus, ctx->stream));
+    CR_CUDA(launch_ewald_sk(ctx->d_reps, 1, ctx->P.ewald_items, ctx->P.ewald_vec, ctx->stream));
     ctx->launches_total += 3;  // occupied slots, S(k), reciprocal forces
   }
   CR_CUDA(launch_md_forces(ctx->P, Q, ctx->d_plist, ctx->d_nparts, (int)ctx->capacity, ctx->stream));
@@ -1860,7 +1866,7 @@ struct cr_batch {
   int *d_pk_type = nullptr, *d_pk_cls = nullptr;
   int8_t *d_pk_state = nullptr;
   bool holds_refs = false;  // the contexts' batch_refs count this batch
-  int ewald_items = 0, ewald_plus = 0;  // largest numbers of Ewald items and nz >= 0 places over the replicas
+  int ewald_items = 0, ewald_vec = 0;  // largest numbers of Ewald items and vectors over the replicas
   // batched MD steps: per-replica parameters on the device and the lengths of
   // the replicas' particle lists
   MdJob *d_md = nullptr;
@@ -1956,7 +1962,7 @@ extern "C" int cr_batch_create(cr_batch **out, cr_ctx *const *ctxs, int32_t n) {
     b->S.chunk = std::max(b->S.chunk, c->S.chunk);
     b->S.ewk = std::max(b->S.ewk, c->S.ewk);
     b->ewald_items = std::max(b->ewald_items, c->P.ewald_items);
-    b->ewald_plus = std::max(b->ewald_plus, c->P.ewald_plus);
+    b->ewald_vec = std::max(b->ewald_vec, c->P.ewald_vec);
     b->grid_x = std::max(b->grid_x, c->P.nact);
   }
   b->ncol = ctxs[0]->P.ncol;
@@ -2152,7 +2158,7 @@ static int batch_sweep_impl(cr_batch *b, uint64_t n_sweeps, uint64_t seed, bool 
         c0->launches_total += 2;
       }
       if (b->ewald_items > 0) {  // S(k) of every replica from scratch at every sweep
-        CR_CUDA(launch_ewald_sk(b->d_reps, n, b->ewald_items, b->ewald_plus, s));
+        CR_CUDA(launch_ewald_sk(b->d_reps, n, b->ewald_items, b->ewald_vec, s));
         c0->launches_total += 2;
       }
       if (persistent) return batch_launch_persistent(b, F, da, swc, sweep0, k0, k1);
@@ -2284,7 +2290,7 @@ static int batch_md_forces(cr_batch *b, int mode, double dt, double gamma, uint6
   cr_ctx *c0 = b->ctx[0];
   const int n = (int)b->ctx.size();
   if (b->ewald_items > 0) {
-    CR_CUDA(launch_ewald_sk(b->d_reps, n, b->ewald_items, b->ewald_plus, c0->stream));
+    CR_CUDA(launch_ewald_sk(b->d_reps, n, b->ewald_items, b->ewald_vec, c0->stream));
     c0->launches_total += 3;  // occupied slots, S(k), reciprocal forces
   }
   const MdParams M = md_params(c0, mode, dt, gamma, seed);

@@ -126,16 +126,16 @@ struct alignas(16) SysParams {
   // column: a thread forms the column's factor e_x e_y once for up to eight
   // vectors, and |nz| is uniform over a warp.
   int ewald_nk, ewald_kmax;
-  int ewald_plus, ewald_items;  // places with nz >= 0; items
+  int ewald_items;
   const float *ek_A;            // [ewald_nk] weights
   const int4 *ek_z;             // [kmax + 4] of |nz|: columns that reach it, the slices' first places (+, -)
-  const int *ek_col;            // nx | ny << 8 of each column
   const int2 *ek_item;          // nx | ny << 8 | (|nz| / 4) << 16, column
   // every vector in the order of nz, ny, nx: n code (three signed bytes),
   // weight bits, place
   int ewald_vec;
   const int4 *ek_vec;
-  float2 *ek_Shi, *ek_Slo;
+  const int *ek_place;  // [ewald_nk] the place's vector, -1 for one outside the half space
+  float2 *ek_Shi, *ek_Slo, *ek_Sf;  // Sf: hi + lo in FP32 from scratch, by vector (the forces)
   double invLd;  // 1 / L in FP64
   int *ek_list, *ek_np;  // occupied slots (the structure-factor kernel's particle list) and their number
   int ek_cap;            // entries of ek_list (the capacity in particles)

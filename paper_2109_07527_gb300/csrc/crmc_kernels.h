@@ -135,6 +135,14 @@ struct LoadJob {
   int n_perm;
 };
 
+// multiprocessors of the current device
+inline int device_sms() {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return sms > 0 ? sms : 1;
+}
+
 // forms of the phase launches; da: the delayed-acceptance set
 size_t phase_smem_bytes(const PhaseShape &S, const PhaseForm &F, bool da);
 int phase_form_count(bool da);
@@ -206,10 +214,10 @@ size_t state_sort_temp_bytes(int cap);
 cudaError_t launch_state_batch(const SysParams *d_reps, const StateBufs *d_bufs, int n_rep, int max_cells,
                                int max_input, int max_cap, long long *d_n_out, int *d_err_out, cudaStream_t s);
 // Ewald: S(k) of every replica of a batch from scratch (the occupied slots
-// listed, then one thread per item of reciprocal vectors, or per |nz| of
-// each column where there are few); max_items, max_plus: the largest
-// ewald_items and ewald_plus over the replicas
-cudaError_t launch_ewald_sk(const SysParams *d_reps, int n_rep, int max_items, int max_plus, cudaStream_t s);
+// listed, then one thread per item of reciprocal vectors, or per vector where
+// there are few); max_items, max_vec: the largest ewald_items and ewald_vec
+// over the replicas
+cudaError_t launch_ewald_sk(const SysParams *d_reps, int n_rep, int max_items, int max_vec, cudaStream_t s);
 // rigid bodies: centre, principal frame, body-frame offsets and momenta from
 // the current configuration (bodies[] carries first, count and mfirst);
 // then, once every body is valid, the members' rigid velocities

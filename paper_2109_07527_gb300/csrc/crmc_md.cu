@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
 #include <cstdint>
 
 #include "crmc_device.cuh"
@@ -428,7 +429,7 @@ constexpr int CELL_THREADS = 256;  // at most
 static inline unsigned cell_groups(int ncell) { return (unsigned)((ncell + CELL_GROUP - 1) / CELL_GROUP); }
 // one system: 256 threads, so that dense cells (a nanoparticle's shell) are
 // done early; many: 64, about what 32 cells hold
-static inline unsigned cell_threads(unsigned groups) { return groups < 8 * 152 ? 256u : 64u; }
+static inline unsigned cell_threads(unsigned groups) { return groups < 8u * (unsigned)device_sms() ? 256u : 64u; }
 template <typename F>
 __device__ __forceinline__ void for_cell_particles(int n, F f) {
   const int lane = threadIdx.x & 31, c0 = blockIdx.x * CELL_GROUP;
@@ -1031,8 +1032,9 @@ __global__ void __launch_bounds__(RB_THREADS) k_body_drift(SysParams P, MdParams
 // F_j = 2 q_j sum_k A'_k k Im(S(k)^* exp(i k.r_j)), Im(...) = C sin - D cos,
 // S = C + i D of the current positions (k_ewald_sk runs just before).  One
 // CTA of 256 threads per four particles of the force kernel's list, which
-// share each vector's loads and decoding (one particle per CTA re-read 24
-// bytes and re-decoded them for 20 flops); the axis factors
+// share each vector's loads and decoding (one particle per CTA re-reads 24
+// bytes and re-decodes them for 20 flops), or per two or one where there are
+// fewer particles than keep the SMs busy (ewf_particles); the axis factors
 // exp(i 2 pi n x / L), n <= kmax, from the coordinate's 0.32 fixed-point
 // fraction (an exact phase reduction); each thread sums every 256th vector in
 // order, the warps by a fixed butterfly, the eight warp sums in warp order;
@@ -1041,7 +1043,6 @@ __global__ void __launch_bounds__(RB_THREADS) k_body_drift(SysParams P, MdParams
 // ---------------------------------------------------------------------------
 constexpr int EWF_THREADS = 256;
 constexpr int EWF_K1 = 33;  // kmax + 1 for kmax <= 32
-constexpr int EWF_P = 4;    // particles per CTA
 
 __device__ __forceinline__ float2 ewf_factor(float x, double invL, int n) {
   const uint32_t U = (uint32_t)(unsigned long long)llrint((double)x * invL * 4294967296.0);
@@ -1051,35 +1052,36 @@ __device__ __forceinline__ float2 ewf_factor(float x, double invL, int n) {
   return make_float2(cs, sn);
 }
 
+template <int NP>
 __device__ __forceinline__ void ewald_forces(const SysParams &P, const MdParams &M) {
-  __shared__ float2 f[EWF_P][3 * EWF_K1];
-  __shared__ float part[EWF_P][EWF_THREADS / 32][3];
-  const int w0 = blockIdx.x * EWF_P, t = threadIdx.x, lane = t & 31, wl = t >> 5, np = min(*M.n_particles, M.max_particles);
+  __shared__ float2 f[NP][3 * EWF_K1];
+  __shared__ float part[NP][EWF_THREADS / 32][3];
+  const int w0 = blockIdx.x * NP, t = threadIdx.x, lane = t & 31, wl = t >> 5, np = min(*M.n_particles, M.max_particles);
   if (w0 >= np) return;  // whole CTA
   const int ewk = P.ewald_kmax + 1;
-  float q[EWF_P];
+  float q[NP];
 #pragma unroll
-  for (int p = 0; p < EWF_P; ++p) q[p] = w0 + p < np ? P.pos[M.plist[w0 + p]].w : 0.0f;
-  for (int i = t; i < EWF_P * 3 * ewk; i += EWF_THREADS) {
+  for (int p = 0; p < NP; ++p) q[p] = w0 + p < np ? P.pos[M.plist[w0 + p]].w : 0.0f;
+  for (int i = t; i < NP * 3 * ewk; i += EWF_THREADS) {
     const int p = i / (3 * ewk), ax = i / ewk - 3 * p, n = i % ewk;
     if (w0 + p >= np) break;
     const float4 r = P.pos[M.plist[w0 + p]];
     f[p][ax * EWF_K1 + n] = ewf_factor(ax == 0 ? r.x : (ax == 1 ? r.y : r.z), P.invLd, n);
   }
   __syncthreads();
-  float gx[EWF_P], gy[EWF_P], gz[EWF_P];
+  float gx[NP], gy[NP], gz[NP];
 #pragma unroll
-  for (int p = 0; p < EWF_P; ++p) gx[p] = gy[p] = gz[p] = 0.0f;
+  for (int p = 0; p < NP; ++p) gx[p] = gy[p] = gz[p] = 0.0f;
 #pragma unroll 2
   for (int i = t; i < P.ewald_vec; i += EWF_THREADS) {
     const int4 v = P.ek_vec[i];
-    const float2 hi = P.ek_Shi[v.z], lo = P.ek_Slo[v.z];
+    const float2 S = P.ek_Sf[i];
     const int nx = (int)(signed char)(v.x & 255), ny = (int)(signed char)((v.x >> 8) & 255),
               nz = (int)(signed char)((v.x >> 16) & 255);
     const int iy = EWF_K1 + abs(ny), iz = 2 * EWF_K1 + abs(nz);  // (nx >= 0)
-    const float C = hi.x + lo.x, D = hi.y + lo.y, A = __int_as_float(v.y);
+    const float C = S.x, D = S.y, A = __int_as_float(v.y);
 #pragma unroll
-    for (int p = 0; p < EWF_P; ++p) {
+    for (int p = 0; p < NP; ++p) {
       if (q[p] == 0.0f) continue;
       const float2 ey = f[p][iy], ez = f[p][iz];
       const float2 e = cmul(cmul(make_float2(ey.x, ny < 0 ? -ey.y : ey.y), f[p][nx]),
@@ -1091,7 +1093,7 @@ __device__ __forceinline__ void ewald_forces(const SysParams &P, const MdParams 
     }
   }
 #pragma unroll
-  for (int p = 0; p < EWF_P; ++p) {
+  for (int p = 0; p < NP; ++p) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       gx[p] += __shfl_xor_sync(0xffffffffu, gx[p], o);
@@ -1105,7 +1107,7 @@ __device__ __forceinline__ void ewald_forces(const SysParams &P, const MdParams 
     }
   }
   __syncthreads();
-  if (t < EWF_P * 3 && w0 + t / 3 < np) {
+  if (t < NP * 3 && w0 + t / 3 < np) {
     const int p = t / 3, ax = t - 3 * p, gi = M.plist[w0 + p];
     float sum = 0.0f;
     for (int k = 0; k < EWF_THREADS / 32; ++k) sum += part[p][k][ax];
@@ -1114,10 +1116,26 @@ __device__ __forceinline__ void ewald_forces(const SysParams &P, const MdParams 
   }
 }
 
-__global__ void __launch_bounds__(EWF_THREADS) k_ewald_forces(SysParams P, MdParams M) { ewald_forces(P, M); }
+template <int NP>
+__global__ void __launch_bounds__(EWF_THREADS) k_ewald_forces(SysParams P, MdParams M) {
+  ewald_forces<NP>(P, M);
+}
+template <int NP>
 __global__ void __launch_bounds__(EWF_THREADS) k_ewald_forces_batch(const SysParams *__restrict__ reps,
                                                                     const MdJob *__restrict__ jobs) {
-  if (reps[blockIdx.y].ewald_nk > 0) ewald_forces(reps[blockIdx.y], jobs[blockIdx.y].M);
+  if (reps[blockIdx.y].ewald_nk > 0) ewald_forces<NP>(reps[blockIdx.y], jobs[blockIdx.y].M);
+}
+
+// the particles that share a CTA, by the capacity in particles (the boxes here
+// hold a quarter of theirs): up to 32 per SM one (a box of 1,160 and 8,578 vectors: 24,
+// 29 and 32 us with one, two and four), up to 128 two (four boxes 75, 60 and 62
+// us), beyond four (eight 143, 114 and 102 us; 64 boxes 1121, 877 and 700 us)
+template <typename F>
+static void ewf_particles(int capacity, int n_rep, F launch) {
+  const long long n = (long long)capacity * n_rep, sms = device_sms();
+  if (n <= 32 * sms) launch(std::integral_constant<int, 1>{});
+  else if (n <= 128 * sms) launch(std::integral_constant<int, 2>{});
+  else launch(std::integral_constant<int, 4>{});
 }
 
 cudaError_t launch_step_advance(StepDyn *dyn, cudaStream_t s) {
@@ -1142,7 +1160,9 @@ cudaError_t launch_md_forces(const SysParams &P, const MdParams &M, int *plist, 
     else if (P.h == 1 && P.nc >= 3) k_md_forces<3, true><<<grid, MD_THREADS, 0, s>>>(P, Q);
     else k_md_forces<0, true><<<grid, MD_THREADS, 0, s>>>(P, Q);
     if (P.ewald_nk > 0)  // S(k) of these positions is current (launch_ewald_sk before this call)
-      k_ewald_forces<<<(unsigned)((max_particles + EWF_P - 1) / EWF_P), EWF_THREADS, 0, s>>>(P, Q);
+      ewf_particles(max_particles, 1, [&](auto np) {
+        k_ewald_forces<np.value><<<(unsigned)((max_particles + np.value - 1) / np.value), EWF_THREADS, 0, s>>>(P, Q);
+      });
     k_md_finish<<<(unsigned)((max_particles + 255) / 256), 256, 0, s>>>(P, Q);
   } else {
     if (P.h == 2 && P.nc >= 5) k_md_forces<5, false><<<grid, MD_THREADS, 0, s>>>(P, Q);
@@ -1158,16 +1178,19 @@ cudaError_t launch_md_forces_batch(const SysParams *d_reps, const MdJob *d_jobs,
   const cudaError_t e = cudaMemsetAsync(n_particles, 0, sizeof(int) * (size_t)n_rep, s);
   if (e != cudaSuccess) return e;
   k_plist_batch<<<dim3((unsigned)((S.cells + 255) / 256), (unsigned)n_rep), 256, 0, s>>>(d_reps, d_jobs);
-  // (eight times the CTAs that 152 SMs hold, over the replicas: the capacities allow for several times
+  // (eight times the CTAs that the SMs hold, over the replicas: the capacities allow for several times
   // the particles there are, and 64 replicas' empty CTAs cost more than the loop)
-  const unsigned share = (unsigned)std::max(8 * 8 * 152 / n_rep, 32);
+  const unsigned share = (unsigned)std::max(8 * 8 * device_sms() / n_rep, 32);
   const dim3 grid(std::min((unsigned)((S.particles + MD_NW - 1) / MD_NW), share), (unsigned)n_rep);
   if (S.variants & 1) k_md_forces_batch<5, true><<<grid, MD_THREADS, 0, s>>>(d_reps, d_jobs);
   if (S.variants & 2) k_md_forces_batch<5, false><<<grid, MD_THREADS, 0, s>>>(d_reps, d_jobs);
   if (S.variants & 4) k_md_forces_batch<3, false><<<grid, MD_THREADS, 0, s>>>(d_reps, d_jobs);
   if (S.variants & 8) k_md_forces_batch<0, false><<<grid, MD_THREADS, 0, s>>>(d_reps, d_jobs);
   if (S.ewald_particles > 0)
-    k_ewald_forces_batch<<<dim3((unsigned)((S.ewald_particles + EWF_P - 1) / EWF_P), (unsigned)n_rep), EWF_THREADS, 0, s>>>(d_reps, d_jobs);
+    ewf_particles(S.ewald_particles, n_rep, [&](auto np) {
+      k_ewald_forces_batch<np.value><<<dim3((unsigned)((S.ewald_particles + np.value - 1) / np.value), (unsigned)n_rep),
+                                       EWF_THREADS, 0, s>>>(d_reps, d_jobs);
+    });
   k_md_finish_batch<<<dim3((unsigned)((S.particles + 255) / 256), (unsigned)n_rep), 256, 0, s>>>(d_reps, d_jobs, C);
   return cudaGetLastError();
 }

@@ -1874,17 +1874,20 @@ __device__ __forceinline__ void phase_task(unsigned char *smem, const PhaseArgs 
 // seat runs the same code.
 //
 // What bounds it: one domain's chain of trials, each some 200 + instructions
-// that one warp fetches and runs once (4.0 of the 13.5 cycles between a warp's
-// instructions wait for instructions, 3.6 at barriers; issue active 24 %).
+// that one warp runs once while the others wait (of the 9.6 cycles between a
+// warp's instructions 2.8 are spent at barriers, 2.2 on fixed latencies, 0.9 on
+// global and 0.9 on shared loads, 0.5 on instruction fetch; issue active 34 %,
+// 12.5 warps per SM; 64 threads per domain and longer code in the trial loop:
+// 13.6 cycles, 3.8 at barriers, 3.2 on instruction fetch, 24 %).
 // With one CTA of 64 threads per domain the densest domain of a colour, coils
 // of a chain with 60 and more beads, lasted as long as two waves of the others.
 // Seats give it four times the threads and the shared memory of four, from the
-// same launch.  13 polyelectrolyte boxes (125 domains a colour each): a sweep
-// 1.03 ms with 64 threads per domain; 0.79 ms with 1/16 of the domains on 256
-// threads and the rest on seats of 64, of which 0.17 ms came from shorter code
-// in the trial loop (one path for the four move forms, loops not unrolled);
-// 64 ragged single chains 0.80 -> 0.55 ms.  A box alone (125 domains for 152
-// SMs) runs fastest with 256 threads for every domain.
+// same launch.  The same sweep of 13 polyelectrolyte boxes (125 domains a colour
+// each): 0.96 ms with 64 threads per domain, 0.82 ms with 1/16 of the domains on
+// 256 threads and the rest on seats of 64; 64 ragged single chains 0.76 ms with
+// 128 threads, 0.65 ms with two seats; one box of 1,000 domains a colour 0.61 and
+// 0.53 ms.  A box alone (125 domains for 152 SMs) runs fastest with 256 threads
+// for every domain.
 // ---------------------------------------------------------------------------
 template <bool LOG, bool DA, bool SEATS>
 __global__ void __launch_bounds__(512, 1)
@@ -2081,11 +2084,8 @@ static cudaError_t launch_sweep_t(const SysParams *d_reps, const PhaseShape &S, 
   cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cr_sweep<DA>, F.threads, smem);
   if (e != cudaSuccess) return e;
   per_sm = std::max(per_sm, 1);
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int total = Q.tasks_total;
-  int grid = std::min(total, per_sm * std::max(sms, 1));
+  int grid = std::min(total, per_sm * device_sms());
   if (max_ctas > 0) grid = std::min(grid, max_ctas);
   if (grid <= 0) return cudaSuccess;
   k_cr_sweep<DA><<<grid, F.threads, smem, s>>>(d_reps, A, sweep, sweep0, k0, k1, Q, dyn);
@@ -2181,9 +2181,9 @@ cudaError_t launch_domain_order(const SysParams *d_reps, int n_rep, int ncol, in
 // Ewald structure factor S(k) = sum_j q_j exp(i k.r_j) of every replica from
 // scratch (at every sweep): k_ewald_list lists each replica's occupied slots
 // (one CTA per replica, cells in order), k_ewald_sk gives each item (up to
-// eight reciprocal vectors) a thread, the particles in tiles of 32 whose axis
-// factors the CTA computes together in shared memory (FP32 products summed
-// per tile, tiles summed in FP64).
+// eight reciprocal vectors) or each vector a thread, the particles in tiles of
+// 32 whose axis factors the CTA computes together in shared memory (FP32
+// products summed per tile, tiles summed in FP64).
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_ewald_list(const SysParams *__restrict__ reps) {
   const SysParams &P = reps[blockIdx.x];
@@ -2220,44 +2220,47 @@ __global__ void __launch_bounds__(256) k_ewald_list(const SysParams *__restrict_
 
 constexpr int EW_TILE = 32;
 constexpr int EW_KMAX = 32;
-constexpr int EW_THREADS = 128;
 
-// FP32 pipes and shared-memory reads bound it: a thread per vector took three
-// factors from shared memory and two complex products for every particle, an
-// item's thread forms e_x e_y once for up to eight vectors and reads each e_z,
-// which is uniform over the warp, once for +nz and -nz (64 boxes of 1,150
-// particles, |n| <= 16, 8,578 vectors: 0.28 ms per 16 boxes before, 0.49 ms per
-// 64 now).  ZS: |nz| per thread, 4 (an item) or, where fewer than two CTAs of
-// items per SM exist (a single box has 10), 1.
-template <int ZS>
-__global__ void __launch_bounds__(EW_THREADS) k_ewald_sk(const SysParams *__restrict__ reps) {
+// FP32 pipes and shared-memory reads bound it where there are many boxes: a
+// thread per vector took three factors from shared memory and two complex
+// products for every particle, an item's thread forms e_x e_y once for up to
+// eight vectors and reads each e_z, which is uniform over the warp, once for +nz
+// and -nz (64 boxes of 1,150 particles, |n| <= 16, 8,578 vectors: 735 us with a
+// vector per thread, 451 us).  A few boxes do not fill the SMs with items (one has
+// 10 CTAs of them) and are bound by a thread's chain: there a thread takes one
+// vector, in the order of nz, ny, nx (consecutive lanes read consecutive factors),
+// and 256 threads share a tile's factors while such CTAs have an SM each, 512
+// beyond (one box 138 us with 256, 145 with 512, 276 by items, 198 with a thread
+// per column and |nz|; 8 boxes 163 and 154; 24 boxes 310 with 512, 344 by items;
+// 32 boxes 407 and 363).
+template <bool ITEMS, int THREADS>
+__global__ void __launch_bounds__(THREADS) k_ewald_sk(const SysParams *__restrict__ reps) {
+  constexpr int NV = ITEMS ? 8 : 1;  // vectors of a thread
   const SysParams &P = reps[blockIdx.y];
-  const int n_work = ZS == 4 ? P.ewald_items : P.ewald_plus;
-  if (P.ewald_nk <= 0 || (int)blockIdx.x * EW_THREADS >= n_work) return;  // uniform over the CTA
+  const int n_work = ITEMS ? P.ewald_items : P.ewald_vec;
+  if (P.ewald_nk <= 0 || (int)blockIdx.x * THREADS >= n_work) return;  // uniform over the CTA
   __shared__ float2 fac[EW_TILE][3][EW_KMAX + 4];
   __shared__ float qt[EW_TILE];
   __shared__ uint32_t ut[EW_TILE][3];
   const int ewk = P.ewald_kmax + 1, np = *P.ek_np;
-  const int i = (int)blockIdx.x * EW_THREADS + (int)threadIdx.x;
+  const int i = (int)blockIdx.x * THREADS + (int)threadIdx.x;
   const bool mine = i < n_work;
   int col = 0, z0 = 0, code = 0;
   if (mine) {
-    if (ZS == 4) {
+    if (ITEMS) {
       const int2 item = P.ek_item[i];
       code = item.x;
       col = item.y;
       z0 = item.x >> 16 << 2;
     } else {
-      while (z0 + 1 < ewk && P.ek_z[z0 + 1].y <= i) ++z0;
-      col = i - P.ek_z[z0].y;
-      code = P.ek_col[col];
+      code = P.ek_vec[i].x;
     }
   }
   int nx, ny, nz;
   ew_decode(code, nx, ny, nz);
-  double re[2 * ZS], im[2 * ZS];
+  double re[NV], im[NV];
 #pragma unroll
-  for (int k = 0; k < 2 * ZS; ++k) re[k] = im[k] = 0.0;
+  for (int k = 0; k < NV; ++k) re[k] = im[k] = 0.0;
   for (int t0 = 0; t0 < np; t0 += EW_TILE) {
     const int nt = min(EW_TILE, np - t0);
     if (threadIdx.x < 3 * nt) {  // the tile's coordinates as 0.32 fixed-point fractions of L
@@ -2267,31 +2270,37 @@ __global__ void __launch_bounds__(EW_THREADS) k_ewald_sk(const SysParams *__rest
       if (ax == 0) qt[p] = r.w;
     }
     __syncthreads();
-    for (int v = threadIdx.x; v < nt * 3 * ewk; v += EW_THREADS) {
+    for (int v = threadIdx.x; v < nt * 3 * ewk; v += THREADS) {
       const int p = v / (3 * ewk), ax = (v / ewk) % 3, n = v % ewk;
-      if (qt[p] != 0.0f) fac[p][ax][n] = ew_factor(ut[p][ax], n);
+      if (!ITEMS || qt[p] != 0.0f) fac[p][ax][n] = ew_factor(ut[p][ax], n);  // (few threads: the test costs more)
     }
     __syncthreads();
     if (mine) {
-      float tr[2 * ZS], ti[2 * ZS];
+      float tr[NV], ti[NV];
 #pragma unroll
-      for (int k = 0; k < 2 * ZS; ++k) tr[k] = ti[k] = 0.0f;
+      for (int k = 0; k < NV; ++k) tr[k] = ti[k] = 0.0f;
       for (int p = 0; p < nt; ++p) {
         const float q = qt[p];
         if (q == 0.0f) continue;
         const float2 xy = ew_xy(ew_axis(fac[p][0], nx), ew_axis(fac[p][1], ny));
+        if constexpr (ITEMS) {
 #pragma unroll
-        for (int k = 0; k < ZS; ++k) {  // (places beyond kmax hold no factor and are not stored)
-          const float2 ez = fac[p][2][z0 + k];
-          const float2 ep = cmul(xy, ez), em = cmul(xy, ew_conj(ez));
-          tr[2 * k] = __fmaf_rn(q, ep.x, tr[2 * k]);
-          ti[2 * k] = __fmaf_rn(q, ep.y, ti[2 * k]);
-          tr[2 * k + 1] = __fmaf_rn(q, em.x, tr[2 * k + 1]);
-          ti[2 * k + 1] = __fmaf_rn(q, em.y, ti[2 * k + 1]);
+          for (int k = 0; k < 4; ++k) {  // (places beyond kmax hold no factor and are not stored)
+            const float2 ez = fac[p][2][z0 + k];
+            const float2 ep = cmul(xy, ez), em = cmul(xy, ew_conj(ez));
+            tr[2 * k] = __fmaf_rn(q, ep.x, tr[2 * k]);
+            ti[2 * k] = __fmaf_rn(q, ep.y, ti[2 * k]);
+            tr[2 * k + 1] = __fmaf_rn(q, em.x, tr[2 * k + 1]);
+            ti[2 * k + 1] = __fmaf_rn(q, em.y, ti[2 * k + 1]);
+          }
+        } else {
+          const float2 e = cmul(xy, ew_axis(fac[p][2], nz));
+          tr[0] = __fmaf_rn(q, e.x, tr[0]);
+          ti[0] = __fmaf_rn(q, e.y, ti[0]);
         }
       }
 #pragma unroll
-      for (int k = 0; k < 2 * ZS; ++k) {
+      for (int k = 0; k < NV; ++k) {
         re[k] += (double)tr[k];
         im[k] += (double)ti[k];
       }
@@ -2299,25 +2308,39 @@ __global__ void __launch_bounds__(EW_THREADS) k_ewald_sk(const SysParams *__rest
     __syncthreads();
   }
   if (!mine) return;
+  // hi + lo at the vector's place (the trials), their FP32 sum in the order of
+  // the vectors (the forces)
+  auto store = [&](int place, int vec, double r, double m) {
+    const float2 hi = make_float2((float)r, (float)m);
+    const float2 lo = make_float2((float)(r - (double)hi.x), (float)(m - (double)hi.y));
+    P.ek_Shi[place] = hi;
+    P.ek_Slo[place] = lo;
+    if (vec >= 0) P.ek_Sf[vec] = make_float2(__fadd_rn(hi.x, lo.x), __fadd_rn(hi.y, lo.y));
+  };
+  if constexpr (ITEMS) {
 #pragma unroll
-  for (int k = 0; k < 2 * ZS; ++k) {
-    const int4 z = P.ek_z[z0 + k / 2];
-    if (col >= z.x || ((k & 1) && z0 + k / 2 == 0)) continue;
-    const int o = col + ((k & 1) ? z.z : z.y);
-    const float hr = (float)re[k], hm = (float)im[k];
-    P.ek_Shi[o] = make_float2(hr, hm);
-    P.ek_Slo[o] = make_float2((float)(re[k] - (double)hr), (float)(im[k] - (double)hm));
+    for (int k = 0; k < NV; ++k) {
+      const int4 z = P.ek_z[z0 + k / 2];
+      if (col >= z.x || ((k & 1) && z0 + k / 2 == 0)) continue;
+      const int o = col + ((k & 1) ? z.z : z.y);
+      store(o, P.ek_place[o], re[k], im[k]);
+    }
+  } else {
+    store(P.ek_vec[i].z, i, re[0], im[0]);
   }
 }
 
-cudaError_t launch_ewald_sk(const SysParams *d_reps, int n_rep, int max_items, int max_plus, cudaStream_t s) {
+cudaError_t launch_ewald_sk(const SysParams *d_reps, int n_rep, int max_items, int max_vec, cudaStream_t s) {
   if (n_rep <= 0 || max_items <= 0) return cudaSuccess;
   k_ewald_list<<<n_rep, 256, 0, s>>>(d_reps);
-  const unsigned g4 = (unsigned)((max_items + EW_THREADS - 1) / EW_THREADS);
-  if ((long long)g4 * n_rep >= 2 * 152)
-    k_ewald_sk<4><<<dim3(g4, (unsigned)n_rep), EW_THREADS, 0, s>>>(d_reps);
+  const unsigned R = (unsigned)n_rep;
+  auto grid = [&](int n, int threads) { return dim3((unsigned)((n + threads - 1) / threads), R); };
+  if ((long long)grid(max_items, 128).x * n_rep >= 2 * device_sms())
+    k_ewald_sk<true, 128><<<grid(max_items, 128), 128, 0, s>>>(d_reps);
+  else if ((long long)grid(max_vec, 256).x * n_rep > device_sms())
+    k_ewald_sk<false, 512><<<grid(max_vec, 512), 512, 0, s>>>(d_reps);
   else
-    k_ewald_sk<1><<<dim3((unsigned)((max_plus + EW_THREADS - 1) / EW_THREADS), (unsigned)n_rep), EW_THREADS, 0, s>>>(d_reps);
+    k_ewald_sk<false, 256><<<grid(max_vec, 256), 256, 0, s>>>(d_reps);
   return cudaGetLastError();
 }
 

@@ -106,15 +106,16 @@ def test_ewald_sums_keep_their_rounding(crmc):
     g.close()
 
 
-def test_many_ewald_boxes_equal_single_ones(crmc):
-    """64 boxes of 16 reciprocal vectors per axis go by items of a column, well past two CTAs of items per SM; a box
-    alone goes by slices."""
+@pytest.mark.parametrize("boxes", [2, 12, 64])
+def test_many_ewald_boxes_equal_single_ones(crmc, boxes):
+    """64 boxes of 16 reciprocal vectors per axis go by items of a column, well past two CTAs of items per SM; few
+    take a vector per thread, and their forces one, two or four particles per CTA."""
     make = lambda r: _electrolyte(20.0, 16, 10 + r, acids=12)
-    b = crmc.Batch([crmc.Context(make(r)) for r in range(64)])
+    b = crmc.Batch([crmc.Context(make(r)) for r in range(boxes)])
     b.md_begin(0.005, 1.0, 7)
     b.sweep(2, 50)
     b.md_end(0.005, 1.0, 7)
-    for r in (0, 31, 63):
+    for r in (0, boxes // 2, boxes - 1):
         g = crmc.Context(make(r))
         g.md_begin(0.005, 1.0, 7 ^ (r << 32))
         g.sweep(g.trials_per_sweep * 2, 50 ^ (r << 32))
