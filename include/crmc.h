@@ -584,9 +584,9 @@ int cr_batch_load(cr_batch *b, const cr_load_args *args);
  * r's entries starting at r * stride (stride >= the largest capacity; xyz and
  * vel hold 3 floats per entry).  cr_batch_state_packed fills the arrays that
  * are not NULL and n[r] (the particles of replica r, ordered by id as
- * cr_state; entries past n[r] in a replica's block are unspecified) with two
- * kernel launches, one copy per array and one synchronisation for the whole
- * batch (contexts above 16,384 particles of capacity take the per-context
+ * cr_state; entries past n[r] in a replica's block are unspecified) with three
+ * or four kernel launches, one copy per array and one synchronisation for the whole
+ * batch (replicas with more than 16,384 inserted ions take the per-context
  * path).  cr_batch_load_packed is cr_load of every replica from such arrays
  * (n[r] in; vel may be NULL), checked on the device like cr_load; its
  * per-particle errors come at the next synchronising call.  A load reads

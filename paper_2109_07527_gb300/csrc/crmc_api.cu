@@ -48,9 +48,10 @@ struct cr_ctx {
   long long *d_lnK = nullptr, *d_lntab = nullptr;
   long long *d_counts = nullptr, *d_kept = nullptr;  // (d_kept: kind counts and statistics of keep_state)
   int *d_perm = nullptr, *d_bond_off = nullptr, *d_bond_nbr = nullptr;
-  // d_counts holds N_KIND + 2 words: [0, N_KIND) kind counts, [N_KIND] ions found by cr_state
-  // (an int), [N_KIND + 1] the error word (an int), read back with one copy
-  int *d_err = nullptr, *d_counter = nullptr;
+  // d_counts holds N_KIND + 3 words: [0, N_KIND) kind counts, [N_KIND] ions found by cr_state
+  // (an int), [N_KIND + 1] the error word (an int), read back with one copy; [N_KIND + 2] the
+  // ions found by a batched read
+  int *d_err = nullptr, *d_counter = nullptr, *d_found = nullptr;
   cr_trial *d_log = nullptr;
   size_t log_cap = 0;
   // dense-domain scratch of the phase kernel and the MD particle list
@@ -733,7 +734,7 @@ extern "C" int cr_init(cr_ctx **out, const cr_system *sys, double pH, const doub
   ALLOC(c->d_stats, 16);
   ALLOC(c->d_lnK, std::max<size_t>(lnK.size(), 1));
   ALLOC(c->d_lntab, P.lnmax);
-  ALLOC(c->d_counts, N_KIND + 2);
+  ALLOC(c->d_counts, N_KIND + 3);
   ALLOC(c->d_kept, N_KIND + 16);
   ALLOC(c->d_perm, std::max(n, 1));
   ALLOC(c->d_bond_off, n + 1);
@@ -827,7 +828,8 @@ extern "C" int cr_init(cr_ctx **out, const cr_system *sys, double pH, const doub
   COPY(c->d_bond_nbr, nbr.data(), nbr.size());
   c->d_counter = (int *)(c->d_counts + N_KIND);
   c->d_err = (int *)(c->d_counts + N_KIND + 1);
-  cudaMemset(c->d_counts, 0, sizeof(long long) * (N_KIND + 2));
+  c->d_found = (int *)(c->d_counts + N_KIND + 2);
+  cudaMemset(c->d_counts, 0, sizeof(long long) * (N_KIND + 3));
   cudaMemset(c->d_present, 0, sizeof(int) * (size_t)std::max(n, 1));
   cudaMemset(c->d_chunk, 0, sizeof(int) * 2 * state_chunks(n));
   COPY(c->d_counts, kinds, (size_t)N_KIND);
@@ -1866,6 +1868,7 @@ struct cr_batch {
   int *d_pk_type = nullptr, *d_pk_cls = nullptr;
   int8_t *d_pk_state = nullptr;
   bool holds_refs = false;  // the contexts' batch_refs count this batch
+  bool few = false;         // the last packed read found at most 768 particles in every replica
   int ewald_items = 0, ewald_vec = 0;  // largest numbers of Ewald items and vectors over the replicas
   // batched MD steps: per-replica parameters on the device and the lengths of
   // the replicas' particle lists
@@ -2645,6 +2648,7 @@ extern "C" int cr_batch_state_packed(cr_batch *b, cr_batch_packed *p) {
     B.chunk = c->d_chunk;
     B.chunk_base = c->d_chunk + state_chunks(c->n_input);
     B.n_ions = c->d_counter;
+    B.n_found = c->d_found;
     B.ion_key = c->d_ion_key;
     B.ion_val = c->d_ion_val;
     B.ion_rank = c->d_ion_rank;
@@ -2660,8 +2664,9 @@ extern "C" int cr_batch_state_packed(cr_batch *b, cr_batch_packed *p) {
     B.state = p->state ? (zs ? zs : b->d_pk_state) + r * S : nullptr;
   }
   CR_CUDA(cudaMemcpyAsync(b->d_sbufs, b->h_sbufs, R * sizeof(StateBufs), cudaMemcpyHostToDevice, s));
-  CR_CUDA(launch_state_batch(b->d_reps, b->d_sbufs, (int)R, max_cells, max_input, (int)capmax, b->d_nout, b->d_errout, s));
-  b->ctx[0]->launches_total += 5;
+  CR_CUDA(launch_state_batch(b->d_reps, b->d_sbufs, (int)R, max_cells, max_input, (int)capmax, b->few, b->d_nout,
+                             b->d_errout, s));
+  b->ctx[0]->launches_total += b->few ? 3 : 4;
   CR_CUDA(cudaMemcpyAsync(b->h_nout, b->d_nout, R * sizeof(long long), cudaMemcpyDeviceToHost, s));
   int *herr = (int *)(b->h_nout + R);
   CR_CUDA(cudaMemcpyAsync(herr, b->d_errout, R * sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -2673,6 +2678,10 @@ extern "C" int cr_batch_state_packed(cr_batch *b, cr_batch_packed *p) {
   if (p->cls && !zc) CR_CUDA(cudaMemcpyAsync(p->cls, b->d_pk_cls, m * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
   if (p->state && !zs) CR_CUDA(cudaMemcpyAsync(p->state, b->d_pk_state, m, cudaMemcpyDeviceToHost, s));
   CR_CUDA(cudaStreamSynchronize(s));
+  const bool was_few = b->few;
+  const auto n_range = std::minmax_element(b->h_nout, b->h_nout + R);
+  b->few = *n_range.first >= 0 && *n_range.second <= 768;
+  if (was_few && *n_range.first < 0) return cr_batch_state_packed(b, p);  // more than a tile after all: with the ranks
   rc = CR_OK;
   for (size_t r = 0; r < R; ++r) {
     p->n[r] = b->h_nout[r];

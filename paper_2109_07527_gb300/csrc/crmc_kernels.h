@@ -80,7 +80,7 @@ struct StateBufs {
   int lo_bits;                    // the low words of ion ids stay below 2^lo_bits
   int *present;                   // [n_input] slot + 1 of each input id, 0 absent
   int *chunk, *chunk_base;        // present ids of each chunk of STATE_CHUNK, and before it
-  int *n_ions;                    // number of inserted ions found
+  int *n_ions, *n_found;          // number of inserted ions found; a copy for the batched kernels
   unsigned long long *ion_key, *ion_key_alt;  // [cap] ion sort keys (the alternates for the device-wide sort)
   int *ion_val, *ion_val_alt;                 // [cap] their slots
   int *ion_rank;                              // [cap] slot of each rank among the ion ids
@@ -208,11 +208,13 @@ cudaError_t launch_state_mark(const SysParams &P, const StateBufs &B, cudaStream
 cudaError_t launch_state_order(const SysParams &P, const StateBufs &B, int n_present, int n_ions, int end_bit,
                                cudaStream_t s, int *launches);
 size_t state_sort_temp_bytes(int cap);
-// every replica of a batch in five launches (marks, ranks, ordering), the counts read
+// every replica of a batch in four launches (marks, sort, ranks, ordering), the counts read
 // on the device; n_out[r] = particles of replica r, -1 when its read needs the
-// per-context path; err_out[r] its error word
+// per-context path; err_out[r] its error word.  one_tile: no ranks, for replicas
+// that are expected to hold few ions (a launch less; one with more gets -1)
 cudaError_t launch_state_batch(const SysParams *d_reps, const StateBufs *d_bufs, int n_rep, int max_cells,
-                               int max_input, int max_cap, long long *d_n_out, int *d_err_out, cudaStream_t s);
+                               int max_input, int max_cap, bool one_tile, long long *d_n_out, int *d_err_out,
+                               cudaStream_t s);
 // Ewald: S(k) of every replica of a batch from scratch (the occupied slots
 // listed, then one thread per item of reciprocal vectors, or per vector where
 // there are few); max_items, max_vec: the largest ewald_items and ewald_vec

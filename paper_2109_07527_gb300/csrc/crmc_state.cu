@@ -84,9 +84,10 @@ __global__ void __launch_bounds__(256) k_state_mark(SysParams P, StateBufs B) {
 }
 
 // Tile blockIdx.x of the n ion keys sorted in place with its slots (a bitonic
-// network in shared memory; the last tile is padded with the largest key), by
-// one CTA; the CTA past the last tile turns the chunks' counts into their
-// exclusive prefix sums (chunk_base) and clears them.
+// network in shared memory over the next power of two, padded with the largest
+// key: a few ions take 15 of its 55 steps), by one CTA; the CTA past the last
+// tile turns the chunks' counts into their exclusive prefix sums (chunk_base)
+// and clears them.
 __device__ __forceinline__ void sort_tile(const StateBufs &B, int n) {
   __shared__ unsigned long long ks[RANK_TILE];
   __shared__ int vs[RANK_TILE];
@@ -118,7 +119,8 @@ __device__ __forceinline__ void sort_tile(const StateBufs &B, int n) {
   if ((int)blockIdx.x * RANK_TILE >= n) return;  // the whole CTA
   ks[t] = i < n ? B.ion_key[i] : ~0ull;
   vs[t] = i < n ? B.ion_val[i] : 0;
-  for (int size = 2; size <= RANK_TILE; size <<= 1)
+  const int m = min(n - (int)blockIdx.x * RANK_TILE, RANK_TILE);  // the tile's keys
+  for (int size = 2; size < 2 * m; size <<= 1)
     for (int stride = size >> 1; stride > 0; stride >>= 1) {
       __syncthreads();
       const int p = t ^ stride;
@@ -164,13 +166,17 @@ __device__ __forceinline__ void rank_tile(const StateBufs &B, int n) {
 
 __global__ void __launch_bounds__(RANK_TILE) k_ion_sort(StateBufs B, int n) { sort_tile(B, n); }
 __global__ void __launch_bounds__(RANK_TILE) k_ion_rank(StateBufs B, int n) { rank_tile(B, n); }
+// (in a batch the counter is read from the copy that the sort leaves, so that
+// the ordering kernel can clear it for the next read)
 __global__ void __launch_bounds__(RANK_TILE) k_ion_sort_batch(const StateBufs *__restrict__ bufs) {
   const StateBufs &B = bufs[blockIdx.y];
-  sort_tile(B, min(*B.n_ions, min(B.cap, STATE_BLOCK_SORT_MAX)));
+  const int n_ions = *B.n_ions;
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *B.n_found = n_ions;
+  sort_tile(B, min(n_ions, min(B.cap, STATE_BLOCK_SORT_MAX)));
 }
 __global__ void __launch_bounds__(RANK_TILE) k_ion_rank_batch(const StateBufs *__restrict__ bufs) {
   const StateBufs &B = bufs[blockIdx.y];
-  rank_tile(B, min(*B.n_ions, min(B.cap, STATE_BLOCK_SORT_MAX)));
+  rank_tile(B, min(*B.n_found, min(B.cap, STATE_BLOCK_SORT_MAX)));
 }
 
 __device__ __forceinline__ void emit(const SysParams &P, const StateBufs &B, int g, int o) {
@@ -246,8 +252,8 @@ __global__ void __launch_bounds__(ORDER_THREADS) k_state_order(SysParams P, Stat
 // device: n from the kind counts, n_ions from the mark kernel.  A replica
 // whose ions exceed the tile ranking (or whose counts are inconsistent) gets
 // n_out = -1 and only its marks cleared.  n_out and err_out receive each
-// replica's particle count and error word; k_state_done clears the ion
-// counters, which every CTA here reads.
+// replica's particle count and error word.  one_tile: no ranks were formed, and
+// a replica of more ions than a tile, whose order is the ranks', is one of those.
 __global__ void __launch_bounds__(256) k_state_mark_batch(const SysParams *__restrict__ reps,
                                                           const StateBufs *__restrict__ bufs) {
   mark_cells(reps[blockIdx.y], bufs[blockIdx.y], blockIdx.x * blockDim.x + threadIdx.x);
@@ -255,32 +261,28 @@ __global__ void __launch_bounds__(256) k_state_mark_batch(const SysParams *__res
 
 __global__ void __launch_bounds__(ORDER_THREADS) k_state_order_batch(const SysParams *__restrict__ reps,
                                                                      const StateBufs *__restrict__ bufs,
-                                                                     int input_chunks, long long *n_out,
-                                                                     int *err_out) {
+                                                                     int input_chunks, int one_tile,
+                                                                     long long *n_out, int *err_out) {
   const int r = blockIdx.y;
   const SysParams &P = reps[r];
   const StateBufs &B = bufs[r];
   const long long *cn = B.counts;
   const long long n = cn[K_A0] + cn[K_A1] + cn[K_B0] + cn[K_B1] + cn[K_XP] + cn[K_XM] + cn[K_SP] + cn[K_SM] + B.n_other;
-  const int n_ions = *B.n_ions;
+  const int n_ions = *B.n_found;
   const long long n_present = n - n_ions;
-  const bool ok = n_ions >= 0 && n_ions <= STATE_BLOCK_SORT_MAX && n <= B.cap && n_present >= 0 &&
+  const bool ok = n_ions >= 0 && n_ions <= (one_tile ? RANK_TILE : STATE_BLOCK_SORT_MAX) && n <= B.cap && n_present >= 0 &&
                   n_present <= B.n_input && *P.err == 0;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     n_out[r] = ok ? n : -1;
     err_out[r] = *P.err;
+    *B.n_ions = 0;
   }
   if (ok) {
-    order_cta(P, B, input_chunks, (int)n_present, n_ions, B.ion_rank);
+    order_cta(P, B, input_chunks, (int)n_present, n_ions, n_ions <= RANK_TILE ? B.ion_val : B.ion_rank);
   } else {
     const int i = blockIdx.x * ORDER_THREADS + threadIdx.x;
     if ((int)blockIdx.x < input_chunks && i < B.n_input) B.present[i] = 0;
   }
-}
-
-__global__ void k_state_done(const StateBufs *__restrict__ bufs, int n) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r < n) *bufs[r].n_ions = 0;
 }
 
 }  // namespace
@@ -334,16 +336,17 @@ cudaError_t launch_state_order(const SysParams &P, const StateBufs &B, int n_pre
 }
 
 cudaError_t launch_state_batch(const SysParams *d_reps, const StateBufs *d_bufs, int n_rep, int max_cells,
-                               int max_input, int max_cap, long long *d_n_out, int *d_err_out, cudaStream_t s) {
+                               int max_input, int max_cap, bool one_tile, long long *d_n_out, int *d_err_out,
+                               cudaStream_t s) {
   const unsigned R = (unsigned)n_rep;
   if (max_cells > 0) k_state_mark_batch<<<dim3((max_cells + 255) / 256, R), 256, 0, s>>>(d_reps, d_bufs);
   const unsigned nt = (unsigned)((std::min(max_cap, STATE_BLOCK_SORT_MAX) + RANK_TILE - 1) / RANK_TILE);
   k_ion_sort_batch<<<dim3(nt + 1, R), RANK_TILE, 0, s>>>(d_bufs);
-  if (nt > 0) k_ion_rank_batch<<<dim3(nt, R), RANK_TILE, 0, s>>>(d_bufs);
+  if (nt > 1 && !one_tile) k_ion_rank_batch<<<dim3(nt, R), RANK_TILE, 0, s>>>(d_bufs);
   const int ic = (max_input + ORDER_THREADS - 1) / ORDER_THREADS;
   const int gx = std::max(ic + (int)nt, 1);
-  k_state_order_batch<<<dim3((unsigned)gx, R), ORDER_THREADS, 0, s>>>(d_reps, d_bufs, ic, d_n_out, d_err_out);
-  k_state_done<<<(R + 127) / 128, 128, 0, s>>>(d_bufs, n_rep);
+  k_state_order_batch<<<dim3((unsigned)gx, R), ORDER_THREADS, 0, s>>>(d_reps, d_bufs, ic, one_tile ? 1 : 0, d_n_out,
+                                                                              d_err_out);
   return cudaGetLastError();
 }
 
