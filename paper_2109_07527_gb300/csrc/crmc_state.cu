@@ -83,11 +83,11 @@ __global__ void __launch_bounds__(256) k_state_mark(SysParams P, StateBufs B) {
   mark_cells(P, B, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
-// Tile blockIdx.x of the n ion keys sorted in place with its slots (a bitonic
-// network in shared memory over the next power of two, padded with the largest
-// key: a few ions take 15 of its 55 steps), by one CTA; the CTA past the last
-// tile turns the chunks' counts into their exclusive prefix sums (chunk_base)
-// and clears them.
+// Tile blockIdx.x of the n ion keys sorted in place with its slots by one CTA: a
+// bitonic network over the next power of two, padded with the largest key, a
+// key per thread (of its 55 steps over 1024 keys the 15 between warps go through
+// shared memory, the others are shuffles).  The CTA past the last tile turns the
+// chunks' counts into their exclusive prefix sums (chunk_base) and clears them.
 __device__ __forceinline__ void sort_tile(const StateBufs &B, int n) {
   __shared__ unsigned long long ks[RANK_TILE];
   __shared__ int vs[RANK_TILE];
@@ -117,28 +117,32 @@ __device__ __forceinline__ void sort_tile(const StateBufs &B, int n) {
   }
   const int i = blockIdx.x * RANK_TILE + t;
   if ((int)blockIdx.x * RANK_TILE >= n) return;  // the whole CTA
-  ks[t] = i < n ? B.ion_key[i] : ~0ull;
-  vs[t] = i < n ? B.ion_val[i] : 0;
+  unsigned long long k = i < n ? B.ion_key[i] : ~0ull;
+  int v = i < n ? B.ion_val[i] : 0;
   const int m = min(n - (int)blockIdx.x * RANK_TILE, RANK_TILE);  // the tile's keys
   for (int size = 2; size < 2 * m; size <<= 1)
     for (int stride = size >> 1; stride > 0; stride >>= 1) {
-      __syncthreads();
-      const int p = t ^ stride;
-      if (p > t) {
-        const unsigned long long a = ks[t], b = ks[p];
-        if ((a > b) == ((t & size) == 0)) {
-          ks[t] = b;
-          ks[p] = a;
-          const int v = vs[t];
-          vs[t] = vs[p];
-          vs[p] = v;
-        }
+      unsigned long long k2;
+      int v2;
+      if (stride >= 32) {
+        __syncthreads();
+        ks[t] = k;
+        vs[t] = v;
+        __syncthreads();
+        k2 = ks[t ^ stride];
+        v2 = vs[t ^ stride];
+      } else {
+        k2 = __shfl_xor_sync(0xffffffffu, k, stride);
+        v2 = __shfl_xor_sync(0xffffffffu, v, stride);
+      }
+      if (((t & stride) == 0) == ((t & size) == 0) ? k2 < k : k2 > k) {
+        k = k2;
+        v = v2;
       }
     }
-  __syncthreads();
   if (i < n) {
-    B.ion_key[i] = ks[t];
-    B.ion_val[i] = vs[t];
+    B.ion_key[i] = k;
+    B.ion_val[i] = v;
   }
 }
 
