@@ -1,5 +1,5 @@
 // crmc_common.h -- data layout and kernel parameter records shared by the
-// host side (crmc_api.cu) and the kernels (crmc_kernels.cu) of libcrmc.so.
+// host side (crmc_api.cu) and the kernels of libcrmc.so.
 //
 // Device layout of one system (cell-major, "slots"):
 //   cnt[ncell]                 used slots of each cell (particles sorted by id)

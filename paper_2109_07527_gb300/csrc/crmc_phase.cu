@@ -1,7 +1,7 @@
 // crmc_phase.cu -- the colour-phase kernel of the CR-MC stage (sm_103a).
 //
-// k_cr_phase: one CTA per active domain of one colour of the 8-colour
-// checkerboard, for one or several replicas (blockIdx.x) in one launch; the
+// k_cr_phase: one CTA, or a seat of one, per active domain of one colour of the
+// 8-colour checkerboard, for one or several replicas (blockIdx.x) in one launch; the
 // domains of a colour are launched densest first (blockIdx.y is the rank in
 // the order k_domain_cost and k_domain_rank compute at the start of every sweep), so that the
 // long CTAs do not form the tail of the launch.

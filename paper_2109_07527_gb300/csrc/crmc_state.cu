@@ -12,7 +12,7 @@
 //
 // 13 polyelectrolyte boxes (11,000 inserted ions each) into device arrays:
 // 377 us with a thread per slot (76), ranks by counting all pairs of keys (251)
-// and two CTAs writing (49); now 72 us (14, 41 and 14).  A box of 87,000
+// and two CTAs writing (49); now 66 us (16, 21 + 17 and 13).  A box of 87,000
 // particles: the marks 38 -> 18 and the writing 202 -> 8 us.
 #include <cuda_runtime.h>
 
